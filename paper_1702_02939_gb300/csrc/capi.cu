@@ -527,9 +527,9 @@ void enqueue_step_suffix(cg_ctx* c, cudaStream_t st) {
   g.list = c->at<int>(c->off.dirty_list);
   g.list_count = &c->ctl()->dirty_count;
   g.list_bits = c->at<unsigned>(c->off.dirty_bits);
-  // one warp per rewritten ring (about 1% of the cells per step): every cell
-  // of the list at once rather than a few per warp one after another
-  run_geom(c, g, st, sm_count() * 16);
+  // two blocks per SM take up to 9728 listed cells at once (usually well
+  // below 1% of the cells are rewritten in a step)
+  run_geom(c, g, st, sm_count() * 2);
   if (c->launch.dir_beside_geom) cudaStreamWaitEvent(st, c->join_terms, 0);
   if (c->launch.ring_order) {
     // the ring-size grouping of the next step, from the rings this step

@@ -12,6 +12,10 @@ struct Ctl;
 constexpr int kGeomThreads = 32;   // one warp: finer blocks than 64 cut k_geom by ~4% at N = 262144
 constexpr int kGeomSh = 10;        // ring slots of k_geom held in shared memory (longer rings: local)
 constexpr int kGeomMinBlocks = 20;  // resident one-warp blocks per SM that k_geom is compiled for
+constexpr int kSlotWarps = 8;       // warps of a block that takes 32 cells, one warp per ring slot
+constexpr int kSlotThreads = 32 * kSlotWarps;
+constexpr int kGeomSlotBlocks = 6;      // resident blocks per SM that k_geom_slots is compiled for
+constexpr int kGeomSlotCells = 155648;  // up to here (1024 cells per SM) k_geom_slots takes all cells
 constexpr int kForceThreads = 128;
 constexpr int kTestThreads = 128;
 constexpr int kRepairWarps = 4;  // warps per repair block
@@ -29,7 +33,8 @@ struct GeomArgs {
   double *A, *P;
   double* energy_out;   // per-cell energy or nullptr
   double2 *fs, *s, *w;  // [CG_RING][n]
-  // Cells to process: list[0 .. *list_count) if list is set, else all.
+  // Cells to process: list[0 .. *list_count) if list is set, else all
+  // (k_geom takes no list: k_geom_slots does).
   const int* list;
   const int* list_count;
   unsigned* list_bits;  // bit of each listed cell, cleared once processed

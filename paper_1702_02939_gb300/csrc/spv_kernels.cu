@@ -20,6 +20,48 @@
 
 namespace cgk {
 
+// The doubled circumcentre h of the triangle (0, a, b), a and b in grid units,
+// and its Jacobian factor s = h / det.  Squared lengths and the determinant
+// exactly in 128-bit integers from the grid offsets; the numerators
+// (b_y |a|^2 - a_y |b|^2, a_x |b|^2 - b_x |a|^2) in 128-bit integers too, from
+// |a|^2 and |b|^2 cut to 62 significant bits by a shift common to the triangle
+// (at least as accurate as FP64 products of the rounded squares), each rounded
+// to double once.
+__device__ __forceinline__ void geom_vertex(long long AX, long long AY, long long BX, long long BY, double2& h,
+                                            double2& s) {
+  const unsigned __int128 LA = (unsigned __int128)((__int128)AX * AX + (__int128)AY * AY);
+  const unsigned __int128 LB = (unsigned __int128)((__int128)BX * BX + (__int128)BY * BY);
+  const double det = i128_to_double((__int128)AX * BY - (__int128)AY * BX);
+  const double r = fx_rcp(det);
+  const int S = max(u128_bits(LA > LB ? LA : LB) - 62, 0);
+  const long long la = (long long)(LA >> S), lb = (long long)(LB >> S);
+  h.x = i128_to_double((__int128)BY * la - (__int128)AY * lb, S) * r;
+  h.y = i128_to_double((__int128)AX * lb - (__int128)BX * la, S) * r;
+  s = make_double2(h.x * r, h.y * r);
+}
+
+// The edge from vertex hp to h: (squared length, inverse length) and its unit
+// vector; a zero-length edge has no direction.
+__device__ __forceinline__ void geom_edge(double2 h, double2 hp, double2& l, double2& e) {
+  const double ex = h.x - hp.x, ey = h.y - hp.y;
+  const double l2 = fma(ex, ex, ey * ey);
+  const double il = (__double_as_longlong(l2) > 0) ? fx_rsqrt(l2) : 0.0;
+  l = make_double2(l2, il);
+  e = make_double2(ex * il, ey * il);
+}
+
+// A, P and the energy of cell i from its accumulated sums; returns (ka, kp).
+__device__ __forceinline__ double2 geom_cell(const GeomArgs& g, int i, double sc, double area, double per) {
+  const double A = 0.125 * area * sc * sc, P = 0.5 * per * sc;
+  g.A[i] = A;
+  g.P[i] = P;
+  const double dA = A - g.A0, dP = fma(-g.p0[i], g.sqrtA0, P);
+  if (g.energy_out) g.energy_out[i] = fma(g.KA * dA, dA, g.KP * dP * dP);
+  // dA/dh = 1/2 perp(h_next - h_prev) (the 1/2, the doubling of g and the
+  // grid scale fold into ka); dP/dh = e_in - e_out (unit edge vectors)
+  return make_double2(g.KA * dA * (0.5 * sc), 2.0 * g.KP * dP);
+}
+
 // One thread per cell.  Writes A, P, force sets fs[a][i] = dE_i/dh_a, and the
 // per-slot Jacobian factor s[a][i] = 2 u_a / det_a (the other factor, w_a / 2,
 // is rebuilt exactly from the integer positions by k_force).
@@ -56,10 +98,8 @@ __global__ void __launch_bounds__(kGeomThreads, kGeomMinBlocks) k_geom(GeomArgs 
   const int cur = g.ctl->cur;
   const long long* __restrict__ X = g.X + (size_t)cur * N;
   const long long* __restrict__ Y = g.Y + (size_t)cur * N;
-  const int total = g.list ? *g.list_count : g.n;
-  for (int item = blockIdx.x * kGeomThreads + t; item < total; item += gridDim.x * kGeomThreads) {
-    const int i = g.list ? g.list[item] : (g.order ? g.order[item] : item);
-    if (g.list_bits) atomicAnd(&g.list_bits[i >> 5], ~(1u << (i & 31)));
+  for (int item = blockIdx.x * kGeomThreads + t; item < g.n; item += gridDim.x * kGeomThreads) {
+    const int i = g.order ? g.order[item] : item;
     const Rep R = g.reps[g.rep[i]];
     const long long Xi = X[i], Yi = Y[i];
     const int m = g.cnt[i];
@@ -115,9 +155,9 @@ __global__ void __launch_bounds__(kGeomThreads, kGeomMinBlocks) k_geom(GeomArgs 
       } else {
         area = fma(-hx, hpy, fma(hpx, hy, area));  // shoelace term, two FMAs
         const double ex = hx - hpx, ey = hy - hpy;
-        const double l2 = ex * ex + ey * ey;
+        const double l2 = fma(ex, ex, ey * ey);
         const double il = (__double_as_longlong(l2) > 0) ? fx_rsqrt(l2) : 0.0;  // zero-length edge: no direction
-        per += l2 * il;
+        per = fma(l2, il, per);
         put(sh_ex, lo_ex, a, ex * il);
         put(sh_ey, lo_ey, a, ey * il);
       }
@@ -128,21 +168,14 @@ __global__ void __launch_bounds__(kGeomThreads, kGeomMinBlocks) k_geom(GeomArgs 
     {  // closing edge h_{m-1} -> h_0 is the incoming edge of vertex 0
       area = fma(-h0x, hpy, fma(hpx, h0y, area));
       const double ex = h0x - hpx, ey = h0y - hpy;
-      const double l2 = ex * ex + ey * ey;
+      const double l2 = fma(ex, ex, ey * ey);
       const double il = (__double_as_longlong(l2) > 0) ? fx_rsqrt(l2) : 0.0;  // zero-length edge: no direction
-      per += l2 * il;
+      per = fma(l2, il, per);
       sh_ex[0][t] = ex * il;
       sh_ey[0][t] = ey * il;
     }
-    const double sc = R.inv_scale;
-    const double A = 0.125 * area * sc * sc, P = 0.5 * per * sc;
-    g.A[i] = A;
-    g.P[i] = P;
-    const double dA = A - g.A0, dP = P - g.p0[i] * g.sqrtA0;
-    if (g.energy_out) g.energy_out[i] = g.KA * dA * dA + g.KP * dP * dP;
-    // dA/dh = 1/2 perp(h_next - h_prev) (the 1/2, the doubling of g and the
-    // grid scale fold into ka); dP/dh = e_in - e_out (unit edge vectors)
-    const double ka = g.KA * dA * (0.5 * sc), kp = 2.0 * g.KP * dP;
+    const double2 k = geom_cell(g, i, R.inv_scale, area, per);
+    const double ka = k.x, kp = k.y;
     for (int a = 0; a < m; ++a) {
       const int ap = (a == 0) ? m - 1 : a - 1;
       const int an = (a + 1 == m) ? 0 : a + 1;
@@ -152,6 +185,96 @@ __global__ void __launch_bounds__(kGeomThreads, kGeomMinBlocks) k_geom(GeomArgs 
       const double dPy = get(sh_ey, lo_ey, a) - get(sh_ey, lo_ey, an);
       g.fs[a * N + i] = make_double2(fma(ka, gx, kp * dPx), fma(ka, gy, kp * dPy));
     }
+  }
+}
+
+// The same pass with one thread per (cell, ring slot): a block takes 32 cells,
+// its warp w the slots w, w + 8 of all of them (lane = cell, so every access
+// is laid out as in k_geom).  The neighbours' offsets, the circumcentres and
+// the edges pass between slots through shared memory; the last warp, whose own
+// slots are rare, adds the area up while the others form the edges, and the
+// first adds up the perimeter and forms the cell's coefficients.  Every
+// operation and its order is k_geom's, so the results are bit-identical.
+__global__ void __launch_bounds__(kSlotThreads, kGeomSlotBlocks) k_geom_slots(GeomArgs g) {
+  __shared__ longlong2 s_off[CG_RING][32];  // neighbour offsets, then (as double2) unit edge vectors
+  __shared__ double2 s_h[CG_RING][32];      // doubled circumcentres
+  __shared__ double2 s_l[CG_RING][32];      // edge ending at the slot: squared length, inverse length
+  __shared__ double2 s_k[32];               // the cell's ka, kp
+  __shared__ double s_area[32];
+  double2(*s_e)[32] = reinterpret_cast<double2(*)[32]>(s_off);
+  const int c = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const size_t N = (size_t)g.n;
+  const int cur = g.ctl->cur;
+  const long long* __restrict__ X = g.X + (size_t)cur * N;
+  const long long* __restrict__ Y = g.Y + (size_t)cur * N;
+  const int total = g.list ? *g.list_count : g.n;
+  for (int base = blockIdx.x * 32; base < total; base += gridDim.x * 32) {
+    const int item = base + c;
+    int i = 0, m = 0;
+    if (item < total) {
+      i = g.list ? g.list[item] : (g.order ? g.order[item] : item);
+      m = g.cnt[i];
+      if (w == 0) {
+        if (g.list_bits) atomicAnd(&g.list_bits[i >> 5], ~(1u << (i & 31)));
+        if ((m < 3 || m > CG_RING) && !g.tolerant) raise_status(g.ctl, kETOPO);
+      }
+      if (m < 3 || m > CG_RING) m = 0;
+    }
+    const Rep& R = g.reps[g.rep[i]];
+    const int* ring = g.nbr + (size_t)i * CG_RING;
+    if (w < m) {
+      const long long Xi = X[i], Yi = Y[i], LX = R.LX, LY = R.LY;
+      for (int a = w; a < m; a += kSlotWarps) {
+        // a ring being rewritten concurrently may hold -1 entries: the cell
+        // itself is read there (the result is discarded and computed again)
+        int j = ring[a];
+        j = ((unsigned)j < (unsigned)g.n) ? j : i;
+        s_off[a][c] = make_longlong2(min_image_i(X[j] - Xi, LX), min_image_i(Y[j] - Yi, LY));
+      }
+    }
+    __syncthreads();
+    for (int a = w; a < m; a += kSlotWarps) {
+      const longlong2 A = s_off[a][c], B = s_off[a + 1 < m ? a + 1 : 0][c];
+      double2 h, sj;
+      geom_vertex(A.x, A.y, B.x, B.y, h, sj);
+      g.s[a * N + i] = sj;
+      s_h[a][c] = h;
+    }
+    __syncthreads();
+    if (w == kSlotWarps - 1) {
+      double area = 0.0;
+      for (int a = 1; a <= m; ++a) {
+        const double2 hp = s_h[a - 1][c], h = s_h[a < m ? a : 0][c];
+        area = fma(-h.x, hp.y, fma(hp.x, h.y, area));
+      }
+      s_area[c] = area;
+    }
+    for (int a = w; a < m; a += kSlotWarps) {
+      const double2 h = s_h[a][c], hp = s_h[a > 0 ? a - 1 : m - 1][c];
+      double2 l, e;
+      geom_edge(h, hp, l, e);
+      s_l[a][c] = l;
+      s_e[a][c] = e;
+    }
+    __syncthreads();
+    if (w == 0 && m) {
+      double per = 0.0;
+      for (int a = 1; a <= m; ++a) {
+        const double2 l = s_l[a < m ? a : 0][c];
+        per = fma(l.x, l.y, per);
+      }
+      s_k[c] = geom_cell(g, i, R.inv_scale, s_area[c], per);
+    }
+    __syncthreads();
+    const double2 k = s_k[c];
+    for (int a = w; a < m; a += kSlotWarps) {
+      const int ap = a > 0 ? a - 1 : m - 1, an = a + 1 < m ? a + 1 : 0;
+      const double2 hp = s_h[ap][c], hn = s_h[an][c], e = s_e[a][c], en = s_e[an][c];
+      const double gx = hn.y - hp.y, gy = hp.x - hn.x;
+      const double dPx = e.x - en.x, dPy = e.y - en.y;
+      g.fs[a * N + i] = make_double2(fma(k.x, gx, k.y * dPx), fma(k.x, gy, k.y * dPy));
+    }
+    __syncthreads();
   }
 }
 
@@ -523,6 +646,18 @@ void launch_order(int n, const int* cnt, int* order, cudaStream_t st) {
 }
 void launch_geom(const GeomArgs& a, cudaStream_t st, int blocks) {
   if (a.n <= 0) return;
+  // A block per 32 cells and a warp per ring slot shortens the chain that one
+  // thread walks by the number of slots: it is faster while the chip is not
+  // full (one pass, us, one thread per cell -> slots: 22.5 -> 10.2 at 256
+  // cells, 26.6 -> 12.3 at 4096, 26.6 -> 16.8 at 16384, 36.9 -> 34.4 at 65536,
+  // 62.7 -> 57.1 at 131072).  Beyond, both fill the FP64 pipe and the warps of
+  // the last slots idle (102 -> 102 at 262144, 337 -> 379 at 10^6).  A list
+  // (the cells whose rings a step rewrote) is short.
+  if (a.list || a.n <= kGeomSlotCells) {
+    const int full = (a.n + 31) / 32;
+    k_geom_slots<<<(blocks > 0 && blocks < full) ? blocks : full, kSlotThreads, 0, st>>>(a);
+    return;
+  }
   const int full = (a.n + kGeomThreads - 1) / kGeomThreads;
   k_geom<<<(blocks > 0 && blocks < full) ? blocks : full, kGeomThreads, 0, st>>>(a);
 }

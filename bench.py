@@ -211,13 +211,13 @@ class ClockSampler:
 
 
 def kernels_launched(steps, loop_iterations, eager=False, ring_order=1, force_beside=0):
-    # per step: begin-topology, test, 4 cell-list kernels, directors, the
+    # per step: begin-topology, test, the cell list, directors, the
     # ring-size grouping (if on), geometry of the new state, force + move;
     # graph only: the geometry fix-up of rewritten rings and, with the force
     # pass beside the rounds, the fix-up list and the force fix-up; per
     # repair round: repair + check
     graph_extra = 0 if eager else 1 + (2 if force_beside else 0)
-    return (9 + (1 if ring_order else 0) + graph_extra) * steps + 2 * loop_iterations
+    return (6 + (1 if ring_order else 0) + graph_extra) * steps + 2 * loop_iterations
 
 
 def host_cpu():

@@ -329,7 +329,7 @@ int cg_autotune(cg_ctx* ctx, int32_t steps_per_trial, size_t flush_bytes, void* 
  *                 neighbours of every cell exactly as cg_get_neighbors()
  *                 returns them for the same positions.
  *   stream      : cudaStream_t (may be 0); the call synchronizes it.
- * Scratch lives in a static device array of the library (about 3.7 MB, held
+ * Scratch lives in a static device array of the library (about 4.7 MB, held
  * by every GPU that loads the library until the process exits); the call
  * makes no device allocation.  All calls share that array: calls whose GPU
  * work overlaps race.  The first call on each device looks the array's address

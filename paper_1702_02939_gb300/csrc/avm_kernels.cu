@@ -143,15 +143,7 @@ __global__ void k_avm_vertices(AvmBuildArgs g) {
 void launch_avm_build(const AvmBuildArgs& a, cudaStream_t st) {
   const int blocks = (a.n + 127) / 128;
   k_avm_count_owned<<<blocks, 128, 0, st>>>(a);
-  CellListArgs sc{};
-  sc.n = a.n;
-  sc.nbins = a.n;
-  sc.ctl = a.ctl;
-  sc.bin_count = a.owned;
-  sc.bin_start = a.base_local;
-  sc.scan_partials = a.base_partial;
-  sc.only_if_flagged = 0;
-  launch_scan(sc, st);
+  launch_scan({a.n, a.owned, a.base_local, a.base_partial}, st);
   k_avm_cell_lists<<<blocks, 128, 0, st>>>(a);
   k_avm_vertices<<<blocks, 128, 0, st>>>(a);
 }
@@ -1374,20 +1366,8 @@ void launch_avm_divide_slots(const DivArgs& d, const int* cslot, const int* vslo
                              int* fv, int* sv, int* svp, cudaStream_t st) {
   const int blocks = blocks_of(d.g.V);  // V = 2n covers the cells too
   k_div_free_flags<<<blocks, kAvmThreads, 0, st>>>(d.g, cslot, vslot, fc, fv);
-  CellListArgs sc_args{};
-  sc_args.ctl = d.g.ctl;
-  sc_args.n = d.g.n;
-  sc_args.nbins = d.g.n;
-  sc_args.bin_count = fc;
-  sc_args.bin_start = sc;
-  sc_args.scan_partials = scp;
-  launch_scan(sc_args, st);
-  sc_args.n = d.g.V;
-  sc_args.nbins = d.g.V;
-  sc_args.bin_count = fv;
-  sc_args.bin_start = sv;
-  sc_args.scan_partials = svp;
-  launch_scan(sc_args, st);
+  launch_scan({d.g.n, fc, sc, scp}, st);
+  launch_scan({d.g.V, fv, sv, svp}, st);
   k_div_free_list<<<blocks, kAvmThreads, 0, st>>>(d, cslot, vslot, fc, sc, scp, fv, sv, svp);
 }
 void launch_avm_divide_begin(const DivArgs& d, cudaStream_t st) {
@@ -1403,20 +1383,8 @@ void launch_avm_divide_round(const DivArgs& d, cudaStream_t st) {
 void launch_avm_sort(const AvmSortArgs& a, cudaStream_t st) {
   const int blocks = blocks_of(a.V);  // V = 2n covers the cells too
   k_avm_sort_keys<<<blocks, kAvmThreads, 0, st>>>(a);
-  CellListArgs sc{};
-  sc.ctl = a.ctl;
-  sc.n = a.V;
-  sc.nbins = a.by_tag ? a.V : (1 << (2 * a.hord_v)) + 1;
-  sc.bin_count = a.kcount_v;
-  sc.bin_start = a.kstart_v;
-  sc.scan_partials = a.kpart_v;
-  launch_scan(sc, st);
-  sc.n = a.n;
-  sc.nbins = a.by_tag ? a.n : (1 << (2 * a.hord_c)) + 1;
-  sc.bin_count = a.kcount_c;
-  sc.bin_start = a.kstart_c;
-  sc.scan_partials = a.kpart_c;
-  launch_scan(sc, st);
+  launch_scan({a.by_tag ? a.V : (1 << (2 * a.hord_v)) + 1, a.kcount_v, a.kstart_v, a.kpart_v}, st);
+  launch_scan({a.by_tag ? a.n : (1 << (2 * a.hord_c)) + 1, a.kcount_c, a.kstart_c, a.kpart_c}, st);
   k_avm_sort_perm<<<blocks, kAvmThreads, 0, st>>>(a);
   k_avm_sort_move<<<blocks, kAvmThreads, 0, st>>>(a);
   const size_t V = (size_t)a.V, n = (size_t)a.n;

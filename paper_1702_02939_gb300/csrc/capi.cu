@@ -32,7 +32,7 @@ struct Offsets {
   size_t tag, nid, nid_alt, rep, cnt, nbr, old_cnt, old_nbr;
   size_t fs, s, w, order;
   size_t flags, list0, list1, dirty_list, dirty_bits, fix_list, fix_bits;
-  size_t bin_count, bin_start, partials, cell_bin, cell_rank, ids;
+  size_t bin_count, bin_slot, bin_head, bin_next;
   size_t reps, ctl, dir_tab;
   size_t io_v0, io_xy;  // staging of cg_run_io: [2][n] v0, [2][2][n] positions
   size_t total;
@@ -94,11 +94,9 @@ Offsets layout(int64_t N, int64_t NB, int64_t NK, int R) {
   o.fix_list = L.take(N * i4);
   o.fix_bits = L.take(((N + 31) / 32) * 4);
   o.bin_count = L.take(NB * i4);
-  o.bin_start = L.take((NB + 1) * i4);
-  o.partials = L.take(((NB + 1 + kScanChunkHost - 1) / kScanChunkHost + 1) * i4);
-  o.cell_bin = L.take(N * i4);
-  o.cell_rank = L.take(N * i4);
-  o.ids = L.take(N * i4);
+  o.bin_slot = L.take(NB * sizeof(int4));
+  o.bin_head = L.take(NB * i4);
+  o.bin_next = L.take(N * i4);
   o.reps = L.take(R * sizeof(Rep));
   o.ctl = L.take(sizeof(Ctl));
   o.dir_tab = L.take(kDirTabEntries * sizeof(double2));
@@ -338,23 +336,26 @@ TestArgs test_args(cg_ctx* c) {
   return t;
 }
 
-CellListArgs cell_list_args(cg_ctx* c, int only_if_flagged) {
+BinArrays bin_arrays(cg_ctx* c) {
+  return {c->at<int>(c->off.bin_count), c->at<int4>(c->off.bin_slot), c->at<int>(c->off.bin_head),
+          c->at<int>(c->off.bin_next)};
+}
+
+CellListArgs cell_list_args(cg_ctx* c) {
   CellListArgs a{};  // every field starts zero or null
   a.n = (int)c->N;
-  a.nbins = (int)c->NB;
   a.reps = c->at<Rep>(c->off.reps);
   a.rep = c->at<int>(c->off.rep);
   a.ctl = c->ctl();
   a.X = c->at<long long>(c->off.X);
   a.Y = c->at<long long>(c->off.Y);
-  a.bin_count = c->at<int>(c->off.bin_count);
-  a.bin_start = c->at<int>(c->off.bin_start);
-  a.cell_bin = c->at<int>(c->off.cell_bin);
-  a.cell_rank = c->at<int>(c->off.cell_rank);
-  a.ids = c->at<int>(c->off.ids);
-  a.scan_partials = c->at<int>(c->off.partials);
-  a.only_if_flagged = only_if_flagged;
+  a.bins = bin_arrays(c);
   return a;
+}
+
+// The list's counts back to zero for the next build.
+void clear_bins(cg_ctx* c, cudaStream_t st) {
+  cudaMemsetAsync(c->at<int>(c->off.bin_count), 0, c->NB * sizeof(int), st);
 }
 
 RepairArgs repair_args(cg_ctx* c, int which_in, int all_cells) {
@@ -368,9 +369,7 @@ RepairArgs repair_args(cg_ctx* c, int which_in, int all_cells) {
   r.X = c->at<long long>(c->off.X);
   r.Y = c->at<long long>(c->off.Y);
   r.tag = c->at<int>(c->off.tag);
-  r.bin_start = c->at<int>(c->off.bin_start);
-  r.bin_partials = c->at<int>(c->off.partials);
-  r.ids = c->at<int>(c->off.ids);
+  r.bins = bin_arrays(c);
   r.cnt = c->at<int>(c->off.cnt);
   r.nbr = c->at<int>(c->off.nbr);
   r.old_cnt = c->at<int>(c->off.old_cnt);
@@ -499,7 +498,7 @@ void enqueue_step_prefix(cg_ctx* c, cudaStream_t st) {
     run_force(c, f, c->side[0]);
   }
   cudaEventRecord(c->join_dir, c->side[0]);
-  launch_cell_list(cell_list_args(c, 0), c->side[1]);
+  launch_cell_list(cell_list_args(c), c->side[1]);
   cudaEventRecord(c->join_list, c->side[1]);
   launch_test(test_args(c), st, test_grid(c));
   cudaStreamWaitEvent(st, c->join_list, 0);
@@ -527,6 +526,8 @@ void enqueue_step_suffix(cg_ctx* c, cudaStream_t st) {
   g.list = c->at<int>(c->off.dirty_list);
   g.list_count = &c->ctl()->dirty_count;
   g.list_bits = c->at<unsigned>(c->off.dirty_bits);
+  g.clear = c->at<int>(c->off.bin_count);  // the rounds are done with the cell list
+  g.n_clear = (int)c->NB;
   // two blocks per SM take up to 9728 listed cells at once (usually well
   // below 1% of the cells are rewritten in a step)
   run_geom(c, g, st, sm_count() * 2);
@@ -590,9 +591,10 @@ int triangulate_all(cg_ctx* c) {
   CG_CUDA(c, cudaMemsetAsync(c->at<unsigned>(c->off.flags), 0, ((c->N + 31) / 32) * 4, st));
   CG_CUDA(c, cudaMemsetAsync(c->at<int>(c->off.bin_count), 0, c->NB * sizeof(int), st));
   launch_begin_topology(c->ctl(), 0, st);
-  launch_cell_list(cell_list_args(c, 0), st);
+  launch_cell_list(cell_list_args(c), st);
   launch_repair(repair_args(c, 0, 1), repair_grid_all(c), st);
   launch_check(check_args(c, 0, 1, 1), check_grid_all(c), st);
+  clear_bins(c, st);
   launch_begin_topology(c->ctl(), 0, st);
   CG_CUDA(c, cudaGetLastError());
   return CG_OK;
@@ -1008,13 +1010,16 @@ int cg_profile_step(cg_ctx* c, int64_t nsteps, double* ms_out, int32_t n_out) {
     launch_begin_topology(c->ctl(), 1, st);
     launch_test(test_args(c), st);
     cudaEventRecord(ev[1], st);
-    launch_cell_list(cell_list_args(c, 1), st);
+    launch_cell_list(cell_list_args(c), st);
     cudaEventRecord(ev[2], st);
     for (int r = 0; r < cap; ++r) {
-      launch_repair(repair_args(c, r & 1, 0), grid, st);
+      RepairArgs ra = repair_args(c, r & 1, 0);
+      ra.record = r == 0;
+      launch_repair(ra, grid, st);
       launch_check(check_args(c, r & 1, r == cap - 1, 0), check_grid(c), st);
     }
     cudaEventRecord(ev[3], st);
+    clear_bins(c, st);
     run_dir(c, dir_args_step(c), st, dir_grid(c));
     cudaEventRecord(ev[4], st);
     if (c->launch.ring_order) run_order(c, st);
@@ -1127,7 +1132,7 @@ int cg_get_neighbors(cg_ctx* c, int32_t* cnt, int32_t* nbr) {
   int rc = read_status(c);
   if (rc) return rc;
   // stage in the old-ring scratch (free outside a step)
-  int* tc = c->at<int>(c->off.cell_bin);
+  int* tc = c->at<int>(c->off.old_cnt);
   int* tn = c->at<int>(c->off.old_nbr);
   launch_gather_ring((int)c->N, c->at<int>(c->off.tag), c->at<int>(c->off.cnt), c->at<int>(c->off.nbr), tc, tn,
                      c->stream);

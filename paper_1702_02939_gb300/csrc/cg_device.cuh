@@ -107,6 +107,18 @@ __device__ __forceinline__ bool last_block(unsigned int* done) {
   return s_last;
 }
 
+// Cell list: a bin holds its first kBinCap cells in place (one 16-byte load
+// with the count); further ones (0.4% of the bins at one cell per bin) hang on
+// a chain, newest first, of exactly count - kBinCap links, so neither heads nor
+// links need clearing.
+constexpr int kBinCap = 4;
+template <class Bins>
+__device__ __forceinline__ void bin_insert(const Bins& l, int b, int i) {
+  const int r = atomicAdd(&l.count[b], 1);
+  if (r < kBinCap) reinterpret_cast<int*>(l.slot + b)[r] = i;
+  else l.next[i] = atomicExch(&l.head[b], i);
+}
+
 // Bins per block of the block-local scans; the global start of bin b is the
 // block-local exclusive prefix plus one offset per scan block.
 constexpr int kScanChunk = 256 * 8;

@@ -38,6 +38,10 @@ struct GeomArgs {
   const int* list;
   const int* list_count;
   unsigned* list_bits;  // bit of each listed cell, cleared once processed
+  // With a list: n_clear integers set to zero on the way (the cell list's
+  // counts for the next step), or null
+  int* clear;
+  int n_clear;
   // Rings may be rewritten concurrently (the pass beside the repair rounds):
   // out-of-range entries are skipped and no status is raised; every cell whose
   // ring changes is processed again afterwards.
@@ -138,15 +142,28 @@ struct TestArgs {
   const int* order;  // processing order of the cells (as GeomArgs), or null
 };
 
+// The cell list's arrays (see kBinCap in cg_device.cuh).
+struct BinArrays {
+  int* count;  // [bins] cells per bin, zero before a build
+  int4* slot;  // [bins] the first kBinCap cells
+  int* head;   // [bins] newest cell past those
+  int* next;   // [n] chain links
+};
 struct CellListArgs {
-  int n, nbins;
+  int n;
   const Rep* reps;
   const int* rep;
   Ctl* ctl;
   const long long *X, *Y;  // [2][n] grid coordinates
-  int *bin_count, *bin_start, *cell_bin, *cell_rank, *ids;
-  int* scan_partials;
-  int only_if_flagged;  // skip when nothing is flagged
+  BinArrays bins;          // counts zero before the build
+};
+
+// Exclusive scan of count[0 .. nbins): block-local prefixes in start[0 ..
+// nbins], one offset per block of kScanChunk in partials (bin_begin).
+struct ScanArgs {
+  int nbins;
+  const int* count;
+  int *start, *partials;
 };
 
 struct RepairArgs {
@@ -157,13 +174,14 @@ struct RepairArgs {
   const double *x, *y;     // [2][n]
   const long long *X, *Y;  // [2][n]
   const int* tag;
-  const int *bin_start, *bin_partials, *ids;
+  BinArrays bins;
   int *cnt, *nbr;
   int *old_cnt, *old_nbr;
   unsigned* flags;
   const int* list_in;
   int which_in;  // count index of list_in
   int all_cells; // process cells 0..n-1 instead of the list
+  int record;    // outside a graph: count the list in the step statistics
   // Rounds inside a conditional (while) graph node: the input list is
   // lists[round & 1] with the round counter read from the control word.
   int dyn;
@@ -205,8 +223,7 @@ void launch_begin_topology(Ctl* ctl, int flip, cudaStream_t st);
 void launch_test(const TestArgs& a, cudaStream_t st, int blocks = 0);
 void launch_cell_list(const CellListArgs& a, cudaStream_t st);
 void launch_repair(const RepairArgs& a, int grid_blocks, cudaStream_t st);
-// exclusive scan of a.bin_count[0..nbins) into (a.bin_start, a.scan_partials)
-void launch_scan(const CellListArgs& a, cudaStream_t st);
+void launch_scan(const ScanArgs& a, cudaStream_t st);
 void launch_check(const CheckArgs& a, int grid_blocks, cudaStream_t st);
 
 // state preparation and user-order transfers

@@ -34,8 +34,6 @@ namespace {
 
 constexpr int kMaxCells = CG_NOALLOC_MAX_CELLS;
 constexpr int kMaxBins = 4 * CG_NOALLOC_MAX_CELLS;
-constexpr int kScanChunk = 256 * 8;  // bins per scan block of the cell-list kernels
-constexpr int kMaxPartials = (kMaxBins + 1 + kScanChunk - 1) / kScanChunk + 1;
 
 // byte offsets inside the static scratch array (all 256-byte aligned)
 constexpr size_t al(size_t b) { return (b + 255) & ~(size_t)255; }
@@ -55,16 +53,14 @@ constexpr size_t kOffFlags = kOffOldNbr + al(4 * (size_t)kMaxCells * CG_RING);
 constexpr size_t kOffList0 = kOffFlags + al(4 * (size_t)((kMaxCells + 31) / 32));
 constexpr size_t kOffList1 = kOffList0 + al(4 * (size_t)kMaxCells);
 constexpr size_t kOffBinCount = kOffList1 + al(4 * (size_t)kMaxCells);
-constexpr size_t kOffBinStart = kOffBinCount + al(4 * (size_t)kMaxBins);
-constexpr size_t kOffPartials = kOffBinStart + al(4 * (size_t)(kMaxBins + 1));
-constexpr size_t kOffCellBin = kOffPartials + al(4 * (size_t)kMaxPartials);
-constexpr size_t kOffCellRank = kOffCellBin + al(4 * (size_t)kMaxCells);
-constexpr size_t kOffIds = kOffCellRank + al(4 * (size_t)kMaxCells);
-constexpr size_t kScratchBytes = kOffIds + al(4 * (size_t)kMaxCells);
+constexpr size_t kOffBinSlot = kOffBinCount + al(4 * (size_t)kMaxBins);
+constexpr size_t kOffBinHead = kOffBinSlot + al(sizeof(int4) * (size_t)kMaxBins);
+constexpr size_t kOffBinNext = kOffBinHead + al(4 * (size_t)kMaxBins);
+constexpr size_t kScratchBytes = kOffBinNext + al(4 * (size_t)kMaxCells);
 
 }  // namespace
 
-// The scratch itself (about 3.7 MB for 16384 cells).
+// The scratch itself (about 4.7 MB for 16384 cells).
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 
 namespace {
@@ -169,19 +165,13 @@ extern "C" int cg_triangulate_noalloc(int32_t n, double Lx, double Ly, const dou
 
   CellListArgs cl{};  // every field starts zero or null
   cl.n = n;
-  cl.nbins = nbins;
   cl.reps = d_rep;
   cl.rep = repi;
   cl.ctl = ctl;
   cl.X = X;
   cl.Y = Y;
-  cl.bin_count = reinterpret_cast<int*>(base + kOffBinCount);
-  cl.bin_start = reinterpret_cast<int*>(base + kOffBinStart);
-  cl.cell_bin = reinterpret_cast<int*>(base + kOffCellBin);
-  cl.cell_rank = reinterpret_cast<int*>(base + kOffCellRank);
-  cl.ids = reinterpret_cast<int*>(base + kOffIds);
-  cl.scan_partials = reinterpret_cast<int*>(base + kOffPartials);
-  cl.only_if_flagged = 0;
+  cl.bins = {reinterpret_cast<int*>(base + kOffBinCount), reinterpret_cast<int4*>(base + kOffBinSlot),
+             reinterpret_cast<int*>(base + kOffBinHead), reinterpret_cast<int*>(base + kOffBinNext)};
   launch_cell_list(cl, st);
 
   RepairArgs ra{};  // every field starts zero or null
@@ -194,9 +184,7 @@ extern "C" int cg_triangulate_noalloc(int32_t n, double Lx, double Ly, const dou
   ra.X = X;
   ra.Y = Y;
   ra.tag = tag;
-  ra.bin_start = cl.bin_start;
-  ra.bin_partials = cl.scan_partials;
-  ra.ids = cl.ids;
+  ra.bins = cl.bins;
   ra.cnt = cnt;
   ra.nbr = nbr;
   ra.old_cnt = reinterpret_cast<int*>(base + kOffOldCnt);

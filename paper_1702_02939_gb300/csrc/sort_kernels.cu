@@ -63,15 +63,7 @@ void launch_sort(const SortArgs& a, cudaStream_t st) {
   if (a.n <= 0) return;
   const int blocks = (a.n + 255) / 256;
   k_sort_keys<<<blocks, 256, 0, st>>>(a);
-  CellListArgs sc{};
-  sc.n = a.n;
-  sc.nbins = a.nkeys;
-  sc.ctl = a.ctl;
-  sc.bin_count = a.key_count;
-  sc.bin_start = a.key_start;
-  sc.scan_partials = a.key_partials;
-  sc.only_if_flagged = 0;
-  launch_scan(sc, st);
+  launch_scan({a.nkeys, a.key_count, a.key_start, a.key_partials}, st);
   k_sort_perm<<<blocks, 256, 0, st>>>(a);
   k_sort_move<<<blocks, 256, 0, st>>>(a);
   k_sort_flip<<<1, 1, 0, st>>>(a.ctl);

@@ -208,6 +208,8 @@ __global__ void __launch_bounds__(kSlotThreads, kGeomSlotBlocks) k_geom_slots(Ge
   const long long* __restrict__ X = g.X + (size_t)cur * N;
   const long long* __restrict__ Y = g.Y + (size_t)cur * N;
   const int total = g.list ? *g.list_count : g.n;
+  if (g.clear)
+    for (int k = blockIdx.x * kSlotThreads + threadIdx.x; k < g.n_clear; k += gridDim.x * kSlotThreads) g.clear[k] = 0;
   for (int base = blockIdx.x * 32; base < total; base += gridDim.x * 32) {
     const int item = base + c;
     int i = 0, m = 0;

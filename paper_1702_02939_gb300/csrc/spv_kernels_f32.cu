@@ -69,6 +69,8 @@ __global__ void __launch_bounds__(kGeomThreads) k_geom_f32(GeomArgs g) {
   float2* sv = as_f2(g.s);
   float2* wv = as_f2(g.w);
   const int total = g.list ? *g.list_count : g.n;
+  if (g.clear)
+    for (int k = blockIdx.x * kGeomThreads + t; k < g.n_clear; k += gridDim.x * kGeomThreads) g.clear[k] = 0;
   for (int item = blockIdx.x * kGeomThreads + t; item < total; item += gridDim.x * kGeomThreads) {
     const int i = g.list ? g.list[item] : (g.order ? g.order[item] : item);
     if (g.list_bits) atomicAnd(&g.list_bits[i >> 5], ~(1u << (i & 31)));

@@ -4,15 +4,17 @@
 // The paper repairs flagged cells on the CPU: a candidate "Delaunay 1-ring"
 // from the locality lemma of Chen et al., reduced to the true neighbours with
 // CGAL (Sussman, arXiv 1702.02939, Sec. 2.C.4).  Here the repair stays on the
-// GPU: each flagged cell's Voronoi polygon is rebuilt by clipping a large
-// square with the bisectors of nearby cells taken from a periodic cell list,
+// GPU: each flagged cell's ring is wrapped around it neighbour by neighbour
+// from the nearby cells of a periodic cell list, every step decided by the
+// exact, perturbed in-circle predicate.  Where that cannot decide (more
+// candidates than a warp holds, a very small box), the cell's Voronoi polygon
+// is rebuilt by clipping a large square with the bisectors of nearby cells,
 // nearest first.  A polygon vertex v_a (circumcentre of i, g_a, g_{a+1})
 // is cut away by candidate j exactly when j lies inside the circle through
-// (i, g_a, g_{a+1}), so every keep/drop decision is the exact, perturbed
-// in-circle predicate and the result is the exact Delaunay ring of i.  The
-// search stops once every unvisited cell is farther than twice the polygon's
-// circumradius (the security radius), which is the locality argument of the
-// paper in its simplest form.
+// (i, g_a, g_{a+1}): the same predicate.  Either way the result is the exact
+// Delaunay ring of i, and the search stops once every unvisited cell is
+// farther than twice the largest circumradius (the security radius), which is
+// the locality argument of the paper in its simplest form.
 #include "cg_device.cuh"
 #include "cg_kernels.h"
 
@@ -24,22 +26,22 @@ constexpr int kScanThreads = 256;
 constexpr int kScanPer = 8;
 static_assert(kScanChunk == kScanThreads * kScanPer, "scan block size");
 
-__global__ void k_bin_count(CellListArgs g) {
-  if (g.only_if_flagged && g.ctl->count[0] == 0) return;
+// The cell list in one pass (see kBinCap): the count of a bin hands out its
+// places.  Bound by the latency of one atomic and one store per cell; four
+// kernels of a counting sort with contiguous bins took 14-23 us where this one
+// takes 4-8 (256 to 262144 cells).
+__global__ void k_bin_cells(CellListArgs g) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= g.n) return;
   const int cur = g.ctl->cur;
-  const Rep R = g.reps[g.rep[i]];
+  const Rep& R = g.reps[g.rep[i]];
   int bx, by;
   bin_of_grid(R, g.X[(size_t)cur * g.n + i], g.Y[(size_t)cur * g.n + i], bx, by);
-  const int b = R.bin0 + by * R.nbx + bx;
-  g.cell_bin[i] = b;
-  g.cell_rank[i] = atomicAdd(&g.bin_count[b], 1);
+  bin_insert(g.bins, R.bin0 + by * R.nbx + bx, i);
 }
 
 // Block-local exclusive scan of bin counts; block totals to scan_partials.
-__global__ void __launch_bounds__(kScanThreads) k_scan_local(CellListArgs g) {
-  if (g.only_if_flagged && g.ctl->count[0] == 0) return;
+__global__ void __launch_bounds__(kScanThreads) k_scan_local(ScanArgs g) {
   __shared__ int warp_tot[kScanThreads / 32];
   const int base = blockIdx.x * kScanChunk + threadIdx.x * kScanPer;
   int v[kScanPer];
@@ -47,7 +49,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_local(CellListArgs g) {
 #pragma unroll
   for (int k = 0; k < kScanPer; ++k) {
     int b = base + k;
-    v[k] = (b < g.nbins) ? g.bin_count[b] : 0;
+    v[k] = (b < g.nbins) ? g.count[b] : 0;
     sum += v[k];
   }
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -65,33 +67,26 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_local(CellListArgs g) {
 #pragma unroll
   for (int k = 0; k < kScanPer; ++k) {
     int b = base + k;
-    if (b < g.nbins) g.bin_start[b] = run;
-    else if (b == g.nbins) g.bin_start[b] = run;  // sentinel
+    if (b < g.nbins) g.start[b] = run;
+    else if (b == g.nbins) g.start[b] = run;  // sentinel
     run += v[k];
   }
   if (threadIdx.x == kScanThreads - 1) {
     int tot = 0;
     for (int w = 0; w < kScanThreads / 32; ++w) tot += warp_tot[w];
-    g.scan_partials[blockIdx.x] = tot;
+    g.partials[blockIdx.x] = tot;
   }
 }
 
-// Exclusive scan of the block totals (one block); also records step statistics.
-__global__ void __launch_bounds__(1024) k_scan_partials(CellListArgs g, int nblocks) {
-  Ctl* ctl = g.ctl;
-  if (threadIdx.x == 0 && g.only_if_flagged) {  // per-step build: record statistics
-    int c = ctl->count[0];
-    ctl->last_flagged = c;
-    ctl->flagged_total += c;
-  }
-  if (g.only_if_flagged && ctl->count[0] == 0) return;
+// Exclusive scan of the block totals (one block).
+__global__ void __launch_bounds__(1024) k_scan_partials(ScanArgs g, int nblocks) {
   __shared__ int buf[1024];
   __shared__ int carry;
   if (threadIdx.x == 0) carry = 0;
   __syncthreads();
   for (int base = 0; base <= nblocks; base += 1024) {
     int idx = base + threadIdx.x;
-    int v = (idx < nblocks) ? g.scan_partials[idx] : 0;
+    int v = (idx < nblocks) ? g.partials[idx] : 0;
     buf[threadIdx.x] = v;
     __syncthreads();
     for (int o = 1; o < 1024; o <<= 1) {
@@ -102,32 +97,18 @@ __global__ void __launch_bounds__(1024) k_scan_partials(CellListArgs g, int nblo
     }
     int excl = carry + buf[threadIdx.x] - v;
     __syncthreads();
-    if (idx < nblocks) g.scan_partials[idx] = excl;
-    else if (idx == nblocks) g.scan_partials[idx] = excl;  // total
+    if (idx < nblocks) g.partials[idx] = excl;
+    else if (idx == nblocks) g.partials[idx] = excl;  // total
     if (threadIdx.x == 1023) carry += buf[1023];
     __syncthreads();
   }
 }
 
-__global__ void k_bin_scatter(CellListArgs g) {
-  if (g.only_if_flagged && g.ctl->count[0] == 0) return;
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= g.n) return;
-  const int b = g.cell_bin[i];
-  g.ids[bin_begin(g.bin_start, g.scan_partials, b) + g.cell_rank[i]] = i;
-  g.bin_count[b] = 0;  // ready for the next build
-}
-
 void launch_cell_list(const CellListArgs& a, cudaStream_t st) {
-  if (a.n <= 0) return;
-  const int nblk = (a.nbins + 1 + kScanChunk - 1) / kScanChunk;
-  k_bin_count<<<(a.n + 255) / 256, 256, 0, st>>>(a);
-  k_scan_local<<<nblk, kScanThreads, 0, st>>>(a);
-  k_scan_partials<<<1, 1024, 0, st>>>(a, nblk);
-  k_bin_scatter<<<(a.n + 255) / 256, 256, 0, st>>>(a);
+  if (a.n > 0) k_bin_cells<<<(a.n + 255) / 256, 256, 0, st>>>(a);
 }
 
-void launch_scan(const CellListArgs& a, cudaStream_t st) {
+void launch_scan(const ScanArgs& a, cudaStream_t st) {
   const int nblk = (a.nbins + 1 + kScanChunk - 1) / kScanChunk;
   k_scan_local<<<nblk, kScanThreads, 0, st>>>(a);
   k_scan_partials<<<1, 1024, 0, st>>>(a, nblk);
@@ -301,11 +282,370 @@ __device__ void process_candidates(Poly& p, int nbuf, const int* s_id, const lon
   __syncwarp();
 }
 
+// ---------------------------------------------------------------------------
+// Repair by gift wrapping: the ring of cell i around it, one neighbour after
+// the other.  With g the last neighbour found, the next one counter-clockwise
+// is the candidate c left of g (g x c > 0) whose circle through (i, g, c) is
+// empty, the one of smallest
+//   s = (|c|^2 - g.c) / (g x c),
+// the signed distance (in units of |g| / 2) of the circle's centre from the
+// middle of g.  Every lane holds two candidates and forms s in FP32 with a
+// bound on its error; usually one candidate alone can be the smallest, else
+// the exact perturbed in-circle predicate picks among those that can.  The
+// nearest candidate starts the ring; a ring that closes on its start is the
+// exact one among the candidates (every step is decided exactly).
+//
+// Against clipping a square by the bisectors of the sorted candidates (below),
+// a ring costs ~6 steps of ~60 instructions instead of a sort and ~10 clips of
+// ~300.
+// ---------------------------------------------------------------------------
+struct WrapLane {  // a candidate as its lane holds it
+  float x, y, l2;  // offset from the cell (real units), its squared length
+  int e;           // entry in the candidate buffer, -1: none
+};
+
+// Bounds lo <= s <= hi of candidate c seen from neighbour g; lo = hi = +inf
+// when c is not left of g, lo = -inf, hi = +inf when FP32 cannot tell.  Inputs
+// carry a relative error <= 2u + u^2 (u = 2^-24, i2f_scaled): a product 4u
+// and its rounding u, the sums at most 3u more, so the numerator is within
+// 10u of the sum of its terms' magnitudes and so is the cross product, which
+// is used where it exceeds 16 times its error (the quotient's error is then
+// below 1.07 times the first-order one, plus the division's 2u and the sums').
+__device__ __forceinline__ void wrap_bounds(float gx, float gy, int ge, const WrapLane& c, const long long* s_X,
+                                            const long long* s_Y, float& lo, float& hi) {
+  const float inf = __int_as_float(0x7f800000), u = 0x1p-24f;
+  lo = hi = inf;
+  if (c.e < 0 || c.e == ge) return;
+  const float t1 = gx * c.y, t2 = gy * c.x, q1 = gx * c.x, q2 = gy * c.y;
+  const float cr = t1 - t2, sc = fabsf(t1) + fabsf(t2), ec = 10.0f * u * sc;
+  const float num = c.l2 - (q1 + q2), sn = c.l2 + fabsf(q1) + fabsf(q2);
+  if (sc > 1e-30f && sn < 1e30f && fabsf(cr) > 16.0f * ec) {
+    if (cr < 0.0f) return;
+    const float s = __fdividef(num, cr);
+    const float e = 1.2f * __fdividef(10.0f * u * sn + fabsf(s) * ec, cr) + 6.0f * u * fabsf(s);
+    lo = s - e;
+    hi = s + e;
+    return;
+  }
+  if (orient_exact(s_X[ge], s_Y[ge], s_X[c.e], s_Y[c.e]) <= 0) return;
+  lo = -inf;
+}
+
+// Signed integers ordered as the floats are.
+__device__ __forceinline__ int float_order(float f) {
+  const int b = __float_as_int(f);
+  return b ^ ((b >> 31) & 0x7fffffff);
+}
+
+// The ring of the cell among the buffered candidates: lane a receives the
+// a-th neighbour's entry, R4 bounds four times the largest squared
+// circumradius.  Returns the number of neighbours, 0 when the ring does not
+// close (within CG_RING).
+__device__ __forceinline__ int wrap_ring(int start, const WrapLane& c0, const WrapLane& c1, const long long* s_X,
+                                         const long long* s_Y, const int* s_tag, int ikey, float sc, double inv_scale,
+                                         int lane, int& mine, float& R4) {
+  const float u = 0x1p-24f;
+  int g = start;
+  float r4 = 0.0f;
+  for (int a = 0; a < CG_RING; ++a) {
+    if (lane == a) mine = g;
+    const float gx = __shfl_sync(0xffffffffu, g < 32 ? c0.x : c1.x, g & 31);
+    const float gy = __shfl_sync(0xffffffffu, g < 32 ? c0.y : c1.y, g & 31);
+    float lo0, hi0, lo1, hi1;
+    wrap_bounds(gx, gy, g, c0, s_X, s_Y, lo0, hi0);
+    wrap_bounds(gx, gy, g, c1, s_X, s_Y, lo1, hi1);
+    const int m = __reduce_min_sync(0xffffffffu, float_order(fminf(hi0, hi1)));
+    const float inf = __int_as_float(0x7f800000);
+    const unsigned b0 = __ballot_sync(0xffffffffu, float_order(lo0) <= m && lo0 < inf);
+    const unsigned b1 = __ballot_sync(0xffffffffu, float_order(lo1) <= m && lo1 < inf);
+    if (!(b0 | b1)) return 0;  // nothing left of g
+    int best = b0 ? __ffs(b0) - 1 : 32 + __ffs(b1) - 1;
+    const bool sure = __popc(b0) + __popc(b1) == 1;
+    if (!sure) {
+      const long long gX = s_X[g], gY = s_Y[g];
+      unsigned r0 = b0, r1 = b1;
+      if (best < 32) r0 &= r0 - 1;
+      else r1 &= r1 - 1;
+      while (r0 | r1) {
+        const int o = r0 ? __ffs(r0) - 1 : 32 + __ffs(r1) - 1;
+        if (r0) r0 &= r0 - 1;
+        else r1 &= r1 - 1;
+        if (incircle_sign(0, 0, gX, gY, s_X[best], s_Y[best], s_X[o], s_Y[o], ikey, s_tag[g], s_tag[best], s_tag[o],
+                          sc) > 0)
+          best = o;
+      }
+    }
+    // the circle's centre is (g + s perp(g)) / 2: 4 r^2 = |g|^2 (1 + s^2)
+    const float hi = best < 32 ? hi0 : hi1, lo = best < 32 ? lo0 : lo1;
+    if (lane == (best & 31)) {
+      const float s = fmaxf(fabsf(hi), fabsf(lo));
+      float r = (gx * gx + gy * gy) * (1.0f + s * s) * (1.0f + 32.0f * u);
+      if (!(s < 1e15f)) r = 4.0f * vertex_r2_bound(s_X[g], s_Y[g], s_X[best], s_Y[best], sc, inv_scale);
+      r4 = fmaxf(r4, r);
+    }
+    if (best == start) {
+      R4 = warp_max(r4);
+      return a + 1;
+    }
+    g = best;
+  }
+  return 0;
+}
+
+// The bin (dx, dy) away from bin (bxi, byi) of the replica, periodic.
+__device__ __forceinline__ int bin_at(const Rep& R, int bxi, int byi, int dx, int dy) {
+  int bx = bxi + dx, by = byi + dy;
+  bx += (bx < 0) ? R.nbx : (bx >= R.nbx ? -R.nbx : 0);
+  by += (by < 0) ? R.nby : (by >= R.nby ? -R.nby : 0);
+  return R.bin0 + by * R.nbx + bx;
+}
+
+// The t-th cell of a bin whose first cells are already loaded (link: the cell
+// this function returned last).
+__device__ __forceinline__ int bin_cell(const BinArrays& l, int bin, int4 first, int t, int link) {
+  return t == 0 ? first.x : t == 1 ? first.y : t == 2 ? first.z : t == 3 ? first.w
+         : t == kBinCap ? l.head[bin] : l.next[link];
+}
+
+// A warp's candidate buffer (offsets from the cell, cell index, perturbation key).
+struct CandBuf {
+  long long X[kCand], Y[kCand];
+  int id[kCand], tag[kCand];
+  float d2[kCand];
+};
+
+// Ring of cell i by clipping, nearest candidates first, bins ring by ring: for
+// any number of candidates and any box.  Lane a receives the a-th neighbour;
+// returns the number of neighbours or a status (negative).
+__device__ __noinline__ int clip_ring(const RepairArgs& g, const Rep& R, const long long* __restrict__ X,
+                                      const long long* __restrict__ Y, int i, CandBuf& buf, int lane, int& gid,
+                                      int& gkey) {
+  const long long Xi = X[i], Yi = Y[i];
+  const int ikey = g.tag[i];
+  const float sc = (float)R.inv_scale;
+  // initial polygon: the square of half-width W (vertices (+-W, +-W)), cut
+  // out by four phantom generators at (+-2W, 0) and (0, +-2W)
+  Poly p;
+  p.m = 4;
+  p.err = 0;
+  p.gX = (lane == 0) ? R.W2 : (lane == 2 ? -R.W2 : 0);
+  p.gY = (lane == 1) ? R.W2 : (lane == 3 ? -R.W2 : 0);
+  p.gid = -1 - (lane & 3);
+  p.gkey = kPhantomKey + (lane & 3);
+  {
+    const float W = 0.5f * i2f_scaled(R.W2, sc);  // power of two: exact
+    p.r2 = 2.0f * W * W;
+    p.R2 = p.r2;
+  }
+  int bxi, byi;
+  bin_of_grid(R, Xi, Yi, bxi, byi);
+  const float bs = (float)R.bsx;  // every bin is at least this wide
+  const int kmax = min((R.nbx - 1) / 2, (R.nby - 1) / 2);
+  int nbuf = 0;
+  bool done = false;
+  for (int k = 0; k <= kmax && !done && !p.err; ++k) {
+    const int nring = (k == 0) ? 1 : 8 * k;
+    for (int base = 0; base < nring && !p.err; base += 32) {
+      const int idx = base + lane;
+      int count = 0, bin = 0, j = 0;
+      int4 first = make_int4(0, 0, 0, 0);
+      if (idx < nring) {
+        int dx, dy;
+        ring_bin(k, idx, dx, dy);
+        bin = bin_at(R, bxi, byi, dx, dy);
+        count = g.bins.count[bin];
+        first = g.bins.slot[bin];
+      }
+      int incl = count;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += t;
+      }
+      const int tot = __shfl_sync(0xffffffffu, incl, 31);
+      if (nbuf + tot > kCand) {
+        process_candidates(p, nbuf, buf.id, buf.X, buf.Y, buf.d2, buf.tag, ikey, sc, R.inv_scale, lane);
+        nbuf = 0;
+        if (tot > kCand) p.err = kECAND;
+      }
+      if (!p.err) {
+        int slot = nbuf + incl - count;
+        bool same = false;  // another cell on exactly this grid point
+        for (int t = 0; t < count; ++t) {
+          j = bin_cell(g.bins, bin, first, t, j);
+          buf.tag[slot] = g.tag[j];
+          buf.id[slot] = j;
+          if (j == i) {
+            buf.d2[slot] = kSelfKey;  // never clips
+            buf.X[slot] = 0;
+            buf.Y[slot] = 0;
+          } else {
+            const long long dX = min_image_i(X[j] - Xi, R.LX), dY = min_image_i(Y[j] - Yi, R.LY);
+            same |= (dX == 0 && dY == 0);
+            const float dx = i2f_scaled(dX, sc), dy = i2f_scaled(dY, sc);
+            buf.d2[slot] = dx * dx + dy * dy;
+            buf.X[slot] = dX;
+            buf.Y[slot] = dY;
+          }
+          ++slot;
+        }
+        nbuf += tot;
+        if (__any_sync(0xffffffffu, same)) p.err = kEDEGEN;  // no bisector between them
+      }
+      __syncwarp();
+    }
+    if (p.err) break;
+    // rings 0..2 are gathered into one batch before clipping
+    if (k < 2 && k < kmax) continue;
+    process_candidates(p, nbuf, buf.id, buf.X, buf.Y, buf.d2, buf.tag, ikey, sc, R.inv_scale, lane);
+    nbuf = 0;
+    // every unvisited cell is farther than k*bs from cell i
+    const float reach = k * bs;
+    if (reach * reach > 4.0f * p.R2 * (1.0f + 1e-3f)) done = true;
+  }
+  if (p.err) return p.err;
+  if (!done) return kEBOX;
+  if (p.m > CG_RING) return kERING;
+  if (__ballot_sync(0xffffffffu, lane < p.m && p.gid < 0)) return kEBOX;
+  gid = p.gid;
+  gkey = p.gkey;
+  return p.m;
+}
+
+// Ring of cell i by gift wrapping over the 25 bins around it, widened bin ring
+// by bin ring until every unseen cell is farther than the diameter of the
+// largest circle; only the ring found so far and the cells within that
+// diameter can then be in the final one.  Lane a receives the a-th neighbour;
+// returns their number, a status (negative), or 0 where clip_ring has to
+// decide (more than kCand candidates, an unbounded or overfull ring, a box too
+// small).
+__device__ __forceinline__ int gift_ring(const RepairArgs& g, const Rep& R, const long long* __restrict__ X,
+                                         const long long* __restrict__ Y, int i, CandBuf& buf, int lane, int& gid,
+                                         int& gkey) {
+  const int kmax = min((R.nbx - 1) / 2, (R.nby - 1) / 2);
+  if (kmax < 2) return 0;
+  const long long Xi = X[i], Yi = Y[i];
+  const int ikey = g.tag[i];
+  const float sc = (float)R.inv_scale, bs = (float)R.bsx;
+  int bxi, byi;
+  bin_of_grid(R, Xi, Yi, bxi, byi);
+  int count = 0, bin = 0;
+  int4 first = make_int4(0, 0, 0, 0);
+  if (lane < 25) {
+    bin = bin_at(R, bxi, byi, lane % 5 - 2, lane / 5 - 2);
+    count = g.bins.count[bin];
+    first = g.bins.slot[bin];
+  }
+  int incl = count;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int t = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += t;
+  }
+  int n = __shfl_sync(0xffffffffu, incl, 31);
+  if (n > kCand) return 0;
+  for (int t = 0, j = 0; t < count; ++t) {
+    j = bin_cell(g.bins, bin, first, t, j);
+    buf.id[incl - count + t] = j;
+  }
+  __syncwarp();
+  // lane e takes entries e and e + 32: every candidate's loads at once
+  bool same = false;
+  auto offset = [&](int e, int j) {
+    const long long dX = min_image_i(X[j] - Xi, R.LX), dY = min_image_i(Y[j] - Yi, R.LY);
+    same |= dX == 0 && dY == 0 && j != i;
+    buf.X[e] = dX;
+    buf.Y[e] = dY;
+  };
+  for (int e = lane; e < n; e += 32) {
+    const int j = buf.id[e];
+    buf.tag[e] = g.tag[j];
+    offset(e, j);
+  }
+  if (__any_sync(0xffffffffu, same)) return kEDEGEN;  // no bisector between them
+  for (int k = 2;;) {
+    WrapLane c0, c1;
+    auto load = [&](WrapLane& c, int e) {
+      c.e = (e < n && buf.id[e] != i) ? e : -1;
+      c.x = c.e < 0 ? 0.0f : i2f_scaled(buf.X[e], sc);
+      c.y = c.e < 0 ? 0.0f : i2f_scaled(buf.Y[e], sc);
+      c.l2 = c.x * c.x + c.y * c.y;
+    };
+    __syncwarp();
+    load(c0, lane);
+    load(c1, lane + 32);
+    const int q0 = c0.e < 0 ? INT_MAX : __float_as_int(c0.l2), q1 = c1.e < 0 ? INT_MAX : __float_as_int(c1.l2);
+    const int q = __reduce_min_sync(0xffffffffu, min(q0, q1));
+    if (q == INT_MAX) return 0;
+    const unsigned b0 = __ballot_sync(0xffffffffu, q0 == q), b1 = __ballot_sync(0xffffffffu, q1 == q);
+    int mine = 0;
+    float R4 = 0.0f;
+    const int m = wrap_ring(b0 ? __ffs(b0) - 1 : 32 + __ffs(b1) - 1, c0, c1, buf.X, buf.Y, buf.tag, ikey, sc,
+                            R.inv_scale, lane, mine, R4);
+    if (m < 3) return 0;
+    gid = buf.id[mine];
+    gkey = buf.tag[mine];
+    n = m;
+    const float need = R4 * (1.0f + 1e-3f);
+    do {
+      // every unseen cell is farther than k bins from cell i
+      const float reach = k * bs;
+      if (reach * reach > need) return m;
+      if (++k > kmax) return 0;
+      if (n == m) {  // the ring to the front of the buffer
+        const long long mX = buf.X[mine], mY = buf.Y[mine];
+        __syncwarp();
+        if (lane < m) {
+          buf.X[lane] = mX;
+          buf.Y[lane] = mY;
+          buf.id[lane] = gid;
+          buf.tag[lane] = gkey;
+        }
+        mine = lane < m ? lane : 0;
+        __syncwarp();
+      }
+      for (int base = 0; base < 8 * k; base += 32) {
+        int cnt = 0, bn = 0, j = 0;
+        int4 f = make_int4(0, 0, 0, 0);
+        if (base + lane < 8 * k) {
+          int dx, dy;
+          ring_bin(k, base + lane, dx, dy);
+          bn = bin_at(R, bxi, byi, dx, dy);
+          cnt = g.bins.count[bn];
+          f = g.bins.slot[bn];
+        }
+        const int most = __reduce_max_sync(0xffffffffu, cnt);
+        for (int t = 0; t < most; ++t) {
+          bool keep = false;
+          long long dX = 0, dY = 0;
+          if (t < cnt) {
+            j = bin_cell(g.bins, bn, f, t, j);
+            dX = min_image_i(X[j] - Xi, R.LX);
+            dY = min_image_i(Y[j] - Yi, R.LY);
+            const float dx = i2f_scaled(dX, sc), dy = i2f_scaled(dY, sc);
+            keep = dx * dx + dy * dy <= need;
+          }
+          const unsigned mask = __ballot_sync(0xffffffffu, keep);
+          if (n + __popc(mask) > kCand) return 0;
+          if (keep) {
+            const int e = n + __popc(mask & ((1u << lane) - 1u));
+            buf.id[e] = j;
+            buf.tag[e] = g.tag[j];
+            buf.X[e] = dX;
+            buf.Y[e] = dY;
+          }
+          n += __popc(mask);
+        }
+      }
+    } while (n == m);  // no new candidate: the ring stands, look farther out
+  }
+}
+
+// One warp per cell.  Bound by latency in a step (a few to a few thousand
+// cells: list entry, cell, replica, bins, candidates, then the ring), by
+// instruction issue when every cell is triangulated.
 __global__ void __launch_bounds__(kRepairWarps * 32) k_repair(RepairArgs g) {
-  __shared__ int s_id[kRepairWarps][kCand];
-  __shared__ long long s_X[kRepairWarps][kCand], s_Y[kRepairWarps][kCand];
-  __shared__ float s_d2[kRepairWarps][kCand];
-  __shared__ int s_tag[kRepairWarps][kCand];  // perturbation keys, loaded with the positions
+  __shared__ CandBuf s_buf[kRepairWarps];
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   const int gw = blockIdx.x * kRepairWarps + wib, nw = gridDim.x * kRepairWarps;
   // stop the round loop unless this round's check asks for another
@@ -313,6 +653,10 @@ __global__ void __launch_bounds__(kRepairWarps * 32) k_repair(RepairArgs g) {
   const int which_in = g.dyn ? (g.ctl->round_count & 1) : g.which_in;
   const int* list_in = g.dyn ? (which_in ? g.lists[1] : g.lists[0]) : g.list_in;
   const int total = g.all_cells ? g.n : g.ctl->count[which_in];
+  if (g.record && blockIdx.x == 0 && threadIdx.x == 0) {
+    g.ctl->last_flagged = total;
+    g.ctl->flagged_total += total;
+  }
   // the list this round's check fills must start empty
   if (!g.all_cells && blockIdx.x == 0 && threadIdx.x == 0) g.ctl->count[which_in ^ 1] = 0;
   if (total == 0) return;
@@ -327,129 +671,22 @@ __global__ void __launch_bounds__(kRepairWarps * 32) k_repair(RepairArgs g) {
 
   for (int item = gw; item < total; item += nw) {
     const int i = g.all_cells ? item : list_in[item];
-    const Rep R = g.reps[g.rep[i]];
-    const long long Xi = X[i], Yi = Y[i];
-    const int ikey = g.tag[i];
-    const float sc = (float)R.inv_scale;
+    const Rep& R = g.reps[g.rep[i]];
     // keep the old ring for the consistency check
     const int oc = g.cnt[i];
     if (lane < CG_RING) g.old_nbr[(size_t)i * CG_RING + lane] = g.nbr[(size_t)i * CG_RING + lane];
     if (lane == 0) g.old_cnt[i] = oc;
 
-    // initial polygon: the square of half-width W (vertices (+-W, +-W)), cut
-    // out by four phantom generators at (+-2W, 0) and (0, +-2W)
-    Poly p;
-    p.m = 4;
-    p.err = 0;
-    p.gX = (lane == 0) ? R.W2 : (lane == 2 ? -R.W2 : 0);
-    p.gY = (lane == 1) ? R.W2 : (lane == 3 ? -R.W2 : 0);
-    p.gid = -1 - (lane & 3);
-    p.gkey = kPhantomKey + (lane & 3);
-    {
-      const float W = 0.5f * i2f_scaled(R.W2, sc);  // power of two: exact
-      p.r2 = 2.0f * W * W;
-      p.R2 = p.r2;
-    }
-    int bxi, byi;
-    bin_of_grid(R, Xi, Yi, bxi, byi);
-    const float bs = (float)R.bsx;  // every bin is at least this wide
-    const int kmax = min((R.nbx - 1) / 2, (R.nby - 1) / 2);
-    int nbuf = 0;
-    bool done = false;
-    // rings 0..2 (25 bins) are gathered in one pass, one bin per lane, unless
-    // they hold more candidates than the buffer; then ring by ring
-    bool batch = kmax >= 2;
-    for (int k = 0; k <= kmax && !done && !p.err; ++k) {
-      const bool first = batch && k == 0;
-      const int nring = first ? 25 : ((k == 0) ? 1 : 8 * k);
-      bool retry = false;
-      for (int base = 0; base < nring && !p.err; base += 32) {
-        const int idx = base + lane;
-        int start = 0, count = 0;
-        if (idx < nring) {
-          int dx, dy;
-          if (first) ring_bin(idx == 0 ? 0 : (idx <= 8 ? 1 : 2), idx == 0 ? 0 : (idx <= 8 ? idx - 1 : idx - 9), dx, dy);
-          else ring_bin(k, idx, dx, dy);
-          int bx = bxi + dx, by = byi + dy;
-          bx += (bx < 0) ? R.nbx : (bx >= R.nbx ? -R.nbx : 0);
-          by += (by < 0) ? R.nby : (by >= R.nby ? -R.nby : 0);
-          const int b = R.bin0 + by * R.nbx + bx;
-          start = bin_begin(g.bin_start, g.bin_partials, b);
-          count = bin_begin(g.bin_start, g.bin_partials, b + 1) - start;
-        }
-        int incl = count;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const int t = __shfl_up_sync(0xffffffffu, incl, o);
-          if (lane >= o) incl += t;
-        }
-        const int tot = __shfl_sync(0xffffffffu, incl, 31);
-        if (first && tot > kCand) {
-          retry = true;
-          break;
-        }
-        if (nbuf + tot > kCand) {
-          process_candidates(p, nbuf, s_id[wib], s_X[wib], s_Y[wib], s_d2[wib], s_tag[wib],
-                             ikey, sc, R.inv_scale, lane);
-          nbuf = 0;
-          if (tot > kCand) p.err = kECAND;
-        }
-        if (!p.err) {
-          int slot = nbuf + incl - count;
-          bool same = false;  // another cell on exactly this grid point
-          for (int t = 0; t < count; ++t) {
-            const int j = g.ids[start + t];
-            s_tag[wib][slot] = g.tag[j];
-            if (j == i) {
-              s_d2[wib][slot] = kSelfKey;  // never clips
-              s_id[wib][slot] = j;
-              s_X[wib][slot] = 0;
-              s_Y[wib][slot] = 0;
-            } else {
-              const long long dX = min_image_i(X[j] - Xi, R.LX), dY = min_image_i(Y[j] - Yi, R.LY);
-              same |= (dX == 0 && dY == 0);
-              const float dx = i2f_scaled(dX, sc), dy = i2f_scaled(dY, sc);
-              s_d2[wib][slot] = dx * dx + dy * dy;
-              s_id[wib][slot] = j;
-              s_X[wib][slot] = dX;
-              s_Y[wib][slot] = dY;
-            }
-            ++slot;
-          }
-          nbuf += tot;
-          if (__any_sync(0xffffffffu, same)) p.err = kEDEGEN;  // no bisector between them
-        }
-        __syncwarp();
-      }
-      if (retry) {  // the ring-by-ring gathering from ring 0
-        batch = false;
-        k = -1;
-        continue;
-      }
-      if (p.err) break;
-      if (first) k = 2;  // rings 1 and 2 are in the batch
-      // rings 0..2 are gathered into one batch before clipping
-      if (k < 2 && k < kmax) continue;
-      process_candidates(p, nbuf, s_id[wib], s_X[wib], s_Y[wib], s_d2[wib], s_tag[wib], ikey,
-                         sc, R.inv_scale, lane);
-      nbuf = 0;
-      // every unvisited cell is farther than k*bs from cell i
-      const float reach = k * bs;
-      if (reach * reach > 4.0f * p.R2 * (1.0f + 1e-3f)) done = true;
-    }
-    int err = p.err;
-    if (!err && !done) err = kEBOX;
-    if (!err) {
-      const unsigned ph = __ballot_sync(0xffffffffu, lane < p.m && p.gid < 0);
-      if (ph) err = kEBOX;
-      if (p.m > CG_RING) err = kERING;
-    }
-    if (err) {
-      if (lane == 0) raise_status(g.ctl, err);
+    int gid = -1, gkey = INT_MAX;
+    int m = gift_ring(g, R, X, Y, i, s_buf[wib], lane, gid, gkey);
+    __syncwarp();
+    if (m == 0) m = clip_ring(g, R, X, Y, i, s_buf[wib], lane, gid, gkey);
+    if (m < 0) {
+      if (lane == 0) raise_status(g.ctl, m);
       continue;
     }
     // canonical CCW ring: start at the smallest tag
-    int kmin = (lane < p.m) ? p.gkey : INT_MAX;
+    int kmin = (lane < m) ? gkey : INT_MAX;
     int lmin = lane;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -457,20 +694,21 @@ __global__ void __launch_bounds__(kRepairWarps * 32) k_repair(RepairArgs g) {
       const int ol = __shfl_xor_sync(0xffffffffu, lmin, o);
       if (ok < kmin || (ok == kmin && ol < lmin)) { kmin = ok; lmin = ol; }
     }
-    if (lane < p.m) {
-      const int slot = (lane - lmin + p.m) % p.m;
-      g.nbr[(size_t)i * CG_RING + slot] = p.gid;
+    if (lane < m) {
+      const int slot = (lane - lmin + m) % m;
+      g.nbr[(size_t)i * CG_RING + slot] = gid;
     } else if (lane < CG_RING) {
       g.nbr[(size_t)i * CG_RING + lane] = -1;
     }
     if (lane == 0) {
-      g.cnt[i] = p.m;
+      g.cnt[i] = m;
       atomicAnd(&g.flags[i >> 5], ~(1u << (i & 31)));
       if (g.dirty_list && !g.all_cells) {
         const unsigned bit = 1u << (i & 31);
         if (!(atomicOr(&g.dirty_bits[i >> 5], bit) & bit)) g.dirty_list[atomicAdd(&g.ctl->dirty_count, 1)] = i;
       }
     }
+    __syncwarp();
   }
 }
 

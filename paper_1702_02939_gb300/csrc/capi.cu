@@ -458,7 +458,7 @@ int geom_grid(const cg_ctx* c) { return sm_count() * c->launch.geom_blocks_per_s
 int test_grid(const cg_ctx* c) { return sm_count() * c->launch.test_blocks_per_sm; }  // 0: full
 // Full triangulation: one warp per cell over every cell.
 int repair_grid_all(const cg_ctx*) { return sm_count() * 16; }
-int check_grid_all(const cg_ctx* c) { return (int)((c->N + 255) / 256); }
+int check_grid_all(const cg_ctx* c) { return check_blocks_all((int)c->N, sm_count()); }
 
 // One time step, enqueued on stream st (also used for capture).
 // One step as captured into the step graph.  When a step starts, the move of

@@ -212,7 +212,7 @@ extern "C" int cg_triangulate_noalloc(int32_t n, double Lx, double Ly, const dou
   ck.which_out = 1;
   ck.last_round = 1;
   ck.all_cells = 1;
-  launch_check(ck, (n + 255) / 256, st);
+  launch_check(ck, check_blocks_all(n, sms), st);
 
   launch_gather_ring(n, tag, cnt, nbr, d_cnt, d_nbr, st);
   if (cudaGetLastError() != cudaSuccess) return CG_ECUDA;

@@ -216,6 +216,15 @@ int fail(cg_ctx* c, int code, const std::string& msg) {
       return fail(ctx, CG_ECUDA, std::string(#call) + ": " + cudaGetErrorString(e_));      \
   } while (0)
 
+// Ring-size grouping of the cells for the geometry and force kernels (always
+// a permutation of the cells, so a stale one is only slower, never wrong).
+const int* order_for(const cg_ctx* c, int bit) {
+  return (c->launch.ring_order & bit) ? c->at<int>(c->off.order) : nullptr;
+}
+void run_order(cg_ctx* c, cudaStream_t st) {
+  launch_order((int)c->N, c->at<int>(c->off.cnt), c->at<int>(c->off.order), st);
+}
+
 GeomArgs geom_args(cg_ctx* c) {
   GeomArgs g{};  // every field starts zero or null
   g.n = (int)c->N;
@@ -241,7 +250,7 @@ GeomArgs geom_args(cg_ctx* c) {
   g.list_count = nullptr;
   g.list_bits = nullptr;
   g.tolerant = 0;
-  g.order = (c->launch.ring_order & 1) ? c->at<int>(c->off.order) : nullptr;
+  g.order = order_for(c, 1);
   return g;
 }
 
@@ -272,14 +281,8 @@ ForceArgs force_args(cg_ctx* c, int integrate) {
   f.seed = c->par.seed;
   f.nrm = c->at<double2>(c->off.nrm);
   f.xi = c->at<double>(c->off.xi);
-  f.order = (c->launch.ring_order & 2) ? c->at<int>(c->off.order) : nullptr;
+  f.order = order_for(c, 2);
   return f;
-}
-
-// Ring-size grouping of the cells for the geometry and force kernels (always
-// a permutation of the cells, so a stale one is only slower, never wrong).
-void run_order(cg_ctx* c, cudaStream_t st) {
-  launch_order((int)c->N, c->at<int>(c->off.cnt), c->at<int>(c->off.order), st);
 }
 
 DirArgs dir_args(cg_ctx* c) {
@@ -332,7 +335,7 @@ TestArgs test_args(cg_ctx* c) {
   t.tag = c->at<int>(c->off.tag);
   t.flags = c->at<unsigned>(c->off.flags);
   t.list = c->at<int>(c->off.list0);
-  t.order = (c->launch.ring_order & 4) ? c->at<int>(c->off.order) : nullptr;
+  t.order = order_for(c, 4);
   return t;
 }
 
@@ -463,24 +466,24 @@ int check_grid_all(const cg_ctx* c) { return check_blocks_all((int)c->N, sm_coun
 // One time step, enqueued on stream st (also used for capture).
 // One step as captured into the step graph.  When a step starts, the move of
 // Eq. 3 from the current state is already computed (the "pending move", in
-// the other position buffer): the step makes it current, then runs three
-// branches — the circumcircle test, the cell-list build, and, at low
-// priority, the director terms (rotation by the previous noise, n(theta),
+// the other position buffer): the step makes it current, then runs two
+// branches — the circumcircle test and the cell list (one kernel for small
+// systems, two side by side for large ones), and, at low priority, the
+// director terms (rotation by the previous noise, n(theta),
 // new noise) followed by the geometry and force sets of the new positions,
 // which overlaps the latency-bound repair rounds (rings rewritten meanwhile
 // are recomputed by the fix-up after the rounds) — and ends with the forces
 // and the next pending move, while the force sets are still in L2.  With
-// dir_beside_geom the director terms take a fourth branch and run beside the
+// dir_beside_geom the director terms take a third branch and run beside the
 // geometry instead of before it.
 void enqueue_step_prefix(cg_ctx* c, cudaStream_t st) {
   launch_begin_topology(c->ctl(), 1, st);
   cudaEventRecord(c->fork, st);
   cudaStreamWaitEvent(c->side[0], c->fork, 0);
-  cudaStreamWaitEvent(c->side[1], c->fork, 0);
   if (c->launch.dir_beside_geom) {
-    cudaStreamWaitEvent(c->side[2], c->fork, 0);
-    run_dir(c, dir_args_step(c), c->side[2], dir_grid(c));
-    cudaEventRecord(c->join_terms, c->side[2]);
+    cudaStreamWaitEvent(c->side[1], c->fork, 0);
+    run_dir(c, dir_args_step(c), c->side[1], dir_grid(c));
+    cudaEventRecord(c->join_terms, c->side[1]);
   } else {
     run_dir(c, dir_args_step(c), c->side[0], dir_grid(c));
   }
@@ -498,9 +501,16 @@ void enqueue_step_prefix(cg_ctx* c, cudaStream_t st) {
     run_force(c, f, c->side[0]);
   }
   cudaEventRecord(c->join_dir, c->side[0]);
-  launch_cell_list(cell_list_args(c), c->side[1]);
-  cudaEventRecord(c->join_list, c->side[1]);
-  launch_test(test_args(c), st, test_grid(c));
+  TestArgs t = test_args(c);
+  if (c->N <= kTestSlotCells) {  // the test fills the cell list on the way
+    t.bins = bin_arrays(c);
+    launch_test(t, st, test_grid(c));
+    return;
+  }
+  cudaStreamWaitEvent(c->side[2], c->fork, 0);
+  launch_cell_list(cell_list_args(c), c->side[2]);
+  cudaEventRecord(c->join_list, c->side[2]);
+  launch_test(t, st, test_grid(c));
   cudaStreamWaitEvent(st, c->join_list, 0);
 }
 
@@ -817,15 +827,15 @@ int cg_create(int32_t R, const cg_replica* reps, const cg_params* params, const 
   c->stream = static_cast<cudaStream_t>(stream);
   int rc = CG_OK;
   do {
-    // the critical path (capture stream, cell-list branch) at the highest
+    // the critical path (capture stream, cell list) at the highest
     // priority, the director branch at the lowest; the priorities take effect
     // when the graph is instantiated with node priorities (dir_low_priority)
     int lo = 0, hi = 0;
     cudaError_t e = cudaDeviceGetStreamPriorityRange(&lo, &hi);
     if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&c->capture, cudaStreamNonBlocking, hi);
     if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&c->side[0], cudaStreamNonBlocking, lo);
-    if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&c->side[1], cudaStreamNonBlocking, hi);
-    if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&c->side[2], cudaStreamNonBlocking, lo);
+    if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&c->side[1], cudaStreamNonBlocking, lo);
+    if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&c->side[2], cudaStreamNonBlocking, hi);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->fork, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->join_dir, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->join_list, cudaEventDisableTiming);

@@ -16,6 +16,10 @@ constexpr int kSlotWarps = 8;       // warps of a block that takes 32 cells, one
 constexpr int kSlotThreads = 32 * kSlotWarps;
 constexpr int kGeomSlotBlocks = 6;      // resident blocks per SM that k_geom_slots is compiled for
 constexpr int kGeomSlotCells = 155648;  // up to here (1024 cells per SM) k_geom_slots takes all cells
+constexpr int kForceSlotBlocks = 6, kTestSlotBlocks = 6, kGeomF32SlotBlocks = 5, kForceF32SlotBlocks = 8;
+// the force and test passes, and the single-precision geometry, take their
+// slot kernels while every cell is resident at once: 152 SMs x 6 blocks x 32
+constexpr int kForceSlotCells = 29184, kTestSlotCells = 29184, kGeomF32SlotCells = 29184;
 constexpr int kForceThreads = 128;
 constexpr int kTestThreads = 128;
 constexpr int kRepairWarps = 4;  // warps per repair block
@@ -130,6 +134,13 @@ void launch_init_dir_tables(double2* tab, cudaStream_t st);
 void launch_dir_terms(int n, const double* theta, const int* tag, unsigned long long seed, long long step,
                       const double2* tab, double* cs, double* sn, double* xi, cudaStream_t st);
 
+// The cell list's arrays (see kBinCap in cg_device.cuh).
+struct BinArrays {
+  int* count;  // [bins] cells per bin, zero before a build
+  int4* slot;  // [bins] the first kBinCap cells
+  int* head;   // [bins] newest cell past those
+  int* next;   // [n] chain links
+};
 struct TestArgs {
   int n;
   const Rep* reps;
@@ -140,15 +151,9 @@ struct TestArgs {
   unsigned* flags;
   int* list;  // list 0
   const int* order;  // processing order of the cells (as GeomArgs), or null
+  BinArrays bins;    // the cell list filled on the way (counts zero before; up to kTestSlotCells), or null arrays
 };
 
-// The cell list's arrays (see kBinCap in cg_device.cuh).
-struct BinArrays {
-  int* count;  // [bins] cells per bin, zero before a build
-  int4* slot;  // [bins] the first kBinCap cells
-  int* head;   // [bins] newest cell past those
-  int* next;   // [n] chain links
-};
 struct CellListArgs {
   int n;
   const Rep* reps;

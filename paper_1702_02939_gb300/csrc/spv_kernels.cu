@@ -338,9 +338,9 @@ __device__ __forceinline__ bool net_force(const ForceArgs& g, int i, double& fx_
     const double Gx = f0.x + f1.x + f2.x, Gy = f0.y + f1.y + f2.y;
     const double2 s = g.s[a * N + i];
     const double wx = i2d_int(bY - aY, -1), wy = i2d_int(aX - bX, -1);
-    const double c = wx * Gx + wy * Gy;
-    fx -= s.x * c;
-    fy -= s.y * c;
+    const double c = fma(wx, Gx, wy * Gy);
+    fx = fma(-s.x, c, fx);
+    fy = fma(-s.y, c, fy);
     j = k;
     pj = pk;
     aX = bX;
@@ -356,25 +356,9 @@ __device__ __forceinline__ bool net_force(const ForceArgs& g, int i, double& fx_
 }
 
 
-// Cell i's net force (integrate 0 or 1) and update of Eq. 3 (integrate 1),
-// or the update alone from the stored forces of the current positions
-// (integrate 2: after a change of v0).
-__device__ __forceinline__ void force_cell(const ForceArgs& g, int i) {
+// The update of Eq. 3 of cell i under the force (fx, fy).
+__device__ __forceinline__ void move_cell(const ForceArgs& g, int i, double fx, double fy) {
   const size_t N = (size_t)g.n;
-  double fx, fy;
-  if (g.integrate == 2) {
-    fx = g.Fx[i];
-    fy = g.Fy[i];
-  } else {
-    if (!net_force(g, i, fx, fy)) {
-      if (g.tolerant) claim_fix(g.fix_bits, g.fix_list, &g.ctl->force_count, i);
-      return;
-    }
-    g.Fx[i] = fx;
-    g.Fy[i] = fy;
-    if (!g.integrate) return;
-  }
-
   // Eq. 3: r <- r + dt (mu F + v0 n(theta)), rounded to the grid and wrapped
   // into the other position buffer; the director rotation
   // theta <- theta + sqrt(2 D_r dt) xi follows at the start of the next step
@@ -416,6 +400,104 @@ __device__ __forceinline__ void force_cell(const ForceArgs& g, int i) {
   g.y[(size_t)nxt * N + i] = i2d_int(Y, -R.q);
   g.X[(size_t)nxt * N + i] = X;
   g.Y[(size_t)nxt * N + i] = Y;
+}
+
+// Cell i's net force (integrate 0 or 1) and update of Eq. 3 (integrate 1),
+// or the update alone from the stored forces of the current positions
+// (integrate 2: after a change of v0).
+__device__ __forceinline__ void force_cell(const ForceArgs& g, int i) {
+  double fx, fy;
+  if (g.integrate == 2) {
+    fx = g.Fx[i];
+    fy = g.Fy[i];
+  } else {
+    if (!net_force(g, i, fx, fy)) {
+      if (g.tolerant) claim_fix(g.fix_bits, g.fix_list, &g.ctl->force_count, i);
+      return;
+    }
+    g.Fx[i] = fx;
+    g.Fy[i] = fy;
+    if (!g.integrate) return;
+  }
+  move_cell(g, i, fx, fy);
+}
+
+// The same with one thread per (cell, ring slot), as k_geom_slots: the slots'
+// triangles in parallel, their contributions added up in ring order by the
+// first warp (bit-identical to force_cell), which then moves the cells.  Rings
+// must not change meanwhile.
+__global__ void __launch_bounds__(kSlotThreads, kForceSlotBlocks) k_force_slots(ForceArgs g) {
+  __shared__ longlong2 s_off[CG_RING][32];  // neighbour offsets
+  __shared__ double2 s_s[CG_RING][32];      // Jacobian factors
+  __shared__ double s_c[CG_RING][32];       // w . G
+  __shared__ int s_j[CG_RING][32];          // neighbours
+  __shared__ int s_p[CG_RING][32];          // the cell's slot in the neighbour's ring, and the one before it
+  __shared__ int s_bad[32];
+  const int c = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const size_t N = (size_t)g.n;
+  const int cur = g.ctl->cur;
+  const long long* __restrict__ X = g.X + (size_t)cur * N;
+  const long long* __restrict__ Y = g.Y + (size_t)cur * N;
+  const int total = g.list ? *g.list_count : g.n;
+  for (int base = blockIdx.x * 32; base < total; base += gridDim.x * 32) {
+    const int item = base + c;
+    int i = 0, m = 0;
+    if (item < total) {
+      i = g.list ? g.list[item] : (g.order ? g.order[item] : item);
+      m = g.cnt[i];
+      if (w == 0) {
+        if (g.list_bits) atomicAnd(&g.list_bits[i >> 5], ~(1u << (i & 31)));
+        if (m < 3 || m > CG_RING) raise_status(g.ctl, kETOPO);
+      }
+      if (m < 3 || m > CG_RING) m = 0;
+    }
+    bool bad = false;
+    if (w == 0) s_bad[c] = 0;
+    if (w < m) {
+      const Rep& R = g.reps[g.rep[i]];
+      const int* ring = g.nbr + (size_t)i * CG_RING;
+      const long long Xi = X[i], Yi = Y[i], LX = R.LX, LY = R.LY;
+      for (int a = w; a < m; a += kSlotWarps) {
+        int j = ring[a];
+        const bool ok = (unsigned)j < (unsigned)g.n;
+        j = ok ? j : i;
+        const int mj = g.cnt[j], p = ring_pos(g.nbr, g.cnt, j, i);
+        bad |= !ok || p < 0;
+        // triangle (i, j, k) is the slot before i's around j and i's slot around k
+        s_p[a][c] = (p < 0 ? 0 : p) | ((p <= 0 ? (mj > 0 ? mj - 1 : 0) : p - 1) << 8);
+        s_j[a][c] = j;
+        s_off[a][c] = make_longlong2(min_image_i(X[j] - Xi, LX), min_image_i(Y[j] - Yi, LY));
+      }
+    }
+    __syncthreads();
+    if (bad) s_bad[c] = 1;
+    for (int a = w; a < m; a += kSlotWarps) {
+      const int an = a + 1 < m ? a + 1 : 0;
+      const double2 f0 = g.fs[a * N + i];
+      const double2 f1 = g.fs[(size_t)(s_p[a][c] >> 8) * N + s_j[a][c]];
+      const double2 f2 = g.fs[(size_t)(s_p[an][c] & 255) * N + s_j[an][c]];
+      s_s[a][c] = g.s[a * N + i];
+      const longlong2 A = s_off[a][c], B = s_off[an][c];
+      const double Gx = f0.x + f1.x + f2.x, Gy = f0.y + f1.y + f2.y;
+      const double wx = i2d_int(B.y - A.y, -1), wy = i2d_int(A.x - B.x, -1);
+      s_c[a][c] = fma(wx, Gx, wy * Gy);
+    }
+    __syncthreads();
+    if (w == 0 && m) {
+      if (s_bad[c]) raise_status(g.ctl, kETOPO);
+      double fx = 0.0, fy = 0.0;
+      for (int a = 0; a < m; ++a) {
+        const double2 sj = s_s[a][c];
+        const double cj = s_c[a][c];
+        fx = fma(-sj.x, cj, fx);
+        fy = fma(-sj.y, cj, fy);
+      }
+      g.Fx[i] = fx;
+      g.Fy[i] = fy;
+      if (g.integrate) move_cell(g, i, fx, fy);
+    }
+    __syncthreads();
+  }
 }
 
 // One thread per cell: the net force (integrate 0 or 1) and the update of
@@ -530,10 +612,35 @@ __device__ __forceinline__ void flag_cell(unsigned* flags, int* list, int* count
   if (!(old & bit)) list[atomicAdd(count, 1)] = c;
 }
 
-// One thread per cell: every edge (i, j_a) with i < j_a must be locally
+// Places cell i in the cell list of the step.
+__device__ __forceinline__ void bin_cell_at(const TestArgs& g, const Rep& R, long long X, long long Y, int i) {
+  int bx, by;
+  bin_of_grid(R, X, Y, bx, by);
+  bin_insert(g.bins, R.bin0 + by * R.nbx + bx, i);
+}
+
+// One ring slot of cell i: its edge (i, j_a) with i < j_a must be locally
 // Delaunay (the far vertex j_{a+1} outside the circle through i, j_{a-1}, j_a)
-// and every triangle owned by i (i its smallest index) positively oriented.
-// Failing quadruples/triangles flag all their cells.
+// and its triangle (i, j_a, j_{a+1}), where i is the smallest index,
+// positively oriented.  A failing quadruple or triangle flags all its cells.
+__device__ __forceinline__ void test_slot(const TestArgs& g, int i, int jp, int ja, int jn, float fpx, float fpy,
+                                          float fax, float fay, float fnx, float fny, long long pX, long long pY,
+                                          long long aX, long long aY, long long nX, long long nY, float sc) {
+  if (i >= ja) return;
+  if (incircle0_sign(fpx, fpy, fax, fay, fnx, fny, pX, pY, aX, aY, nX, nY, g.tag, i, jp, ja, jn, sc) > 0) {
+    flag_cell(g.flags, g.list, &g.ctl->count[0], i);
+    flag_cell(g.flags, g.list, &g.ctl->count[0], jp);
+    flag_cell(g.flags, g.list, &g.ctl->count[0], ja);
+    flag_cell(g.flags, g.list, &g.ctl->count[0], jn);
+  }
+  if (i < jn && orient0_sign(fax, fay, fnx, fny, aX, aY, nX, nY) <= 0) {
+    flag_cell(g.flags, g.list, &g.ctl->count[0], i);
+    flag_cell(g.flags, g.list, &g.ctl->count[0], ja);
+    flag_cell(g.flags, g.list, &g.ctl->count[0], jn);
+  }
+}
+
+// One thread per cell: every slot of its ring.
 __device__ __forceinline__ void test_cell(const TestArgs& g, int i, const long long* __restrict__ X,
                                           const long long* __restrict__ Y) {
   const Rep R = g.reps[g.rep[i]];
@@ -568,23 +675,7 @@ __device__ __forceinline__ void test_cell(const TestArgs& g, int i, const long l
     } else {
       jn = jfirst; nX = fX; nY = fY; fnx = ffx; fny = ffy;
     }
-    if (i < ja) {
-      // triangle (i, j_{a-1}, j_a) CCW; j_{a+1} must be outside its circle
-      int s = incircle0_sign(fpx, fpy, fax, fay, fnx, fny, pX, pY, aX, aY, nX, nY, g.tag, i, jp, ja, jn, sc);
-      if (s > 0) {
-        flag_cell(g.flags, g.list, &g.ctl->count[0], i);
-        flag_cell(g.flags, g.list, &g.ctl->count[0], jp);
-        flag_cell(g.flags, g.list, &g.ctl->count[0], ja);
-        flag_cell(g.flags, g.list, &g.ctl->count[0], jn);
-      }
-    }
-    if (i < ja && i < jn) {
-      if (orient0_sign(fax, fay, fnx, fny, aX, aY, nX, nY) <= 0) {
-        flag_cell(g.flags, g.list, &g.ctl->count[0], i);
-        flag_cell(g.flags, g.list, &g.ctl->count[0], ja);
-        flag_cell(g.flags, g.list, &g.ctl->count[0], jn);
-      }
-    }
+    test_slot(g, i, jp, ja, jn, fpx, fpy, fax, fay, fnx, fny, pX, pY, aX, aY, nX, nY, sc);
     jp = ja; pX = aX; pY = aY; fpx = fax; fpy = fay;
     ja = jn; aX = nX; aY = nY; fax = fnx; fay = fny;
   }
@@ -599,6 +690,56 @@ __global__ void __launch_bounds__(kTestThreads) k_test(TestArgs g) {
   const long long* __restrict__ Y = g.Y + (size_t)cur * N;
   for (int item = blockIdx.x * kTestThreads + threadIdx.x; item < g.n; item += gridDim.x * kTestThreads)
     test_cell(g, g.order ? g.order[item] : item, X, Y);
+}
+
+// The same with one thread per (cell, ring slot), as k_geom_slots: offsets and
+// their float values pass between slots through shared memory; the first warp
+// places the cells in the cell list.
+__global__ void __launch_bounds__(kSlotThreads, kTestSlotBlocks) k_test_slots(TestArgs g) {
+  __shared__ longlong2 s_off[CG_RING][32];
+  __shared__ float2 s_f[CG_RING][32];
+  __shared__ int s_j[CG_RING][32];
+  const int c = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const size_t N = (size_t)g.n;
+  const int cur = g.ctl->cur;
+  const long long* __restrict__ X = g.X + (size_t)cur * N;
+  const long long* __restrict__ Y = g.Y + (size_t)cur * N;
+  for (int base = blockIdx.x * 32; base < g.n; base += gridDim.x * 32) {
+    const int item = base + c;
+    int i = 0, m = 0;
+    float sc = 0.0f;
+    if (item < g.n) {
+      i = g.order ? g.order[item] : item;
+      m = g.cnt[i];
+      const Rep& R = g.reps[g.rep[i]];
+      sc = (float)R.inv_scale;
+      const long long Xi = X[i], Yi = Y[i], LX = R.LX, LY = R.LY;
+      if (w == 0) {
+        if (g.bins.count) bin_cell_at(g, R, Xi, Yi, i);
+        if (m < 3 || m > CG_RING) raise_status(g.ctl, kETOPO);
+      }
+      if (m < 3 || m > CG_RING) m = 0;
+      const int* ring = g.nbr + (size_t)i * CG_RING;
+      for (int a = w; a < m; a += kSlotWarps) {
+        const int j = ring[a];
+        const long long dX = min_image_i(X[j] - Xi, LX), dY = min_image_i(Y[j] - Yi, LY);
+        s_j[a][c] = j;
+        s_off[a][c] = make_longlong2(dX, dY);
+        s_f[a][c] = make_float2(i2f_scaled(dX, sc), i2f_scaled(dY, sc));
+      }
+    }
+    __syncthreads();
+    for (int a = w; a < m; a += kSlotWarps) {
+      const int p = a > 0 ? a - 1 : m - 1, n = a + 1 < m ? a + 1 : 0;
+      const int ja = s_j[a][c];
+      if (i >= ja) continue;
+      const float2 fp = s_f[p][c], fa = s_f[a][c], fn = s_f[n][c];
+      const longlong2 op = s_off[p][c], oa = s_off[a][c], on = s_off[n][c];
+      test_slot(g, i, s_j[p][c], ja, s_j[n][c], fp.x, fp.y, fa.x, fa.y, fn.x, fn.y, op.x, op.y, oa.x, oa.y, on.x,
+                on.y, sc);
+    }
+    __syncthreads();
+  }
 }
 
 // Ring-size grouping of each chunk of kOrderChunk cells (see launch_order):
@@ -665,6 +806,15 @@ void launch_geom(const GeomArgs& a, cudaStream_t st, int blocks) {
 }
 void launch_force(const ForceArgs& a, cudaStream_t st, int blocks) {
   if (a.n <= 0) return;
+  // While all cells fit on the chip at once, a warp per slot shortens the chain
+  // of gathers (one pass, us: 14.3 -> 9.4 at 256 cells, 14.3 -> 10.2 at 4096,
+  // 16.4 -> 12.3 at 16384); beyond, the lanes that idle in the last slots and
+  // the barriers cost more (18.4 -> 24.6 at 65536).
+  if (!a.tolerant && a.integrate != 2 && (a.list || a.n <= kForceSlotCells)) {
+    const int full = (a.n + 31) / 32;
+    k_force_slots<<<(blocks > 0 && blocks < full) ? blocks : full, kSlotThreads, 0, st>>>(a);
+    return;
+  }
   const int full = (a.n + kForceThreads - 1) / kForceThreads;
   k_force<<<(blocks > 0 && blocks < full) ? blocks : full, kForceThreads, 0, st>>>(a);
 }
@@ -674,6 +824,13 @@ void launch_force_fix_list(const ForceFixArgs& a, int blocks, cudaStream_t st) {
 void launch_begin_topology(Ctl* ctl, int flip, cudaStream_t st) { k_begin_topology<<<1, 1, 0, st>>>(ctl, flip); }
 void launch_test(const TestArgs& a, cudaStream_t st, int blocks) {
   if (a.n <= 0) return;
+  // As for the force: 13.6 -> 11.4 us at 1024 cells (cell list included),
+  // 16.9 -> 14.0 at 16384, 18.5 -> 19.4 at 65536.
+  if (a.n <= kTestSlotCells) {
+    const int full = (a.n + 31) / 32;
+    k_test_slots<<<(blocks > 0 && blocks < full) ? blocks : full, kSlotThreads, 0, st>>>(a);
+    return;
+  }
   const int full = (a.n + kTestThreads - 1) / kTestThreads;
   k_test<<<(blocks > 0 && blocks < full) ? blocks : full, kTestThreads, 0, st>>>(a);
 }

@@ -51,6 +51,37 @@ __device__ __forceinline__ float det_f(long long ax, long long ay, long long bx,
   return neg ? -f : f;
 }
 
+// The circumcentre (relative to the cell) of its neighbours a and b and the
+// Jacobian factor h / det; l: squared lengths of a and b.
+__device__ __forceinline__ void vertex_f(long long gax, long long gay, long long gbx, long long gby, float ax, float ay,
+                                         float la, float bx, float by, float lb, float sc, float2& h, float2& s) {
+  const float r = 1.0f / det_f(gax, gay, gbx, gby, sc);  // 1 / ((r_j - r_i) x (r_k - r_i))
+  const float hr = 0.5f * r;
+  h = make_float2(fmaf(by, la, -(ay * lb)) * hr, fmaf(ax, lb, -(bx * la)) * hr);
+  s = make_float2(h.x * r, h.y * r);
+}
+
+// The edge from vertex hp to h: (squared length, inverse length) and its unit
+// vector; a zero-length edge has no direction.
+__device__ __forceinline__ void edge_f(float2 h, float2 hp, float2& l, float2& e) {
+  const float ex = h.x - hp.x, ey = h.y - hp.y;
+  const float l2 = fmaf(ex, ex, ey * ey);
+  const float il = l2 > 0.f ? rsqrtf(l2) : 0.f;
+  l = make_float2(l2, il);
+  e = make_float2(ex * il, ey * il);
+}
+
+// A, P and the energy of cell i from its accumulated sums; returns (ka, kp).
+__device__ __forceinline__ float2 cell_f(const GeomArgs& g, int i, float area, float per) {
+  const float A = 0.5f * area, P = per;
+  g.A[i] = A;
+  g.P[i] = P;
+  const float dA = A - (float)g.A0, dP = P - (float)(g.p0[i] * g.sqrtA0);
+  if (g.energy_out) g.energy_out[i] = (double)fmaf((float)g.KA * dA, dA, (float)g.KP * dP * dP);
+  // dA/dh = 1/2 perp(h_next - h_prev); dP/dh = e_in - e_out
+  return make_float2((float)g.KA * dA, 2.0f * (float)g.KP * dP);
+}
+
 }  // namespace
 
 // One thread per cell (grid-stride; optional list of cells; tolerant mode for
@@ -68,12 +99,8 @@ __global__ void __launch_bounds__(kGeomThreads) k_geom_f32(GeomArgs g) {
   float2* fs = as_f2(g.fs);
   float2* sv = as_f2(g.s);
   float2* wv = as_f2(g.w);
-  const int total = g.list ? *g.list_count : g.n;
-  if (g.clear)
-    for (int k = blockIdx.x * kGeomThreads + t; k < g.n_clear; k += gridDim.x * kGeomThreads) g.clear[k] = 0;
-  for (int item = blockIdx.x * kGeomThreads + t; item < total; item += gridDim.x * kGeomThreads) {
-    const int i = g.list ? g.list[item] : (g.order ? g.order[item] : item);
-    if (g.list_bits) atomicAnd(&g.list_bits[i >> 5], ~(1u << (i & 31)));
+  for (int item = blockIdx.x * kGeomThreads + t; item < g.n; item += gridDim.x * kGeomThreads) {
+    const int i = g.order ? g.order[item] : item;
     const Rep R = g.reps[g.rep[i]];
     const float sc = (float)R.inv_scale;
     const long long Xi = X[i], Yi = Y[i];
@@ -90,7 +117,7 @@ __global__ void __launch_bounds__(kGeomThreads) k_geom_f32(GeomArgs g) {
     long long g0x, g0y;
     float d0x, d0y;
     rel_f(R, X, Y, Xi, Yi, nb(0), sc, g0x, g0y, d0x, d0y);
-    const float l0 = d0x * d0x + d0y * d0y;
+    const float l0 = fmaf(d0x, d0x, d0y * d0y);
     float ax = d0x, ay = d0y, la = l0;
     long long gax = g0x, gay = g0y;
     float hpx = 0.f, hpy = 0.f, h0x = 0.f, h0y = 0.f;
@@ -100,51 +127,42 @@ __global__ void __launch_bounds__(kGeomThreads) k_geom_f32(GeomArgs g) {
       long long gbx, gby;
       if (a + 1 < m) {
         rel_f(R, X, Y, Xi, Yi, nb(a + 1), sc, gbx, gby, bx, by);
-        lb = bx * bx + by * by;
+        lb = fmaf(bx, bx, by * by);
       } else {
         bx = d0x; by = d0y; lb = l0;
         gbx = g0x; gby = g0y;
       }
-      const float det = det_f(gax, gay, gbx, gby, sc);  // (r_j - r_i) x (r_k - r_i)
-      const float r = 1.0f / det;
-      const float hr = 0.5f * r;
-      const float hx = (by * la - ay * lb) * hr;  // circumcentre relative to r_i
-      const float hy = (ax * lb - bx * la) * hr;
-      sv[a * N + i] = make_float2(hx * r, hy * r);
+      float2 h, sj;
+      vertex_f(gax, gay, gbx, gby, ax, ay, la, bx, by, lb, sc, h, sj);
+      const float hx = h.x, hy = h.y;
+      sv[a * N + i] = sj;
       wv[a * N + i] = make_float2(by - ay, ax - bx);
       sh_hx[a][t] = hx;
       sh_hy[a][t] = hy;
       if (a == 0) {
         h0x = hx; h0y = hy;
       } else {
-        area += hpx * hy - hx * hpy;
-        const float ex = hx - hpx, ey = hy - hpy;
-        const float l2 = ex * ex + ey * ey;
-        const float il = l2 > 0.f ? rsqrtf(l2) : 0.f;  // a zero-length edge has no direction
-        per += l2 * il;
-        sh_ex[a][t] = ex * il;
-        sh_ey[a][t] = ey * il;
+        area += fmaf(hpx, hy, -(hx * hpy));
+        float2 l, e;
+        edge_f(h, make_float2(hpx, hpy), l, e);
+        per = fmaf(l.x, l.y, per);
+        sh_ex[a][t] = e.x;
+        sh_ey[a][t] = e.y;
       }
       hpx = hx; hpy = hy;
       ax = bx; ay = by; la = lb;
       gax = gbx; gay = gby;
     }
     {  // closing edge h_{m-1} -> h_0 is the incoming edge of vertex 0
-      area += hpx * h0y - h0x * hpy;
-      const float ex = h0x - hpx, ey = h0y - hpy;
-      const float l2 = ex * ex + ey * ey;
-      const float il = l2 > 0.f ? rsqrtf(l2) : 0.f;
-      per += l2 * il;
-      sh_ex[0][t] = ex * il;
-      sh_ey[0][t] = ey * il;
+      area += fmaf(hpx, h0y, -(h0x * hpy));
+      float2 l, e;
+      edge_f(make_float2(h0x, h0y), make_float2(hpx, hpy), l, e);
+      per = fmaf(l.x, l.y, per);
+      sh_ex[0][t] = e.x;
+      sh_ey[0][t] = e.y;
     }
-    const float A = 0.5f * area, P = per;
-    g.A[i] = A;
-    g.P[i] = P;
-    const float dA = A - (float)g.A0, dP = P - (float)(g.p0[i] * g.sqrtA0);
-    if (g.energy_out) g.energy_out[i] = (double)((float)g.KA * dA * dA + (float)g.KP * dP * dP);
-    // dA/dh = 1/2 perp(h_next - h_prev); dP/dh = e_in - e_out
-    const float ka = (float)g.KA * dA, kp = 2.0f * (float)g.KP * dP;
+    const float2 k = cell_f(g, i, area, per);
+    const float ka = k.x, kp = k.y;
     for (int a = 0; a < m; ++a) {
       const int ap = (a == 0) ? m - 1 : a - 1;
       const int an = (a + 1 == m) ? 0 : a + 1;
@@ -152,6 +170,93 @@ __global__ void __launch_bounds__(kGeomThreads) k_geom_f32(GeomArgs g) {
       const float dPx = sh_ex[a][t] - sh_ex[an][t], dPy = sh_ey[a][t] - sh_ey[an][t];
       fs[a * N + i] = make_float2(fmaf(ka, gx, kp * dPx), fmaf(ka, gy, kp * dPy));
     }
+  }
+}
+
+// The same pass with one thread per (cell, ring slot), as k_geom_slots.
+__global__ void __launch_bounds__(kSlotThreads, kGeomF32SlotBlocks) k_geom_f32_slots(GeomArgs g) {
+  __shared__ longlong2 s_off[CG_RING][32];  // neighbour offsets, exact
+  __shared__ float2 s_d[CG_RING][32];       // and rounded, then unit edge vectors
+  __shared__ float2 s_h[CG_RING][32];       // circumcentres
+  __shared__ float2 s_l[CG_RING][32];       // edge ending at the slot: squared length, inverse length
+  __shared__ float2 s_k[32];                // the cell's ka, kp
+  const int c = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const size_t N = (size_t)g.n;
+  const int cur = g.ctl->cur;
+  const long long* __restrict__ X = g.X + (size_t)cur * N;
+  const long long* __restrict__ Y = g.Y + (size_t)cur * N;
+  float2* fs = as_f2(g.fs);
+  float2* sv = as_f2(g.s);
+  float2* wv = as_f2(g.w);
+  const int total = g.list ? *g.list_count : g.n;
+  if (g.clear)
+    for (int k = blockIdx.x * kSlotThreads + threadIdx.x; k < g.n_clear; k += gridDim.x * kSlotThreads) g.clear[k] = 0;
+  for (int base = blockIdx.x * 32; base < total; base += gridDim.x * 32) {
+    const int item = base + c;
+    int i = 0, m = 0;
+    float sc = 0.f;
+    if (item < total) {
+      i = g.list ? g.list[item] : (g.order ? g.order[item] : item);
+      m = g.cnt[i];
+      if (w == 0) {
+        if (g.list_bits) atomicAnd(&g.list_bits[i >> 5], ~(1u << (i & 31)));
+        if ((m < 3 || m > CG_RING) && !g.tolerant) raise_status(g.ctl, kETOPO);
+      }
+      if (m < 3 || m > CG_RING) m = 0;
+    }
+    if (w < m) {
+      const Rep& R = g.reps[g.rep[i]];
+      sc = (float)R.inv_scale;
+      const int* ring = g.nbr + (size_t)i * CG_RING;
+      const long long Xi = X[i], Yi = Y[i], LX = R.LX, LY = R.LY;
+      for (int a = w; a < m; a += kSlotWarps) {
+        int j = ring[a];
+        j = ((unsigned)j < (unsigned)g.n) ? j : i;
+        const long long dX = min_image_i(X[j] - Xi, LX), dY = min_image_i(Y[j] - Yi, LY);
+        s_off[a][c] = make_longlong2(dX, dY);
+        s_d[a][c] = make_float2(i2f_scaled(dX, sc), i2f_scaled(dY, sc));
+      }
+    }
+    __syncthreads();
+    for (int a = w; a < m; a += kSlotWarps) {
+      const int an = a + 1 < m ? a + 1 : 0;
+      const longlong2 A = s_off[a][c], B = s_off[an][c];
+      const float2 da = s_d[a][c], db = s_d[an][c];
+      float2 h, sj;
+      vertex_f(A.x, A.y, B.x, B.y, da.x, da.y, fmaf(da.x, da.x, da.y * da.y), db.x, db.y,
+               fmaf(db.x, db.x, db.y * db.y), sc, h, sj);
+      sv[a * N + i] = sj;
+      wv[a * N + i] = make_float2(db.y - da.y, da.x - db.x);
+      s_h[a][c] = h;
+    }
+    __syncthreads();
+    for (int a = w; a < m; a += kSlotWarps) {
+      float2 l, e;
+      edge_f(s_h[a][c], s_h[a > 0 ? a - 1 : m - 1][c], l, e);
+      s_l[a][c] = l;
+      s_d[a][c] = e;
+    }
+    __syncthreads();
+    if (w == 0 && m) {
+      float area = 0.f, per = 0.f;
+      for (int a = 1; a <= m; ++a) {
+        const int b = a < m ? a : 0;
+        const float2 hp = s_h[a - 1][c], h = s_h[b][c], l = s_l[b][c];
+        area += fmaf(hp.x, h.y, -(h.x * hp.y));
+        per = fmaf(l.x, l.y, per);
+      }
+      s_k[c] = cell_f(g, i, area, per);
+    }
+    __syncthreads();
+    const float2 k = s_k[c];
+    for (int a = w; a < m; a += kSlotWarps) {
+      const int ap = a > 0 ? a - 1 : m - 1, an = a + 1 < m ? a + 1 : 0;
+      const float2 hp = s_h[ap][c], hn = s_h[an][c], e = s_d[a][c], en = s_d[an][c];
+      const float gx = hn.y - hp.y, gy = hp.x - hn.x;
+      const float dPx = e.x - en.x, dPy = e.y - en.y;
+      fs[a * N + i] = make_float2(fmaf(k.x, gx, k.y * dPx), fmaf(k.x, gy, k.y * dPy));
+    }
+    __syncthreads();
   }
 }
 
@@ -198,9 +303,9 @@ __device__ __forceinline__ bool net_force_f32(const ForceArgs& g, int i, float& 
     const float2 f2 = fs[(size_t)(pk < 0 ? 0 : pk) * N + k];
     const float Gx = f0.x + f1.x + f2.x, Gy = f0.y + f1.y + f2.y;
     const float2 s = sv[a * N + i], w = wv[a * N + i];
-    const float c = w.x * Gx + w.y * Gy;
-    fx -= s.x * c;
-    fy -= s.y * c;
+    const float c = fmaf(w.x, Gx, w.y * Gy);
+    fx = fmaf(-s.x, c, fx);
+    fy = fmaf(-s.y, c, fy);
     j = k;
     pj = pk;
   }
@@ -213,25 +318,10 @@ __device__ __forceinline__ bool net_force_f32(const ForceArgs& g, int i, float& 
   return true;
 }
 
-// Cell i's net force and, as in k_force, the move of Eq. 3 accumulated in
-// FP64 and rounded to the grid (integrate 2: the move alone from the stored
-// forces, which hold the FP32 values exactly).
-__device__ __forceinline__ void force_cell_f32(const ForceArgs& g, int i) {
+// The move of Eq. 3 of cell i under the force (fx, fy), accumulated in FP64 and
+// rounded to the grid.
+__device__ __forceinline__ void move_cell_f32(const ForceArgs& g, int i, float fx, float fy) {
   const size_t N = (size_t)g.n;
-  float fx, fy;
-  if (g.integrate == 2) {
-    fx = (float)g.Fx[i];
-    fy = (float)g.Fy[i];
-  } else {
-    if (!net_force_f32(g, i, fx, fy)) {
-      if (g.tolerant) claim_fix(g.fix_bits, g.fix_list, &g.ctl->force_count, i);
-      return;
-    }
-    g.Fx[i] = fx;
-    g.Fy[i] = fy;
-    if (!g.integrate) return;
-  }
-
   const int cur = g.ctl->cur;
   const Rep R = g.reps[g.rep[i]];
   const double xi = g.x[(size_t)cur * N + i], yi = g.y[(size_t)cur * N + i];
@@ -271,6 +361,92 @@ __device__ __forceinline__ void force_cell_f32(const ForceArgs& g, int i) {
   g.Y[(size_t)nxt * N + i] = Yn;
 }
 
+// Cell i's net force and, as in k_force, the move of Eq. 3 accumulated in
+// FP64 and rounded to the grid (integrate 2: the move alone from the stored
+// forces, which hold the FP32 values exactly).
+__device__ __forceinline__ void force_cell_f32(const ForceArgs& g, int i) {
+  float fx, fy;
+  if (g.integrate == 2) {
+    fx = (float)g.Fx[i];
+    fy = (float)g.Fy[i];
+  } else {
+    if (!net_force_f32(g, i, fx, fy)) {
+      if (g.tolerant) claim_fix(g.fix_bits, g.fix_list, &g.ctl->force_count, i);
+      return;
+    }
+    g.Fx[i] = fx;
+    g.Fy[i] = fy;
+    if (!g.integrate) return;
+  }
+  move_cell_f32(g, i, fx, fy);
+}
+
+// The same with one thread per (cell, ring slot), as k_force_slots.
+__global__ void __launch_bounds__(kSlotThreads, kForceF32SlotBlocks) k_force_f32_slots(ForceArgs g) {
+  __shared__ float2 s_s[CG_RING][32];  // Jacobian factors
+  __shared__ float s_c[CG_RING][32];   // w . G
+  __shared__ int s_j[CG_RING][32];     // neighbours
+  __shared__ int s_p[CG_RING][32];     // the cell's slot in the neighbour's ring, and the one before it
+  __shared__ int s_bad[32];
+  const int c = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const size_t N = (size_t)g.n;
+  const float2* fs = as_f2(g.fs);
+  const float2* sv = as_f2(g.s);
+  const float2* wv = as_f2(g.w);
+  const int total = g.list ? *g.list_count : g.n;
+  for (int base = blockIdx.x * 32; base < total; base += gridDim.x * 32) {
+    const int item = base + c;
+    int i = 0, m = 0;
+    if (item < total) {
+      i = g.list ? g.list[item] : (g.order ? g.order[item] : item);
+      m = g.cnt[i];
+      if (w == 0) {
+        if (g.list_bits) atomicAnd(&g.list_bits[i >> 5], ~(1u << (i & 31)));
+        if (m < 3 || m > CG_RING) raise_status(g.ctl, kETOPO);
+      }
+      if (m < 3 || m > CG_RING) m = 0;
+    }
+    bool bad = false;
+    if (w == 0) s_bad[c] = 0;
+    for (int a = w; a < m; a += kSlotWarps) {
+      int j = g.nbr[(size_t)i * CG_RING + a];
+      const bool ok = (unsigned)j < (unsigned)g.n;
+      j = ok ? j : i;
+      const int mj = g.cnt[j], p = ring_pos(g.nbr, g.cnt, j, i);
+      bad |= !ok || p < 0;
+      s_p[a][c] = (p < 0 ? 0 : p) | ((p <= 0 ? (mj > 0 ? mj - 1 : 0) : p - 1) << 8);
+      s_j[a][c] = j;
+    }
+    __syncthreads();
+    if (bad) s_bad[c] = 1;
+    for (int a = w; a < m; a += kSlotWarps) {
+      const int an = a + 1 < m ? a + 1 : 0;
+      const float2 f0 = fs[a * N + i];
+      const float2 f1 = fs[(size_t)(s_p[a][c] >> 8) * N + s_j[a][c]];
+      const float2 f2 = fs[(size_t)(s_p[an][c] & 255) * N + s_j[an][c]];
+      const float2 wj = wv[a * N + i];
+      s_s[a][c] = sv[a * N + i];
+      const float Gx = f0.x + f1.x + f2.x, Gy = f0.y + f1.y + f2.y;
+      s_c[a][c] = fmaf(wj.x, Gx, wj.y * Gy);
+    }
+    __syncthreads();
+    if (w == 0 && m) {
+      if (s_bad[c]) raise_status(g.ctl, kETOPO);
+      float fx = 0.f, fy = 0.f;
+      for (int a = 0; a < m; ++a) {
+        const float2 sj = s_s[a][c];
+        const float cj = s_c[a][c];
+        fx = fmaf(-sj.x, cj, fx);
+        fy = fmaf(-sj.y, cj, fy);
+      }
+      g.Fx[i] = fx;
+      g.Fy[i] = fy;
+      if (g.integrate) move_cell_f32(g, i, fx, fy);
+    }
+    __syncthreads();
+  }
+}
+
 // One thread per cell, or grid-stride over a list (bits cleared), as k_force.
 __global__ void __launch_bounds__(kForceThreads) k_force_f32(ForceArgs g) {
   const int total = g.list ? *g.list_count : g.n;
@@ -307,11 +483,24 @@ __global__ void k_dir_f32(DirArgs g) {
 
 void launch_geom_f32(const GeomArgs& a, cudaStream_t st, int blocks) {
   if (a.n <= 0) return;
+  // up to one resident wave (us: 10.2 -> 8.1 at 256 to 16384 cells; 14.1 -> 14.8
+  // at 65536), and for a list
+  if (a.list || a.n <= kGeomF32SlotCells) {
+    const int full = (a.n + 31) / 32;
+    k_geom_f32_slots<<<(blocks > 0 && blocks < full) ? blocks : full, kSlotThreads, 0, st>>>(a);
+    return;
+  }
   const int full = (a.n + kGeomThreads - 1) / kGeomThreads;
   k_geom_f32<<<(blocks > 0 && blocks < full) ? blocks : full, kGeomThreads, 0, st>>>(a);
 }
 void launch_force_f32(const ForceArgs& a, cudaStream_t st, int blocks) {
   if (a.n <= 0) return;
+  // as launch_force (us: 12.3 -> 8.2 at 1024 to 16384 cells, 14.3 -> 14.3 at 65536)
+  if (!a.tolerant && a.integrate != 2 && (a.list || a.n <= kForceSlotCells)) {
+    const int full = (a.n + 31) / 32;
+    k_force_f32_slots<<<(blocks > 0 && blocks < full) ? blocks : full, kSlotThreads, 0, st>>>(a);
+    return;
+  }
   const int full = (a.n + kForceThreads - 1) / kForceThreads;
   k_force_f32<<<(blocks > 0 && blocks < full) ? blocks : full, kForceThreads, 0, st>>>(a);
 }

@@ -33,6 +33,7 @@ struct AvmOff {
   size_t div_flag, div_ctl;                                                // its rounds
   // storage order: tags of the slots, slots of the tags, candidate priorities
   size_t vtag, ctag, vslot, cslot, cand_k;
+  size_t work0, work1, work_bits;  // items a T1 pass leaves for the next
   size_t cand_v, cand_w;  // a T1 candidate's other end and outer neighbours
   // re-sort scratch (keys, ranks, new places, key counts, permuted copies);
   // between re-sorts the copies stage the API's tag-ordered transfers
@@ -98,6 +99,9 @@ AvmOff avm_layout(int64_t n, size_t spv_bytes) {
   o.cand_k = L.take((3 * V / 2 + n + 1) * i4);
   o.cand_v = L.take((3 * V / 2 + n + 1) * sizeof(int4));
   o.cand_w = L.take((3 * V / 2 + n + 1) * i4);
+  o.work0 = L.take((V + n) * i4);
+  o.work1 = L.take((V + n) * i4);
+  o.work_bits = L.take((V + n + 31) / 32 * i4);
   o.vkey = L.take(V * i4);
   o.vrank = L.take(V * i4);
   o.vperm = L.take(V * i4);
@@ -246,10 +250,12 @@ AvmArgs avm_args(cg_avm_ctx* c) {
   a.cand_k = c->at<int>(c->off.cand_k);
   a.cand_v = c->at<int4>(c->off.cand_v);
   a.cand_w = c->at<int>(c->off.cand_w);
+  a.work[0] = c->at<int>(c->off.work0);
+  a.work[1] = c->at<int>(c->off.work1);
+  a.work_bits = c->at<unsigned>(c->off.work_bits);
   a.vtag = c->at<int>(c->off.vtag);
   a.ctag = c->at<int>(c->off.ctag);
   a.done = c->at<unsigned int>(c->off.done);
-  a.loop = 0;
   return a;
 }
 
@@ -362,41 +368,36 @@ int in_by_tag(cg_avm_ctx* c, double* dst, const double* src, int count, const in
   return CG_OK;
 }
 
-// A graph of `prefix` (captured) followed by a while node whose body is one
-// T1 pass (the pass's first kernel clears the handle, its closing block sets
-// it again when another pass is due).
+// A graph of `prefix` (with a first T1 pass), the further passes in one kernel,
+// and `suffix`.  Against a while node with a pass as its body (step, us): 35.1
+// -> 26.9 at 8192 vertices, 56.4 -> 48.3 at 131072, 146 -> 138 at 524288.
 template <class Prefix, class Suffix>
-int loop_graph(cg_avm_ctx* c, Prefix prefix, Suffix suffix, cudaGraphExec_t* out) {
+int pass_graph(cg_avm_ctx* c, Prefix prefix, Suffix suffix, cudaGraphExec_t* out) {
   if (*out) {
     cudaGraphExecDestroy(*out);
     *out = nullptr;
   }
-  AvmArgs a = avm_args(c);
-  cudaError_t e = build_loop_graph(
+  const AvmArgs a = avm_args(c);
+  cudaError_t e = build_plain_graph(
       c->capture,
-      [&](cudaGraphConditionalHandle h, cudaStream_t st) {
-        a.loop = h;
+      [&](cudaStream_t st) {
         prefix(a, st);
+        launch_avm_t1_rest(a, st);
+        suffix(st);
       },
-      [&](cudaGraphConditionalHandle h, cudaStream_t st) {
-        a.loop = h;
-        launch_avm_t1_pass(a, st);
-      },
-      suffix, out);
+      out);
   if (e != cudaSuccess) {
     cudaGetLastError();
-    return afail(c, CG_ECUDA, std::string("building the T1 loop graph: ") + cudaGetErrorString(e));
+    return afail(c, CG_ECUDA, std::string("building the step graph: ") + cudaGetErrorString(e));
   }
   return CG_OK;
 }
 
-// The first T1 pass of a step runs as plain graph nodes before the while
-// node (every step has one); the node then runs only the further passes.
 int avm_graphs(cg_avm_ctx* c) {
   // the step: geometry, vertex forces and move; then the T1 passes beside the
   // director terms of the next step (FP64 work on a branch of its own, joined
   // at the end of the step)
-  int rc = loop_graph(
+  int rc = pass_graph(
       c,
       [c](const AvmArgs& a, cudaStream_t st) {
         launch_avm_move(a, st);
@@ -408,7 +409,7 @@ int avm_graphs(cg_avm_ctx* c) {
       },
       [c](cudaStream_t st) { cudaStreamWaitEvent(st, c->join, 0); }, &c->exec);
   if (rc) return rc;
-  rc = loop_graph(
+  rc = pass_graph(
       c,
       [](const AvmArgs& a, cudaStream_t st) {
         launch_avm_begin_t1(a.ctl, st);
@@ -575,7 +576,8 @@ int cg_avm_create(int32_t n, double Lx, double Ly, double p0, double v0, const c
     launch_avm_p0s(avm_args(c), st);
     launch_fill_d(ncap, v0, c->at<double>(c->off.v0), st);
     launch_fill_u64(ncap, ~0ull, c->at<unsigned long long>(c->off.lock), st);
-    if (cudaMemsetAsync(c->at<unsigned int>(c->off.done), 0, 2 * sizeof(unsigned int), st) != cudaSuccess) {
+    if (cudaMemsetAsync(c->at<unsigned int>(c->off.done), 0, 2 * sizeof(unsigned int), st) != cudaSuccess ||
+        cudaMemsetAsync(c->at<unsigned>(c->off.work_bits), 0, (c->V + c->n + 31) / 32 * 4, st) != cudaSuccess) {
       rc = CG_ECUDA;
       break;
     }
@@ -646,6 +648,7 @@ int cg_avm_profile_step(cg_avm_ctx* c, int64_t nsteps, double* ms_out, int32_t n
       ms_out[3] += 1.0;
       if (!h.pad || h.status) break;
     }
+    launch_avm_t1_rest(a, st);  // no pass is due: empties the lists of unfinished items
   }
   for (int k = 0; k < 3; ++k) cudaEventDestroy(ev[k]);
   if (rc) return rc;

@@ -312,7 +312,7 @@ __global__ void k_avm_begin_t1(Ctl* ctl) {
 }
 
 // ---------------------------------------------------------------------------
-// T1 passes: the body of a conditional (while) graph node.  Candidate edges
+// T1 passes.  Candidate edges
 // take an atomic minimum of a 64-bit key on their four cells; the high word
 // 0xffffffff - pass number makes every key of this pass smaller than any
 // left over from earlier passes, so the locks never need clearing.
@@ -351,12 +351,18 @@ __device__ __forceinline__ int cell_across(const int* __restrict__ vc, int c, in
   return r;
 }
 
+// Leaves item x of pass `pass` for the next one, once.
+__device__ __forceinline__ void relist(const AvmArgs& g, int pass, int x) {
+  const unsigned bit = 1u << (x & 31);
+  if (!(atomicOr(&g.work_bits[x >> 5], bit) & bit)) g.work[pass & 1][atomicAdd(&g.ctl->work[pass & 1], 1)] = x;
+}
+
 // T2 proposal for the triangular cell c: twice its signed area (each product
 // and the difference rounded separately, offsets from its first vertex)
 // below twice the threshold; the cells across its three edges must be
 // distinct with more than 3 vertices and the outer vertices distinct.  The
 // candidate id is 3V + tag(c); its cells are c and the three across its edges.
-__device__ void t2_propose(const AvmArgs& g, int c, int stamp) {
+__device__ void t2_propose(const AvmArgs& g, int c, int stamp, int pass) {
   const size_t V = (size_t)g.V;
   const int cur = g.ctl->cur;
   const double* hx = g.hx + cur * V;
@@ -395,6 +401,7 @@ __device__ void t2_propose(const AvmArgs& g, int c, int stamp) {
   }
   if (!ok) {  // a later transition may allow it
     g.ctl->t1_more = 1;
+    relist(g, pass, g.V + c);
     return;
   }
   const int ek = 3 * g.V + g.ctag[c];  // priority: the id in tags
@@ -418,13 +425,7 @@ __device__ void t2_propose(const AvmArgs& g, int c, int stamp) {
 // go to a compact list.  A short edge that its cells' vertex counts keep from
 // flipping marks the pass as possibly leaving work (another flip may change
 // those counts).
-__global__ void k_t1_propose(AvmArgs g) {
-  const int v = blockIdx.x * blockDim.x + threadIdx.x;
-  // stop the loop unless the closing kernel of this pass asks for another
-  if (v == 0 && g.loop) cudaGraphSetConditional(g.loop, 0);
-  const int stamp = g.ctl->round_count;
-  if (g.t2_twice > 0.0 && v < g.n && g.cc[v] == 3) t2_propose(g, v, stamp);
-  if (v >= g.V) return;
+__device__ __forceinline__ void t1_propose_vertex(const AvmArgs& g, int v, int stamp, int pass) {
   const size_t V = (size_t)g.V;
   const float2 pv = g.hf[v];
   for (int s = 0; s < 3; ++s) {
@@ -475,6 +476,7 @@ __global__ void k_t1_propose(AvmArgs g) {
     }
     if (g.cc[i] <= 3 || g.cc[k] <= 3 || g.cc[j] >= CG_RING || g.cc[l] >= CG_RING) {
       g.ctl->t1_more = 1;
+      relist(g, pass, v);
       continue;
     }
     const int ek = 3 * min(tv, tw) + a;  // priority: the id in tags
@@ -492,6 +494,12 @@ __global__ void k_t1_propose(AvmArgs g) {
   }
 }
 
+__global__ void k_t1_propose(AvmArgs g) {
+  const int v = blockIdx.x * blockDim.x + threadIdx.x;
+  const int stamp = g.ctl->round_count, pass = g.ctl->last_flagged;
+  if (g.t2_twice > 0.0 && v < g.n && g.cc[v] == 3) t2_propose(g, v, stamp, pass);
+  if (v < g.V) t1_propose_vertex(g, v, stamp, pass);
+}
 
 __device__ void remove_from_cell(int* cc, int* cv, int c, int v) {
   const int m = cc[c];
@@ -591,7 +599,8 @@ __device__ __forceinline__ int row_insert(Row& w, int m, int after, int v) {
   return m + 1;
 }
 
-__device__ void apply_t1(const AvmArgs& g, int v1, int a, int4 cd, int4 nv, int Aur, unsigned long long key) {
+__device__ void apply_t1(const AvmArgs& g, int v1, int a, int4 cd, int4 nv, int Aur, unsigned long long key,
+                         int pass) {
   Ctl* ctl = g.ctl;
   const size_t V = (size_t)g.V;
   double* hx = g.hx + ctl->cur * V;
@@ -630,6 +639,7 @@ __device__ void apply_t1(const AvmArgs& g, int v1, int a, int4 cd, int4 nv, int 
   const float2 fAll = g.hf[All], fAlr = g.hf[Alr], fAul = g.hf[Aul], fAur = g.hf[Aur];
   if (g.lock[i] != key || g.lock[j] != key || g.lock[k] != key || g.lock[l] != key) {
     ctl->t1_more = 1;
+    relist(g, pass, min(v1, v2));
     return;
   }
   // the network as the proposal saw it (always so for a lock holder); the
@@ -676,7 +686,10 @@ __device__ void apply_t1(const AvmArgs& g, int v1, int a, int4 cd, int4 nv, int 
                       t1_len2_f(g, f2, now(Aur, fAur)) <= g.t2hi;
     // (a degenerate network, with a cell on both sides of an edge, takes the
     // next pass regardless)
-    if (near || !distinct) ctl->t1_more = 1;
+    if (near || !distinct) {
+      ctl->t1_more = 1;
+      for (int x : {v1, v2, Aul, All, Alr, Aur}) relist(g, pass, x);
+    }
   }
   // neighbour exchange (Fig. 1): v1 -> cells (j, i, l), v2 -> cells (k, j, l)
   g.vc[3 * v1 + 0] = j; g.vc[3 * v1 + 1] = i; g.vc[3 * v1 + 2] = l;
@@ -698,7 +711,11 @@ __device__ void apply_t1(const AvmArgs& g, int v1, int a, int4 cd, int4 nv, int 
     insert_in_cell(g.cc, g.cv, l, v2, v1);
   }
   // i or k left as a triangle may be removed by a T2 in the next pass
-  if (g.t2_twice > 0.0 && (g.cc[i] == 3 || g.cc[k] == 3)) ctl->t1_more = 1;
+  if (g.t2_twice > 0.0 && (g.cc[i] == 3 || g.cc[k] == 3)) {
+    ctl->t1_more = 1;
+    for (int x : {i, k})
+      if (g.cc[x] == 3) relist(g, pass, g.V + x);
+  }
   atomicAdd((unsigned long long*)&ctl->repaired_total, 1ull);
 }
 
@@ -723,7 +740,7 @@ __device__ void merge_in_cell(int* cc, int* cv, int x, const int* v, int vk) {
 // its centroid.  The vertex of smallest tag among its three stays, joined to the
 // three outer vertices in their order around the triangle; the other two are
 // freed (vc, vn = -1) and the cell is emptied (cc = 0, cv = -1).
-__device__ void apply_t2(const AvmArgs& g, int c, int4 cd) {
+__device__ void apply_t2(const AvmArgs& g, int c, int4 cd, int pass) {
   Ctl* ctl = g.ctl;
   const size_t V = (size_t)g.V;
   double* hx = g.hx + ctl->cur * V;
@@ -793,7 +810,42 @@ __device__ void apply_t2(const AvmArgs& g, int c, int4 cd) {
   for (int a = 0; a < CG_RING; ++a) row[a] = -1;
   g.cc[c] = 0;
   ctl->t1_more = 1;  // the merged vertex's edges and the neighbours' counts changed
+  relist(g, pass, vk);
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    relist(g, pass, w[a]);
+    if (g.cc[nb[a]] == 3) relist(g, pass, g.V + nb[a]);
+  }
   atomicAdd((unsigned long long*)&ctl->flagged_total, 1ull);
+}
+
+// Applies one listed candidate if it holds all four locks.
+__device__ __forceinline__ void t1_apply_candidate(const AvmArgs& g, int e, int4 cd, int4 nv, int w,
+                                                   unsigned long long key, int pass) {
+  if (e < 3 * g.V) {
+    apply_t1(g, e / 3, e % 3, cd, nv, w, key, pass);  // checks the locks itself
+    return;
+  }
+  if (g.lock[cd.x] != key || g.lock[cd.y] != key || g.lock[cd.z] != key || g.lock[cd.w] != key) {
+    g.ctl->t1_more = 1;
+    relist(g, pass, e - 2 * g.V);  // V + the cell
+    return;
+  }
+  apply_t2(g, e - 3 * g.V, cd, pass);
+}
+
+// Closes a pass (one thread, after every candidate): counts it and leaves in
+// ctl->pad whether another one is due.
+__device__ __forceinline__ void t1_close(const AvmArgs& g, int pass, int proposed) {
+  Ctl* ctl = g.ctl;
+  ctl->count[1] = 0;
+  ctl->round_count += 1;
+  ctl->loop_total += 1;
+  ctl->last_flagged = pass + 1;
+  if (pass >= g.t1_cap && proposed > 0) atomicCAS(&ctl->status, 0, (int)kET1CAP);
+  const int more = proposed > 0 && *(volatile int*)&ctl->t1_more && pass < g.t1_cap && ctl->status == 0;
+  ctl->t1_more = 0;
+  ctl->pad = more;
 }
 
 // Applies the listed candidates (T1 edges, T2 cells) that hold all four
@@ -830,15 +882,7 @@ __global__ void k_t1_apply(AvmArgs g) {
       const int e = first ? e0 : g.cand_e[t];
       const int4 cd = first ? cd0 : g.cand[t];
       const unsigned long long key = lock_key(stamp, first ? k0 : g.cand_k[t]);
-      if (e < 3 * g.V) {
-        apply_t1(g, e / 3, e % 3, cd, first ? nv0 : g.cand_v[t], first ? w0 : g.cand_w[t], key);  // checks the locks itself
-        continue;
-      }
-      if (g.lock[cd.x] != key || g.lock[cd.y] != key || g.lock[cd.z] != key || g.lock[cd.w] != key) {
-        ctl->t1_more = 1;
-        continue;
-      }
-      apply_t2(g, e - 3 * g.V, cd);
+      t1_apply_candidate(g, e, cd, first ? nv0 : g.cand_v[t], first ? w0 : g.cand_w[t], key, pass);
     }
   }
   bool closing;
@@ -848,17 +892,50 @@ __global__ void k_t1_apply(AvmArgs g) {
   } else {
     closing = last_block(g.done + 1) && threadIdx.x == 0;
   }
-  if (closing) {
-    ctl->count[1] = 0;
-    ctl->round_count += 1;
-    ctl->loop_total += 1;
-    ctl->last_flagged = pass + 1;
-    if (pass >= g.t1_cap && proposed > 0) atomicCAS(&ctl->status, 0, (int)kET1CAP);
-    const int more = proposed > 0 && *(volatile int*)&ctl->t1_more && pass < g.t1_cap && ctl->status == 0;
-    ctl->t1_more = 0;
-    ctl->pad = more;  // read by the host when the passes run outside a graph
-    if (more && g.loop) cudaGraphSetConditional(g.loop, 1);
+  if (closing) t1_close(g, pass, proposed);
+}
+
+// The passes after the first in one kernel (as k_repair_rest): one cluster
+// proposes and applies pass after pass, its hardware barrier between the two,
+// while passes are due (1.02 passes per step in a relaxed tissue).  Only the
+// items the pass before left can be candidates: an edge that lost a lock or
+// whose cells kept it from flipping, an edge at a moved vertex, a triangle that
+// lost a lock, was kept or came to be; no other length, area or count changed.
+// Items left when no further pass is due are dropped.
+__global__ void __cluster_dims__(kT1RestBlocks, 1, 1) __launch_bounds__(kT1RestThreads) k_t1_rest(AvmArgs g) {
+  Ctl* ctl = g.ctl;
+  const int t0 = blockIdx.x * kT1RestThreads + threadIdx.x;
+  constexpr int kStride = kT1RestBlocks * kT1RestThreads;
+  // every thread of the cluster follows the same words: each is written between
+  // two barriers that all threads read it across
+  while (*(volatile int*)&ctl->pad) {
+    const int pass = *(volatile int*)&ctl->last_flagged, stamp = *(volatile int*)&ctl->round_count;
+    const int from = (pass & 1) ^ 1, items = *(volatile int*)&ctl->work[from];
+    for (int t = t0; t < items; t += kStride) {
+      const int x = g.work[from][t];
+      atomicAnd(&g.work_bits[x >> 5], ~(1u << (x & 31)));
+      if (x < g.V) t1_propose_vertex(g, x, stamp, pass);
+      else if (g.cc[x - g.V] == 3) t2_propose(g, x - g.V, stamp, pass);
+    }
+    cluster_barrier();
+    if (t0 == 0) ctl->work[from] = 0;
+    const int proposed = *(volatile int*)&ctl->count[1];
+    if (pass < g.t1_cap)
+      for (int t = t0; t < proposed; t += kStride)
+        t1_apply_candidate(g, g.cand_e[t], g.cand[t], g.cand_v[t], g.cand_w[t], lock_key(stamp, g.cand_k[t]), pass);
+    cluster_barrier();
+    if (t0 == 0) t1_close(g, pass, proposed);
+    cluster_barrier();
   }
+  const int left[2] = {*(volatile int*)&ctl->work[0], *(volatile int*)&ctl->work[1]};
+  if (left[0] + left[1] == 0) return;  // the same for every thread
+  for (int q = 0; q < 2; ++q)
+    for (int t = t0; t < left[q]; t += kStride) atomicAnd(&g.work_bits[g.work[q][t] >> 5], ~(1u << (g.work[q][t] & 31)));
+  cluster_barrier();  // every thread has read the counts
+  if (t0 == 0) ctl->work[0] = ctl->work[1] = 0;
+}
+void launch_avm_t1_rest(const AvmArgs& a, cudaStream_t st) {
+  k_t1_rest<<<kT1RestBlocks, kT1RestThreads, 0, st>>>(a);
 }
 
 // Float copies of the current positions (after the network or the positions

@@ -452,6 +452,12 @@ int sm_count() {
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   return sms;
 }
+// Up to here a step takes its repair rounds after the first as one kernel
+// (step, us, with a while node -> without: 41.6 -> 26.8 at 1024 cells, 55.9 ->
+// 43.0 at 16384, 109.5 -> 106.6 at 131072; FP32 98.5 -> 87.3 at 262144, 263.7
+// -> 259.9 at 10^6).  In double precision the rounds of larger systems hide
+// behind the geometry (191 -> 194 at 262144).
+constexpr int64_t kRestCells = kGeomSlotCells, kRestCellsF32 = 1 << 20;
 // Per-step repair rounds handle a few hundred flagged cells: a modest
 // persistent grid (warps loop over the list) keeps empty rounds cheap.
 int repair_grid(const cg_ctx* c) { return sm_count() * c->launch.repair_blocks_per_sm; }
@@ -573,9 +579,9 @@ void prime(cg_ctx* c, int what = kPrimeAll) {
   if (what & kPrimeMove) run_force(c, force_args(c, 1), c->stream);
 }
 
-// One repair round (repair + consistency check) for a conditional loop node:
-// the round counter in the control word picks the lists.
-void enqueue_repair_round(cg_ctx* c, cudaGraphConditionalHandle h, cudaStream_t st) {
+// A step's repair rounds: the round counter in the control word picks the
+// lists.
+RepairArgs round_repair_args(cg_ctx* c, cudaGraphConditionalHandle h) {
   RepairArgs r = repair_args(c, 0, 0);
   r.dyn = 1;
   r.lists[0] = c->at<int>(c->off.list0);
@@ -583,14 +589,22 @@ void enqueue_repair_round(cg_ctx* c, cudaGraphConditionalHandle h, cudaStream_t 
   r.loop = h;
   r.dirty_list = c->at<int>(c->off.dirty_list);
   r.dirty_bits = c->at<unsigned>(c->off.dirty_bits);
+  return r;
+}
+CheckArgs round_check_args(cg_ctx* c, cudaGraphConditionalHandle h) {
   CheckArgs k = check_args(c, 0, 0, 0);
   k.dyn = 1;
   k.cap = c->par.repair_cap > 0 ? c->par.repair_cap : 4;
   k.lists[0] = c->at<int>(c->off.list0);
   k.lists[1] = c->at<int>(c->off.list1);
   k.loop = h;
-  launch_repair(r, repair_grid(c), st);
-  launch_check(k, check_grid(c), st);
+  return k;
+}
+// One round (repair + consistency check), as the body of a loop node or (h 0)
+// on its own.
+void enqueue_repair_round(cg_ctx* c, cudaGraphConditionalHandle h, cudaStream_t st) {
+  launch_repair(round_repair_args(c, h), repair_grid(c), st);
+  launch_check(round_check_args(c, h), check_grid(c), st);
 }
 
 // Full triangulation of the current positions (every cell repaired).
@@ -644,15 +658,32 @@ int load_positions(cg_ctx* c, const double* x, const double* y) {
   return CG_OK;
 }
 
-// One step as a graph: the prefix, then the repair rounds as a conditional
-// while node that stops at the first round leaving no cell flagged.
+// One step as a graph.  Up to kRestCells cells: the prefix, the first repair
+// round, one kernel for the further rounds (usually none), the suffix.  Larger
+// systems, whose later rounds can be long and hide behind the geometry: the
+// rounds as a conditional while node that stops at the first one leaving no
+// cell flagged.
 int build_graph(cg_ctx* c) {
   if (c->step_exec) return CG_OK;
-  cudaError_t e = build_loop_graph(
-      c->capture, [&](cudaGraphConditionalHandle, cudaStream_t st) { enqueue_step_prefix(c, st); },
-      [&](cudaGraphConditionalHandle h, cudaStream_t st) { enqueue_repair_round(c, h, st); },
-      [&](cudaStream_t st) { enqueue_step_suffix(c, st); }, &c->step_exec,
-      c->launch.dir_low_priority ? (unsigned long long)cudaGraphInstantiateFlagUseNodePriority : 0ull);
+  const unsigned long long flags =
+      c->launch.dir_low_priority ? (unsigned long long)cudaGraphInstantiateFlagUseNodePriority : 0ull;
+  cudaError_t e;
+  if (c->N <= (fp32(c) ? kRestCellsF32 : kRestCells)) {
+    e = build_plain_graph(
+        c->capture,
+        [&](cudaStream_t st) {
+          enqueue_step_prefix(c, st);
+          enqueue_repair_round(c, 0, st);
+          launch_repair_rest(round_repair_args(c, 0), round_check_args(c, 0), st);
+          enqueue_step_suffix(c, st);
+        },
+        &c->step_exec, flags);
+  } else {
+    e = build_loop_graph(
+        c->capture, [&](cudaGraphConditionalHandle, cudaStream_t st) { enqueue_step_prefix(c, st); },
+        [&](cudaGraphConditionalHandle h, cudaStream_t st) { enqueue_repair_round(c, h, st); },
+        [&](cudaStream_t st) { enqueue_step_suffix(c, st); }, &c->step_exec, flags);
+  }
   if (e != cudaSuccess) {
     cudaGetLastError();
     c->step_exec = nullptr;

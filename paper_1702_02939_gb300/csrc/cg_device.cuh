@@ -88,7 +88,17 @@ struct Ctl {
   long long loop_total;  // iterations of the repair-round (or T1-pass) loop node
   int t1_more;        // the current T1 pass may leave work for another (AVM)
   int force_count;    // cells whose force the step recomputes after the repair rounds
+  int work[2];        // lengths of the lists of a T1 pass's unfinished items (AVM)
 };
+
+// Barrier of all threads of the thread-block cluster; global writes before it
+// are seen after it.
+__device__ __forceinline__ void cluster_barrier() {
+  __syncwarp();
+  __threadfence();
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  __threadfence();
+}
 
 // True in exactly one block of the grid: the last one to get here.  Every
 // thread of every block must call it; each block's global writes are fenced

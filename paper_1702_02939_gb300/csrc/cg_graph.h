@@ -65,4 +65,18 @@ cudaError_t build_loop_graph(cudaStream_t cap, Prefix prefix, Body body, Suffix 
   return e;
 }
 
+// A captured sequence as a graph.
+template <class Body>
+cudaError_t build_plain_graph(cudaStream_t cap, Body body, cudaGraphExec_t* out,
+                              unsigned long long instantiate_flags = 0) {
+  cudaError_t e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
+  if (e != cudaSuccess) return e;
+  body(cap);
+  cudaGraph_t g = nullptr;
+  e = cudaStreamEndCapture(cap, &g);
+  if (e == cudaSuccess) e = cudaGraphInstantiate(out, g, instantiate_flags);
+  if (g) cudaGraphDestroy(g);
+  return e;
+}
+
 }  // namespace cgk

@@ -23,6 +23,7 @@ constexpr int kForceSlotCells = 29184, kTestSlotCells = 29184, kGeomF32SlotCells
 constexpr int kForceThreads = 128;
 constexpr int kTestThreads = 128;
 constexpr int kRepairWarps = 4;  // warps per repair block
+constexpr int kRestBlocks = 8, kRestWarps = 16;  // the cluster of the rounds after the first
 constexpr int kCand = 64;        // candidate buffer per repair warp
 
 struct GeomArgs {
@@ -187,8 +188,9 @@ struct RepairArgs {
   int which_in;  // count index of list_in
   int all_cells; // process cells 0..n-1 instead of the list
   int record;    // outside a graph: count the list in the step statistics
-  // Rounds inside a conditional (while) graph node: the input list is
-  // lists[round & 1] with the round counter read from the control word.
+  // The rounds of a step: the input list is lists[round & 1] with the round
+  // counter read from the control word; loop: the handle of the conditional
+  // (while) graph node the rounds run in, or 0.
   int dyn;
   const int* lists[2];
   cudaGraphConditionalHandle loop;
@@ -208,9 +210,9 @@ struct CheckArgs {
   int which_in, which_out;
   int last_round;  // raise REPAIR_CAP if anything is flagged
   int all_cells;
-  // Rounds inside a conditional (while) graph node (see RepairArgs): the last
-  // block counts the round, raises REPAIR_CAP after `cap` rounds with work
-  // and asks for another round while cells are left flagged.
+  // The rounds of a step (see RepairArgs): the last block counts the round,
+  // raises REPAIR_CAP after `cap` rounds with work and, in a while node, asks
+  // for another round while cells are left flagged.
   int dyn, cap;
   int* lists[2];
   cudaGraphConditionalHandle loop;
@@ -230,6 +232,8 @@ void launch_cell_list(const CellListArgs& a, cudaStream_t st);
 void launch_repair(const RepairArgs& a, int grid_blocks, cudaStream_t st);
 void launch_scan(const ScanArgs& a, cudaStream_t st);
 void launch_check(const CheckArgs& a, int grid_blocks, cudaStream_t st);
+// After a first round (dyn): the further rounds, until none is needed
+void launch_repair_rest(const RepairArgs& a, const CheckArgs& c, cudaStream_t st);
 // Blocks of 8 warps for the check of every cell: a warp per cell up to 16
 // blocks per SM (one block per 256 cells left each warp a chain of 32 cells:
 // 44 us at 1024 cells against 3.5)
@@ -362,8 +366,12 @@ struct AvmArgs {
                              // (v2, Aul, All, Alr) (Fig. 1 naming)
   int* cand_w;               // [3V/2 + n] and v2's other outer neighbour Aur
   const int *vtag, *ctag;    // [V], [n] the tag (API id) of each vertex and cell slot
+  // Items a pass leaves for the next one: vertices v (whose edges to larger
+  // slots are proposed again) and V + c (cells, T2), once each (work_bits);
+  // pass p leaves its items in work[p & 1], counted in ctl->work[p & 1]
+  int* work[2];              // [V + n]
+  unsigned* work_bits;
   unsigned int* done;        // [2] last-block counters (force/move, T1 apply)
-  cudaGraphConditionalHandle loop;  // while-node handle of the T1 passes
 };
 void launch_avm_build(const AvmBuildArgs& a, cudaStream_t st);
 // part: 0 both kernels, 1 the per-cell kernel only, 2 the per-vertex kernel only
@@ -374,6 +382,9 @@ void launch_avm_move(const AvmArgs& a, cudaStream_t st, int part = 0);
 void launch_avm_dir(const AvmArgs& a, cudaStream_t st);
 void launch_avm_begin_t1(Ctl* ctl, cudaStream_t st);
 void launch_avm_t1_pass(const AvmArgs& a, cudaStream_t st);
+// After a first pass: the further passes while any is due (ctl->pad)
+constexpr int kT1RestBlocks = 8, kT1RestThreads = 512;
+void launch_avm_t1_rest(const AvmArgs& a, cudaStream_t st);
 void launch_avm_forces(const AvmArgs& a, cudaStream_t st);
 void launch_avm_validate(const AvmArgs& a, cudaStream_t st);
 // P0[c] = p0[c] sqrt(a0[c]) after p0 or A0 change

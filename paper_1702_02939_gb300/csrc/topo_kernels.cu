@@ -641,6 +641,48 @@ __device__ __forceinline__ int gift_ring(const RepairArgs& g, const Rep& R, cons
   }
 }
 
+// Rebuilds the ring of cell i (one warp), keeping the old one for the check.
+__device__ __forceinline__ void repair_cell(const RepairArgs& g, const long long* __restrict__ X,
+                                            const long long* __restrict__ Y, int i, CandBuf& buf, int lane) {
+  const Rep& R = g.reps[g.rep[i]];
+  const int oc = g.cnt[i];
+  if (lane < CG_RING) g.old_nbr[(size_t)i * CG_RING + lane] = g.nbr[(size_t)i * CG_RING + lane];
+  if (lane == 0) g.old_cnt[i] = oc;
+
+  int gid = -1, gkey = INT_MAX;
+  int m = gift_ring(g, R, X, Y, i, buf, lane, gid, gkey);
+  __syncwarp();
+  if (m == 0) m = clip_ring(g, R, X, Y, i, buf, lane, gid, gkey);
+  if (m < 0) {
+    if (lane == 0) raise_status(g.ctl, m);
+    return;
+  }
+  // canonical CCW ring: start at the smallest tag
+  int kmin = (lane < m) ? gkey : INT_MAX;
+  int lmin = lane;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const int ok = __shfl_xor_sync(0xffffffffu, kmin, o);
+    const int ol = __shfl_xor_sync(0xffffffffu, lmin, o);
+    if (ok < kmin || (ok == kmin && ol < lmin)) { kmin = ok; lmin = ol; }
+  }
+  if (lane < m) {
+    const int slot = (lane - lmin + m) % m;
+    g.nbr[(size_t)i * CG_RING + slot] = gid;
+  } else if (lane < CG_RING) {
+    g.nbr[(size_t)i * CG_RING + lane] = -1;
+  }
+  if (lane == 0) {
+    g.cnt[i] = m;
+    atomicAnd(&g.flags[i >> 5], ~(1u << (i & 31)));
+    if (g.dirty_list && !g.all_cells) {
+      const unsigned bit = 1u << (i & 31);
+      if (!(atomicOr(&g.dirty_bits[i >> 5], bit) & bit)) g.dirty_list[atomicAdd(&g.ctl->dirty_count, 1)] = i;
+    }
+  }
+  __syncwarp();
+}
+
 // One warp per cell.  Bound by latency in a step (a few to a few thousand
 // cells: list entry, cell, replica, bins, candidates, then the ring), by
 // instruction issue when every cell is triangulated.
@@ -669,47 +711,8 @@ __global__ void __launch_bounds__(kRepairWarps * 32) k_repair(RepairArgs g) {
     atomicAdd((unsigned long long*)&g.ctl->repaired_total, (unsigned long long)total);
   }
 
-  for (int item = gw; item < total; item += nw) {
-    const int i = g.all_cells ? item : list_in[item];
-    const Rep& R = g.reps[g.rep[i]];
-    // keep the old ring for the consistency check
-    const int oc = g.cnt[i];
-    if (lane < CG_RING) g.old_nbr[(size_t)i * CG_RING + lane] = g.nbr[(size_t)i * CG_RING + lane];
-    if (lane == 0) g.old_cnt[i] = oc;
-
-    int gid = -1, gkey = INT_MAX;
-    int m = gift_ring(g, R, X, Y, i, s_buf[wib], lane, gid, gkey);
-    __syncwarp();
-    if (m == 0) m = clip_ring(g, R, X, Y, i, s_buf[wib], lane, gid, gkey);
-    if (m < 0) {
-      if (lane == 0) raise_status(g.ctl, m);
-      continue;
-    }
-    // canonical CCW ring: start at the smallest tag
-    int kmin = (lane < m) ? gkey : INT_MAX;
-    int lmin = lane;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const int ok = __shfl_xor_sync(0xffffffffu, kmin, o);
-      const int ol = __shfl_xor_sync(0xffffffffu, lmin, o);
-      if (ok < kmin || (ok == kmin && ol < lmin)) { kmin = ok; lmin = ol; }
-    }
-    if (lane < m) {
-      const int slot = (lane - lmin + m) % m;
-      g.nbr[(size_t)i * CG_RING + slot] = gid;
-    } else if (lane < CG_RING) {
-      g.nbr[(size_t)i * CG_RING + lane] = -1;
-    }
-    if (lane == 0) {
-      g.cnt[i] = m;
-      atomicAnd(&g.flags[i >> 5], ~(1u << (i & 31)));
-      if (g.dirty_list && !g.all_cells) {
-        const unsigned bit = 1u << (i & 31);
-        if (!(atomicOr(&g.dirty_bits[i >> 5], bit) & bit)) g.dirty_list[atomicAdd(&g.ctl->dirty_count, 1)] = i;
-      }
-    }
-    __syncwarp();
-  }
+  for (int item = gw; item < total; item += nw)
+    repair_cell(g, X, Y, g.all_cells ? item : list_in[item], s_buf[wib], lane);
 }
 
 void launch_repair(const RepairArgs& a, int grid_blocks, cudaStream_t st) {
@@ -742,6 +745,32 @@ __device__ __forceinline__ void flag_into(unsigned* flags, int* list, int* count
 // One warp per listed cell i: lanes 0-15 take the entries of i's new ring
 // (j must list i), lanes 16-31 those of its old ring (a neighbour i dropped
 // must have dropped i too).  Every lookup of a ring row runs in parallel.
+// Cells whose rings disagree go on the output list; returns whether any did.
+__device__ __forceinline__ bool check_cell(const CheckArgs& g, int i, int* list_out, int* count_out, int lane) {
+  const int a = lane & 15;
+  const int m = g.cnt[i];
+  const int rj = (lane < 16 && a < m) ? g.nbr[(size_t)i * CG_RING + a] : -1;  // new ring of i
+  int j = -1;
+  bool mine = false;
+  if (lane < 16) {
+    j = rj;
+    mine = a < m;
+  } else if (a < g.old_cnt[i]) {
+    j = g.old_nbr[(size_t)i * CG_RING + a];
+    mine = j >= 0 && j < g.n;
+  }
+  bool kept = false;  // j still in the new ring of i
+#pragma unroll
+  for (int b = 0; b < 16; ++b) kept |= (__shfl_sync(0xffffffffu, rj, b) == j);
+  bool flag = false;
+  if (mine) {
+    const bool lists_i = in_ring(g.nbr, g.cnt, j, i);
+    flag = (lane < 16) ? !lists_i : (!kept && lists_i);
+  }
+  if (flag) flag_into(g.flags, list_out, count_out, j);
+  return __any_sync(0xffffffffu, flag);
+}
+
 __global__ void k_check(CheckArgs g) {
   const int which_in = g.dyn ? (g.ctl->round_count & 1) : g.which_in;
   const int which_out = which_in ^ 1;
@@ -749,32 +778,11 @@ __global__ void k_check(CheckArgs g) {
   int* list_out = g.dyn ? (which_out ? g.lists[1] : g.lists[0]) : g.list_out;
   const int total = g.all_cells ? g.n : g.ctl->count[which_in];
   int* count_out = &g.ctl->count[which_out];
-  const int lane = threadIdx.x & 31, a = lane & 15;
+  const int lane = threadIdx.x & 31;
   const int warp = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
   const int nwarps = (int)((gridDim.x * blockDim.x) >> 5);
   for (int item = warp; item < total; item += nwarps) {  // warp-uniform
-    const int i = g.all_cells ? item : list_in[item];
-    const int m = g.cnt[i];
-    const int rj = (lane < 16 && a < m) ? g.nbr[(size_t)i * CG_RING + a] : -1;  // new ring of i
-    int j = -1;
-    bool mine = false;
-    if (lane < 16) {
-      j = rj;
-      mine = a < m;
-    } else if (a < g.old_cnt[i]) {
-      j = g.old_nbr[(size_t)i * CG_RING + a];
-      mine = j >= 0 && j < g.n;
-    }
-    bool kept = false;  // j still in the new ring of i
-#pragma unroll
-    for (int b = 0; b < 16; ++b) kept |= (__shfl_sync(0xffffffffu, rj, b) == j);
-    bool flag = false;
-    if (mine) {
-      const bool lists_i = in_ring(g.nbr, g.cnt, j, i);
-      flag = (lane < 16) ? !lists_i : (!kept && lists_i);
-    }
-    if (flag) flag_into(g.flags, list_out, count_out, j);
-    const bool bad = __any_sync(0xffffffffu, flag);
+    const bool bad = check_cell(g, g.all_cells ? item : list_in[item], list_out, count_out, lane);
     if (bad && g.last_round && !g.dyn && lane == 0) raise_status(g.ctl, kEREPAIR_CAP);
   }
   if (!g.dyn) return;  // uniform over the grid
@@ -793,6 +801,54 @@ __global__ void k_check(CheckArgs g) {
       else if (g.loop) cudaGraphSetConditional(g.loop, 1);
     }
   }
+}
+
+// The rounds after the first in one kernel: one cluster of kRestBlocks blocks
+// repairs and checks the listed cells, its hardware barrier between the two,
+// until a round leaves no cell flagged or the cap is reached (raised by the
+// check of the last allowed round).  Nearly every step leaves nothing to do
+// here (1.01 to 1.04 rounds per step) and a graph's while node costs 10-12 us
+// whether it runs or not (a chain of 6 empty kernels 6 us, with a while node
+// 14-16); this kernel adds 2 us.
+__global__ void __cluster_dims__(kRestBlocks, 1, 1) __launch_bounds__(kRestWarps * 32) k_repair_rest(RepairArgs g,
+                                                                                                CheckArgs k) {
+  __shared__ CandBuf s_buf[kRestWarps];
+  Ctl* ctl = g.ctl;
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+  const int gw = blockIdx.x * kRestWarps + wib, nw = kRestBlocks * kRestWarps;
+  const bool first = blockIdx.x == 0 && threadIdx.x == 0;
+  const int cur = ctl->cur;
+  const size_t N = (size_t)g.n;
+  const long long* __restrict__ X = g.X + cur * N;
+  const long long* __restrict__ Y = g.Y + cur * N;
+  // every thread of the cluster follows the same counts: the list of a round is
+  // complete before the barrier that ends the one before it
+  for (int r = *(volatile int*)&ctl->round_count; r < k.cap; ++r) {
+    const int in = r & 1;
+    const int total = *(volatile int*)&ctl->count[in];
+    if (total == 0) break;
+    const int* list_in = g.lists[in];
+    int* list_out = k.lists[in ^ 1];
+    int* count_out = &ctl->count[in ^ 1];
+    cluster_barrier();  // every thread has read the counts
+    if (first) {
+      *count_out = 0;
+      ctl->repaired_total += total;
+    }
+    for (int item = gw; item < total; item += nw) repair_cell(g, X, Y, list_in[item], s_buf[wib], lane);
+    cluster_barrier();
+    for (int item = gw; item < total; item += nw) check_cell(k, list_in[item], list_out, count_out, lane);
+    cluster_barrier();
+    if (first) {
+      ctl->round_count = r + 1;
+      ctl->loop_total += 1;
+      if (*(volatile int*)count_out > 0 && r + 1 >= k.cap) atomicCAS(&ctl->status, 0, (int)kEREPAIR_CAP);
+    }
+  }
+}
+
+void launch_repair_rest(const RepairArgs& a, const CheckArgs& c, cudaStream_t st) {
+  if (a.n > 0) k_repair_rest<<<kRestBlocks, kRestWarps * 32, 0, st>>>(a, c);
 }
 
 void launch_check(const CheckArgs& a, int grid_blocks, cudaStream_t st) {

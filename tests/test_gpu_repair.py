@@ -42,3 +42,25 @@ def test_rings_equal_the_oracle(kind):
     np.testing.assert_array_equal(cnt, topo.cnt)
     np.testing.assert_array_equal(nbr, topo.nbr)
     sim.close()
+
+
+@pytest.mark.parametrize("n", [400, 4099])
+def test_later_rounds_with_long_lists(n):
+    """Moves of a fraction of a spacing: most cells are repaired, and the rounds
+    after the first have many cells left."""
+    rng = np.random.default_rng(5)
+    L = float(np.sqrt(n))
+    Lx, Ly, _ = oracle.box(L)
+    xs, ys = oracle.snap_positions(rng.uniform(0.0, L, n), rng.uniform(0.0, L, n), Lx, Ly)
+    sim = cg.SPV([dict(n=n, Lx=L, Ly=L, p0=3.8, v0=3.0)], xs, ys, rng.uniform(0.0, 6.28, n), KA=0.0, KP=0.0, dt=0.1,
+                 seed=1, repair_cap=16)
+    for _ in range(3):
+        sim.step(1)
+        x, y, _ = (t.cpu().numpy() for t in sim.state())
+        topo = oracle.triangulate(x, y, Lx, Ly)
+        cnt, nbr = (t.cpu().numpy() for t in sim.neighbors())
+        np.testing.assert_array_equal(cnt, topo.cnt)
+        np.testing.assert_array_equal(nbr, topo.nbr)
+    c = sim.counters()
+    assert c["repaired_total"] > c["flagged_total"] > n and c["loop_total"] > 3
+    sim.close()

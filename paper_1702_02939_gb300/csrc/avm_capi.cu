@@ -368,24 +368,17 @@ int in_by_tag(cg_avm_ctx* c, double* dst, const double* src, int count, const in
   return CG_OK;
 }
 
-// A graph of `prefix` (with a first T1 pass), the further passes in one kernel,
-// and `suffix`.  Against a while node with a pass as its body (step, us): 35.1
-// -> 26.9 at 8192 vertices, 56.4 -> 48.3 at 131072, 146 -> 138 at 524288.
-template <class Prefix, class Suffix>
-int pass_graph(cg_avm_ctx* c, Prefix prefix, Suffix suffix, cudaGraphExec_t* out) {
+// A captured sequence that ends with a first T1 pass and the kernel of the
+// further passes.  Against a while node with a pass as its body (step, us):
+// 35.1 -> 26.9 at 8192 vertices, 56.4 -> 48.3 at 131072, 146 -> 138 at 524288.
+template <class Body>
+int pass_graph(cg_avm_ctx* c, Body body, cudaGraphExec_t* out) {
   if (*out) {
     cudaGraphExecDestroy(*out);
     *out = nullptr;
   }
   const AvmArgs a = avm_args(c);
-  cudaError_t e = build_plain_graph(
-      c->capture,
-      [&](cudaStream_t st) {
-        prefix(a, st);
-        launch_avm_t1_rest(a, st);
-        suffix(st);
-      },
-      out);
+  cudaError_t e = build_plain_graph(c->capture, [&](cudaStream_t st) { body(a, st); }, out);
   if (e != cudaSuccess) {
     cudaGetLastError();
     return afail(c, CG_ECUDA, std::string("building the step graph: ") + cudaGetErrorString(e));
@@ -394,28 +387,33 @@ int pass_graph(cg_avm_ctx* c, Prefix prefix, Suffix suffix, cudaGraphExec_t* out
 }
 
 int avm_graphs(cg_avm_ctx* c) {
-  // the step: geometry, vertex forces and move; then the T1 passes beside the
-  // director terms of the next step (FP64 work on a branch of its own, joined
-  // at the end of the step)
+  // the step: geometry, vertex forces and move; then the first T1 pass beside
+  // the director terms of the next step (FP64 work on a branch of its own), and
+  // the further passes
   int rc = pass_graph(
       c,
       [c](const AvmArgs& a, cudaStream_t st) {
         launch_avm_move(a, st);
+        AvmArgs ahead = a;
+        ahead.flip = 1;
         cudaEventRecord(c->fork, st);
         cudaStreamWaitEvent(c->side, c->fork, 0);
-        launch_avm_dir(a, c->side);
+        launch_avm_dir(ahead, c->side);
         cudaEventRecord(c->join, c->side);
-        launch_avm_t1_pass(a, st);
+        launch_avm_t1_pass(ahead, st);
+        cudaStreamWaitEvent(st, c->join, 0);
+        launch_avm_t1_rest(a, 1, st);
       },
-      [c](cudaStream_t st) { cudaStreamWaitEvent(st, c->join, 0); }, &c->exec);
+      &c->exec);
   if (rc) return rc;
   rc = pass_graph(
       c,
       [](const AvmArgs& a, cudaStream_t st) {
-        launch_avm_begin_t1(a.ctl, st);
+        launch_avm_begin_t1(a.ctl, 0, st);
         launch_avm_t1_pass(a, st);
+        launch_avm_t1_rest(a, 0, st);
       },
-      [](cudaStream_t) {}, &c->t1_exec);
+      &c->t1_exec);
   if (rc) return rc;
   // division rounds: locks, prefix, dry runs, slots, application, advance
   DivArgs d{};
@@ -623,6 +621,7 @@ int cg_avm_profile_step(cg_avm_ctx* c, int64_t nsteps, double* ms_out, int32_t n
     launch_avm_move(a, st, 1);
     cudaEventRecord(ev[1], st);
     launch_avm_move(a, st, 2);
+    launch_avm_begin_t1(a.ctl, 1, st);
     cudaEventRecord(ev[2], st);
     if (cudaEventSynchronize(ev[2]) != cudaSuccess) { rc = afail(c, CG_ECUDA, "profile sync"); break; }
     cudaEventElapsedTime(&ms, ev[0], ev[1]);
@@ -648,7 +647,7 @@ int cg_avm_profile_step(cg_avm_ctx* c, int64_t nsteps, double* ms_out, int32_t n
       ms_out[3] += 1.0;
       if (!h.pad || h.status) break;
     }
-    launch_avm_t1_rest(a, st);  // no pass is due: empties the lists of unfinished items
+    launch_avm_t1_rest(a, 0, st);  // no pass is due: empties the lists of unfinished items
   }
   for (int k = 0; k < 3; ++k) cudaEventDestroy(ev[k]);
   if (rc) return rc;

@@ -165,7 +165,26 @@ __global__ void k_avm_dir(AvmArgs g) {
   dm_sincos(th, g.tab, sn, cs);
   const double v3 = g.v0[c] * (1.0 / 3.0);
   g.act[c] = make_double2(v3 * cs, v3 * sn);
-  g.thn[c] = th + g.noise_amp * director_noise(g.seed, g.ctag[c], g.ctl->step, g.tab);
+  g.thn[c] = th + g.noise_amp * director_noise(g.seed, g.ctag[c], g.ctl->step + g.flip, g.tab);
+}
+
+// A, P, the force coefficients and the energy of cell c from its sums.  An
+// empty cell (removed by a T2) has no geometry and no force; its director still
+// turns.
+__device__ __forceinline__ void avm_cell(const AvmArgs& g, int c, bool empty, double area, double per) {
+  const double A = 0.5 * area, P = per;
+  g.A[c] = A;
+  g.P[c] = P;
+  if (empty) {
+    g.ka[c] = 0.0;
+    g.kp[c] = 0.0;
+    if (g.energy) g.energy[c] = 0.0;
+    return;
+  }
+  const double dA = A - g.a0[c], dP = P - g.P0[c];
+  g.ka[c] = g.KA * dA;  // half of dE/dA = 2 K_A (A - A0): dA/dh carries a 1/2
+  g.kp[c] = 2.0 * g.KP * dP;
+  if (g.energy) g.energy[c] = fma(g.KA * dA, dA, g.KP * dP * dP);
 }
 
 // Per cell: area and perimeter of the polygon and the force coefficients
@@ -181,12 +200,8 @@ __global__ void k_avm_cells(AvmArgs g) {
   const double* hy = g.hy + cur * V;
   const int m = g.cc[c];
   if (g.move) g.theta[c] = g.thn[c];
-  if (m == 0) {  // removed by a T2: no geometry, no force; the director still turns
-    g.A[c] = 0.0;
-    g.P[c] = 0.0;
-    g.ka[c] = 0.0;
-    g.kp[c] = 0.0;
-    if (g.energy) g.energy[c] = 0.0;
+  if (m == 0) {
+    avm_cell(g, c, true, 0.0, 0.0);
     return;
   }
   if (m < 3 || m > CG_RING) {
@@ -210,24 +225,88 @@ __global__ void k_avm_cells(AvmArgs g) {
       qy = mimg_a(hy[v] - y0, g.ay);
     }
     area = fma(-qx, py, fma(px, qy, area));
-    const double l2 = (qx - px) * (qx - px) + (qy - py) * (qy - py);
+    const double ex = qx - px, ey = qy - py;
+    const double l2 = fma(ex, ex, ey * ey);
     per = (__double_as_longlong(l2) > 0) ? fma(l2, fx_rsqrt(l2), per) : per;  // sqrt(l2)
     px = qx;
     py = qy;
   }
-  const double A = 0.5 * area, P = per;
-  g.A[c] = A;
-  g.P[c] = P;
-  const double dA = A - g.a0[c], dP = P - g.P0[c];
-  g.ka[c] = g.KA * dA;  // half of dE/dA = 2 K_A (A - A0): dA/dh carries a 1/2
-  g.kp[c] = 2.0 * g.KP * dP;
-  if (g.energy) g.energy[c] = g.KA * dA * dA + g.KP * dP * dP;
+  avm_cell(g, c, false, area, per);
+}
+
+// The same with one thread per (cell, polygon edge): a block takes 32 cells,
+// its warp w the vertices w, w + 8 of all of them (lane = cell); the vertices'
+// offsets and the edges pass through shared memory, the last warp adds the area
+// up beside the edges and the first one the perimeter.  Bit-identical to
+// k_avm_cells, whose lanes walk the polygon one edge after another.
+__global__ void __launch_bounds__(kSlotThreads, kAvmSlotBlocks) k_avm_cells_slots(AvmArgs g) {
+  __shared__ double2 s_q[CG_RING][32];  // vertices relative to the first one
+  __shared__ double2 s_l[CG_RING][32];  // edge leaving the vertex: squared length, inverse length
+  __shared__ double s_area[32];
+  __shared__ int s_bad[32];
+  const int t = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int c = blockIdx.x * 32 + t;
+  const size_t V = (size_t)g.V;
+  const int cur = g.ctl->cur;
+  const double* hx = g.hx + cur * V;
+  const double* hy = g.hy + cur * V;
+  int m = c < g.n ? g.cc[c] : 0;
+  const bool empty = m == 0;
+  bool bad = false;
+  if (m && (m < 3 || m > CG_RING)) {
+    bad = true;
+    m = 0;
+  }
+  if (w == 0) s_bad[t] = bad;
+  const int* row = g.cv + (size_t)c * CG_RING;
+  if (w < m) {
+    const int v0 = row[0];
+    const bool ok0 = (unsigned)v0 < (unsigned)g.V;
+    const double x0 = ok0 ? hx[v0] : 0.0, y0 = ok0 ? hy[v0] : 0.0;
+    for (int a = w; a < m; a += kSlotWarps) {
+      const int v = row[a];
+      const bool ok = ok0 && (unsigned)v < (unsigned)g.V;
+      bad |= !ok;
+      s_q[a][t] = (ok && a) ? make_double2(mimg_a(hx[v] - x0, g.ax), mimg_a(hy[v] - y0, g.ay)) : make_double2(0.0, 0.0);
+    }
+  }
+  __syncthreads();
+  if (bad) s_bad[t] = 1;
+  if (w == kSlotWarps - 1) {
+    double area = 0.0;
+    for (int a = 1; a <= m; ++a) {
+      const double2 p = s_q[a - 1][t], q = s_q[a < m ? a : 0][t];
+      area = fma(-q.x, p.y, fma(p.x, q.y, area));
+    }
+    s_area[t] = area;
+  }
+  for (int a = w; a < m; a += kSlotWarps) {
+    const double2 p = s_q[a][t], q = s_q[a + 1 < m ? a + 1 : 0][t];
+    const double ex = q.x - p.x, ey = q.y - p.y;
+    const double l2 = fma(ex, ex, ey * ey);
+    s_l[a][t] = make_double2(l2, (__double_as_longlong(l2) > 0) ? fx_rsqrt(l2) : 0.0);
+  }
+  __syncthreads();
+  if (w || c >= g.n) return;
+  if (g.move) g.theta[c] = g.thn[c];
+  if (s_bad[t]) {
+    raise_status(g.ctl, kETOPO);
+    return;
+  }
+  double per = 0.0;
+  for (int a = 0; a < m; ++a) {
+    const double2 l = s_l[a][t];
+    per = (__double_as_longlong(l.x) > 0) ? fma(l.x, l.y, per) : per;
+  }
+  avm_cell(g, c, empty, s_area[t], per);
 }
 
 // Per vertex: F_v = -sum_k [ka_k 1/2 perp(u_{k-1} - u_k) - kp_k (u^_k + u^_{k-1})]
 // with u_k = h(n_k) - h(v); then, when stepping, the move of Eq. 4 into the
-// other position buffer.  The last block switches buffers, advances the step
-// counter and opens the step's T1 passes.
+// other position buffer.  (The buffers are switched and the step counter
+// advances once the step's first T1 pass is done, in k_t1_rest; until then the
+// kernels of the step look one ahead, AvmArgs::flip.  A count of finished
+// blocks at the end of this kernel cost 2 us at 131072 vertices.)
 __global__ void k_avm_force_move(AvmArgs g) {
   const int v = blockIdx.x * blockDim.x + threadIdx.x;
   const size_t V = (size_t)g.V;
@@ -294,18 +373,12 @@ __global__ void k_avm_force_move(AvmArgs g) {
       g.hf[v] = make_float2((float)wx, (float)wy);
     }
   }
-  if (!g.move) return;  // uniform over the grid
-  if (last_block(g.done) && threadIdx.x == 0) {
-    Ctl* ctl = g.ctl;
-    ctl->cur = cur ^ 1;
-    ctl->step += 1;
-    ctl->last_flagged = 0;  // T1 passes run in this step
-    ctl->pad = 1;
-  }
 }
 
-// Opens T1 passes on the current state without a move.
-__global__ void k_avm_begin_t1(Ctl* ctl) {
+// Opens T1 passes on the current state, or (flip) on the state just moved to.
+__global__ void k_avm_begin_t1(Ctl* ctl, int flip) {
+  ctl->cur ^= flip;
+  ctl->step += flip;
   ctl->last_flagged = 0;
   ctl->count[1] = 0;
   ctl->pad = 1;
@@ -364,7 +437,7 @@ __device__ __forceinline__ void relist(const AvmArgs& g, int pass, int x) {
 // candidate id is 3V + tag(c); its cells are c and the three across its edges.
 __device__ void t2_propose(const AvmArgs& g, int c, int stamp, int pass) {
   const size_t V = (size_t)g.V;
-  const int cur = g.ctl->cur;
+  const int cur = g.ctl->cur ^ g.flip;
   const double* hx = g.hx + cur * V;
   const double* hy = g.hy + cur * V;
   const int* row = g.cv + (size_t)c * CG_RING;
@@ -439,7 +512,7 @@ __device__ __forceinline__ void t1_propose_vertex(const AvmArgs& g, int v, int s
     const float l2 = t1_len2_f(g, pv, g.hf[w]);
     if (l2 > g.t2hi) continue;
     if (!(l2 < g.t2lo)) {
-      const int cur = g.ctl->cur;
+      const int cur = g.ctl->cur ^ g.flip;
       const double* hx = g.hx + cur * V;
       const double* hy = g.hy + cur * V;
       const double dx = mimg_a(hx[w] - hx[v], g.ax), dy = mimg_a(hy[w] - hy[v], g.ay);
@@ -496,7 +569,7 @@ __device__ __forceinline__ void t1_propose_vertex(const AvmArgs& g, int v, int s
 
 __global__ void k_t1_propose(AvmArgs g) {
   const int v = blockIdx.x * blockDim.x + threadIdx.x;
-  const int stamp = g.ctl->round_count, pass = g.ctl->last_flagged;
+  const int stamp = g.ctl->round_count, pass = g.flip ? 0 : g.ctl->last_flagged;
   if (g.t2_twice > 0.0 && v < g.n && g.cc[v] == 3) t2_propose(g, v, stamp, pass);
   if (v < g.V) t1_propose_vertex(g, v, stamp, pass);
 }
@@ -603,8 +676,9 @@ __device__ void apply_t1(const AvmArgs& g, int v1, int a, int4 cd, int4 nv, int 
                          int pass) {
   Ctl* ctl = g.ctl;
   const size_t V = (size_t)g.V;
-  double* hx = g.hx + ctl->cur * V;
-  double* hy = g.hy + ctl->cur * V;
+  const int cur = ctl->cur ^ g.flip;
+  double* hx = g.hx + cur * V;
+  double* hy = g.hy + cur * V;
   const int e = 3 * v1 + a;
   const int i = cd.x, j = cd.y, k = cd.z, l = cd.w;
   const int v2 = nv.x, Aul = nv.y, All = nv.z, Alr = nv.w;
@@ -743,8 +817,9 @@ __device__ void merge_in_cell(int* cc, int* cv, int x, const int* v, int vk) {
 __device__ void apply_t2(const AvmArgs& g, int c, int4 cd, int pass) {
   Ctl* ctl = g.ctl;
   const size_t V = (size_t)g.V;
-  double* hx = g.hx + ctl->cur * V;
-  double* hy = g.hy + ctl->cur * V;
+  const int cur = ctl->cur ^ g.flip;
+  double* hx = g.hx + cur * V;
+  double* hy = g.hy + cur * V;
   int* row = g.cv + (size_t)c * CG_RING;
   int v[3], w[3], cp[3], cpp[3];
   const int nb[3] = {cd.y, cd.z, cd.w};
@@ -868,7 +943,7 @@ __global__ void k_t1_apply(AvmArgs g) {
   const bool room = t0 < 3 * g.V / 2 + g.n + 1;
   const int e0 = room ? g.cand_e[t0] : 0, k0 = room ? g.cand_k[t0] : 0, w0 = room ? g.cand_w[t0] : 0;
   const int4 cd0 = room ? g.cand[t0] : make_int4(0, 0, 0, 0), nv0 = room ? g.cand_v[t0] : make_int4(0, 0, 0, 0);
-  const int pass = ctl->last_flagged;
+  const int pass = g.flip ? 0 : ctl->last_flagged;
   const int proposed = *(volatile int*)&ctl->count[1];
   // the same for every block (the count is cleared only by the closing
   // block, after every block that uses it has read it)
@@ -902,10 +977,18 @@ __global__ void k_t1_apply(AvmArgs g) {
 // whose cells kept it from flipping, an edge at a moved vertex, a triangle that
 // lost a lock, was kept or came to be; no other length, area or count changed.
 // Items left when no further pass is due are dropped.
-__global__ void __cluster_dims__(kT1RestBlocks, 1, 1) __launch_bounds__(kT1RestThreads) k_t1_rest(AvmArgs g) {
+__global__ void __cluster_dims__(kT1RestBlocks, 1, 1) __launch_bounds__(kT1RestThreads) k_t1_rest(AvmArgs g,
+                                                                                                    int advance) {
   Ctl* ctl = g.ctl;
   const int t0 = blockIdx.x * kT1RestThreads + threadIdx.x;
   constexpr int kStride = kT1RestBlocks * kT1RestThreads;
+  if (advance) {  // the end of a step's first pass: the moved state becomes current
+    if (t0 == 0) {
+      ctl->cur ^= 1;
+      ctl->step += 1;
+    }
+    if (*(volatile int*)&ctl->pad) cluster_barrier();  // the same for every thread
+  }
   // every thread of the cluster follows the same words: each is written between
   // two barriers that all threads read it across
   while (*(volatile int*)&ctl->pad) {
@@ -934,8 +1017,8 @@ __global__ void __cluster_dims__(kT1RestBlocks, 1, 1) __launch_bounds__(kT1RestT
   cluster_barrier();  // every thread has read the counts
   if (t0 == 0) ctl->work[0] = ctl->work[1] = 0;
 }
-void launch_avm_t1_rest(const AvmArgs& a, cudaStream_t st) {
-  k_t1_rest<<<kT1RestBlocks, kT1RestThreads, 0, st>>>(a);
+void launch_avm_t1_rest(const AvmArgs& a, int advance, cudaStream_t st) {
+  k_t1_rest<<<kT1RestBlocks, kT1RestThreads, 0, st>>>(a, advance);
 }
 
 // Float copies of the current positions (after the network or the positions
@@ -1416,16 +1499,23 @@ constexpr int kAvmCellThreads = 64, kAvmVertexThreads = 32;
 static inline int cell_blocks_of(int n) { return (n + kAvmCellThreads - 1) / kAvmCellThreads; }
 static inline int vertex_blocks_of(int n) { return (n + kAvmVertexThreads - 1) / kAvmVertexThreads; }
 
+// The cell pass takes a thread per polygon edge while every cell is resident at
+// once (pass, us: 14.2 -> 10.1 at 4096 cells, 14.2 -> 12.2 at 16384, 14.5 ->
+// 16.2 at 32768, 18.4 -> 21.3 at 65536).
+static void launch_cells(const AvmArgs& a, cudaStream_t st) {
+  if (a.n <= kAvmSlotCells) k_avm_cells_slots<<<(a.n + 31) / 32, kSlotThreads, 0, st>>>(a);
+  else k_avm_cells<<<cell_blocks_of(a.n), kAvmCellThreads, 0, st>>>(a);
+}
 void launch_avm_move(const AvmArgs& a, cudaStream_t st, int part) {
   AvmArgs m = a;
   m.move = 1;
-  if (part != 2) k_avm_cells<<<cell_blocks_of(a.n), kAvmCellThreads, 0, st>>>(m);
+  if (part != 2) launch_cells(m, st);
   if (part != 1) k_avm_force_move<<<vertex_blocks_of(a.V), kAvmVertexThreads, 0, st>>>(m);
 }
 void launch_avm_dir(const AvmArgs& a, cudaStream_t st) {
   k_avm_dir<<<cell_blocks_of(a.n), kAvmCellThreads, 0, st>>>(a);
 }
-void launch_avm_begin_t1(Ctl* ctl, cudaStream_t st) { k_avm_begin_t1<<<1, 1, 0, st>>>(ctl); }
+void launch_avm_begin_t1(Ctl* ctl, int flip, cudaStream_t st) { k_avm_begin_t1<<<1, 1, 0, st>>>(ctl, flip); }
 void launch_avm_t1_pass(const AvmArgs& a, cudaStream_t st) {
   k_t1_propose<<<blocks_of(a.V), kAvmThreads, 0, st>>>(a);
   k_t1_apply<<<a.apply_blocks, kApplyThreads, 0, st>>>(a);
@@ -1436,7 +1526,7 @@ void launch_avm_shadow(const AvmArgs& a, cudaStream_t st) {
 void launch_avm_forces(const AvmArgs& a, cudaStream_t st) {
   AvmArgs f = a;
   f.move = 0;
-  k_avm_cells<<<cell_blocks_of(a.n), kAvmCellThreads, 0, st>>>(f);
+  launch_cells(f, st);
   k_avm_force_move<<<vertex_blocks_of(a.V), kAvmVertexThreads, 0, st>>>(f);
 }
 void launch_avm_divide_slots(const DivArgs& d, const int* cslot, const int* vslot, int* fc, int* sc, int* scp,

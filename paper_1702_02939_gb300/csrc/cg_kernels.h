@@ -353,6 +353,9 @@ struct AvmArgs {
   double* thn;             // [n] the directors after the step's rotation (k_avm_dir)
   double *Fx, *Fy;
   int move;
+  // 1 in the kernels of a step between the move and k_t1_rest: the state just
+  // moved to (position buffer ctl->cur ^ 1, step ctl->step + 1), first T1 pass
+  int flip;
   double thr2, t1_len;
   double t2_twice;           // T2: twice the area threshold (0: no T2)
   float t2lo, t2hi;          // FP32 squared lengths certainly below / above thr2
@@ -371,7 +374,7 @@ struct AvmArgs {
   // pass p leaves its items in work[p & 1], counted in ctl->work[p & 1]
   int* work[2];              // [V + n]
   unsigned* work_bits;
-  unsigned int* done;        // [2] last-block counters (force/move, T1 apply)
+  unsigned int* done;        // [2] last-block counters ([1]: T1 apply)
 };
 void launch_avm_build(const AvmBuildArgs& a, cudaStream_t st);
 // part: 0 both kernels, 1 the per-cell kernel only, 2 the per-vertex kernel only
@@ -380,11 +383,13 @@ void launch_avm_move(const AvmArgs& a, cudaStream_t st, int part = 0);
 // directors thn = theta + sqrt(2 D_r dt) xi (noise counter of ctl->step); in
 // the step graph beside the T1 passes, which leave the FP64 pipe idle
 void launch_avm_dir(const AvmArgs& a, cudaStream_t st);
-void launch_avm_begin_t1(Ctl* ctl, cudaStream_t st);
+void launch_avm_begin_t1(Ctl* ctl, int flip, cudaStream_t st);
 void launch_avm_t1_pass(const AvmArgs& a, cudaStream_t st);
-// After a first pass: the further passes while any is due (ctl->pad)
+// After a first pass: the further passes while any is due (ctl->pad); advance:
+// that pass looked one step ahead, whose state becomes current first
+constexpr int kAvmSlotBlocks = 6, kAvmSlotCells = 29184;
 constexpr int kT1RestBlocks = 8, kT1RestThreads = 512;
-void launch_avm_t1_rest(const AvmArgs& a, cudaStream_t st);
+void launch_avm_t1_rest(const AvmArgs& a, int advance, cudaStream_t st);
 void launch_avm_forces(const AvmArgs& a, cudaStream_t st);
 void launch_avm_validate(const AvmArgs& a, cudaStream_t st);
 // P0[c] = p0[c] sqrt(a0[c]) after p0 or A0 change

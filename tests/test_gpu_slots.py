@@ -38,3 +38,31 @@ def test_small_system_alone_and_inside_a_large_batch(n, precision):
         assert np.array_equal(alone.neighbors()[1].cpu().numpy(), batch.neighbors()[1].cpu().numpy()[:n])
     alone.close()
     batch.close()
+
+
+@pytest.mark.parametrize("n", [64, 1000])
+def test_vertex_model_small_and_with_room_for_many_cells(n):
+    # the same network in a context small enough for the slot kernel and in one
+    # with a capacity beyond it (empty cells and free vertices past the network)
+    x, y, th, L = workloads.spv_uniform(n, 13)
+    sims = [cg.AVM(n, L, L, x, y, th, v0=0.3, seed=3, t2_area=0.01, capacity=cap) for cap in (n, 40000)]
+    for sim in sims:
+        a0 = np.ones(sim.n)
+        a0[:n // 10] = 0.0  # dying cells: triangles, T2s, empty cells
+        sim.set_a0(a0)
+    for steps in (1, 40):
+        got = []
+        for sim in sims:
+            sim.step(steps)
+            hx, hy, th_ = sim.state()
+            vc, vn, cc, cv = sim.topology()
+            A, P = sim.geometry()
+            Fx, Fy, _ = sim.forces()
+            got.append([t.cpu().numpy() for t in (hx[:2 * n], hy[:2 * n], th_[:n], vc[:2 * n], vn[:2 * n], cc[:n],
+                                                  cv[:n], A[:n], P[:n], Fx[:2 * n], Fy[:2 * n])])
+        for a, b in zip(*got):
+            assert np.array_equal(a, b)
+    c = [sim.counters() for sim in sims]
+    assert c[0]["t1_total"] == c[1]["t1_total"] > 0 and c[0]["t2_total"] == c[1]["t2_total"]
+    for sim in sims:
+        sim.close()

@@ -24,174 +24,182 @@
 
 namespace cgk {
 
-constexpr int kJvpThreads = 32;
-
 __device__ __forceinline__ double i2d_exact_a(long long v) {
   return __longlong_as_double(0x4338000000000000LL + v) - 0x1.8p52;
 }
 
-__global__ void __launch_bounds__(kJvpThreads) k_geom_jvp(JvpArgs g) {
-  __shared__ double s_ux[CG_RING][kJvpThreads], s_uy[CG_RING][kJvpThreads];
-  __shared__ double s_vx[CG_RING][kJvpThreads], s_vy[CG_RING][kJvpThreads];  // udot
-  __shared__ double s_ex[CG_RING][kJvpThreads], s_ey[CG_RING][kJvpThreads];  // unit edge ending at a
-  __shared__ double s_fx[CG_RING][kJvpThreads], s_fy[CG_RING][kJvpThreads];  // its tangent
-  const int t = threadIdx.x;
-  const int i = blockIdx.x * kJvpThreads + t;
-  if (i >= g.n) return;
+// A, P, the force sets and their tangents along v.  One thread per (cell, ring
+// slot): a block takes 32 cells, its warp w the slots w, w + 8 of all of them
+// (lane = cell).  Offsets, circumcentres, edges and their tangents pass
+// between slots through shared memory; the first warp adds up the cell's sums
+// while the last one forms the director's cotangent.  One thread per cell left
+// each lane a chain of ~400 FP64 operations per slot (41 us at 4096 cells, one
+// warp per SM); this way 14 us.  Divisions and square roots by fx_rcp and
+// fx_rsqrt (within 1 ulp, no FP64 instruction).
+__global__ void __launch_bounds__(kSlotThreads, kJvpSlotBlocks) k_geom_jvp(JvpArgs g) {
+  __shared__ double2 s_a[CG_RING][32], s_t[CG_RING][32];  // offsets and tangents, then unit edges and theirs
+  __shared__ double2 s_u[CG_RING][32], s_v[CG_RING][32];  // circumcentres and their tangents
+  __shared__ double2 s_A[CG_RING][32], s_P[CG_RING][32];  // terms of A and P and their tangents
+  __shared__ double2 s_k[32], s_kd[32];                   // ka, kp and their tangents
+  const int c = threadIdx.x & 31, w = threadIdx.x >> 5;
   const size_t N = (size_t)g.n;
-  const int cur = g.ctl->cur;
-  const long long* __restrict__ X = g.X + (size_t)cur * N;
-  const long long* __restrict__ Y = g.Y + (size_t)cur * N;
-  const Rep R = g.reps[g.rep[i]];
-  const double sc = R.inv_scale;
-  const long long Xi = X[i], Yi = Y[i];
-  const int m = g.cnt[i];
-  if (m < 3 || m > CG_RING) {
-    raise_status(g.ctl, kETOPO);
-    return;
-  }
-  const int* ring = g.nbr + (size_t)i * CG_RING;
-  const double2 vi = g.v[i];
-
-  const int j0 = ring[0];
-  const double d0x = i2d_exact_a(min_image_i(X[j0] - Xi, R.LX)) * sc;
-  const double d0y = i2d_exact_a(min_image_i(Y[j0] - Yi, R.LY)) * sc;
-  const double2 v0 = g.v[j0];
-  const double t0x = v0.x - vi.x, t0y = v0.y - vi.y;
-  double ax = d0x, ay = d0y, adx = t0x, ady = t0y;
-  for (int a = 0; a < m; ++a) {
-    double bx, by, bdx, bdy;
-    if (a + 1 < m) {
-      const int j = ring[a + 1];
-      bx = i2d_exact_a(min_image_i(X[j] - Xi, R.LX)) * sc;
-      by = i2d_exact_a(min_image_i(Y[j] - Yi, R.LY)) * sc;
-      const double2 vj = g.v[j];
-      bdx = vj.x - vi.x;
-      bdy = vj.y - vi.y;
-    } else {
-      bx = d0x; by = d0y; bdx = t0x; bdy = t0y;
+  const int i = blockIdx.x * 32 + c;
+  const size_t off = g.flat ? 0 : (size_t)g.ctl->cur * N;
+  const long long* __restrict__ X = g.X + off;
+  const long long* __restrict__ Y = g.Y + off;
+  int m = 0;
+  double2 vi = make_double2(0.0, 0.0);
+  if (i < g.n) {
+    m = g.cnt[i];
+    if (m < 3 || m > CG_RING) {
+      if (w == 0) raise_status(g.ctl, kETOPO);
+      m = 0;
     }
-    const double la = ax * ax + ay * ay, lb = bx * bx + by * by;
-    const double det = ax * by - ay * bx;
-    const double r = 1.0 / det;
-    const double ux = 0.5 * (by * la - ay * lb) * r;
-    const double uy = 0.5 * (ax * lb - bx * la) * r;
-    const double ra = (ax - ux) * adx + (ay - uy) * ady;
-    const double rb = (bx - ux) * bdx + (by - uy) * bdy;
-    const double udx = (by * ra - ay * rb) * r;
-    const double udy = (ax * rb - bx * ra) * r;
-    const double detd = adx * by + ax * bdy - ady * bx - ay * bdx;
+    vi = g.v[i];
+    const Rep& R = g.reps[g.rep[i]];
+    const double sc = R.inv_scale;
+    const long long Xi = X[i], Yi = Y[i], LX = R.LX, LY = R.LY;
+    for (int a = w; a < m; a += kSlotWarps) {
+      const int j = g.nbr[(size_t)i * CG_RING + a];
+      const double2 vj = g.v[j];
+      s_a[a][c] = make_double2(i2d_exact_a(min_image_i(X[j] - Xi, LX)) * sc, i2d_exact_a(min_image_i(Y[j] - Yi, LY)) * sc);
+      s_t[a][c] = make_double2(vj.x - vi.x, vj.y - vi.y);
+    }
+  }
+  __syncthreads();
+  for (int a = w; a < m; a += kSlotWarps) {
+    const int an = a + 1 < m ? a + 1 : 0;
+    const double2 A = s_a[a][c], B = s_a[an][c], Ad = s_t[a][c], Bd = s_t[an][c];
+    const double la = A.x * A.x + A.y * A.y, lb = B.x * B.x + B.y * B.y;
+    const double r = fx_rcp(A.x * B.y - A.y * B.x);
+    const double ux = 0.5 * (B.y * la - A.y * lb) * r;
+    const double uy = 0.5 * (A.x * lb - B.x * la) * r;
+    const double ra = (A.x - ux) * Ad.x + (A.y - uy) * Ad.y;
+    const double rb = (B.x - ux) * Bd.x + (B.y - uy) * Bd.y;
+    const double udx = (B.y * ra - A.y * rb) * r;
+    const double udy = (A.x * rb - B.x * ra) * r;
+    const double detd = Ad.x * B.y + A.x * Bd.y - Ad.y * B.x - A.y * Bd.x;
     g.s[a * N + i] = make_double2(ux * r, uy * r);
     g.sd[a * N + i] = make_double2(udx * r - ux * detd * r * r, udy * r - uy * detd * r * r);
-    g.w[a * N + i] = make_double2(by - ay, ax - bx);
-    g.wd[a * N + i] = make_double2(bdy - ady, adx - bdx);
-    s_ux[a][t] = ux; s_uy[a][t] = uy;
-    s_vx[a][t] = udx; s_vy[a][t] = udy;
-    ax = bx; ay = by; adx = bdx; ady = bdy;
+    g.w[a * N + i] = make_double2(B.y - A.y, A.x - B.x);
+    g.wd[a * N + i] = make_double2(Bd.y - Ad.y, Ad.x - Bd.x);
+    s_u[a][c] = make_double2(ux, uy);
+    s_v[a][c] = make_double2(udx, udy);
   }
-  double A = 0.0, Ad = 0.0, P = 0.0, Pd = 0.0;
-  for (int a = 0; a < m; ++a) {
-    const int ap = (a == 0) ? m - 1 : a - 1;
-    const double px = s_ux[ap][t], py = s_uy[ap][t], pdx = s_vx[ap][t], pdy = s_vy[ap][t];
-    const double hx = s_ux[a][t], hy = s_uy[a][t], hdx = s_vx[a][t], hdy = s_vy[a][t];
-    A += px * hy - hx * py;
-    Ad += pdx * hy + px * hdy - hdx * py - hx * pdy;
-    const double ex = hx - px, ey = hy - py, edx = hdx - pdx, edy = hdy - pdy;
-    const double len = sqrt(ex * ex + ey * ey);
-    const double il = 1.0 / len;
+  __syncthreads();
+  for (int a = w; a < m; a += kSlotWarps) {
+    const int ap = a > 0 ? a - 1 : m - 1;
+    const double2 p = s_u[ap][c], pd = s_v[ap][c], h = s_u[a][c], hd = s_v[a][c];
+    s_A[a][c] = make_double2(p.x * h.y - h.x * p.y, pd.x * h.y + p.x * hd.y - hd.x * p.y - h.x * pd.y);
+    const double ex = h.x - p.x, ey = h.y - p.y, edx = hd.x - pd.x, edy = hd.y - pd.y;
+    const double l2 = ex * ex + ey * ey;
+    const double il = fx_rsqrt(l2);
     const double nx = ex * il, ny = ey * il;
     const double dl = nx * edx + ny * edy;
-    P += len;
-    Pd += dl;
-    s_ex[a][t] = nx; s_ey[a][t] = ny;
-    s_fx[a][t] = (edx - nx * dl) * il;
-    s_fy[a][t] = (edy - ny * dl) * il;
+    s_P[a][c] = make_double2(l2 * il, dl);
+    s_a[a][c] = make_double2(nx, ny);
+    s_t[a][c] = make_double2((edx - nx * dl) * il, (edy - ny * dl) * il);
   }
-  A *= 0.5;
-  Ad *= 0.5;
-  const double P0 = g.p0[i] * g.sqrtA0;
-  double ka, kp, kad, kpd;
-  if (g.coefA) {
-    ka = g.coefA[i]; kp = g.coefP[i]; kad = 0.0; kpd = 0.0;
-  } else {
-    ka = 2.0 * g.KA * (A - g.A0); kp = 2.0 * g.KP * (P - P0);
-    kad = 2.0 * g.KA * Ad; kpd = 2.0 * g.KP * Pd;
-  }
-  if (g.A) g.A[i] = A;
-  if (g.P) g.P[i] = P;
-  if (g.Adot) g.Adot[i] = Ad;
-  if (g.Pdot) g.Pdot[i] = Pd;
-  if (g.gp0) {  // parameter cotangents along v = g_{t+1}
-    g.gp0[i] += g.dtmu * 2.0 * g.KP * g.sqrtA0 * Pd;
-    g.gKA[i] += -g.dtmu * 2.0 * (A - g.A0) * Ad;
-    g.gKP[i] += -g.dtmu * 2.0 * (P - P0) * Pd;
+  __syncthreads();
+  if (w == kSlotWarps - 1 && m && g.gp0) {
     double sn, cs;
     sincos(g.theta[i], &sn, &cs);
     g.gv0[i] += g.dt * (vi.x * cs + vi.y * sn);
   }
-  for (int a = 0; a < m; ++a) {
-    const int ap = (a == 0) ? m - 1 : a - 1;
-    const int an = (a + 1 == m) ? 0 : a + 1;
-    const double gx = 0.5 * (s_uy[an][t] - s_uy[ap][t]), gy = 0.5 * (s_ux[ap][t] - s_ux[an][t]);
-    const double gdx = 0.5 * (s_vy[an][t] - s_vy[ap][t]), gdy = 0.5 * (s_vx[ap][t] - s_vx[an][t]);
-    const double qx = s_ex[a][t] - s_ex[an][t], qy = s_ey[a][t] - s_ey[an][t];
-    const double qdx = s_fx[a][t] - s_fx[an][t], qdy = s_fy[a][t] - s_fy[an][t];
-    g.fs[a * N + i] = make_double2(ka * gx + kp * qx, ka * gy + kp * qy);
-    g.fsd[a * N + i] = make_double2(kad * gx + ka * gdx + kpd * qx + kp * qdx, kad * gy + ka * gdy + kpd * qy + kp * qdy);
+  if (w == 0 && m) {
+    double A = 0.0, Ad = 0.0, P = 0.0, Pd = 0.0;
+    for (int a = 0; a < m; ++a) {
+      const double2 tA = s_A[a][c], tP = s_P[a][c];
+      A += tA.x;
+      Ad += tA.y;
+      P += tP.x;
+      Pd += tP.y;
+    }
+    A *= 0.5;
+    Ad *= 0.5;
+    const double P0 = g.p0[i] * g.sqrtA0;
+    double ka, kp, kad, kpd;
+    if (g.coefA) {
+      ka = g.coefA[i]; kp = g.coefP[i]; kad = 0.0; kpd = 0.0;
+    } else {
+      ka = 2.0 * g.KA * (A - g.A0); kp = 2.0 * g.KP * (P - P0);
+      kad = 2.0 * g.KA * Ad; kpd = 2.0 * g.KP * Pd;
+    }
+    s_k[c] = make_double2(ka, kp);
+    s_kd[c] = make_double2(kad, kpd);
+    if (g.Adot) g.Adot[i] = Ad;
+    if (g.Pdot) g.Pdot[i] = Pd;
+    if (g.gp0) {  // parameter cotangents along v = g_{t+1}
+      g.gp0[i] += g.dtmu * 2.0 * g.KP * g.sqrtA0 * Pd;
+      g.gKA[i] += -g.dtmu * 2.0 * (A - g.A0) * Ad;
+      g.gKP[i] += -g.dtmu * 2.0 * (P - P0) * Pd;
+    }
   }
-}
-
-__device__ __forceinline__ int ring_pos_a(const int* __restrict__ nbr, const int* __restrict__ cnt, int j, int i) {
-  const int* row = nbr + (size_t)j * CG_RING;
-  const int mj = cnt[j];
-  for (int b = 0; b < mj; ++b)
-    if (row[b] == i) return b;
-  return -1;
+  __syncthreads();
+  const double2 k = s_k[c], kd = s_kd[c];
+  for (int a = w; a < m; a += kSlotWarps) {
+    const int ap = a > 0 ? a - 1 : m - 1, an = a + 1 < m ? a + 1 : 0;
+    const double2 hn = s_u[an][c], hp = s_u[ap][c], vn = s_v[an][c], vp = s_v[ap][c];
+    const double gx = 0.5 * (hn.y - hp.y), gy = 0.5 * (hp.x - hn.x);
+    const double gdx = 0.5 * (vn.y - vp.y), gdy = 0.5 * (vp.x - vn.x);
+    const double2 e = s_a[a][c], en = s_a[an][c], ed = s_t[a][c], end = s_t[an][c];
+    const double qx = e.x - en.x, qy = e.y - en.y;
+    const double qdx = ed.x - end.x, qdy = ed.y - end.y;
+    g.fs[a * N + i] = make_double2(k.x * gx + k.y * qx, k.x * gy + k.y * qy);
+    g.fsd[a * N + i] = make_double2(kd.x * gx + k.x * gdx + kd.y * qx + k.y * qdx,
+                                    kd.x * gy + k.x * gdy + kd.y * qy + k.y * qdy);
+  }
 }
 
 // H g = -Fdot and the cotangent update g <- g - dt mu H g (in place: this
-// kernel reads only per-slot data written by k_geom_jvp).
-__global__ void k_force_jvp(JvpArgs g) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= g.n) return;
+// kernel reads only per-slot data written by k_geom_jvp).  One thread per
+// (cell, ring slot) as k_geom_jvp; the first warp adds the slots' terms up in
+// ring order.
+__global__ void __launch_bounds__(kSlotThreads, kJvpSlotBlocks) k_force_jvp(JvpArgs g) {
+  __shared__ double2 s_s[CG_RING][32], s_sd[CG_RING][32], s_c[CG_RING][32];
+  __shared__ int s_j[CG_RING][32], s_p[CG_RING][32];
+  __shared__ int s_bad[32];
+  const int c = threadIdx.x & 31, w = threadIdx.x >> 5;
   const size_t N = (size_t)g.n;
-  const int m = g.cnt[i];
-  if (m < 3 || m > CG_RING) return;
-  const int* ring = g.nbr + (size_t)i * CG_RING;
-  const int jfirst = ring[0];
-  const int pfirst = ring_pos_a(g.nbr, g.cnt, jfirst, i);
-  int j = jfirst, pj = pfirst;
-  bool bad = pfirst < 0;
-  double Fdx = 0.0, Fdy = 0.0, Fx = 0.0, Fy = 0.0;
-  for (int a = 0; a < m; ++a) {
-    int k, pk;
-    if (a + 1 < m) {
-      k = ring[a + 1];
-      pk = ring_pos_a(g.nbr, g.cnt, k, i);
-      bad |= pk < 0;
-    } else {
-      k = jfirst;
-      pk = pfirst;
-    }
-    const int mj = g.cnt[j];
-    const int bj = (pj <= 0) ? (mj > 0 ? mj - 1 : 0) : pj - 1;
-    const int bk = pk < 0 ? 0 : pk;
-    const double2 f0 = g.fs[a * N + i], f1 = g.fs[(size_t)bj * N + j], f2 = g.fs[(size_t)bk * N + k];
-    const double2 e0 = g.fsd[a * N + i], e1 = g.fsd[(size_t)bj * N + j], e2 = g.fsd[(size_t)bk * N + k];
+  const int i = blockIdx.x * 32 + c;
+  int m = i < g.n ? g.cnt[i] : 0;
+  if (m < 3 || m > CG_RING) m = 0;
+  bool bad = false;
+  if (w == 0) s_bad[c] = 0;
+  for (int a = w; a < m; a += kSlotWarps) {
+    const int j = g.nbr[(size_t)i * CG_RING + a];
+    const int mj = g.cnt[j], p = ring_pos(g.nbr, g.cnt, j, i);
+    bad |= p < 0;
+    // triangle (i, j, k) is the slot before i's around j and i's slot around k
+    s_p[a][c] = (p < 0 ? 0 : p) | ((p <= 0 ? (mj > 0 ? mj - 1 : 0) : p - 1) << 8);
+    s_j[a][c] = j;
+  }
+  __syncthreads();
+  if (bad) s_bad[c] = 1;
+  for (int a = w; a < m; a += kSlotWarps) {
+    const int an = a + 1 < m ? a + 1 : 0;
+    const size_t o0 = a * N + i, o1 = (size_t)(s_p[a][c] >> 8) * N + s_j[a][c],
+                 o2 = (size_t)(s_p[an][c] & 255) * N + s_j[an][c];
+    const double2 f0 = g.fs[o0], f1 = g.fs[o1], f2 = g.fs[o2];
+    const double2 e0 = g.fsd[o0], e1 = g.fsd[o1], e2 = g.fsd[o2];
+    const double2 wj = g.w[o0], wd = g.wd[o0];
+    s_s[a][c] = g.s[o0];
+    s_sd[a][c] = g.sd[o0];
     const double Gx = f0.x + f1.x + f2.x, Gy = f0.y + f1.y + f2.y;
     const double Gdx = e0.x + e1.x + e2.x, Gdy = e0.y + e1.y + e2.y;
-    const double2 s = g.s[a * N + i], sd = g.sd[a * N + i];
-    const double2 w = g.w[a * N + i], wd = g.wd[a * N + i];
-    const double c = w.x * Gx + w.y * Gy;
-    const double cd = wd.x * Gx + wd.y * Gy + w.x * Gdx + w.y * Gdy;
-    Fx -= s.x * c;
-    Fy -= s.y * c;
-    Fdx -= sd.x * c + s.x * cd;
-    Fdy -= sd.y * c + s.y * cd;
-    j = k;
-    pj = pk;
+    s_c[a][c] = make_double2(wj.x * Gx + wj.y * Gy, wd.x * Gx + wd.y * Gy + wj.x * Gdx + wj.y * Gdy);
   }
-  if (bad) raise_status(g.ctl, kETOPO);
+  __syncthreads();
+  if (w || !m) return;
+  double Fdx = 0.0, Fdy = 0.0, Fx = 0.0, Fy = 0.0;
+  for (int a = 0; a < m; ++a) {
+    const double2 sj = s_s[a][c], sd = s_sd[a][c], cc = s_c[a][c];
+    Fx -= sj.x * cc.x;
+    Fy -= sj.y * cc.x;
+    Fdx -= sd.x * cc.x + sj.x * cc.y;
+    Fdy -= sd.y * cc.x + sj.y * cc.y;
+  }
+  if (s_bad[c]) raise_status(g.ctl, kETOPO);
   if (g.F) g.F[i] = make_double2(Fx, Fy);
   if (g.Hv) g.Hv[i] = make_double2(-Fdx, -Fdy);
   if (g.update) {
@@ -232,6 +240,17 @@ __global__ void k_reduce2(int n, const double* a, const double* b, double* out) 
   }
 }
 
+// Ring i as 16-byte words.
+__device__ __forceinline__ void copy_row(int* dst, const int* src, int i) {
+  const int4* q = reinterpret_cast<const int4*>(src + (size_t)i * CG_RING);
+  const int4 r0 = q[0], r1 = q[1], r2 = q[2], r3 = q[3];
+  int4* d = reinterpret_cast<int4*>(dst + (size_t)i * CG_RING);
+  d[0] = r0;
+  d[1] = r1;
+  d[2] = r2;
+  d[3] = r3;
+}
+
 // Snapshot of the current state (positions of the current buffer, grid
 // coordinates, directors, rings, control word) to / from a flat buffer.
 __global__ void k_snapshot(int n, int save, Ctl* ctl, double* x, double* y, long long* X, long long* Y, double* theta,
@@ -245,13 +264,13 @@ __global__ void k_snapshot(int n, int save, Ctl* ctl, double* x, double* y, long
       s.X[i] = X[cur * N + i]; s.Y[i] = Y[cur * N + i];
       s.theta[i] = theta[i];
       s.cnt[i] = cnt[i];
-      for (int a = 0; a < CG_RING; ++a) s.nbr[(size_t)i * CG_RING + a] = nbr[(size_t)i * CG_RING + a];
+      copy_row(s.nbr, nbr, i);
     } else {
       x[cur * N + i] = s.x[i]; y[cur * N + i] = s.y[i];
       X[cur * N + i] = s.X[i]; Y[cur * N + i] = s.Y[i];
       theta[i] = s.theta[i];
       cnt[i] = s.cnt[i];
-      for (int a = 0; a < CG_RING; ++a) nbr[(size_t)i * CG_RING + a] = s.nbr[(size_t)i * CG_RING + a];
+      copy_row(nbr, s.nbr, i);
     }
   }
   if (i == 0) {
@@ -262,14 +281,14 @@ __global__ void k_snapshot(int n, int save, Ctl* ctl, double* x, double* y, long
 
 void launch_snapshot(int n, int save, Ctl* ctl, double* x, double* y, long long* X, long long* Y, double* theta,
                      int* cnt, int* nbr, const Snapshot& s, cudaStream_t st) {
-  k_snapshot<<<(n + 255) / 256, 256, 0, st>>>(n, save, ctl, x, y, X, Y, theta, cnt, nbr, s);
+  k_snapshot<<<(n + 127) / 128, 128, 0, st>>>(n, save, ctl, x, y, X, Y, theta, cnt, nbr, s);
 }
 
 void launch_geom_jvp(const JvpArgs& a, cudaStream_t st) {
-  if (a.n > 0) k_geom_jvp<<<(a.n + kJvpThreads - 1) / kJvpThreads, kJvpThreads, 0, st>>>(a);
+  if (a.n > 0) k_geom_jvp<<<(a.n + 31) / 32, kSlotThreads, 0, st>>>(a);
 }
 void launch_force_jvp(const JvpArgs& a, cudaStream_t st) {
-  if (a.n > 0) k_force_jvp<<<(a.n + 127) / 128, 128, 0, st>>>(a);
+  if (a.n > 0) k_force_jvp<<<(a.n + 31) / 32, kSlotThreads, 0, st>>>(a);
 }
 void launch_combine_final(int n, const double* gx, const double* gy, const double2* F, double2* g, cudaStream_t st) {
   if (n > 0) k_combine_final<<<(n + 255) / 256, 256, 0, st>>>(n, gx, gy, F, g);

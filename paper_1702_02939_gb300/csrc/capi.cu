@@ -778,7 +778,6 @@ JvpArgs jvp_args(cg_ctx* c, char* bw, const BwdLayout& b) {
   a.dtmu = c->par.dt * c->par.mu;
   a.coefA = a.coefP = nullptr;
   a.v = reinterpret_cast<double2*>(bw + b.v);
-  a.A = a.P = nullptr;
   a.Adot = a.Pdot = nullptr;
   a.fs = c->at<double2>(c->off.fs);
   a.s = c->at<double2>(c->off.s);
@@ -1571,8 +1570,16 @@ int cg_backward(cg_ctx* c, int64_t nsteps, int32_t ckpt_every, void* d_bw, size_
       snapshot(c, 1, snapshot_at(bw + b.seg + (t - t0) * b.snap_bytes, c->N));
       if (t + 1 < t1) CG_CUDA(c, cudaGraphLaunch(c->step_exec, st));
     }
-    for (int64_t t = t1 - 1; t >= t0; --t) {  // the tangent kernels compute their own geometry
-      snapshot(c, 0, snapshot_at(bw + b.seg + (t - t0) * b.snap_bytes, c->N), 0);
+    // the tangent kernels compute their own geometry, from the saved states
+    // in place
+    for (int64_t t = t1 - 1; t >= t0; --t) {
+      const Snapshot s = snapshot_at(bw + b.seg + (t - t0) * b.snap_bytes, c->N);
+      a.X = s.X;
+      a.Y = s.Y;
+      a.flat = 1;
+      a.cnt = s.cnt;
+      a.nbr = s.nbr;
+      a.theta = s.theta;
       launch_geom_jvp(a, st);
       launch_force_jvp(a, st);
     }

@@ -289,20 +289,21 @@ struct JvpArgs {
   const Rep* reps;
   const int* rep;
   Ctl* ctl;
-  const long long *X, *Y;  // [2][n]
+  const long long *X, *Y;  // [2][n] (buffer ctl->cur), or (flat) [n] of a snapshot
+  int flat;
   const int *cnt, *nbr;
   const double* p0;
   const double* theta;
   double A0, sqrtA0, KA, KP, dt, dtmu;
   const double *coefA, *coefP;  // loss coefficients instead of 2K(A-A0), 2K(P-P0), or null
   double2* v;                   // tangent / running cotangent per cell
-  double *A, *P;                // optional outputs
   double *Adot, *Pdot;          // optional outputs: tangents of A and P along v
   double2 *fs, *fsd, *s, *sd, *w, *wd;  // [CG_RING][n]
   double *gp0, *gv0, *gKA, *gKP;        // per-cell accumulators, or null
   double2 *F, *Hv;                      // optional outputs of k_force_jvp
   int update;                           // v <- v - dt mu H v
 };
+constexpr int kJvpSlotBlocks = 4;       // resident blocks per SM of the tangent kernels
 struct Snapshot {
   double *x, *y, *theta;
   long long *X, *Y;

@@ -28,7 +28,7 @@ struct AvmOff {
   size_t spv, spv_bytes;
   size_t hx, hy, hf, vc, vn, cc, cv, theta, thn, p0, v0, a0, P0, A, P, ka, kp, energy, act, Fx, Fy, lock, cand_e, cand,
       done;
-  size_t owned, base_local, base_partial, xs, ys, cnt, nbr, scalar, ctl, dir_tab;
+  size_t owned, base_local, base_partial, xs, ys, cnt, nbr, scalar, partial, ctl, dir_tab;
   size_t div_cells, div_dirs, div_made, div_cslots, div_vslots, div_lock;  // staging of cg_avm_divide
   size_t div_flag, div_ctl;                                                // its rounds
   // storage order: tags of the slots, slots of the tags, candidate priorities
@@ -82,6 +82,7 @@ AvmOff avm_layout(int64_t n, size_t spv_bytes) {
   o.cnt = L.take(n * i4);
   o.nbr = L.take(n * CG_RING * i4);
   o.scalar = L.take(4 * d);
+  o.partial = L.take(kReduceBlocks * d);
   o.ctl = L.take(sizeof(Ctl));
   o.dir_tab = L.take(kDirTabEntries * sizeof(double2));
   o.div_cells = L.take(n * i4);
@@ -658,13 +659,22 @@ int cg_avm_sync(cg_avm_ctx* c) { return c ? avm_status(c) : CG_EINVAL; }
 
 int cg_avm_get_state(cg_avm_ctx* c, double* hx, double* hy, double* theta) {
   if (!c) return CG_EINVAL;
+  const size_t V = c->V;
+  const int* vtag = c->at<int>(c->off.vtag);
+  const int* ctag = c->at<int>(c->off.ctag);
+  if (!c->broken && all_in_place({hx, hy, theta}, sizeof(double))) {
+    // straight into the caller's buffers, one synchronisation
+    launch_gather3(c->V, vtag, c->ctl(), c->at<double>(c->off.hx), c->at<double>(c->off.hy), nullptr, V, hx, hy,
+                   nullptr, c->stream);
+    launch_gather3(c->n, ctag, c->ctl(), nullptr, nullptr, c->at<double>(c->off.theta), 0, nullptr, nullptr, theta,
+                   c->stream);
+    AV_CUDA(c, cudaGetLastError());
+    return avm_status(c);
+  }
   int rc = avm_status(c);
   if (rc) return rc;
   Ctl h;
   AV_CUDA(c, cudaMemcpy(&h, c->ctl(), sizeof(Ctl), cudaMemcpyDeviceToHost));
-  const size_t V = c->V;
-  const int* vtag = c->at<int>(c->off.vtag);
-  const int* ctag = c->at<int>(c->off.ctag);
   // staging: the permuted-copy arrays of the re-sort (3V ints >= V doubles)
   if ((rc = out_by_tag(c, hx, c->at<double>(c->off.hx) + h.cur * V, c->V, vtag, c->at<double>(c->off.vc_s))))
     return rc;
@@ -676,6 +686,13 @@ int cg_avm_get_state(cg_avm_ctx* c, double* hx, double* hy, double* theta) {
 
 int cg_avm_get_topology(cg_avm_ctx* c, int32_t* vc, int32_t* vn, int32_t* cc, int32_t* cv) {
   if (!c) return CG_EINVAL;
+  if (!c->broken && c->permuted && vc && vn && cc && cv && all_in_place({vc, vn, cc, cv}, sizeof(int4))) {
+    // straight into the caller's buffers, one synchronisation
+    launch_avm_topology_by_tag(avm_args(c), c->at<int>(c->off.vslot), c->at<int>(c->off.cslot), vc, vn, cc, cv,
+                               c->stream);
+    AV_CUDA(c, cudaGetLastError());
+    return avm_status(c);
+  }
   int rc = avm_status(c);
   if (rc) return rc;
   const int *svc = c->at<int>(c->off.vc), *svn = c->at<int>(c->off.vn);
@@ -771,7 +788,8 @@ int cg_avm_get_forces(cg_avm_ctx* c, double* Fx, double* Fy, double* energy) {
       launch_gather_d(c->n, c->at<int>(c->off.ctag), a.energy, c->at<double>(c->off.theta_s), c->stream);
       e = c->at<double>(c->off.theta_s);
     }
-    launch_reduce_sum(c->n, e, c->at<double>(c->off.scalar), c->stream);
+    launch_reduce_sum(c->n, e, c->at<double>(c->off.scalar), c->at<double>(c->off.partial),
+                      c->at<unsigned int>(c->off.done), c->stream);
     AV_CUDA(c, cudaMemcpyAsync(energy, c->at<double>(c->off.scalar), sizeof(double), cudaMemcpyDeviceToHost, c->stream));
   }
   return avm_status(c);

@@ -1475,15 +1475,20 @@ __global__ void k_avm_topology_by_tag(AvmArgs g, const int* vslot, const int* cs
       if (vn_out) vn_out[3 * t + k] = (unsigned)w < (unsigned)g.V ? g.vtag[w] : -1;
     }
   }
-  if (t < g.n) {
-    const int c = cslot[t];
+  // V = 2 n: two threads per cell, each half of its list
+  if (t < 2 * g.n) {
+    const int u = t >> 1, h = (t & 1) * 8;
+    const int c = cslot[u];
     const int m = g.cc[c];
-    if (cc_out) cc_out[t] = m;
-    if (cv_out)
-      for (int a = 0; a < CG_RING; ++a) {
-        const int v = g.cv[(size_t)c * CG_RING + a];
-        cv_out[(size_t)t * CG_RING + a] = (a < m && (unsigned)v < (unsigned)g.V) ? g.vtag[v] : -1;
-      }
+    if (cc_out && h == 0) cc_out[u] = m;
+    if (cv_out) {
+      const int4* row = reinterpret_cast<const int4*>(g.cv + (size_t)c * CG_RING + h);
+      int4* out = reinterpret_cast<int4*>(cv_out + (size_t)u * CG_RING + h);
+      auto tag = [&](int a, int v) { return (a < m && (unsigned)v < (unsigned)g.V) ? g.vtag[v] : -1; };
+      const int4 p = row[0], q = row[1];
+      out[0] = make_int4(tag(h, p.x), tag(h + 1, p.y), tag(h + 2, p.z), tag(h + 3, p.w));
+      out[1] = make_int4(tag(h + 4, q.x), tag(h + 5, q.y), tag(h + 6, q.z), tag(h + 7, q.w));
+    }
   }
 }
 

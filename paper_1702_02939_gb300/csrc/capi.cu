@@ -28,7 +28,7 @@ struct Layout {
 struct Offsets {
   size_t key, rank, perm, key_count, key_start, key_partials, theta_alt, p0_alt, v0_alt, tag_alt, rep_alt,
       cnt_alt, nbr_alt;
-  size_t x, y, X, Y, theta, p0, v0, A, P, Fx, Fy, ecell, tmp, tmp2, scalar, nrm, xi;
+  size_t x, y, X, Y, theta, p0, v0, A, P, Fx, Fy, ecell, tmp, tmp2, scalar, partial, nrm, xi;
   size_t tag, nid, nid_alt, rep, cnt, nbr, old_cnt, old_nbr;
   size_t fs, s, w, order;
   size_t flags, list0, list1, dirty_list, dirty_bits, fix_list, fix_bits;
@@ -72,6 +72,7 @@ Offsets layout(int64_t N, int64_t NB, int64_t NK, int R) {
   o.tmp = L.take(N * d);
   o.tmp2 = L.take(N * d);
   o.scalar = L.take(4 * d);
+  o.partial = L.take(kReduceBlocks * d);
   o.nrm = L.take(N * sizeof(double2));
   o.xi = L.take(N * d);
   o.tag = L.take(N * i4);
@@ -611,7 +612,6 @@ void enqueue_repair_round(cg_ctx* c, cudaGraphConditionalHandle h, cudaStream_t 
 int triangulate_all(cg_ctx* c) {
   cudaStream_t st = c->stream;
   CG_CUDA(c, cudaMemsetAsync(c->at<int>(c->off.cnt), 0, c->N * sizeof(int), st));
-  CG_CUDA(c, cudaMemsetAsync(c->at<int>(c->off.nbr), 0xff, c->N * CG_RING * sizeof(int), st));
   CG_CUDA(c, cudaMemsetAsync(c->at<unsigned>(c->off.flags), 0, ((c->N + 31) / 32) * 4, st));
   CG_CUDA(c, cudaMemsetAsync(c->at<int>(c->off.bin_count), 0, c->NB * sizeof(int), st));
   launch_begin_topology(c->ctl(), 0, st);
@@ -636,26 +636,29 @@ int read_status(cg_ctx* c) {
   return CG_OK;
 }
 
-int load_positions(cg_ctx* c, const double* x, const double* y) {
+// Positions (and directors, or null) from the caller's buffers, read in place
+// when they are device memory.
+int load_state(cg_ctx* c, const double* x, const double* y, const double* theta) {
   cudaStream_t st = c->stream;
-  double* tx = c->at<double>(c->off.tmp);
-  double* ty = c->at<double>(c->off.tmp2);
-  CG_CUDA(c, cudaMemcpyAsync(tx, x, c->N * sizeof(double), cudaMemcpyDefault, st));
-  CG_CUDA(c, cudaMemcpyAsync(ty, y, c->N * sizeof(double), cudaMemcpyDefault, st));
-  // user order == storage order until the first sort; scatter through tags
-  double* sx = c->at<double>(c->off.A);  // staging in storage order
-  double* sy = c->at<double>(c->off.P);
-  launch_scatter_d((int)c->N, c->at<int>(c->off.tag), tx, sx, st);
-  launch_scatter_d((int)c->N, c->at<int>(c->off.tag), ty, sy, st);
-  Ctl h;
-  CG_CUDA(c, cudaMemcpyAsync(&h, c->ctl(), sizeof(Ctl), cudaMemcpyDeviceToHost, st));
-  CG_CUDA(c, cudaStreamSynchronize(st));
-  const size_t cur = (size_t)h.cur;
-  launch_snap((int)c->N, c->at<Rep>(c->off.reps), c->at<int>(c->off.rep), sx, sy,
-              c->at<double>(c->off.x) + cur * c->N, c->at<double>(c->off.y) + cur * c->N,
-              c->at<long long>(c->off.X) + cur * c->N, c->at<long long>(c->off.Y) + cur * c->N, c->ctl(), st);
+  const double* src[3] = {x, y, theta};
+  double* stage[3] = {c->at<double>(c->off.tmp), c->at<double>(c->off.tmp2), c->at<double>(c->off.ecell)};
+  for (int k = 0; k < 3; ++k) {
+    if (!src[k] || in_place(src[k], sizeof(double))) continue;
+    CG_CUDA(c, cudaMemcpyAsync(stage[k], src[k], c->N * sizeof(double), cudaMemcpyDefault, st));
+    src[k] = stage[k];
+  }
+  launch_load_state((int)c->N, c->at<Rep>(c->off.reps), c->at<int>(c->off.rep), c->at<int>(c->off.tag), src[0], src[1],
+                    src[2], c->at<double>(c->off.x), c->at<double>(c->off.y), c->at<long long>(c->off.X),
+                    c->at<long long>(c->off.Y), c->at<double>(c->off.theta), c->ctl(), st);
   CG_CUDA(c, cudaGetLastError());
   return CG_OK;
+}
+
+// A status read back earlier refuses the call (kernels check the status word
+// themselves where a caller's buffer would be written).
+int refuse_seen(cg_ctx* c) {
+  if (!c->seen_status) return CG_OK;
+  return fail(c, c->seen_status, std::string("device status: ") + cg_status_string(c->seen_status));
 }
 
 // One step as a graph.  Up to kRestCells cells: the prefix, the first repair
@@ -901,13 +904,10 @@ int cg_create(int32_t R, const cg_replica* reps, const cg_params* params, const 
     TRY(cudaMemcpyAsync(c->ctl(), &h, sizeof(Ctl), cudaMemcpyHostToDevice, st));
     TRY(cudaMemsetAsync(c->at<int>(c->off.key_count), 0, c->NK * sizeof(int), st));
     TRY(cudaMemsetAsync(c->at<int>(c->off.cnt), 0, c->N * sizeof(int), st));
-    TRY(cudaMemcpyAsync(c->at<double>(c->off.tmp), theta, c->N * sizeof(double), cudaMemcpyDefault, st));
 #undef TRY
     if (rc) break;
     launch_init_dir_tables(c->at<double2>(c->off.dir_tab), st);
-    launch_scatter_d((int)c->N, c->at<int>(c->off.tag), c->at<double>(c->off.tmp), c->at<double>(c->off.theta), st);
-    launch_check_finite((int)c->N, c->at<double>(c->off.theta), c->ctl(), st);
-    rc = load_positions(c, x, y);
+    rc = load_state(c, x, y, theta);
     if (rc) break;
     launch_sort(sort_args(c), st);  // spatial order before the first triangulation
     if (cudaMemsetAsync(c->at<unsigned>(c->off.dirty_bits), 0, ((c->N + 31) / 32) * 4, st) != cudaSuccess ||
@@ -1087,13 +1087,22 @@ int cg_sync(cg_ctx* c) {
 
 int cg_get_state(cg_ctx* c, double* x, double* y, double* theta) {
   if (!c) return CG_EINVAL;
+  const int* tag = c->at<int>(c->off.tag);
+  if (all_in_place({x, y, theta}, sizeof(double))) {
+    // one kernel into the caller's buffers and one synchronisation
+    const int rc = refuse_seen(c);
+    if (rc) return rc;
+    launch_gather3((int)c->N, tag, c->ctl(), c->at<double>(c->off.x), c->at<double>(c->off.y),
+                   c->at<double>(c->off.theta), c->N, x, y, theta, c->stream);
+    CG_CUDA(c, cudaGetLastError());
+    return read_status(c);
+  }
   int rc = read_status(c);
   if (rc) return rc;
   Ctl h;
   CG_CUDA(c, cudaMemcpy(&h, c->ctl(), sizeof(Ctl), cudaMemcpyDeviceToHost));
   const size_t cur = (size_t)h.cur;
   cudaStream_t st = c->stream;
-  const int* tag = c->at<int>(c->off.tag);
   double* tmp = c->at<double>(c->off.tmp);
   const double* srcs[3] = {c->at<double>(c->off.x) + cur * c->N, c->at<double>(c->off.y) + cur * c->N,
                            c->at<double>(c->off.theta)};
@@ -1109,16 +1118,9 @@ int cg_get_state(cg_ctx* c, double* x, double* y, double* theta) {
 
 int cg_set_state(cg_ctx* c, const double* x, const double* y, const double* theta) {
   if (!c || !x || !y) return CG_EINVAL;
-  int rc = read_status(c);
+  int rc = refuse_seen(c);
   if (rc) return rc;
-  if (theta) {
-    CG_CUDA(c, cudaMemcpyAsync(c->at<double>(c->off.tmp), theta, c->N * sizeof(double), cudaMemcpyDefault,
-                               c->stream));
-    launch_scatter_d((int)c->N, c->at<int>(c->off.tag), c->at<double>(c->off.tmp), c->at<double>(c->off.theta),
-                     c->stream);
-    launch_check_finite((int)c->N, c->at<double>(c->off.theta), c->ctl(), c->stream);
-  }
-  rc = load_positions(c, x, y);
+  rc = load_state(c, x, y, theta);
   if (rc) return rc;
   rc = triangulate_all(c);
   if (rc) return rc;
@@ -1126,39 +1128,44 @@ int cg_set_state(cg_ctx* c, const double* x, const double* y, const double* thet
   return read_status(c);
 }
 
-static int compute_forces(cg_ctx* c, int want_energy) {
-  GeomArgs g = geom_args(c);
-  if (want_energy) g.energy_out = c->at<double>(c->off.ecell);
-  run_geom(c, g, c->stream);
-  run_force(c, force_args(c, 0), c->stream);
-  if (want_energy) launch_reduce_sum((int)c->N, c->at<double>(c->off.ecell), c->at<double>(c->off.scalar), c->stream);
-  CG_CUDA(c, cudaGetLastError());
-  return CG_OK;
-}
-
-static int gather_out(cg_ctx* c, const double* src, double* dst) {
-  if (!dst) return CG_OK;
+// Two per-cell arrays to the caller.
+static int gather_out(cg_ctx* c, const double* s0, const double* s1, double* d0, double* d1) {
+  const int* tag = c->at<int>(c->off.tag);
+  if (all_in_place({d0, d1}, sizeof(double))) {
+    launch_gather3((int)c->N, tag, c->ctl(), s0, s1, nullptr, 0, d0, d1, nullptr, c->stream);
+    CG_CUDA(c, cudaGetLastError());
+    return CG_OK;
+  }
+  const double* srcs[2] = {s0, s1};
+  double* dsts[2] = {d0, d1};
   double* tmp = c->at<double>(c->off.tmp);
-  launch_gather_d((int)c->N, c->at<int>(c->off.tag), src, tmp, c->stream);
-  CG_CUDA(c, cudaMemcpyAsync(dst, tmp, c->N * sizeof(double), cudaMemcpyDefault, c->stream));
-  CG_CUDA(c, cudaStreamSynchronize(c->stream));
+  for (int k = 0; k < 2; ++k) {
+    if (!dsts[k]) continue;
+    launch_gather_d((int)c->N, tag, srcs[k], tmp, c->stream);
+    CG_CUDA(c, cudaMemcpyAsync(dsts[k], tmp, c->N * sizeof(double), cudaMemcpyDefault, c->stream));
+    CG_CUDA(c, cudaStreamSynchronize(c->stream));
+  }
   return CG_OK;
 }
 
 int cg_get_geometry(cg_ctx* c, double* A, double* P) {
   if (!c) return CG_EINVAL;
-  int rc = compute_forces(c, 0);
-  if (!rc) rc = gather_out(c, c->at<double>(c->off.A), A);
-  if (!rc) rc = gather_out(c, c->at<double>(c->off.P), P);
+  run_geom(c, geom_args(c), c->stream);
+  int rc = gather_out(c, c->at<double>(c->off.A), c->at<double>(c->off.P), A, P);
   if (rc) return rc;
   return read_status(c);
 }
 
 int cg_get_forces(cg_ctx* c, double* Fx, double* Fy, double* energy) {
   if (!c) return CG_EINVAL;
-  int rc = compute_forces(c, energy != nullptr);
-  if (!rc) rc = gather_out(c, c->at<double>(c->off.Fx), Fx);
-  if (!rc) rc = gather_out(c, c->at<double>(c->off.Fy), Fy);
+  GeomArgs g = geom_args(c);
+  if (energy) g.energy_out = c->at<double>(c->off.ecell);
+  run_geom(c, g, c->stream);
+  run_force(c, force_args(c, 0), c->stream);
+  if (energy)
+    launch_reduce_sum((int)c->N, c->at<double>(c->off.ecell), c->at<double>(c->off.scalar),
+                      c->at<double>(c->off.partial), &c->ctl()->done, c->stream);
+  int rc = gather_out(c, c->at<double>(c->off.Fx), c->at<double>(c->off.Fy), Fx, Fy);
   if (rc) return rc;
   if (energy) {
     CG_CUDA(c, cudaMemcpyAsync(energy, c->at<double>(c->off.scalar), sizeof(double), cudaMemcpyDeviceToHost,
@@ -1169,25 +1176,30 @@ int cg_get_forces(cg_ctx* c, double* Fx, double* Fy, double* energy) {
 
 int cg_get_neighbors(cg_ctx* c, int32_t* cnt, int32_t* nbr) {
   if (!c || !cnt || !nbr) return CG_EINVAL;
-  int rc = read_status(c);
+  const bool direct = all_in_place({cnt, nbr}, sizeof(int));
+  int rc = direct ? refuse_seen(c) : read_status(c);
   if (rc) return rc;
-  // stage in the old-ring scratch (free outside a step)
-  int* tc = c->at<int>(c->off.old_cnt);
-  int* tn = c->at<int>(c->off.old_nbr);
-  launch_gather_ring((int)c->N, c->at<int>(c->off.tag), c->at<int>(c->off.cnt), c->at<int>(c->off.nbr), tc, tn,
+  // host buffers: staged in the old-ring scratch (free outside a step)
+  int* tc = direct ? cnt : c->at<int>(c->off.old_cnt);
+  int* tn = direct ? nbr : c->at<int>(c->off.old_nbr);
+  launch_gather_ring((int)c->N, c->at<int>(c->off.tag), c->at<int>(c->off.cnt), c->at<int>(c->off.nbr), c->ctl(), tc, tn,
                      c->stream);
-  CG_CUDA(c, cudaMemcpyAsync(cnt, tc, c->N * sizeof(int), cudaMemcpyDefault, c->stream));
-  CG_CUDA(c, cudaMemcpyAsync(nbr, tn, c->N * CG_RING * sizeof(int), cudaMemcpyDefault, c->stream));
+  if (!direct) {
+    CG_CUDA(c, cudaMemcpyAsync(cnt, tc, c->N * sizeof(int), cudaMemcpyDefault, c->stream));
+    CG_CUDA(c, cudaMemcpyAsync(nbr, tn, c->N * CG_RING * sizeof(int), cudaMemcpyDefault, c->stream));
+  }
   return read_status(c);
 }
 
 static int set_percell(cg_ctx* c, const double* src, size_t off) {
   if (!c || !src) return CG_EINVAL;
-  double* tmp = c->at<double>(c->off.tmp);
-  CG_CUDA(c, cudaMemcpyAsync(tmp, src, c->N * sizeof(double), cudaMemcpyDefault, c->stream));
-  launch_scatter_d((int)c->N, c->at<int>(c->off.tag), tmp, c->at<double>(off), c->stream);
+  if (!in_place(src, sizeof(double))) {
+    double* tmp = c->at<double>(c->off.tmp);
+    CG_CUDA(c, cudaMemcpyAsync(tmp, src, c->N * sizeof(double), cudaMemcpyDefault, c->stream));
+    src = tmp;
+  }
+  launch_scatter_d((int)c->N, c->at<int>(c->off.tag), src, c->at<double>(off), c->stream);
   launch_check_finite((int)c->N, c->at<double>(off), c->ctl(), c->stream);
-  CG_CUDA(c, cudaStreamSynchronize(c->stream));
   return read_status(c);
 }
 
@@ -1246,6 +1258,7 @@ int cg_set_moduli(cg_ctx* c, double KA, double KP) {
   if (!c || !std::isfinite(KA) || !std::isfinite(KP)) return CG_EINVAL;
   int rc = read_status(c);
   if (rc) return rc;
+  if (KA == c->par.KA && KP == c->par.KP) return CG_OK;  // nothing depends on anything new
   c->par.KA = KA;
   c->par.KP = KP;
   if (c->step_exec) {  // kernel parameters are baked into the graph: capture again

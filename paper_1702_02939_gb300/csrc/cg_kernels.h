@@ -3,6 +3,7 @@
 #include <cstddef>
 #include <cstdint>
 #include <cuda_runtime.h>
+#include <initializer_list>
 
 namespace cgk {
 
@@ -243,9 +244,38 @@ inline int check_blocks_all(int n, int sms) {
 }
 
 // state preparation and user-order transfers
+// Positions (and directors, or null) in user order into the current buffers,
+// positions snapped to the grid; a position far outside the box or a director
+// that is not finite raises CG_EINVAL.
+void launch_load_state(int n, const Rep* reps, const int* rep, const int* tag, const double* xin, const double* yin,
+                       const double* tin, double* x2, double* y2, long long* X2, long long* Y2, double* theta, Ctl* ctl,
+                       cudaStream_t st);
 void launch_snap(int n, const Rep* reps, const int* rep, const double* xin, const double* yin, double* x,
                  double* y, long long* X, long long* Y, Ctl* ctl, cudaStream_t st);
 void launch_gather_d(int n, const int* tag, const double* src, double* dst_user, cudaStream_t st);
+// Up to three per-cell (or per-vertex) arrays into user order at once, straight
+// into the caller's device buffers (null: skipped); nothing is written when a
+// status is raised.  stride: the first two are pairs of buffers that far apart,
+// ctl->cur the current one (0: single arrays).
+void launch_gather3(int n, const int* tag, const Ctl* ctl, const double* s0, const double* s1, const double* s2,
+                    size_t stride, double* d0, double* d1, double* d2, cudaStream_t st);
+// p where a kernel can write or read it in place (device memory of the current
+// device, aligned), else null
+inline void* in_place(const void* p, size_t align) {
+  cudaPointerAttributes a;
+  int dev = -1;
+  if (!p || ((uintptr_t)p & (align - 1)) || cudaGetDevice(&dev) != cudaSuccess ||
+      cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  return a.type == cudaMemoryTypeDevice && a.device == dev ? const_cast<void*>(p) : nullptr;
+}
+inline bool all_in_place(std::initializer_list<const void*> ps, size_t align) {
+  for (const void* p : ps)
+    if (p && !in_place(p, align)) return false;
+  return true;
+}
 void launch_check_finite(int n, const double* v, Ctl* ctl, cudaStream_t st);
 void launch_scatter_d(int n, const int* tag, const double* src_user, double* dst, cudaStream_t st);
 void launch_scatter_i(int n, const int* tag, const int* src_user, int* dst, cudaStream_t st);
@@ -261,9 +291,13 @@ void launch_halo_unpack(int n, const int* tag, const int* slot, const Rep* reps,
 // destination is skipped
 void launch_gather_cur_xy(int n, const int* tag, const double* x2, const double* y2, const Ctl* ctl, int pending,
                           double* dst_x, double* dst_y, cudaStream_t st);
-void launch_gather_ring(int n, const int* tag, const int* cnt, const int* nbr, int* cnt_user, int* nbr_user,
-                        cudaStream_t st);
-void launch_reduce_sum(int n, const double* v, double* out, cudaStream_t st);
+// (nothing is written when a status is raised)
+void launch_gather_ring(int n, const int* tag, const int* cnt, const int* nbr, const Ctl* ctl, int* cnt_user,
+                        int* nbr_user, cudaStream_t st);
+// sum of v into *out; partial: scratch of kReduceBlocks doubles, done: a zeroed
+// counter (left zero)
+constexpr int kReduceBlocks = 128;
+void launch_reduce_sum(int n, const double* v, double* out, double* partial, unsigned int* done, cudaStream_t st);
 
 // Hilbert re-sort of all per-cell state (sort_kernels.cu)
 struct SortArgs {

@@ -120,12 +120,22 @@ bool make_rep(int n, double Lx, double Ly, Rep& p) {
   return true;
 }
 
-__global__ void k_noalloc_index(int n, int* tag, int* rep) {
+// What every call starts from (the array keeps the previous call's contents):
+// zero control word, flags, bin counts and ring counts, the replica's constants
+// and the identity order, in one kernel.
+__global__ void k_noalloc_begin(int n, int nbins, Rep rep, Rep* d_rep, Ctl* ctl, unsigned* flags, int* bin_count,
+                                int* cnt, int* tag, int* repi) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) {
-    tag[i] = i;
-    rep[i] = 0;
+  if (i == 0) {
+    *d_rep = rep;
+    *ctl = Ctl{};
   }
+  if (i < nbins) bin_count[i] = 0;
+  if (i >= n) return;
+  tag[i] = i;
+  repi[i] = 0;
+  cnt[i] = 0;
+  if ((i & 31) == 0) flags[i >> 5] = 0u;
 }
 
 }  // namespace
@@ -153,14 +163,9 @@ extern "C" int cg_triangulate_noalloc(int32_t n, double Lx, double Ly, const dou
   unsigned* flags = reinterpret_cast<unsigned*>(base + kOffFlags);
   const int nbins = rep.nbx * rep.nby;
 
-  // state that must start at zero (the array keeps the previous call's contents)
-  if (cudaMemsetAsync(ctl, 0, sizeof(Ctl), st) != cudaSuccess) return CG_ECUDA;
-  if (cudaMemsetAsync(flags, 0, 4 * (size_t)((n + 31) / 32), st) != cudaSuccess) return CG_ECUDA;
-  if (cudaMemsetAsync(base + kOffBinCount, 0, 4 * (size_t)nbins, st) != cudaSuccess) return CG_ECUDA;
-  if (cudaMemsetAsync(cnt, 0, 4 * (size_t)n, st) != cudaSuccess) return CG_ECUDA;
-  if (cudaMemsetAsync(nbr, 0xff, 4 * (size_t)n * CG_RING, st) != cudaSuccess) return CG_ECUDA;
-  if (cudaMemcpyAsync(d_rep, &rep, sizeof(Rep), cudaMemcpyHostToDevice, st) != cudaSuccess) return CG_ECUDA;
-  k_noalloc_index<<<(n + 255) / 256, 256, 0, st>>>(n, tag, repi);
+  const int items = n > nbins ? n : nbins;
+  k_noalloc_begin<<<(items + 255) / 256, 256, 0, st>>>(n, nbins, rep, d_rep, ctl, flags,
+                                                       reinterpret_cast<int*>(base + kOffBinCount), cnt, tag, repi);
   launch_snap(n, d_rep, repi, d_x, d_y, x, y, X, Y, ctl, st);
 
   CellListArgs cl{};  // every field starts zero or null
@@ -214,7 +219,7 @@ extern "C" int cg_triangulate_noalloc(int32_t n, double Lx, double Ly, const dou
   ck.all_cells = 1;
   launch_check(ck, check_blocks_all(n, sms), st);
 
-  launch_gather_ring(n, tag, cnt, nbr, d_cnt, d_nbr, st);
+  launch_gather_ring(n, tag, cnt, nbr, ctl, d_cnt, d_nbr, st);
   if (cudaGetLastError() != cudaSuccess) return CG_ECUDA;
   // the status word read on the caller's stream, behind the kernels above
   int status = 0;

@@ -859,12 +859,8 @@ void launch_check(const CheckArgs& a, int grid_blocks, cudaStream_t st) {
 // ---------------------------------------------------------------------------
 // State preparation and user-order transfers.
 // ---------------------------------------------------------------------------
-__global__ void k_snap(int n, const Rep* reps, const int* rep, const double* xin, const double* yin, double* x,
-                       double* y, long long* X, long long* Y, Ctl* ctl) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const Rep R = reps[rep[i]];
-  const double xv = xin[i], yv = yin[i];
+__device__ __forceinline__ void snap_cell(const Rep& R, int i, double xv, double yv, double* x, double* y, long long* X,
+                                          long long* Y, Ctl* ctl) {
   if (!(xv >= -R.Lx && xv < 2.0 * R.Lx && yv >= -R.Ly && yv < 2.0 * R.Ly)) {
     raise_status(ctl, kEINVAL);
     x[i] = y[i] = 0.0;
@@ -880,10 +876,38 @@ __global__ void k_snap(int n, const Rep* reps, const int* rep, const double* xin
   y[i] = (double)Yv * R.inv_scale;
 }
 
+__global__ void k_snap(int n, const Rep* reps, const int* rep, const double* xin, const double* yin, double* x,
+                       double* y, long long* X, long long* Y, Ctl* ctl) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) snap_cell(reps[rep[i]], i, xin[i], yin[i], x, y, X, Y, ctl);
+}
+
 void launch_snap(int n, const Rep* reps, const int* rep, const double* xin, const double* yin, double* x, double* y,
                  long long* X, long long* Y, Ctl* ctl, cudaStream_t st) {
   if (n <= 0) return;
   k_snap<<<(n + 255) / 256, 256, 0, st>>>(n, reps, rep, xin, yin, x, y, X, Y, ctl);
+}
+
+__global__ void k_load_state(int n, const Rep* reps, const int* rep, const int* tag, const double* xin,
+                             const double* yin, const double* tin, double* x2, double* y2, long long* X2,
+                             long long* Y2, double* theta, Ctl* ctl) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const int u = tag[i];
+  const size_t off = (size_t)ctl->cur * n;
+  snap_cell(reps[rep[i]], i, xin[u], yin[u], x2 + off, y2 + off, X2 + off, Y2 + off, ctl);
+  if (tin) {
+    const double th = tin[u];
+    theta[i] = th;
+    if (!isfinite(th)) raise_status(ctl, kEINVAL);
+  }
+}
+
+void launch_load_state(int n, const Rep* reps, const int* rep, const int* tag, const double* xin, const double* yin,
+                       const double* tin, double* x2, double* y2, long long* X2, long long* Y2, double* theta, Ctl* ctl,
+                       cudaStream_t st) {
+  if (n <= 0) return;
+  k_load_state<<<(n + 255) / 256, 256, 0, st>>>(n, reps, rep, tag, xin, yin, tin, x2, y2, X2, Y2, theta, ctl);
 }
 
 // Inputs handed in from outside must be finite (directors, p0, v0).
@@ -899,6 +923,20 @@ __global__ void k_gather_d(int n, const int* tag, const double* src, double* dst
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) dst[tag[i]] = src[i];
 }
+__global__ void k_gather3(int n, const int* tag, const Ctl* ctl, const double* s0, const double* s1, const double* s2,
+                          size_t stride, double* d0, double* d1, double* d2) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n || ctl->status) return;
+  const size_t at = ctl->cur * stride + i;
+  const int u = tag[i];
+  if (d0) d0[u] = s0[at];
+  if (d1) d1[u] = s1[at];
+  if (d2) d2[u] = s2[i];
+}
+void launch_gather3(int n, const int* tag, const Ctl* ctl, const double* s0, const double* s1, const double* s2,
+                    size_t stride, double* d0, double* d1, double* d2, cudaStream_t st) {
+  if (n > 0) k_gather3<<<(n + 255) / 256, 256, 0, st>>>(n, tag, ctl, s0, s1, s2, stride, d0, d1, d2);
+}
 // Current positions (buffer ctl->cur of x2, y2, each [2][n]) in user order.
 __global__ void k_gather_cur_xy(int n, const int* tag, const double* x2, const double* y2, const Ctl* ctl,
                                 int pending, double* dst_x, double* dst_y) {
@@ -913,27 +951,38 @@ __global__ void k_scatter_d(int n, const int* tag, const double* src, double* ds
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) dst[i] = src[tag[i]];
 }
-__global__ void k_gather_ring(int n, const int* tag, const int* cnt, const int* nbr, int* cnt_u, int* nbr_u) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
+// Rings in user order: a thread per (cell, slot), so the rows are read and
+// written whole.
+__global__ void k_gather_ring(int n, const int* tag, const int* cnt, const int* nbr, const Ctl* ctl, int* cnt_u,
+                              int* nbr_u) {
+  const int i = blockIdx.x * 16 + (threadIdx.x >> 4), a = threadIdx.x & 15;
+  if (i >= n || ctl->status) return;
   const int t = tag[i], m = cnt[i];
-  cnt_u[t] = m;
-  for (int a = 0; a < CG_RING; ++a) {
-    const int j = (a < m) ? nbr[(size_t)i * CG_RING + a] : -1;
-    nbr_u[(size_t)t * CG_RING + a] = (j >= 0 && j < n) ? tag[j] : -1;
-  }
+  const int j = (a < m) ? nbr[(size_t)i * CG_RING + a] : -1;
+  if (a == 0) cnt_u[t] = m;
+  nbr_u[(size_t)t * CG_RING + a] = (j >= 0 && j < n) ? tag[j] : -1;
 }
-__global__ void __launch_bounds__(1024) k_reduce_sum(int n, const double* v, double* out) {
-  __shared__ double buf[1024];
-  double s = 0.0;
-  for (int i = threadIdx.x; i < n; i += 1024) s += v[i];
-  buf[threadIdx.x] = s;
-  __syncthreads();
-  for (int o = 512; o > 0; o >>= 1) {
-    if (threadIdx.x < o) buf[threadIdx.x] += buf[threadIdx.x + o];
+// Sums over fixed shares of the array, the last block to finish adds them up
+// (one block alone took 60 us at 262144 values).
+__global__ void __launch_bounds__(256) k_reduce_sum(int n, const double* v, double* out, double* partial,
+                                                    unsigned int* done) {
+  __shared__ double buf[256];
+  auto total = [&](double s) {
+    buf[threadIdx.x] = s;
     __syncthreads();
-  }
-  if (threadIdx.x == 0) *out = buf[0];
+    for (int o = 128; o > 0; o >>= 1) {
+      if (threadIdx.x < o) buf[threadIdx.x] += buf[threadIdx.x + o];
+      __syncthreads();
+    }
+    return buf[0];
+  };
+  double s = 0.0;
+  for (int i = blockIdx.x * 256 + threadIdx.x; i < n; i += kReduceBlocks * 256) s += v[i];
+  s = total(s);
+  if (threadIdx.x == 0) partial[blockIdx.x] = s;
+  if (!last_block(done)) return;
+  s = total(threadIdx.x < kReduceBlocks ? *(volatile double*)&partial[threadIdx.x] : 0.0);
+  if (threadIdx.x == 0) *out = s;
 }
 
 void launch_gather_d(int n, const int* tag, const double* src, double* dst_user, cudaStream_t st) {
@@ -1021,12 +1070,12 @@ void launch_halo_unpack(int n, const int* tag, const int* slot, const Rep* reps,
                         const long long* in, double* x2, double* y2, long long* X2, long long* Y2, cudaStream_t st) {
   if (n > 0) k_halo_unpack<<<(n + 255) / 256, 256, 0, st>>>(n, tag, slot, reps, rep, ctl, in, x2, y2, X2, Y2);
 }
-void launch_gather_ring(int n, const int* tag, const int* cnt, const int* nbr, int* cnt_user, int* nbr_user,
-                        cudaStream_t st) {
-  if (n > 0) k_gather_ring<<<(n + 255) / 256, 256, 0, st>>>(n, tag, cnt, nbr, cnt_user, nbr_user);
+void launch_gather_ring(int n, const int* tag, const int* cnt, const int* nbr, const Ctl* ctl, int* cnt_user,
+                        int* nbr_user, cudaStream_t st) {
+  if (n > 0) k_gather_ring<<<(n + 15) / 16, 256, 0, st>>>(n, tag, cnt, nbr, ctl, cnt_user, nbr_user);
 }
-void launch_reduce_sum(int n, const double* v, double* out, cudaStream_t st) {
-  k_reduce_sum<<<1, 1024, 0, st>>>(n, v, out);
+void launch_reduce_sum(int n, const double* v, double* out, double* partial, unsigned int* done, cudaStream_t st) {
+  k_reduce_sum<<<kReduceBlocks, 256, 0, st>>>(n, v, out, partial, done);
 }
 
 }  // namespace cgk

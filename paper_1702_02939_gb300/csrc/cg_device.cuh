@@ -228,31 +228,54 @@ __device__ __forceinline__ double fast_rsqrt(double x) {
 // its top 64 bits rounded to 53 with a sticky bit for the rest (a carry out
 // of the mantissa lands in the exponent field); times 2^e2 (exact).
 __device__ __forceinline__ double i128_to_double(__int128 v, int e2 = 0) {
-  const bool neg = v < 0;
-  const unsigned __int128 a = neg ? (unsigned __int128)(-v) : (unsigned __int128)v;
+  const long long sgn = (long long)(v >> 127);
+  const unsigned __int128 a = (unsigned __int128)((v ^ (__int128)sgn) - (__int128)sgn);
   const unsigned long long hi = (unsigned long long)(a >> 64), lo = (unsigned long long)a;
-  int nb;  // significant bits
-  unsigned long long top;
-  bool sticky;
-  if (hi) {
-    const int lz = __clzll((long long)hi);
-    nb = 128 - lz;
-    const unsigned __int128 sh = a << lz;
-    top = (unsigned long long)(sh >> 64);
-    sticky = (unsigned long long)sh != 0;
-  } else if (lo) {
-    const int lz = __clzll((long long)lo);
-    nb = 64 - lz;
-    top = lo << lz;
-    sticky = false;
-  } else {
-    return 0.0;
-  }
-  unsigned long long m = top >> 11;
-  const unsigned long long rem = top & 0x7ff;
-  if (rem > 0x400 || (rem == 0x400 && (sticky || (m & 1)))) m += 1;
-  const unsigned long long bits = ((unsigned long long)(nb + 1021 + e2) << 52) + m;
-  return __longlong_as_double((long long)(bits | (neg ? 0x8000000000000000ull : 0ull)));
+  const unsigned long long H = hi ? hi : lo, L = hi ? lo : 0ull;
+  if (!H) return 0.0;
+  const int lz = __clzll((long long)H);
+  const unsigned long long top = ((H << lz) | ((L >> 1) >> (63 - lz))) | ((L << lz) ? 1ull : 0ull);
+  const unsigned long long m = top >> 11;
+  const unsigned long long up = ((unsigned)top & 0x7ffu) + ((unsigned)m & 1u) > 0x400u ? 1ull : 0ull;
+  const unsigned long long bits = ((unsigned long long)((hi ? 128 : 64) - lz + 1021 + e2) << 52) + m + up;
+  return __longlong_as_double((long long)(bits | ((unsigned long long)sgn & 0x8000000000000000ull)));
+}
+
+// Exact products of grid offsets (|offset| <= 2^49) from 25-bit halves: every
+// partial product is one 32 x 32 -> 64 multiply-add and no sum overflows, where
+// a signed 64 x 64 -> 128 product takes some thirty instructions.
+__device__ __forceinline__ long long wmul(int a, int b) { return (long long)a * b; }
+// p2 2^(2h) + p1 2^h + p0
+template <int h>
+__device__ __forceinline__ __int128 join3(long long p2, long long p1, long long p0) {
+  constexpr long long mask = (1LL << h) - 1;
+  const long long q = p1 + (p0 >> h), s = p2 + (q >> h);
+  const unsigned long long low = ((unsigned long long)(q & mask) << h) | (unsigned long long)(p0 & mask);
+  return ((__int128)s << (2 * h)) | (__int128)low;
+}
+// (a x b)
+__device__ __forceinline__ __int128 cross_exact(long long ax, long long ay, long long bx, long long by) {
+  constexpr int h = 25, mask = (1 << h) - 1;
+  const int ax1 = (int)(ax >> h), ax0 = (int)ax & mask, ay1 = (int)(ay >> h), ay0 = (int)ay & mask;
+  const int bx1 = (int)(bx >> h), bx0 = (int)bx & mask, by1 = (int)(by >> h), by0 = (int)by & mask;
+  return join3<h>(wmul(ax1, by1) - wmul(ay1, bx1),
+                  wmul(ax1, by0) + wmul(ax0, by1) - wmul(ay1, bx0) - wmul(ay0, bx1),
+                  wmul(ax0, by0) - wmul(ay0, bx0));
+}
+// |a|^2
+__device__ __forceinline__ unsigned __int128 norm2_exact(long long ax, long long ay) {
+  constexpr int h = 25, mask = (1 << h) - 1;
+  const int ax1 = (int)(ax >> h), ax0 = (int)ax & mask, ay1 = (int)(ay >> h), ay0 = (int)ay & mask;
+  return (unsigned __int128)join3<h>(wmul(ax1, ax1) + wmul(ay1, ay1), 2 * (wmul(ax1, ax0) + wmul(ay1, ay0)),
+                                     wmul(ax0, ax0) + wmul(ay0, ay0));
+}
+// b l - a k for offsets a, b and 0 <= k, l < 2^62, from 31-bit halves
+__device__ __forceinline__ __int128 scaled_diff_exact(long long b, long long l, long long a, long long k) {
+  constexpr int h = 31, mask = 0x7fffffff;
+  const int b1 = (int)(b >> h), b0 = (int)b & mask, a1 = (int)(a >> h), a0 = (int)a & mask;
+  const int l1 = (int)(l >> h), l0 = (int)l & mask, k1 = (int)(k >> h), k0 = (int)k & mask;
+  return join3<h>(wmul(b1, l1) - wmul(a1, k1),
+                  (wmul(b0, l1) - wmul(a0, k1)) + (wmul(b1, l0) - wmul(a1, k0)), wmul(b0, l0) - wmul(a0, k0));
 }
 
 // Puts cell i on a list once per use of the bitmap: the caller that sets
@@ -268,49 +291,62 @@ __device__ __forceinline__ int u128_bits(unsigned __int128 v) {
   return hi ? 128 - __clzll((long long)hi) : 64 - __clzll((long long)lo);
 }
 
+// The low 64 bits of v >> S, 0 <= S < 64.
+__device__ __forceinline__ unsigned long long shr128(unsigned __int128 v, int S) {
+  return ((unsigned long long)v >> S) | (((unsigned long long)(v >> 64) << 1) << (63 - S));
+}
+
 // 1/d and 1/sqrt(x) with the refinement on the integer pipes: the mantissa
-// (53 bits) in fixed point, an FP32 hardware seed (rcp/rsqrt.approx of the
-// mantissa's top 23 bits, relative error ~2^-22), one third-order step in
-// Q1.62 (r (1 + e + e^2) with e = 1 - m r; y (1 + e/2 + 3 e^2/8) with
-// e = 1 - m y^2; the error left is ~e^3 ~ 2^-66), and one rounding to double
-// with the exponent put back: within 1 ulp, like fast_rcp / fast_rsqrt, with
-// no FP64 instruction.  Zero, subnormal, infinite and NaN inputs take the
-// FP64 functions.
-__device__ __forceinline__ long long seed_q62(float yf) {  // yf in (0.5, 1]: yf 2^62
+// (53 bits) in fixed point, an FP32 hardware seed of its top 23 bits (rcp/
+// rsqrt.approx, relative error ~2^-22), lowered by 2^-21 so that the residual
+// e is positive and every product unsigned, one step of the series (1 + e +
+// e^2; 1 + e/2 + 3 e^2/8 + 5 e^3/16) whose small powers of e take 32-bit
+// products, and one rounding to double with the exponent put back: within 0.51
+// ulp and no FP64 instruction.  Zero, subnormal, huge, infinite and NaN inputs
+// take the FP64 functions.
+//
+// Three (five) signed 64 x 64 -> 128 products and a general conversion took
+// about 140 (260) instructions; this takes about 50 (60).
+__device__ __forceinline__ unsigned long long seed_q63(float yf) {  // yf in (0.5, 1]: yf (1 - 2^-21) 2^63
   const int b = __float_as_int(yf);
-  const long long mant = (long long)((b & 0x7fffff) | 0x800000);
-  return mant << (39 + ((b >> 23) & 0xff) - 127);  // 62 - 23 + exponent (0 or -1)
+  const unsigned long long mant = (unsigned long long)((b & 0x7fffff) | 0x800000) << (40 + ((b >> 23) & 0xff) - 127);
+  return mant - (mant >> 21);
+}
+// Y 2^-63 (Y in (2^62, 2^63]) times 2^k as a double
+__device__ __forceinline__ double q63_to_double(unsigned long long Y, int k, unsigned long long sgn) {
+  const unsigned long long q = (Y + 512ull) >> 10;  // 2^53 times the value, in (2^52, 2^53]
+  return __longlong_as_double((long long)((((unsigned long long)(1021 + k) << 52) + q) | sgn));
 }
 __device__ __forceinline__ double fx_rcp(double d) {
   const long long b = __double_as_longlong(d);
   const int ef = (int)((b >> 52) & 0x7ff);
-  if (ef == 0 || ef == 0x7ff) return fast_rcp(d);
-  const long long m = (b & 0xFFFFFFFFFFFFFLL) | 0x10000000000000LL;  // mantissa in [1, 2) times 2^52
+  if (ef == 0 || ef > 2040) return fast_rcp(d);
+  const unsigned long long M = ((unsigned long long)b << 11) | 0x8000000000000000ull;  // mantissa times 2^63
   float yf;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(yf) : "f"(__int_as_float(0x3f800000 | (int)((b >> 29) & 0x7fffff))));
-  long long y = seed_q62(yf);
-  const long long e = kQOne - mulq(m << 10, y);  // 1 - m y
-  y += mulq(y, e + mulq(e, e));
-  const double r = q2d(y, -62 - (ef - 1023));
-  return b < 0 ? -r : r;
+  const unsigned long long Y = seed_q63(yf);
+  const unsigned long long e = (unsigned long long)kQOne - __umul64hi(M, Y);  // 1 - m y, times 2^62, below 2^42
+  const unsigned e16 = (unsigned)(e >> 16);
+  const unsigned long long t = e + (((unsigned long long)e16 * e16) >> 30);
+  return q63_to_double(Y + __umul64hi(Y, t << 2), 1023 - ef, (unsigned long long)b & 0x8000000000000000ull);
 }
 __device__ __forceinline__ double fx_rsqrt(double x) {
   const long long b = __double_as_longlong(x);
   const int ef = (int)((b >> 52) & 0x7ff);
   if (ef == 0 || ef == 0x7ff || b < 0) return fast_rsqrt(x);
   const int E = ef - 1023, odd = E & 1;
-  const long long m = (b & 0xFFFFFFFFFFFFFLL) | 0x10000000000000LL;
-  // x = m' 2^(E - odd) with m' = m 2^(odd - 52) in [1, 4), held as m' 2^61
-  const long long mq61 = m << (9 + odd);
+  // x = m' 2^(E - odd) with m' in [1, 4), held as m' 2^62
+  const unsigned long long M = (((unsigned long long)b & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull) << (10 + odd);
   float yf;
   asm("rsqrt.approx.ftz.f32 %0, %1;"
       : "=f"(yf)
       : "f"(__int_as_float((odd ? 0x40000000 : 0x3f800000) | (int)((b >> 29) & 0x7fffff))));
-  long long y = seed_q62(yf);
-  const long long my2 = (long long)(((__int128)mq61 * mulq(y, y)) >> 61);  // m' y^2 in Q1.62
-  const long long e = kQOne - my2;
-  y += mulq(y, mulq(e, (kQOne >> 1) + mulq(e, 3 * (kQOne >> 3))));
-  return q2d(y, -62 - (E - odd) / 2);
+  const unsigned long long Y = seed_q63(yf);
+  const unsigned long long e = (unsigned long long)kQOne - __umul64hi(M, __umul64hi(Y, Y) << 2);  // 1 - m' y^2
+  const unsigned e16 = (unsigned)(e >> 16);
+  const unsigned long long e2 = ((unsigned long long)e16 * e16) >> 30, e3 = (e2 * e16) >> 46;
+  const unsigned long long t = (e >> 1) + ((3ull * e2) >> 3) + ((5ull * e3) >> 4);
+  return q63_to_double(Y + __umul64hi(Y, t << 2), -((E - odd) >> 1), 0ull);
 }
 
 // Standard normal for (seed, cell tag, step), cosine branch of Box-Muller,

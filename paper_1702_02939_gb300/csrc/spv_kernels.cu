@@ -27,16 +27,15 @@ namespace cgk {
 // |a|^2 and |b|^2 cut to 62 significant bits by a shift common to the triangle
 // (at least as accurate as FP64 products of the rounded squares), each rounded
 // to double once.
-__device__ __forceinline__ void geom_vertex(long long AX, long long AY, long long BX, long long BY, double2& h,
-                                            double2& s) {
-  const unsigned __int128 LA = (unsigned __int128)((__int128)AX * AX + (__int128)AY * AY);
-  const unsigned __int128 LB = (unsigned __int128)((__int128)BX * BX + (__int128)BY * BY);
-  const double det = i128_to_double((__int128)AX * BY - (__int128)AY * BX);
-  const double r = fx_rcp(det);
+// (LA, LB: the exact squared lengths.)
+__device__ __forceinline__ void geom_vertex(long long AX, long long AY, unsigned __int128 LA, long long BX,
+                                            long long BY, unsigned __int128 LB, double2& h, double2& s) {
+  const double r = fx_rcp(i128_to_double(cross_exact(AX, AY, BX, BY)));
+  // |offsets| < 2^49 and the cut squares < 2^62: the numerators fit in 113 bits
   const int S = max(u128_bits(LA > LB ? LA : LB) - 62, 0);
-  const long long la = (long long)(LA >> S), lb = (long long)(LB >> S);
-  h.x = i128_to_double((__int128)BY * la - (__int128)AY * lb, S) * r;
-  h.y = i128_to_double((__int128)AX * lb - (__int128)BX * la, S) * r;
+  const long long la = (long long)shr128(LA, S), lb = (long long)shr128(LB, S);
+  h.x = i128_to_double(scaled_diff_exact(BY, la, AY, lb), S) * r;
+  h.y = i128_to_double(scaled_diff_exact(AX, lb, BX, la), S) * r;
   s = make_double2(h.x * r, h.y * r);
 }
 
@@ -115,15 +114,9 @@ __global__ void __launch_bounds__(kGeomThreads, kGeomMinBlocks) k_geom(GeomArgs 
       return ((unsigned)j < (unsigned)g.n) ? j : i;
     };
 
-    // squared lengths and the triangle determinants exactly in 128-bit
-    // integers from the grid offsets; the doubled circumcentre g = num / det
-    // with num = (b_y |a|^2 - a_y |b|^2, a_x |b|^2 - b_x |a|^2) in 128-bit
-    // integers too, from |a|^2 and |b|^2 cut to 62 significant bits by a
-    // shift common to the triangle (at least as accurate as FP64 products
-    // of the rounded squares), each rounded to double once
     const int j0 = nb(0);
     const long long D0X = min_image_i(X[j0] - Xi, R.LX), D0Y = min_image_i(Y[j0] - Yi, R.LY);
-    const unsigned __int128 L0 = (unsigned __int128)((__int128)D0X * D0X + (__int128)D0Y * D0Y);
+    const unsigned __int128 L0 = norm2_exact(D0X, D0Y);
     unsigned __int128 LA = L0;
     long long AX = D0X, AY = D0Y;
     double hpx = 0.0, hpy = 0.0, h0x = 0.0, h0y = 0.0;
@@ -135,19 +128,14 @@ __global__ void __launch_bounds__(kGeomThreads, kGeomMinBlocks) k_geom(GeomArgs 
         const int j = nb(a + 1);
         BX = min_image_i(X[j] - Xi, R.LX);
         BY = min_image_i(Y[j] - Yi, R.LY);
-        LB = (unsigned __int128)((__int128)BX * BX + (__int128)BY * BY);
+        LB = norm2_exact(BX, BY);
       } else {
         BX = D0X; BY = D0Y; LB = L0;
       }
-      // (r_j - r_i) x (r_k - r_i)
-      const double det = i128_to_double((__int128)AX * BY - (__int128)AY * BX);
-      const double r = fx_rcp(det);
-      // |offsets| < 2^49 and the cut squares < 2^62: the numerators fit in 113 bits
-      const int S = max(u128_bits(LA > LB ? LA : LB) - 62, 0);
-      const long long la = (long long)(LA >> S), lb = (long long)(LB >> S);
-      const double hx = i128_to_double((__int128)BY * la - (__int128)AY * lb, S) * r;
-      const double hy = i128_to_double((__int128)AX * lb - (__int128)BX * la, S) * r;
-      g.s[a * N + i] = make_double2(hx * r, hy * r);
+      double2 h, sj;
+      geom_vertex(AX, AY, LA, BX, BY, LB, h, sj);
+      const double hx = h.x, hy = h.y;
+      g.s[a * N + i] = sj;
       put(sh_hx, lo_hx, a, hx);
       put(sh_hy, lo_hy, a, hy);
       if (a == 0) {
@@ -238,7 +226,7 @@ __global__ void __launch_bounds__(kSlotThreads, kGeomSlotBlocks) k_geom_slots(Ge
     for (int a = w; a < m; a += kSlotWarps) {
       const longlong2 A = s_off[a][c], B = s_off[a + 1 < m ? a + 1 : 0][c];
       double2 h, sj;
-      geom_vertex(A.x, A.y, B.x, B.y, h, sj);
+      geom_vertex(A.x, A.y, norm2_exact(A.x, A.y), B.x, B.y, norm2_exact(B.x, B.y), h, sj);
       g.s[a * N + i] = sj;
       s_h[a][c] = h;
     }

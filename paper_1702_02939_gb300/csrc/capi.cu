@@ -458,7 +458,7 @@ int sm_count() {
 // 43.0 at 16384, 109.5 -> 106.6 at 131072; FP32 98.5 -> 87.3 at 262144, 263.7
 // -> 259.9 at 10^6).  In double precision the rounds of larger systems hide
 // behind the geometry (191 -> 194 at 262144).
-constexpr int64_t kRestCells = kGeomSlotCells, kRestCellsF32 = 1 << 20;
+constexpr int64_t kRestCells = 155648, kRestCellsF32 = 1 << 20;
 // Per-step repair rounds handle a few hundred flagged cells: a modest
 // persistent grid (warps loop over the list) keeps empty rounds cheap.
 int repair_grid(const cg_ctx* c) { return sm_count() * c->launch.repair_blocks_per_sm; }

@@ -330,23 +330,69 @@ __device__ __forceinline__ double fx_rcp(double d) {
   const unsigned long long t = e + (((unsigned long long)e16 * e16) >> 30);
   return q63_to_double(Y + __umul64hi(Y, t << 2), 1023 - ef, (unsigned long long)b & 0x8000000000000000ull);
 }
-__device__ __forceinline__ double fx_rsqrt(double x) {
-  const long long b = __double_as_longlong(x);
-  const int ef = (int)((b >> 52) & 0x7ff);
-  if (ef == 0 || ef == 0x7ff || b < 0) return fast_rsqrt(x);
-  const int E = ef - 1023, odd = E & 1;
-  // x = m' 2^(E - odd) with m' in [1, 4), held as m' 2^62
-  const unsigned long long M = (((unsigned long long)b & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull) << (10 + odd);
+// 2^63 / sqrt(m') for m' in [1, 4), given as M = m' 2^62.
+__device__ __forceinline__ unsigned long long rsqrt_q63(unsigned long long M) {
+  const int odd = (int)(M >> 63);
   float yf;
   asm("rsqrt.approx.ftz.f32 %0, %1;"
       : "=f"(yf)
-      : "f"(__int_as_float((odd ? 0x40000000 : 0x3f800000) | (int)((b >> 29) & 0x7fffff))));
+      : "f"(__int_as_float((odd ? 0x40000000 : 0x3f800000) | (int)((unsigned)(M >> (39 + odd)) & 0x7fffffu))));
   const unsigned long long Y = seed_q63(yf);
   const unsigned long long e = (unsigned long long)kQOne - __umul64hi(M, __umul64hi(Y, Y) << 2);  // 1 - m' y^2
   const unsigned e16 = (unsigned)(e >> 16);
   const unsigned long long e2 = ((unsigned long long)e16 * e16) >> 30, e3 = (e2 * e16) >> 46;
   const unsigned long long t = (e >> 1) + ((3ull * e2) >> 3) + ((5ull * e3) >> 4);
-  return q63_to_double(Y + __umul64hi(Y, t << 2), -((E - odd) >> 1), 0ull);
+  return Y + __umul64hi(Y, t << 2);
+}
+__device__ __forceinline__ double fx_rsqrt(double x) {
+  const long long b = __double_as_longlong(x);
+  const int ef = (int)((b >> 52) & 0x7ff);
+  if (ef == 0 || ef == 0x7ff || b < 0) return fast_rsqrt(x);
+  const int E = ef - 1023, odd = E & 1;
+  // x = m' 2^(E - odd) with m' in [1, 4)
+  const unsigned long long M = (((unsigned long long)b & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull) << (10 + odd);
+  return q63_to_double(rsqrt_q63(M), -((E - odd) >> 1), 0ull);
+}
+
+// A 64-bit integer rounded to the nearest double (ties to even), times 2^e2.
+__device__ __forceinline__ double i64_to_double(long long v, int e2 = 0) {
+  const long long sgn = v >> 63;
+  const unsigned long long a = (unsigned long long)((v ^ sgn) - sgn);
+  if (!a) return 0.0;
+  const int lz = __clzll((long long)a);
+  const unsigned long long top = a << lz, m = top >> 11;
+  const unsigned long long up = ((unsigned)top & 0x7ffu) + ((unsigned)m & 1u) > 0x400u ? 1ull : 0ull;
+  const unsigned long long bits = ((unsigned long long)(64 - lz + 1021 + e2) << 52) + m + up;
+  return __longlong_as_double((long long)(bits | ((unsigned long long)sgn & 0x8000000000000000ull)));
+}
+
+// ---- polygon of a cell in 64-bit fixed point: vertices as integers below 2^56
+// in a unit common to the cell, 2^(top - 55) with 2^top the leading bit of its
+// largest vertex coordinate ----
+__device__ __forceinline__ int exponent_of(double x) { return (int)((__double_as_longlong(x) >> 52) & 0x7ff); }
+__device__ __forceinline__ long long to_fixed(double x, int top) {
+  const long long b = __double_as_longlong(x);
+  const int d = top - (int)((b >> 52) & 0x7ff);
+  const long long m = (((b & 0xFFFFFFFFFFFFFLL) | 0x10000000000000LL) << 3) >> (d < 63 ? (d > 0 ? d : 0) : 63);
+  return b < 0 ? -m : m;
+}
+// The edge from hp to h: its length (truncated to a unit) and its unit vector in
+// Q1.61 (zero for an edge of length zero).
+__device__ __forceinline__ void edge_fixed(longlong2 h, longlong2 hp, longlong2& u, unsigned long long& len) {
+  const long long ex = h.x - hp.x, ey = h.y - hp.y, sx = ex >> 63, sy = ey >> 63;
+  const unsigned long long ax = (unsigned long long)((ex ^ sx) - sx), ay = (unsigned long long)((ey ^ sy) - sy);
+  const unsigned long long mx = ax > ay ? ax : ay;
+  u = make_longlong2(0, 0);
+  len = 0;
+  if (!mx) return;
+  const int sh = __clzll((long long)mx) - 2;  // the larger component to [2^61, 2^62)
+  const unsigned long long X = ax << sh, Y = ay << sh;
+  const unsigned long long q = __umul64hi(X << 1, X << 1) + __umul64hi(Y << 1, Y << 1);  // length^2 2^-62, < 2^63
+  const int big = (int)(q >> 62);
+  const unsigned long long M = big ? q : q << 2, r = rsqrt_q63(M);
+  const long long ux = (long long)__umul64hi(X << (1 - big), r), uy = (long long)__umul64hi(Y << (1 - big), r);
+  u = make_longlong2((ux ^ sx) - sx, (uy ^ sy) - sy);
+  len = __umul64hi(M, r) >> (sh - big);
 }
 
 // Standard normal for (seed, cell tag, step), cosine branch of Box-Muller,

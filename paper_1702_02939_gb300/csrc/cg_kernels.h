@@ -11,12 +11,12 @@ struct Rep;
 struct Ctl;
 
 constexpr int kGeomThreads = 32;   // one warp: finer blocks than 64 cut k_geom by ~4% at N = 262144
-constexpr int kGeomSh = 10;        // ring slots of k_geom held in shared memory (longer rings: local)
-constexpr int kGeomMinBlocks = 20;  // resident one-warp blocks per SM that k_geom is compiled for
+constexpr int kGeomSh = 8;        // ring slots of k_geom held in shared memory (longer rings: local)
+constexpr int kGeomMinBlocks = 24;  // resident one-warp blocks per SM that k_geom is compiled for
 constexpr int kSlotWarps = 8;       // warps of a block that takes 32 cells, one warp per ring slot
 constexpr int kSlotThreads = 32 * kSlotWarps;
-constexpr int kGeomSlotBlocks = 6;      // resident blocks per SM that k_geom_slots is compiled for
-constexpr int kGeomSlotCells = 155648;  // up to here (1024 cells per SM) k_geom_slots takes all cells
+constexpr int kGeomSlotBlocks = 5;      // resident blocks per SM that k_geom_slots is compiled for
+constexpr int kGeomSlotCells = 97280;  // up to here (640 cells per SM) k_geom_slots takes all cells
 constexpr int kForceSlotBlocks = 6, kTestSlotBlocks = 6, kGeomF32SlotBlocks = 5, kForceF32SlotBlocks = 8;
 // the force and test passes, and the single-precision geometry, take their
 // slot kernels while every cell is resident at once: 152 SMs x 6 blocks x 32

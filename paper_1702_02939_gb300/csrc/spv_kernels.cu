@@ -39,26 +39,51 @@ __device__ __forceinline__ void geom_vertex(long long AX, long long AY, unsigned
   s = make_double2(h.x * r, h.y * r);
 }
 
-// The edge from vertex hp to h: (squared length, inverse length) and its unit
-// vector; a zero-length edge has no direction.
-__device__ __forceinline__ void geom_edge(double2 h, double2 hp, double2& l, double2& e) {
-  const double ex = h.x - hp.x, ey = h.y - hp.y;
-  const double l2 = fma(ex, ex, ey * ey);
-  const double il = (__double_as_longlong(l2) > 0) ? fx_rsqrt(l2) : 0.0;
-  l = make_double2(l2, il);
-  e = make_double2(ex * il, ey * il);
-}
+// Twice the signed area of a polygon whose vertices (components below 2^56) are
+// added in turn, starting from its last one: the 28-bit halves' products add up
+// in 64 bits over at most CG_RING edges.
+struct PolygonArea {
+  long long p2 = 0, p1 = 0, p0 = 0;
+  int qx1, qx0, qy1, qy0;
+  static constexpr int mask = (1 << 28) - 1;
+  __device__ __forceinline__ void start(longlong2 q) {
+    qx1 = (int)(q.x >> 28);
+    qx0 = (int)q.x & mask;
+    qy1 = (int)(q.y >> 28);
+    qy0 = (int)q.y & mask;
+  }
+  __device__ __forceinline__ void add(longlong2 h) {
+    const int x1 = (int)(h.x >> 28), x0 = (int)h.x & mask, y1 = (int)(h.y >> 28), y0 = (int)h.y & mask;
+    p2 += wmul(qx1, y1) - wmul(qy1, x1);
+    p1 += wmul(qx1, y0) + wmul(qx0, y1) - wmul(qy1, x0) - wmul(qy0, x1);
+    p0 += wmul(qx0, y0) - wmul(qy0, x0);
+    qx1 = x1; qx0 = x0; qy1 = y1; qy0 = y0;
+  }
+  __device__ __forceinline__ __int128 total() const { return join3<28>(p2, p1, p0); }
+};
 
-// A, P and the energy of cell i from its accumulated sums; returns (ka, kp).
-__device__ __forceinline__ double2 geom_cell(const GeomArgs& g, int i, double sc, double area, double per) {
-  const double A = 0.125 * area * sc * sc, P = 0.5 * per * sc;
+// A, P and the energy of cell i from its sums over the doubled circumcentres in
+// fixed point (one unit 2^unit grid units); returns (ka, kp) for differences of
+// fixed-point vertices and of Q1.61 unit vectors.
+__device__ __forceinline__ double2 geom_cell_fixed(const GeomArgs& g, int i, double sc, __int128 area,
+                                                   unsigned long long per, int unit) {
+  const double A = 0.125 * i128_to_double(area, 2 * unit) * sc * sc;
+  const double P = 0.5 * i64_to_double((long long)per, unit) * sc;
   g.A[i] = A;
   g.P[i] = P;
   const double dA = A - g.A0, dP = fma(-g.p0[i], g.sqrtA0, P);
   if (g.energy_out) g.energy_out[i] = fma(g.KA * dA, dA, g.KP * dP * dP);
   // dA/dh = 1/2 perp(h_next - h_prev) (the 1/2, the doubling of g and the
   // grid scale fold into ka); dP/dh = e_in - e_out (unit edge vectors)
-  return make_double2(g.KA * dA * (0.5 * sc), 2.0 * g.KP * dP);
+  const double ka = g.KA * dA * (0.5 * sc), kp = 2.0 * g.KP * dP;
+  return make_double2(ka * __longlong_as_double((long long)(1023 + unit) << 52), kp * 0x1p-61);
+}
+// dE/dh at a vertex from its neighbours hp, hn on the polygon and the unit
+// vectors of the edges ending (e) and leaving (en) there.
+__device__ __forceinline__ double2 force_set(double2 k, longlong2 hp, longlong2 hn, longlong2 e, longlong2 en) {
+  const double gx = i64_to_double(hn.y - hp.y), gy = i64_to_double(hp.x - hn.x);
+  const double dPx = i64_to_double(e.x - en.x), dPy = i64_to_double(e.y - en.y);
+  return make_double2(fma(k.x, gx, k.y * dPx), fma(k.x, gy, k.y * dPy));
 }
 
 // One thread per cell.  Writes A, P, force sets fs[a][i] = dE_i/dh_a, and the
@@ -71,13 +96,19 @@ __device__ __forceinline__ double2 geom_cell(const GeomArgs& g, int i, double sc
 // (A x 2^-2q, P x 2^-q, dA/dh x 2^-q).  The circumcentres are kept doubled,
 // g_a = 2 h_a = num / det: every use is homogeneous in h, so the factor 2
 // (exact) folds into the per-cell constants (A x 1/4, P x 1/2, dA/dh x 1/2,
-// s x 2 against w / 2) and the results equal those of h itself bit for bit.
-// Integer-to-double conversions run on the integer pipes (i2d_int).
+// s x 2 against w / 2).
 //
-// Per ring slot the kernel keeps the circumcentre and the unit vector of the
-// edge ending there for the force-set pass: the first kGeomSh slots in shared
-// memory (10 KB per one-warp block, so that 20 blocks fit on an SM), the
-// slots of longer rings (rare) in local memory.
+// The polygon (edges, lengths, unit vectors, area, differences) is formed in
+// 64-bit fixed point in a unit common to the cell, three bits finer than a
+// double holds its largest vertex: FP64 instructions issue at 1/74 of the FP32
+// rate, and 61 per cell remain of 139.  One pass at 262144 cells 94.2 -> 82.9
+// us, at 10^6 315 -> 270; what bounds it now is the latency and issue of the
+// integer sequences at 24 warps per SM.
+//
+// Per ring slot the kernel keeps the circumcentre, then its fixed-point value
+// and the unit vector of the edge ending there, for the force-set pass: the
+// first kGeomSh slots in shared memory (8 KB per one-warp block, so that 24
+// blocks fit on an SM), the slots of longer rings (rare) in local memory.
 __global__ void __launch_bounds__(kGeomThreads, kGeomMinBlocks) k_geom(GeomArgs g) {
   __shared__ double sh_hx[kGeomSh][kGeomThreads];
   __shared__ double sh_hy[kGeomSh][kGeomThreads];
@@ -119,8 +150,7 @@ __global__ void __launch_bounds__(kGeomThreads, kGeomMinBlocks) k_geom(GeomArgs 
     const unsigned __int128 L0 = norm2_exact(D0X, D0Y);
     unsigned __int128 LA = L0;
     long long AX = D0X, AY = D0Y;
-    double hpx = 0.0, hpy = 0.0, h0x = 0.0, h0y = 0.0;
-    double area = 0.0, per = 0.0;
+    int top = 0;
     for (int a = 0; a < m; ++a) {
       long long BX, BY;
       unsigned __int128 LB;
@@ -134,62 +164,74 @@ __global__ void __launch_bounds__(kGeomThreads, kGeomMinBlocks) k_geom(GeomArgs 
       }
       double2 h, sj;
       geom_vertex(AX, AY, LA, BX, BY, LB, h, sj);
-      const double hx = h.x, hy = h.y;
       g.s[a * N + i] = sj;
-      put(sh_hx, lo_hx, a, hx);
-      put(sh_hy, lo_hy, a, hy);
-      if (a == 0) {
-        h0x = hx; h0y = hy;
-      } else {
-        area = fma(-hx, hpy, fma(hpx, hy, area));  // shoelace term, two FMAs
-        const double ex = hx - hpx, ey = hy - hpy;
-        const double l2 = fma(ex, ex, ey * ey);
-        const double il = (__double_as_longlong(l2) > 0) ? fx_rsqrt(l2) : 0.0;  // zero-length edge: no direction
-        per = fma(l2, il, per);
-        put(sh_ex, lo_ex, a, ex * il);
-        put(sh_ey, lo_ey, a, ey * il);
-      }
-      hpx = hx; hpy = hy;
+      put(sh_hx, lo_hx, a, h.x);
+      put(sh_hy, lo_hy, a, h.y);
+      top = max(top, max(exponent_of(h.x), exponent_of(h.y)));
       LA = LB;
       AX = BX; AY = BY;
     }
-    {  // closing edge h_{m-1} -> h_0 is the incoming edge of vertex 0
-      area = fma(-h0x, hpy, fma(hpx, h0y, area));
-      const double ex = h0x - hpx, ey = h0y - hpy;
-      const double l2 = fma(ex, ex, ey * ey);
-      const double il = (__double_as_longlong(l2) > 0) ? fx_rsqrt(l2) : 0.0;  // zero-length edge: no direction
-      per = fma(l2, il, per);
-      sh_ex[0][t] = ex * il;
-      sh_ey[0][t] = ey * il;
+    // the polygon in fixed point, one unit 2^unit grid units: the vertices and
+    // the unit vectors of the edges ending there take the circumcentres' places
+    const int unit = top - 1023 - 55;
+    auto vertex = [&](int a) {
+      return make_longlong2(to_fixed(get(sh_hx, lo_hx, a), top), to_fixed(get(sh_hy, lo_hy, a), top));
+    };
+    auto keep = [&](double (&sh)[kGeomSh][kGeomThreads], double* lo, int a, long long v) {
+      put(sh, lo, a, __longlong_as_double(v));
+    };
+    PolygonArea area;
+    unsigned long long per = 0;
+    longlong2 H = vertex(m - 1);
+    area.start(H);
+    for (int a = 0; a < m; ++a) {
+      const longlong2 hp = H;
+      H = vertex(a);
+      area.add(H);
+      longlong2 e;
+      unsigned long long len;
+      edge_fixed(H, hp, e, len);
+      per += len;
+      keep(sh_hx, lo_hx, a, H.x);
+      keep(sh_hy, lo_hy, a, H.y);
+      keep(sh_ex, lo_ex, a, e.x);
+      keep(sh_ey, lo_ey, a, e.y);
     }
-    const double2 k = geom_cell(g, i, R.inv_scale, area, per);
-    const double ka = k.x, kp = k.y;
+    const double2 k = geom_cell_fixed(g, i, R.inv_scale, area.total(), per, unit);
+    auto fixed = [&](const double (&sh)[kGeomSh][kGeomThreads], const double* lo, int a) {
+      return __double_as_longlong(get(sh, lo, a));
+    };
     for (int a = 0; a < m; ++a) {
       const int ap = (a == 0) ? m - 1 : a - 1;
       const int an = (a + 1 == m) ? 0 : a + 1;
-      const double gx = get(sh_hy, lo_hy, an) - get(sh_hy, lo_hy, ap);
-      const double gy = get(sh_hx, lo_hx, ap) - get(sh_hx, lo_hx, an);
-      const double dPx = get(sh_ex, lo_ex, a) - get(sh_ex, lo_ex, an);
-      const double dPy = get(sh_ey, lo_ey, a) - get(sh_ey, lo_ey, an);
-      g.fs[a * N + i] = make_double2(fma(ka, gx, kp * dPx), fma(ka, gy, kp * dPy));
+      g.fs[a * N + i] = force_set(
+          k, make_longlong2(fixed(sh_hx, lo_hx, ap), fixed(sh_hy, lo_hy, ap)),
+          make_longlong2(fixed(sh_hx, lo_hx, an), fixed(sh_hy, lo_hy, an)),
+          make_longlong2(fixed(sh_ex, lo_ex, a), fixed(sh_ey, lo_ey, a)),
+          make_longlong2(fixed(sh_ex, lo_ex, an), fixed(sh_ey, lo_ey, an)));
     }
   }
 }
 
-// The same pass with one thread per (cell, ring slot): a block takes 32 cells,
-// its warp w the slots w, w + 8 of all of them (lane = cell, so every access
-// is laid out as in k_geom).  The neighbours' offsets, the circumcentres and
-// the edges pass between slots through shared memory; the last warp, whose own
-// slots are rare, adds the area up while the others form the edges, and the
-// first adds up the perimeter and forms the cell's coefficients.  Every
-// operation and its order is k_geom's, so the results are bit-identical.
+// The pass with one thread per (cell, ring slot): a block takes 32 cells, its
+// warp w the slots w, w + 8 of all of them (lane = cell, so every access is
+// coalesced).  The neighbours' offsets, the circumcentres and the edges pass
+// between slots through shared memory; the last warp, whose own slots are rare,
+// adds the area up while the others form the edges, and the first adds up the
+// perimeter and forms the cell's coefficients.
+//
+// The polygon itself (edges, lengths, unit vectors, area, differences) is
+// formed in 64-bit fixed point, with at least three bits more than a double
+// holds: 8 FP64 operations per slot remain of 21.
 __global__ void __launch_bounds__(kSlotThreads, kGeomSlotBlocks) k_geom_slots(GeomArgs g) {
-  __shared__ longlong2 s_off[CG_RING][32];  // neighbour offsets, then (as double2) unit edge vectors
+  __shared__ longlong2 s_off[CG_RING][32];  // neighbour offsets, then unit edge vectors (Q1.61)
   __shared__ double2 s_h[CG_RING][32];      // doubled circumcentres
-  __shared__ double2 s_l[CG_RING][32];      // edge ending at the slot: squared length, inverse length
-  __shared__ double2 s_k[32];               // the cell's ka, kp
-  __shared__ double s_area[32];
-  double2(*s_e)[32] = reinterpret_cast<double2(*)[32]>(s_off);
+  __shared__ longlong2 s_H[CG_RING][32];    // and in fixed point
+  __shared__ unsigned long long s_len[CG_RING][32];  // length of the edge ending at the slot
+  __shared__ double2 s_k[32];               // the cell's ka, kp, in the units of the differences
+  __shared__ longlong2 s_area[32];
+  __shared__ int s_top[32];                 // largest exponent of the cell's circumcentres
+  longlong2(*s_e)[32] = s_off;
   const int c = threadIdx.x & 31, w = threadIdx.x >> 5;
   const size_t N = (size_t)g.n;
   const int cur = g.ctl->cur;
@@ -210,6 +252,7 @@ __global__ void __launch_bounds__(kSlotThreads, kGeomSlotBlocks) k_geom_slots(Ge
       }
       if (m < 3 || m > CG_RING) m = 0;
     }
+    if (w == 0) s_top[c] = 0;
     const Rep& R = g.reps[g.rep[i]];
     const int* ring = g.nbr + (size_t)i * CG_RING;
     if (w < m) {
@@ -223,46 +266,52 @@ __global__ void __launch_bounds__(kSlotThreads, kGeomSlotBlocks) k_geom_slots(Ge
       }
     }
     __syncthreads();
+    int top = 0;
     for (int a = w; a < m; a += kSlotWarps) {
       const longlong2 A = s_off[a][c], B = s_off[a + 1 < m ? a + 1 : 0][c];
       double2 h, sj;
       geom_vertex(A.x, A.y, norm2_exact(A.x, A.y), B.x, B.y, norm2_exact(B.x, B.y), h, sj);
       g.s[a * N + i] = sj;
       s_h[a][c] = h;
+      top = max(top, max(exponent_of(h.x), exponent_of(h.y)));
     }
+    if (top) atomicMax(&s_top[c], top);
     __syncthreads();
+    top = s_top[c];
+    const int unit = top - 1023 - 55;  // one fixed-point unit is 2^unit grid units
     if (w == kSlotWarps - 1) {
-      double area = 0.0;
-      for (int a = 1; a <= m; ++a) {
-        const double2 hp = s_h[a - 1][c], h = s_h[a < m ? a : 0][c];
-        area = fma(-h.x, hp.y, fma(hp.x, h.y, area));
-      }
-      s_area[c] = area;
+      PolygonArea area;
+      auto vertex = [&](int a) {
+        const double2 h = s_h[a][c];
+        return make_longlong2(to_fixed(h.x, top), to_fixed(h.y, top));
+      };
+      if (m) area.start(vertex(m - 1));
+      for (int a = 0; a < m; ++a) area.add(vertex(a));
+      const __int128 t = area.total();
+      s_area[c] = make_longlong2((long long)t, (long long)(t >> 64));
     }
     for (int a = w; a < m; a += kSlotWarps) {
       const double2 h = s_h[a][c], hp = s_h[a > 0 ? a - 1 : m - 1][c];
-      double2 l, e;
-      geom_edge(h, hp, l, e);
-      s_l[a][c] = l;
+      const longlong2 H = make_longlong2(to_fixed(h.x, top), to_fixed(h.y, top));
+      longlong2 e;
+      unsigned long long len;
+      edge_fixed(H, make_longlong2(to_fixed(hp.x, top), to_fixed(hp.y, top)), e, len);
+      s_H[a][c] = H;
       s_e[a][c] = e;
+      s_len[a][c] = len;
     }
     __syncthreads();
     if (w == 0 && m) {
-      double per = 0.0;
-      for (int a = 1; a <= m; ++a) {
-        const double2 l = s_l[a < m ? a : 0][c];
-        per = fma(l.x, l.y, per);
-      }
-      s_k[c] = geom_cell(g, i, R.inv_scale, s_area[c], per);
+      unsigned long long per = 0;
+      for (int a = 0; a < m; ++a) per += s_len[a][c];
+      const longlong2 t = s_area[c];
+      s_k[c] = geom_cell_fixed(g, i, R.inv_scale, ((__int128)t.y << 64) | (unsigned long long)t.x, per, unit);
     }
     __syncthreads();
     const double2 k = s_k[c];
     for (int a = w; a < m; a += kSlotWarps) {
       const int ap = a > 0 ? a - 1 : m - 1, an = a + 1 < m ? a + 1 : 0;
-      const double2 hp = s_h[ap][c], hn = s_h[an][c], e = s_e[a][c], en = s_e[an][c];
-      const double gx = hn.y - hp.y, gy = hp.x - hn.x;
-      const double dPx = e.x - en.x, dPy = e.y - en.y;
-      g.fs[a * N + i] = make_double2(fma(k.x, gx, k.y * dPx), fma(k.x, gy, k.y * dPy));
+      g.fs[a * N + i] = force_set(k, s_H[ap][c], s_H[an][c], s_e[a][c], s_e[an][c]);
     }
     __syncthreads();
   }
@@ -779,11 +828,11 @@ void launch_geom(const GeomArgs& a, cudaStream_t st, int blocks) {
   if (a.n <= 0) return;
   // A block per 32 cells and a warp per ring slot shortens the chain that one
   // thread walks by the number of slots: it is faster while the chip is not
-  // full (one pass, us, one thread per cell -> slots: 22.5 -> 10.2 at 256
-  // cells, 26.6 -> 12.3 at 4096, 26.6 -> 16.8 at 16384, 36.9 -> 34.4 at 65536,
-  // 62.7 -> 57.1 at 131072).  Beyond, both fill the FP64 pipe and the warps of
-  // the last slots idle (102 -> 102 at 262144, 337 -> 379 at 10^6).  A list
-  // (the cells whose rings a step rewrote) is short.
+  // full (one pass, us, one thread per cell -> slots: 20.5 -> 10.2 at 256
+  // cells, 22.5 -> 11.5 at 4096, 22.5 -> 16.4 at 16384, 34.8 -> 32.8 at 65536).
+  // Beyond, the warps of the last slots idle (51 -> 55 at 131072, 83 -> 98 at
+  // 262144, 270 -> 364 at 10^6).  A list (the cells whose rings a step rewrote)
+  // is short.
   if (a.list || a.n <= kGeomSlotCells) {
     const int full = (a.n + 31) / 32;
     k_geom_slots<<<(blocks > 0 && blocks < full) ? blocks : full, kSlotThreads, 0, st>>>(a);

@@ -719,8 +719,10 @@ __device__ __forceinline__ void test_cell(const TestArgs& g, int i, const long l
 }
 
 // Grid-stride over cells (a smaller grid leaves room on every SM for the
-// FP64 branch that runs beside the test).
-__global__ void __launch_bounds__(kTestThreads) k_test(TestArgs g) {
+// FP64 branch that runs beside the test).  Bound by the latency of the
+// neighbours' gathers: 64 registers (108 before, two blocks fewer on an SM)
+// take 82 -> 68 us at 10^6 cells.
+__global__ void __launch_bounds__(kTestThreads, 8) k_test(TestArgs g) {
   const size_t N = (size_t)g.n;
   const int cur = g.ctl->cur;
   const long long* __restrict__ X = g.X + (size_t)cur * N;

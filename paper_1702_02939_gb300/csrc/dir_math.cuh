@@ -69,6 +69,9 @@ __host__ __device__ constexpr long long qdiv(long long d) { return (kQOne + d / 
 __device__ __forceinline__ long long mulq(long long a, long long b) {
   return (long long)(((__int128)a * (__int128)b) >> 62);
 }
+// The same for |a| < 1/2 (in Q1.62 below 2^61): one signed high product, where
+// the low half and the 128-bit shift cost half as much again.
+__device__ __forceinline__ long long mulq_small(long long a, long long b) { return __mul64hi(a << 2, b); }
 // x 2^62 for |x| < 2, truncated toward zero, on the integer pipes
 __device__ __forceinline__ long long d2q(double x) {
   const long long b = __double_as_longlong(x);
@@ -104,11 +107,11 @@ __device__ __forceinline__ double q2d(long long v, int k) {
 // sin(r) and cos(r) - 1 in Q1.62 for r (Q1.62) with |r| <= 0.0125 (Taylor to
 // r^7 and r^6; the first omitted terms are below 2^-70).
 __device__ __forceinline__ void dm_small_q(long long r, long long& s, long long& c_minus_1) {
-  const long long r2 = mulq(r, r);
-  const long long ps = -qdiv(6) + mulq(r2, qdiv(120) - mulq(r2, qdiv(5040)));
-  s = r + mulq(mulq(r2, r), ps);
-  const long long pc = -(kQOne / 2) + mulq(r2, qdiv(24) - mulq(r2, qdiv(720)));
-  c_minus_1 = mulq(r2, pc);
+  const long long r2 = mulq_small(r, r);
+  const long long ps = -qdiv(6) + mulq_small(r2, qdiv(120) - mulq_small(r2, qdiv(5040)));
+  s = r + mulq_small(mulq_small(r2, r), ps);
+  const long long pc = -(kQOne / 2) + mulq_small(r2, qdiv(24) - mulq_small(r2, qdiv(720)));
+  c_minus_1 = mulq_small(r2, pc);
 }
 
 // (sin theta, cos theta).  theta = j pi/128 + r with j = rint(128 theta / pi)
@@ -131,8 +134,8 @@ __device__ __forceinline__ void dm_sincos(double th, const double2* __restrict__
   long long sr, cm;
   dm_small_q(d2q(r), sr, cm);
   const longlong2 t = __ldg(reinterpret_cast<const longlong2*>(tab + kDirTabQ) + j);  // (S, C) in Q1.62
-  s = q2d(t.x + mulq(t.x, cm) + mulq(t.y, sr), -62);
-  c = q2d(t.y + mulq(t.y, cm) - mulq(t.x, sr), -62);
+  s = q2d(t.x + mulq_small(cm, t.x) + mulq_small(sr, t.y), -62);
+  c = q2d(t.y + mulq_small(cm, t.y) - mulq_small(sr, t.x), -62);
 }
 
 // cos(pi t) for t = v 2^-52, v in [1, 2^53] (t in (0, 2]) given as the
@@ -150,7 +153,7 @@ __device__ __forceinline__ double dm_cospi_grid52(unsigned long long v, const do
   long long sr, cm;
   dm_small_q(rq, sr, cm);
   const longlong2 tt = __ldg(reinterpret_cast<const longlong2*>(tab + kDirTabQ) + j);
-  return q2d(tt.y + mulq(tt.y, cm) - mulq(tt.x, sr), -62);
+  return q2d(tt.y + mulq_small(cm, tt.y) - mulq_small(sr, tt.x), -62);
 }
 
 // ln u for a positive normal u: u = 2^k m, m in [M0, 2 M0).  With c_j the
@@ -168,12 +171,12 @@ __device__ __forceinline__ double dm_log(double u, const double2* __restrict__ t
   const double r = fma(m, t.x, -1.0);
   const long long rq = d2q(r);
   long long p = qdiv(7);
-  p = -qdiv(6) + mulq(rq, p);
-  p = qdiv(5) + mulq(rq, p);
-  p = -(kQOne / 4) + mulq(rq, p);
-  p = qdiv(3) + mulq(rq, p);
-  p = -(kQOne / 2) + mulq(rq, p);
-  p = kQOne + mulq(rq, p);
+  p = -qdiv(6) + mulq_small(rq, p);
+  p = qdiv(5) + mulq_small(rq, p);
+  p = -(kQOne / 4) + mulq_small(rq, p);
+  p = qdiv(3) + mulq_small(rq, p);
+  p = -(kQOne / 2) + mulq_small(rq, p);
+  p = kQOne + mulq_small(rq, p);
   const double l1p = r * q2d(p, -62);
   return fma(dm_i2d(k), 0x1.62e42fefa39efp-1, t.y + l1p);  // + k ln 2
 }

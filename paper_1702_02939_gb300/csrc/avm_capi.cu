@@ -144,6 +144,8 @@ struct cg_avm_ctx {
   cudaStream_t side = nullptr;                     // the director branch of the step graph
   cudaEvent_t fork = nullptr, join = nullptr;
   cudaGraphExec_t exec = nullptr;     // one step
+  cudaGraphExec_t steps_exec = nullptr;  // kGraphSteps steps (built once a run is long)
+  int64_t host_step = 0;                 // steps enqueued
   cudaGraphExec_t t1_exec = nullptr;  // T1 passes alone
   cudaGraphExec_t div_exec = nullptr;  // the division rounds of cg_avm_divide
   int sms = 0;
@@ -387,25 +389,42 @@ int pass_graph(cg_avm_ctx* c, Body body, cudaGraphExec_t* out) {
   return CG_OK;
 }
 
-int avm_graphs(cg_avm_ctx* c) {
-  // the step: geometry, vertex forces and move; then the first T1 pass beside
-  // the director terms of the next step (FP64 work on a branch of its own), and
-  // the further passes
-  int rc = pass_graph(
+// The step: geometry, vertex forces and move; then the first T1 pass beside the
+// director terms of the next step (FP64 work on a branch of its own), and the
+// further passes.
+void enqueue_step(cg_avm_ctx* c, const AvmArgs& a, cudaStream_t st) {
+  launch_avm_move(a, st);
+  AvmArgs ahead = a;
+  ahead.flip = 1;
+  cudaEventRecord(c->fork, st);
+  cudaStreamWaitEvent(c->side, c->fork, 0);
+  launch_avm_dir(ahead, c->side);
+  cudaEventRecord(c->join, c->side);
+  launch_avm_t1_pass(ahead, st);
+  cudaStreamWaitEvent(st, c->join, 0);
+  launch_avm_t1_rest(a, 1, st);
+}
+
+// Several steps per graph launch once a run is long: a launch costs the device
+// about 3.5 us between steps of 20-50 us (as many_steps of the Voronoi model).
+constexpr int kGraphSteps = 8;
+constexpr int64_t kLongRun = 64;
+constexpr int kManyStepCells = 1 << 17;
+bool many_steps(cg_avm_ctx* c) {
+  if (c->steps_exec) return true;
+  if (c->host_step < kLongRun || c->n > kManyStepCells) return false;
+  const int rc = pass_graph(
       c,
       [c](const AvmArgs& a, cudaStream_t st) {
-        launch_avm_move(a, st);
-        AvmArgs ahead = a;
-        ahead.flip = 1;
-        cudaEventRecord(c->fork, st);
-        cudaStreamWaitEvent(c->side, c->fork, 0);
-        launch_avm_dir(ahead, c->side);
-        cudaEventRecord(c->join, c->side);
-        launch_avm_t1_pass(ahead, st);
-        cudaStreamWaitEvent(st, c->join, 0);
-        launch_avm_t1_rest(a, 1, st);
+        for (int k = 0; k < kGraphSteps; ++k) enqueue_step(c, a, st);
       },
-      &c->exec);
+      &c->steps_exec);
+  if (rc) c->last_error.clear();  // single steps do
+  return rc == CG_OK;
+}
+
+int avm_graphs(cg_avm_ctx* c) {
+  int rc = pass_graph(c, [c](const AvmArgs& a, cudaStream_t st) { enqueue_step(c, a, st); }, &c->exec);
   if (rc) return rc;
   rc = pass_graph(
       c,
@@ -597,9 +616,16 @@ int cg_avm_create(int32_t n, double Lx, double Ly, double p0, double v0, const c
 int cg_avm_step(cg_avm_ctx* c, int64_t nsteps) {
   if (!c || nsteps < 0) return CG_EINVAL;
   if (c->broken) return afail(c, CG_EINVAL, "context holds a device error: " + c->last_error);
-  for (int64_t s = 0; s < nsteps; ++s) {
-    AV_CUDA(c, cudaGraphLaunch(c->exec, c->stream));
-    if (c->par.sort_every > 0 && ++c->since_sort >= c->par.sort_every) {
+  for (int64_t s = 0; s < nsteps;) {
+    // steps to go before the end of the call or the next re-sort
+    int64_t left = nsteps - s;
+    if (c->par.sort_every > 0) left = std::min<int64_t>(left, c->par.sort_every - c->since_sort);
+    const int k = left >= kGraphSteps && many_steps(c) ? kGraphSteps : 1;
+    AV_CUDA(c, cudaGraphLaunch(k > 1 ? c->steps_exec : c->exec, c->stream));
+    s += k;
+    c->host_step += k;
+    c->since_sort += k;
+    if (c->par.sort_every > 0 && c->since_sort >= c->par.sort_every) {
       const int rc = enqueue_sort(c, 0);
       if (rc) return rc;
     }
@@ -919,6 +945,7 @@ int cg_avm_get_tags(cg_avm_ctx* c, int32_t* vtag, int32_t* ctag) {
 int cg_avm_destroy(cg_avm_ctx* c) {
   if (!c) return CG_EINVAL;
   if (c->exec) cudaGraphExecDestroy(c->exec);
+  if (c->steps_exec) cudaGraphExecDestroy(c->steps_exec);
   if (c->t1_exec) cudaGraphExecDestroy(c->t1_exec);
   if (c->div_exec) cudaGraphExecDestroy(c->div_exec);
   if (c->capture) cudaStreamDestroy(c->capture);

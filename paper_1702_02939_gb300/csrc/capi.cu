@@ -194,6 +194,7 @@ struct cg_ctx {
   cg_launch launch{4, 4, 4, 1, 0, 8, 1, 5, 0};    // launch shapes of the step graph
   std::vector<cg_replica> user_reps;           // as passed to cg_create
   cudaGraphExec_t step_exec = nullptr;
+  cudaGraphExec_t steps_exec = nullptr;  // kGraphSteps steps (built once a run is long)
   int graph_steps = 0;
   int seen_status = 0;  // a device status read back earlier (the context then stays refused)
   std::string last_error;
@@ -661,6 +662,18 @@ int refuse_seen(cg_ctx* c) {
   return fail(c, c->seen_status, std::string("device status: ") + cg_status_string(c->seen_status));
 }
 
+// The step without a loop node.
+void enqueue_plain_step(cg_ctx* c, cudaStream_t st) {
+  enqueue_step_prefix(c, st);
+  enqueue_repair_round(c, 0, st);
+  launch_repair_rest(round_repair_args(c, 0), round_check_args(c, 0), st);
+  enqueue_step_suffix(c, st);
+}
+bool plain_step(const cg_ctx* c) { return c->N <= (fp32(c) ? kRestCellsF32 : kRestCells); }
+unsigned long long graph_flags(const cg_ctx* c) {
+  return c->launch.dir_low_priority ? (unsigned long long)cudaGraphInstantiateFlagUseNodePriority : 0ull;
+}
+
 // One step as a graph.  Up to kRestCells cells: the prefix, the first repair
 // round, one kernel for the further rounds (usually none), the suffix.  Larger
 // systems, whose later rounds can be long and hide behind the geometry: the
@@ -668,24 +681,15 @@ int refuse_seen(cg_ctx* c) {
 // cell flagged.
 int build_graph(cg_ctx* c) {
   if (c->step_exec) return CG_OK;
-  const unsigned long long flags =
-      c->launch.dir_low_priority ? (unsigned long long)cudaGraphInstantiateFlagUseNodePriority : 0ull;
   cudaError_t e;
-  if (c->N <= (fp32(c) ? kRestCellsF32 : kRestCells)) {
-    e = build_plain_graph(
-        c->capture,
-        [&](cudaStream_t st) {
-          enqueue_step_prefix(c, st);
-          enqueue_repair_round(c, 0, st);
-          launch_repair_rest(round_repair_args(c, 0), round_check_args(c, 0), st);
-          enqueue_step_suffix(c, st);
-        },
-        &c->step_exec, flags);
+  if (plain_step(c)) {
+    e = build_plain_graph(c->capture, [&](cudaStream_t st) { enqueue_plain_step(c, st); }, &c->step_exec,
+                          graph_flags(c));
   } else {
     e = build_loop_graph(
         c->capture, [&](cudaGraphConditionalHandle, cudaStream_t st) { enqueue_step_prefix(c, st); },
         [&](cudaGraphConditionalHandle h, cudaStream_t st) { enqueue_repair_round(c, h, st); },
-        [&](cudaStream_t st) { enqueue_step_suffix(c, st); }, &c->step_exec, flags);
+        [&](cudaStream_t st) { enqueue_step_suffix(c, st); }, &c->step_exec, graph_flags(c));
   }
   if (e != cudaSuccess) {
     cudaGetLastError();
@@ -693,6 +697,35 @@ int build_graph(cg_ctx* c) {
     return fail(c, CG_ECUDA, std::string("step graph: ") + cudaGetErrorString(e));
   }
   return CG_OK;
+}
+
+// A graph launch costs the device about 3.5 us between steps, which a small
+// system's step of 20-45 us feels: once a context has taken kLongRun steps, the
+// steps of a call go kGraphSteps at a time (the graph is built then, beside the
+// steps in flight; contexts of a few steps never pay for it).
+constexpr int kGraphSteps = 8;
+constexpr int64_t kLongRun = 64, kManyStepCells = 1 << 16;
+bool many_steps(cg_ctx* c) {
+  if (c->steps_exec) return true;
+  if (c->host_step < kLongRun || c->N > kManyStepCells || !plain_step(c)) return false;
+  if (build_plain_graph(
+          c->capture,
+          [&](cudaStream_t st) {
+            for (int k = 0; k < kGraphSteps; ++k) enqueue_plain_step(c, st);
+          },
+          &c->steps_exec, graph_flags(c)) != cudaSuccess) {
+    cudaGetLastError();
+    c->steps_exec = nullptr;  // single steps do
+    return false;
+  }
+  return true;
+}
+void drop_graphs(cg_ctx* c) {
+  for (cudaGraphExec_t* g : {&c->step_exec, &c->steps_exec})
+    if (*g) {
+      cudaGraphExecDestroy(*g);
+      *g = nullptr;
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -932,13 +965,19 @@ int cg_create(int32_t R, const cg_replica* reps, const cg_params* params, const 
 
 int cg_step(cg_ctx* c, int64_t nsteps) {
   if (!c || nsteps < 0) return CG_EINVAL;
-  for (int64_t s = 0; s < nsteps; ++s) {
-    if (c->par.sort_every > 0 && c->host_step > 0 && c->host_step % c->par.sort_every == 0) {
+  const int64_t every = c->par.sort_every;
+  for (int64_t s = 0; s < nsteps;) {
+    if (every > 0 && c->host_step > 0 && c->host_step % every == 0) {
       launch_sort(sort_args(c), c->stream);
       prime(c);
     }
-    CG_CUDA(c, cudaGraphLaunch(c->step_exec, c->stream));
-    ++c->host_step;
+    // steps to go before the end of the call or the next re-sort
+    int64_t left = nsteps - s;
+    if (every > 0) left = std::min<int64_t>(left, every - c->host_step % every);
+    const bool many = left >= kGraphSteps && many_steps(c);
+    CG_CUDA(c, cudaGraphLaunch(many ? c->steps_exec : c->step_exec, c->stream));
+    s += many ? kGraphSteps : 1;
+    c->host_step += many ? kGraphSteps : 1;
   }
   return CG_OK;
 }
@@ -1261,10 +1300,7 @@ int cg_set_moduli(cg_ctx* c, double KA, double KP) {
   if (KA == c->par.KA && KP == c->par.KP) return CG_OK;  // nothing depends on anything new
   c->par.KA = KA;
   c->par.KP = KP;
-  if (c->step_exec) {  // kernel parameters are baked into the graph: capture again
-    cudaGraphExecDestroy(c->step_exec);
-    c->step_exec = nullptr;
-  }
+  drop_graphs(c);  // kernel parameters are baked into the graphs: capture again
   rc = build_graph(c);
   if (rc) return rc;
   prime(c, kPrimeGeom | kPrimeMove);  // the force sets and the pending move depend on the moduli
@@ -1289,10 +1325,7 @@ int cg_set_launch(cg_ctx* c, const cg_launch* l) {
   int rc = read_status(c);
   if (rc) return rc;
   c->launch = *l;
-  if (c->step_exec) {
-    cudaGraphExecDestroy(c->step_exec);
-    c->step_exec = nullptr;
-  }
+  drop_graphs(c);
   return build_graph(c);
 }
 
@@ -1669,7 +1702,7 @@ int64_t cg_num_cells(const cg_ctx* c) { return c ? c->N : -1; }
 
 int cg_destroy(cg_ctx* c) {
   if (!c) return CG_EINVAL;
-  if (c->step_exec) cudaGraphExecDestroy(c->step_exec);
+  drop_graphs(c);
   if (c->capture) cudaStreamDestroy(c->capture);
   for (cudaStream_t sd : c->side)
     if (sd) cudaStreamDestroy(sd);

@@ -64,3 +64,25 @@ def test_vertex_model_transfers(sort_every):
         for a, b in zip(got["device"], got[where]):
             assert np.array_equal(a, b)
     sim.close()
+
+
+@pytest.mark.parametrize("sort_every", [0, 20])
+def test_many_steps_per_launch_equal_single_steps(sort_every):
+    """Past the first 64 steps a call's steps go several per graph launch; the
+    result is that of one call per step, through re-sorts and changed moduli."""
+    n = 150
+    x, y, th, L = workloads.spv_uniform(n, 6)
+    for make in (lambda: cg.SPV([dict(n=n, Lx=L, Ly=L, p0=3.8, v0=0.2)], x, y, th, seed=3, sort_every=sort_every),
+                 lambda: cg.AVM(n, L, L, x, y, th, v0=0.2, seed=3, sort_every=sort_every)):
+        got = []
+        for single in (False, True):
+            sim = make()
+            for steps in (70, 19, 7, 33):
+                for _ in range(steps if single else 1):
+                    sim.step(1 if single else steps)
+                if isinstance(sim, cg.SPV) and steps == 19:
+                    sim.set_moduli(1.5, 0.5)
+            got.append([t.cpu().numpy() for t in sim.state()])
+            sim.close()
+        for a, b in zip(*got):
+            assert np.array_equal(a, b)

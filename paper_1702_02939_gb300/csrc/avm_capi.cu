@@ -210,6 +210,12 @@ AvmArgs avm_args(cg_avm_ctx* c) {
   a.Ly = c->Ly;
   a.ax = axis(c->Lx);
   a.ay = axis(c->Ly);
+  int ex;
+  const double fr = std::frexp(std::fmax(c->Lx, c->Ly), &ex);
+  if (fr == 0.5) --ex;  // the smallest power of two >= the sides (positions are below them)
+  a.top = ex - 1 + 1023;
+  a.LXI = (long long)std::ldexp(c->Lx, 62 - ex);
+  a.LYI = (long long)std::ldexp(c->Ly, 62 - ex);
   a.Lxf = (float)c->Lx;
   a.Lyf = (float)c->Ly;
   a.hx = c->at<double>(c->off.hx);

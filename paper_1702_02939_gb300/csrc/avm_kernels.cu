@@ -51,6 +51,14 @@ __device__ __forceinline__ double wrap_d(double v, double L) {
   return r >= L ? 0.0 : r;
 }
 
+// A position in [0, 2^(top - 1022)) in units of 2^-62 of that power of two.
+__device__ __forceinline__ long long position_fixed(double h, int top) {
+  const long long b = __double_as_longlong(h);
+  const int d = top - (int)((b >> 52) & 0x7ff);
+  const long long m = (((b & 0xFFFFFFFFFFFFFLL) | 0x10000000000000LL) << 9) >> (d < 63 ? (d > 0 ? d : 0) : 63);
+  return b < 0 ? -m : m;
+}
+
 // Reduction into [0, L) with the common case (already inside; +0 included)
 // decided on the integer pipe.
 __device__ __forceinline__ double wrap_a(double v, const Axis& a) {
@@ -191,59 +199,22 @@ __device__ __forceinline__ void avm_cell(const AvmArgs& g, int c, bool empty, do
 // ka = 2 K_A (A - A0) and kp = 2 K_P (P - P0); when stepping, the director
 // takes its rotated value thn (k_avm_dir computed it, with the activity act
 // of the current director, before the step).
-__global__ void k_avm_cells(AvmArgs g) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= g.n) return;
-  const size_t V = (size_t)g.V;
-  const int cur = g.ctl->cur;
-  const double* hx = g.hx + cur * V;
-  const double* hy = g.hy + cur * V;
-  const int m = g.cc[c];
-  if (g.move) g.theta[c] = g.thn[c];
-  if (m == 0) {
-    avm_cell(g, c, true, 0.0, 0.0);
-    return;
-  }
-  if (m < 3 || m > CG_RING) {
-    raise_status(g.ctl, kETOPO);
-    return;
-  }
-  const int* row = g.cv + (size_t)c * CG_RING;
-  for (int a = 0; a < m; ++a)
-    if ((unsigned)row[a] >= (unsigned)g.V) {
-      raise_status(g.ctl, kETOPO);
-      return;
-    }
-  const int v0 = row[0];
-  const double x0 = hx[v0], y0 = hy[v0];
-  double px = 0.0, py = 0.0, area = 0.0, per = 0.0;
-  for (int a = 1; a <= m; ++a) {
-    double qx = 0.0, qy = 0.0;
-    if (a < m) {
-      const int v = row[a];
-      qx = mimg_a(hx[v] - x0, g.ax);
-      qy = mimg_a(hy[v] - y0, g.ay);
-    }
-    area = fma(-qx, py, fma(px, qy, area));
-    const double ex = qx - px, ey = qy - py;
-    const double l2 = fma(ex, ex, ey * ey);
-    per = (__double_as_longlong(l2) > 0) ? fma(l2, fx_rsqrt(l2), per) : per;  // sqrt(l2)
-    px = qx;
-    py = qy;
-  }
-  avm_cell(g, c, false, area, per);
-}
-
-// The same with one thread per (cell, polygon edge): a block takes 32 cells,
-// its warp w the vertices w, w + 8 of all of them (lane = cell); the vertices'
-// offsets and the edges pass through shared memory, the last warp adds the area
-// up beside the edges and the first one the perimeter.  Bit-identical to
-// k_avm_cells, whose lanes walk the polygon one edge after another.
-__global__ void __launch_bounds__(kSlotThreads, kAvmSlotBlocks) k_avm_cells_slots(AvmArgs g) {
-  __shared__ double2 s_q[CG_RING][32];  // vertices relative to the first one
-  __shared__ double2 s_l[CG_RING][32];  // edge leaving the vertex: squared length, inverse length
-  __shared__ double s_area[32];
-  __shared__ int s_bad[32];
+//
+// One thread per (cell, polygon edge): a block takes 32 cells, its warp w the
+// vertices w, w + 8 of all of them (lane = cell); the vertices pass through
+// shared memory, the last warp adds the area up beside the edges and the first
+// one the perimeter.  (One thread per cell walks the polygon edge by edge: pass,
+// us, 14.2 -> 9.4 at 4096 cells, 12.6 -> 10.3 at 16384, 18.3 -> 17.4 at 65536.)
+//
+// All of it in 64-bit fixed point: positions in units of 2^-62 of the box's
+// power of two (nine bits finer than a double holds a position), differences
+// scaled so that the cell's largest one has 56 bits; ten FP64 operations per
+// cell remain of about 60.
+__global__ void __launch_bounds__(kSlotThreads, kAvmSlotBlocks) k_avm_cells(AvmArgs g) {
+  __shared__ longlong2 s_q[CG_RING][32];            // vertices relative to the first one
+  __shared__ unsigned long long s_len[CG_RING][32];  // edge leaving the vertex
+  __shared__ longlong2 s_area[32];
+  __shared__ int s_bits[32], s_bad[32];
   const int t = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int c = blockIdx.x * 32 + t;
   const size_t V = (size_t)g.V;
@@ -257,34 +228,48 @@ __global__ void __launch_bounds__(kSlotThreads, kAvmSlotBlocks) k_avm_cells_slot
     bad = true;
     m = 0;
   }
-  if (w == 0) s_bad[t] = bad;
+  if (w == 0) {
+    s_bad[t] = bad;
+    s_bits[t] = 0;
+  }
   const int* row = g.cv + (size_t)c * CG_RING;
+  int bits = 0;
   if (w < m) {
     const int v0 = row[0];
     const bool ok0 = (unsigned)v0 < (unsigned)g.V;
-    const double x0 = ok0 ? hx[v0] : 0.0, y0 = ok0 ? hy[v0] : 0.0;
+    const long long x0 = position_fixed(ok0 ? hx[v0] : 0.0, g.top), y0 = position_fixed(ok0 ? hy[v0] : 0.0, g.top);
     for (int a = w; a < m; a += kSlotWarps) {
       const int v = row[a];
       const bool ok = ok0 && (unsigned)v < (unsigned)g.V;
       bad |= !ok;
-      s_q[a][t] = (ok && a) ? make_double2(mimg_a(hx[v] - x0, g.ax), mimg_a(hy[v] - y0, g.ay)) : make_double2(0.0, 0.0);
+      longlong2 q = make_longlong2(0, 0);
+      if (ok && a) {
+        q = make_longlong2(min_image_i(position_fixed(hx[v], g.top) - x0, g.LXI),
+                           min_image_i(position_fixed(hy[v], g.top) - y0, g.LYI));
+        bits = max(bits, 64 - __clzll((q.x ^ (q.x >> 63)) | (q.y ^ (q.y >> 63))));
+      }
+      s_q[a][t] = q;
     }
   }
   __syncthreads();
   if (bad) s_bad[t] = 1;
-  if (w == kSlotWarps - 1) {
-    double area = 0.0;
-    for (int a = 1; a <= m; ++a) {
-      const double2 p = s_q[a - 1][t], q = s_q[a < m ? a : 0][t];
-      area = fma(-q.x, p.y, fma(p.x, q.y, area));
-    }
-    s_area[t] = area;
+  if (bits) atomicMax(&s_bits[t], bits);
+  __syncthreads();
+  const int sh = s_bits[t] - 56, unit = g.top - 1022 - 62 + sh;  // one unit is 2^unit of length
+  auto vertex = [&](int a) {
+    const longlong2 q = s_q[a][t];
+    return sh > 0 ? make_longlong2(q.x >> sh, q.y >> sh) : make_longlong2(q.x * (1LL << -sh), q.y * (1LL << -sh));
+  };
+  if (w == kSlotWarps - 1 && m) {
+    PolygonArea area;
+    area.start(vertex(m - 1));
+    for (int a = 0; a < m; ++a) area.add(vertex(a));
+    const __int128 sum = area.total();
+    s_area[t] = make_longlong2((long long)sum, (long long)(sum >> 64));
   }
   for (int a = w; a < m; a += kSlotWarps) {
-    const double2 p = s_q[a][t], q = s_q[a + 1 < m ? a + 1 : 0][t];
-    const double ex = q.x - p.x, ey = q.y - p.y;
-    const double l2 = fma(ex, ex, ey * ey);
-    s_l[a][t] = make_double2(l2, (__double_as_longlong(l2) > 0) ? fx_rsqrt(l2) : 0.0);
+    EdgeFixed e;
+    s_len[a][t] = e.set(vertex(a + 1 < m ? a + 1 : 0), vertex(a)) ? e.length() : 0ull;
   }
   __syncthreads();
   if (w || c >= g.n) return;
@@ -293,12 +278,11 @@ __global__ void __launch_bounds__(kSlotThreads, kAvmSlotBlocks) k_avm_cells_slot
     raise_status(g.ctl, kETOPO);
     return;
   }
-  double per = 0.0;
-  for (int a = 0; a < m; ++a) {
-    const double2 l = s_l[a][t];
-    per = (__double_as_longlong(l.x) > 0) ? fma(l.x, l.y, per) : per;
-  }
-  avm_cell(g, c, empty, s_area[t], per);
+  unsigned long long per = 0;
+  for (int a = 0; a < m; ++a) per += s_len[a][t];
+  const longlong2 sum = s_area[t];
+  const __int128 area = m ? ((__int128)sum.y << 64) | (unsigned long long)sum.x : (__int128)0;
+  avm_cell(g, c, empty, i128_to_double(area, 2 * unit), i64_to_double((long long)per, unit));
 }
 
 // Per vertex: F_v = -sum_k [ka_k 1/2 perp(u_{k-1} - u_k) - kp_k (u^_k + u^_{k-1})]
@@ -1504,12 +1488,8 @@ constexpr int kAvmCellThreads = 64, kAvmVertexThreads = 32;
 static inline int cell_blocks_of(int n) { return (n + kAvmCellThreads - 1) / kAvmCellThreads; }
 static inline int vertex_blocks_of(int n) { return (n + kAvmVertexThreads - 1) / kAvmVertexThreads; }
 
-// The cell pass takes a thread per polygon edge while every cell is resident at
-// once (pass, us: 14.2 -> 10.1 at 4096 cells, 14.2 -> 12.2 at 16384, 14.5 ->
-// 16.2 at 32768, 18.4 -> 21.3 at 65536).
 static void launch_cells(const AvmArgs& a, cudaStream_t st) {
-  if (a.n <= kAvmSlotCells) k_avm_cells_slots<<<(a.n + 31) / 32, kSlotThreads, 0, st>>>(a);
-  else k_avm_cells<<<cell_blocks_of(a.n), kAvmCellThreads, 0, st>>>(a);
+  k_avm_cells<<<(a.n + 31) / 32, kSlotThreads, 0, st>>>(a);
 }
 void launch_avm_move(const AvmArgs& a, cudaStream_t st, int part) {
   AvmArgs m = a;

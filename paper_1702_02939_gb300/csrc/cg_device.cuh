@@ -378,22 +378,61 @@ __device__ __forceinline__ long long to_fixed(double x, int top) {
 }
 // The edge from hp to h: its length (truncated to a unit) and its unit vector in
 // Q1.61 (zero for an edge of length zero).
+struct EdgeFixed {
+  unsigned long long X, Y, M, r;  // |components| shifted up, squared length, its inverse root
+  long long sx, sy;
+  int sh, big;
+  __device__ __forceinline__ bool set(longlong2 h, longlong2 hp) {  // false: length zero
+    const long long ex = h.x - hp.x, ey = h.y - hp.y;
+    sx = ex >> 63;
+    sy = ey >> 63;
+    const unsigned long long ax = (unsigned long long)((ex ^ sx) - sx), ay = (unsigned long long)((ey ^ sy) - sy);
+    const unsigned long long mx = ax > ay ? ax : ay;
+    if (!mx) return false;
+    sh = __clzll((long long)mx) - 2;  // the larger component to [2^61, 2^62)
+    X = ax << sh;
+    Y = ay << sh;
+    const unsigned long long q = __umul64hi(X << 1, X << 1) + __umul64hi(Y << 1, Y << 1);  // length^2 2^-62, < 2^63
+    big = (int)(q >> 62);
+    M = big ? q : q << 2;
+    r = rsqrt_q63(M);
+    return true;
+  }
+  __device__ __forceinline__ unsigned long long length() const { return __umul64hi(M, r) >> (sh - big); }
+  __device__ __forceinline__ longlong2 unit() const {
+    const long long ux = (long long)__umul64hi(X << (1 - big), r), uy = (long long)__umul64hi(Y << (1 - big), r);
+    return make_longlong2((ux ^ sx) - sx, (uy ^ sy) - sy);
+  }
+};
 __device__ __forceinline__ void edge_fixed(longlong2 h, longlong2 hp, longlong2& u, unsigned long long& len) {
-  const long long ex = h.x - hp.x, ey = h.y - hp.y, sx = ex >> 63, sy = ey >> 63;
-  const unsigned long long ax = (unsigned long long)((ex ^ sx) - sx), ay = (unsigned long long)((ey ^ sy) - sy);
-  const unsigned long long mx = ax > ay ? ax : ay;
-  u = make_longlong2(0, 0);
-  len = 0;
-  if (!mx) return;
-  const int sh = __clzll((long long)mx) - 2;  // the larger component to [2^61, 2^62)
-  const unsigned long long X = ax << sh, Y = ay << sh;
-  const unsigned long long q = __umul64hi(X << 1, X << 1) + __umul64hi(Y << 1, Y << 1);  // length^2 2^-62, < 2^63
-  const int big = (int)(q >> 62);
-  const unsigned long long M = big ? q : q << 2, r = rsqrt_q63(M);
-  const long long ux = (long long)__umul64hi(X << (1 - big), r), uy = (long long)__umul64hi(Y << (1 - big), r);
-  u = make_longlong2((ux ^ sx) - sx, (uy ^ sy) - sy);
-  len = __umul64hi(M, r) >> (sh - big);
+  EdgeFixed e;
+  const bool any = e.set(h, hp);
+  u = any ? e.unit() : make_longlong2(0, 0);
+  len = any ? e.length() : 0ull;
 }
+
+// Twice the signed area of a polygon whose vertices (components below 2^56) are
+// added in turn, starting from its last one: the 28-bit halves' products add up
+// in 64 bits over at most CG_RING edges.
+struct PolygonArea {
+  long long p2 = 0, p1 = 0, p0 = 0;
+  int qx1, qx0, qy1, qy0;
+  static constexpr int mask = (1 << 28) - 1;
+  __device__ __forceinline__ void start(longlong2 q) {
+    qx1 = (int)(q.x >> 28);
+    qx0 = (int)q.x & mask;
+    qy1 = (int)(q.y >> 28);
+    qy0 = (int)q.y & mask;
+  }
+  __device__ __forceinline__ void add(longlong2 h) {
+    const int x1 = (int)(h.x >> 28), x0 = (int)h.x & mask, y1 = (int)(h.y >> 28), y0 = (int)h.y & mask;
+    p2 += wmul(qx1, y1) - wmul(qy1, x1);
+    p1 += wmul(qx1, y0) + wmul(qx0, y1) - wmul(qy1, x0) - wmul(qy0, x1);
+    p0 += wmul(qx0, y0) - wmul(qy0, x0);
+    qx1 = x1; qx0 = x0; qy1 = y1; qy0 = y0;
+  }
+  __device__ __forceinline__ __int128 total() const { return join3<28>(p2, p1, p0); }
+};
 
 // Standard normal for (seed, cell tag, step), cosine branch of Box-Muller,
 // with the table-driven ln and cos(pi .) of dir_math.cuh (tab: the 512-entry

@@ -372,6 +372,8 @@ struct AvmArgs {
   Ctl* ctl;
   double Lx, Ly;
   Axis ax, ay;
+  int top;                  // exponent field of the doubles just below the power of two that holds the box
+  long long LXI, LYI;       // the box in units of 2^-62 of that power
   float Lxf, Lyf;           // lengths for the FP32 T1 filter
   double *hx, *hy;         // [2][V]
   int *vc, *vn, *cc, *cv;
@@ -422,7 +424,7 @@ void launch_avm_begin_t1(Ctl* ctl, int flip, cudaStream_t st);
 void launch_avm_t1_pass(const AvmArgs& a, cudaStream_t st);
 // After a first pass: the further passes while any is due (ctl->pad); advance:
 // that pass looked one step ahead, whose state becomes current first
-constexpr int kAvmSlotBlocks = 6, kAvmSlotCells = 29184;
+constexpr int kAvmSlotBlocks = 6;
 constexpr int kT1RestBlocks = 8, kT1RestThreads = 512;
 void launch_avm_t1_rest(const AvmArgs& a, int advance, cudaStream_t st);
 void launch_avm_forces(const AvmArgs& a, cudaStream_t st);

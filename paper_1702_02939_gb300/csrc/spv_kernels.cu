@@ -39,29 +39,6 @@ __device__ __forceinline__ void geom_vertex(long long AX, long long AY, unsigned
   s = make_double2(h.x * r, h.y * r);
 }
 
-// Twice the signed area of a polygon whose vertices (components below 2^56) are
-// added in turn, starting from its last one: the 28-bit halves' products add up
-// in 64 bits over at most CG_RING edges.
-struct PolygonArea {
-  long long p2 = 0, p1 = 0, p0 = 0;
-  int qx1, qx0, qy1, qy0;
-  static constexpr int mask = (1 << 28) - 1;
-  __device__ __forceinline__ void start(longlong2 q) {
-    qx1 = (int)(q.x >> 28);
-    qx0 = (int)q.x & mask;
-    qy1 = (int)(q.y >> 28);
-    qy0 = (int)q.y & mask;
-  }
-  __device__ __forceinline__ void add(longlong2 h) {
-    const int x1 = (int)(h.x >> 28), x0 = (int)h.x & mask, y1 = (int)(h.y >> 28), y0 = (int)h.y & mask;
-    p2 += wmul(qx1, y1) - wmul(qy1, x1);
-    p1 += wmul(qx1, y0) + wmul(qx0, y1) - wmul(qy1, x0) - wmul(qy0, x1);
-    p0 += wmul(qx0, y0) - wmul(qy0, x0);
-    qx1 = x1; qx0 = x0; qy1 = y1; qy0 = y0;
-  }
-  __device__ __forceinline__ __int128 total() const { return join3<28>(p2, p1, p0); }
-};
-
 // A, P and the energy of cell i from its sums over the doubled circumcentres in
 // fixed point (one unit 2^unit grid units); returns (ka, kp) for differences of
 // fixed-point vertices and of Q1.61 unit vectors.

@@ -42,8 +42,8 @@ def test_small_system_alone_and_inside_a_large_batch(n, precision):
 
 @pytest.mark.parametrize("n", [64, 1000])
 def test_vertex_model_small_and_with_room_for_many_cells(n):
-    # the same network in a context small enough for the slot kernel and in one
-    # with a capacity beyond it (empty cells and free vertices past the network)
+    # the same network in a context of its size and in one with room for many more
+    # cells (empty cells and free vertices past the network)
     x, y, th, L = workloads.spv_uniform(n, 13)
     sims = [cg.AVM(n, L, L, x, y, th, v0=0.3, seed=3, t2_area=0.01, capacity=cap) for cap in (n, 40000)]
     for sim in sims:

@@ -733,7 +733,9 @@ void drop_graphs(cg_ctx* c) {
 // ---------------------------------------------------------------------------
 struct BwdLayout {
   size_t snap_bytes = 0;                 // one state snapshot
-  size_t snaps = 0, seg = 0;             // checkpoints (+ final state), segment states
+  // checkpoints (+ final state), the input states of the last segment's steps
+  // (kept by the run) and of the segment being recomputed
+  size_t snaps = 0, last = 0, seg = 0;
   size_t v, fsd, sd, wd, gp0, gv0, gKA, gKP, cA, cP, gx, gy, F, red;
   size_t total = 0;
 };
@@ -750,6 +752,7 @@ BwdLayout bwd_layout(int64_t N, int64_t nsteps, int32_t every) {
   b.snap_bytes = s.total;
   const int64_t nck = (nsteps + every - 1) / every;
   b.snaps = L.take((size_t)(nck + 1) * b.snap_bytes);
+  b.last = L.take((size_t)std::min<int64_t>(every, nsteps) * b.snap_bytes);
   b.seg = L.take((size_t)every * b.snap_bytes);
   b.v = L.take(N * sizeof(double2));
   b.fsd = L.take(N * CG_RING * sizeof(double2));
@@ -1560,6 +1563,10 @@ int cg_run_checkpointed(cg_ctx* c, int64_t nsteps, int32_t ckpt_every, void* d_b
   const int64_t nck = (nsteps + ckpt_every - 1) / ckpt_every;
   for (int64_t t = 0; t < nsteps; ++t) {
     if (t % ckpt_every == 0) snapshot(c, 1, snapshot_at(bw + b.snaps + (t / ckpt_every) * b.snap_bytes, c->N));
+    // the last segment is the first the reverse pass needs: its steps' states
+    // are kept now, so that it is not run again
+    const int64_t in_last = t - (nck - 1) * ckpt_every;
+    if (in_last >= 0) snapshot(c, 1, snapshot_at(bw + b.last + in_last * b.snap_bytes, c->N));
     CG_CUDA(c, cudaGraphLaunch(c->step_exec, c->stream));
   }
   snapshot(c, 1, snapshot_at(bw + b.snaps + nck * b.snap_bytes, c->N));
@@ -1582,7 +1589,6 @@ int cg_backward(cg_ctx* c, int64_t nsteps, int32_t ckpt_every, void* d_bw, size_
   const int* tag = c->at<int>(c->off.tag);
   const int64_t nck = (nsteps + ckpt_every - 1) / ckpt_every;
   const Snapshot fin = snapshot_at(bw + b.snaps + nck * b.snap_bytes, c->N);
-  snapshot(c, 0, fin, 0);  // the tangent kernels compute their own geometry
   // cotangents of the final state, in storage order
   double* tmp = c->at<double>(c->off.tmp);
   const double* srcs[4] = {gxT, gyT, gAT, gPT};
@@ -1594,8 +1600,19 @@ int cg_backward(cg_ctx* c, int64_t nsteps, int32_t ckpt_every, void* d_bw, size_
   }
   JvpArgs a = jvp_args(c, bw, b);
   CG_CUDA(c, cudaMemsetAsync(a.v, 0, c->N * sizeof(double2), st));
+  // the tangent kernels compute their own geometry, from the saved states in
+  // place
+  auto use = [](JvpArgs& j, const Snapshot& s) {
+    j.X = s.X;
+    j.Y = s.Y;
+    j.flat = 1;
+    j.cnt = s.cnt;
+    j.nbr = s.nbr;
+    j.theta = s.theta;
+  };
   {
     JvpArgs f = a;
+    use(f, fin);
     f.coefA = dsts[2];
     f.coefP = dsts[3];
     f.F = reinterpret_cast<double2*>(bw + b.F);
@@ -1611,21 +1628,16 @@ int cg_backward(cg_ctx* c, int64_t nsteps, int32_t ckpt_every, void* d_bw, size_
   a.update = 1;
   for (int64_t ck = nck - 1; ck >= 0; --ck) {
     const int64_t t0 = ck * ckpt_every, t1 = std::min<int64_t>(t0 + ckpt_every, nsteps);
-    snapshot(c, 0, snapshot_at(bw + b.snaps + ck * b.snap_bytes, c->N));
-    for (int64_t t = t0; t < t1; ++t) {  // recompute the segment, keeping every step's input state
-      snapshot(c, 1, snapshot_at(bw + b.seg + (t - t0) * b.snap_bytes, c->N));
-      if (t + 1 < t1) CG_CUDA(c, cudaGraphLaunch(c->step_exec, st));
+    const size_t states = ck == nck - 1 ? b.last : b.seg;
+    if (ck < nck - 1) {
+      snapshot(c, 0, snapshot_at(bw + b.snaps + ck * b.snap_bytes, c->N));
+      for (int64_t t = t0; t < t1; ++t) {  // recompute the segment, keeping every step's input state
+        snapshot(c, 1, snapshot_at(bw + b.seg + (t - t0) * b.snap_bytes, c->N));
+        if (t + 1 < t1) CG_CUDA(c, cudaGraphLaunch(c->step_exec, st));
+      }
     }
-    // the tangent kernels compute their own geometry, from the saved states
-    // in place
     for (int64_t t = t1 - 1; t >= t0; --t) {
-      const Snapshot s = snapshot_at(bw + b.seg + (t - t0) * b.snap_bytes, c->N);
-      a.X = s.X;
-      a.Y = s.Y;
-      a.flat = 1;
-      a.cnt = s.cnt;
-      a.nbr = s.nbr;
-      a.theta = s.theta;
+      use(a, snapshot_at(bw + states + (t - t0) * b.snap_bytes, c->N));
       launch_geom_jvp(a, st);
       launch_force_jvp(a, st);
     }

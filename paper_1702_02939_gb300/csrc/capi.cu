@@ -662,11 +662,15 @@ int refuse_seen(cg_ctx* c) {
   return fail(c, c->seen_status, std::string("device status: ") + cg_status_string(c->seen_status));
 }
 
-// The step without a loop node.
+// The step without a loop node.  The 128 warps of the further rounds' cluster do
+// the first round of a small system too (a few to some hundred cells), two
+// kernels fewer.
+constexpr int64_t kClusterCells = 4096;
 void enqueue_plain_step(cg_ctx* c, cudaStream_t st) {
   enqueue_step_prefix(c, st);
-  enqueue_repair_round(c, 0, st);
-  launch_repair_rest(round_repair_args(c, 0), round_check_args(c, 0), st);
+  const bool cluster_only = c->N <= kClusterCells;
+  if (!cluster_only) enqueue_repair_round(c, 0, st);
+  launch_repair_rest(round_repair_args(c, 0), round_check_args(c, 0), cluster_only, st);
   enqueue_step_suffix(c, st);
 }
 bool plain_step(const cg_ctx* c) { return c->N <= (fp32(c) ? kRestCellsF32 : kRestCells); }

@@ -233,8 +233,9 @@ void launch_cell_list(const CellListArgs& a, cudaStream_t st);
 void launch_repair(const RepairArgs& a, int grid_blocks, cudaStream_t st);
 void launch_scan(const ScanArgs& a, cudaStream_t st);
 void launch_check(const CheckArgs& a, int grid_blocks, cudaStream_t st);
-// After a first round (dyn): the further rounds, until none is needed
-void launch_repair_rest(const RepairArgs& a, const CheckArgs& c, cudaStream_t st);
+// After a first round (dyn): the further rounds, until none is needed;
+// every_round: the first one too
+void launch_repair_rest(const RepairArgs& a, const CheckArgs& c, int every_round, cudaStream_t st);
 // Blocks of 8 warps for the check of every cell: a warp per cell up to 16
 // blocks per SM (one block per 256 cells left each warp a chain of 32 cells:
 // 44 us at 1024 cells against 3.5)

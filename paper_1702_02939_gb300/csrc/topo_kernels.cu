@@ -811,7 +811,8 @@ __global__ void k_check(CheckArgs g) {
 // whether it runs or not (a chain of 6 empty kernels 6 us, with a while node
 // 14-16); this kernel adds 2 us.
 __global__ void __cluster_dims__(kRestBlocks, 1, 1) __launch_bounds__(kRestWarps * 32) k_repair_rest(RepairArgs g,
-                                                                                                CheckArgs k) {
+                                                                                                CheckArgs k,
+                                                                                                int every_round) {
   __shared__ CandBuf s_buf[kRestWarps];
   Ctl* ctl = g.ctl;
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
@@ -823,9 +824,14 @@ __global__ void __cluster_dims__(kRestBlocks, 1, 1) __launch_bounds__(kRestWarps
   const long long* __restrict__ Y = g.Y + cur * N;
   // every thread of the cluster follows the same counts: the list of a round is
   // complete before the barrier that ends the one before it
-  for (int r = *(volatile int*)&ctl->round_count; r < k.cap; ++r) {
+  for (int r = every_round ? 0 : *(volatile int*)&ctl->round_count; r < k.cap; ++r) {
     const int in = r & 1;
     const int total = *(volatile int*)&ctl->count[in];
+    if (every_round && r == 0 && first) {  // the first round's statistics (k_check's otherwise)
+      ctl->last_flagged = total;
+      ctl->flagged_total += total;
+      if (total == 0) ctl->loop_total += 1;
+    }
     if (total == 0) break;
     const int* list_in = g.lists[in];
     int* list_out = k.lists[in ^ 1];
@@ -847,8 +853,8 @@ __global__ void __cluster_dims__(kRestBlocks, 1, 1) __launch_bounds__(kRestWarps
   }
 }
 
-void launch_repair_rest(const RepairArgs& a, const CheckArgs& c, cudaStream_t st) {
-  if (a.n > 0) k_repair_rest<<<kRestBlocks, kRestWarps * 32, 0, st>>>(a, c);
+void launch_repair_rest(const RepairArgs& a, const CheckArgs& c, int every_round, cudaStream_t st) {
+  if (a.n > 0) k_repair_rest<<<kRestBlocks, kRestWarps * 32, 0, st>>>(a, c, every_round);
 }
 
 void launch_check(const CheckArgs& a, int grid_blocks, cudaStream_t st) {

@@ -623,6 +623,24 @@ __device__ __forceinline__ int orient0_sign(float fax, float fay, float fbx, flo
   return orient_exact(ax, ay, bx, by);
 }
 
+// Whether s lies outside the circle through 0, q, r (counter-clockwise), and
+// whether b lies left of a seen from 0, by the float values alone (real units,
+// relative to the first point): false also where they leave it open.
+// Determinants and bounds are those of incircle0_sign and orient0_sign.
+__device__ __forceinline__ bool outside_for_sure(float2 q, float2 r, float2 s) {
+  const float la = q.x * q.x + q.y * q.y, lb = r.x * r.x + r.y * r.y, lc = s.x * s.x + s.y * s.y;
+  const float t1 = r.x * s.y, t2 = r.y * s.x, t3 = s.x * q.y, t4 = s.y * q.x, t5 = q.x * r.y, t6 = q.y * r.x;
+  const float det = la * (t1 - t2) + lb * (t3 - t4) + lc * (t5 - t6);
+  const float perm = la * (fabsf(t1) + fabsf(t2)) + lb * (fabsf(t3) + fabsf(t4)) + lc * (fabsf(t5) + fabsf(t6));
+  const float bound = 2.0e-6f * perm;
+  return bound > 1.0e-30f && bound < 1.0e30f && det > bound;
+}
+__device__ __forceinline__ bool left_for_sure(float2 a, float2 b) {
+  const float l = a.x * b.y, r = a.y * b.x;
+  const float bound = 1.0e-6f * (fabsf(l) + fabsf(r));
+  return bound > 1.0e-30f && l - r > bound;
+}
+
 // ----------------------------------------------------------------------------
 // Shared by the FP64 and FP32 step kernels.
 // ----------------------------------------------------------------------------

@@ -23,6 +23,7 @@ constexpr int kForceSlotBlocks = 6, kTestSlotBlocks = 6, kGeomF32SlotBlocks = 5,
 constexpr int kForceSlotCells = 29184, kTestSlotCells = 29184, kGeomF32SlotCells = 29184;
 constexpr int kForceThreads = 128;
 constexpr int kTestThreads = 128;
+constexpr int kTestAhead = 4;     // neighbours that k_test loads together (a multiple of 4)
 constexpr int kRepairWarps = 4;  // warps per repair block
 constexpr int kRestBlocks = 8, kRestWarps = 16;  // the cluster of the rounds after the first
 constexpr int kCand = 64;        // candidate buffer per repair warp

@@ -654,52 +654,85 @@ __device__ __forceinline__ void test_slot(const TestArgs& g, int i, int jp, int 
   }
 }
 
+// The same from the grid, out of line: the one-thread pass comes here where
+// slot_open leaves a slot open.
+static __device__ __noinline__ void test_slot_exact(const TestArgs* args, const long long* __restrict__ X,
+                                                    const long long* __restrict__ Y, int i, int jp, int ja, int jn) {
+  const TestArgs& g = *args;
+  const Rep& R = g.reps[g.rep[i]];
+  const float sc = (float)R.inv_scale;
+  const long long Xi = X[i], Yi = Y[i], LX = R.LX, LY = R.LY;
+  const long long pX = min_image_i(X[jp] - Xi, LX), pY = min_image_i(Y[jp] - Yi, LY);
+  const long long aX = min_image_i(X[ja] - Xi, LX), aY = min_image_i(Y[ja] - Yi, LY);
+  const long long nX = min_image_i(X[jn] - Xi, LX), nY = min_image_i(Y[jn] - Yi, LY);
+  test_slot(g, i, jp, ja, jn, i2f_scaled(pX, sc), i2f_scaled(pY, sc), i2f_scaled(aX, sc), i2f_scaled(aY, sc),
+            i2f_scaled(nX, sc), i2f_scaled(nY, sc), pX, pY, aX, aY, nX, nY, sc);
+}
+
+// Whether the float offsets (real units) of j_{a-1}, j_a and j_{a+1} leave open
+// that the slot is sound.
+__device__ __forceinline__ bool slot_open(int i, int ja, int jn, float2 fp, float2 fa, float2 fn) {
+  return i < ja && !(outside_for_sure(fp, fa, fn) && (i >= jn || left_for_sure(fa, fn)));
+}
+
 // One thread per cell: every slot of its ring.
 __device__ __forceinline__ void test_cell(const TestArgs& g, int i, const long long* __restrict__ X,
                                           const long long* __restrict__ Y) {
-  const Rep R = g.reps[g.rep[i]];
+  const Rep& R = g.reps[g.rep[i]];
   const float sc = (float)R.inv_scale;
-  const long long Xi = X[i], Yi = Y[i];
+  const long long Xi = X[i], Yi = Y[i], LX = R.LX, LY = R.LY;
   const int m = g.cnt[i];
   if (m < 3 || m > CG_RING) {
     raise_status(g.ctl, kETOPO);
     return;
   }
   const int* ring = g.nbr + (size_t)i * CG_RING;
-  // sliding window over (j_{a-1}, j_a, j_{a+1}): grid offsets (exact) and
-  // their float values, each converted once
-  int jp = ring[m - 1], ja = ring[0];
-  long long pX = min_image_i(X[jp] - Xi, R.LX), pY = min_image_i(Y[jp] - Yi, R.LY);
-  long long aX = min_image_i(X[ja] - Xi, R.LX), aY = min_image_i(Y[ja] - Yi, R.LY);
-  float fpx = i2f_scaled(pX, sc), fpy = i2f_scaled(pY, sc);
-  float fax = i2f_scaled(aX, sc), fay = i2f_scaled(aY, sc);
-  const long long fX = aX, fY = aY;
-  const float ffx = fax, ffy = fay;
-  const int jfirst = ja;
-  for (int a = 0; a < m; ++a) {
-    int jn;
-    long long nX, nY;
-    float fnx, fny;
-    if (a + 1 < m) {
-      jn = ring[a + 1];
-      nX = min_image_i(X[jn] - Xi, R.LX);
-      nY = min_image_i(Y[jn] - Yi, R.LY);
-      fnx = i2f_scaled(nX, sc);
-      fny = i2f_scaled(nY, sc);
-    } else {
-      jn = jfirst; nX = fX; nY = fY; fnx = ffx; fny = ffy;
+  auto offset = [&](int j) {
+    return make_float2(i2f_scaled(min_image_i(X[j] - Xi, LX), sc), i2f_scaled(min_image_i(Y[j] - Yi, LY), sc));
+  };
+  // sliding window over (j_{a-1}, j_a, j_{a+1}); the neighbours come kTestAhead
+  // at a time, so that their gathers are in flight together
+  int ja = 0, jfirst = 0;
+  unsigned open = 0;  // the slots to decide in full
+  float2 fp = offset(ring[m - 1]), fa = make_float2(0.0f, 0.0f), ffirst = fa;
+  for (int a0 = 0; a0 < m; a0 += kTestAhead) {
+    int jn[kTestAhead];
+    float2 fn[kTestAhead];
+#pragma unroll
+    for (int q = 0; q < kTestAhead; q += 4) {
+      const int4 r = *reinterpret_cast<const int4*>(ring + a0 + q);
+      jn[q] = r.x; jn[q + 1] = r.y; jn[q + 2] = r.z; jn[q + 3] = r.w;
     }
-    test_slot(g, i, jp, ja, jn, fpx, fpy, fax, fay, fnx, fny, pX, pY, aX, aY, nX, nY, sc);
-    jp = ja; pX = aX; pY = aY; fpx = fax; fpy = fay;
-    ja = jn; aX = nX; aY = nY; fax = fnx; fay = fny;
+#pragma unroll
+    for (int q = 0; q < kTestAhead; ++q) fn[q] = offset(a0 + q < m ? jn[q] : i);
+#pragma unroll
+    for (int q = 0; q < kTestAhead; ++q) {
+      if (a0 + q >= m) break;
+      if (a0 + q == 0) {
+        jfirst = jn[0];
+        ffirst = fn[0];
+      } else {
+        if (slot_open(i, ja, jn[q], fp, fa, fn[q])) open |= 1u << (a0 + q - 1);
+        fp = fa;
+      }
+      ja = jn[q];
+      fa = fn[q];
+    }
+  }
+  if (slot_open(i, ja, jfirst, fp, fa, ffirst)) open |= 1u << (m - 1);
+  for (; open; open &= open - 1) {
+    const int a = __ffs((int)open) - 1;
+    test_slot_exact(&g, X, Y, i, ring[a > 0 ? a - 1 : m - 1], ring[a], ring[a + 1 < m ? a + 1 : 0]);
   }
 }
 
 // Grid-stride over cells (a smaller grid leaves room on every SM for the
 // FP64 branch that runs beside the test).  Bound by the latency of the
-// neighbours' gathers: 64 registers (108 before, two blocks fewer on an SM)
-// take 82 -> 68 us at 10^6 cells.
-__global__ void __launch_bounds__(kTestThreads, 8) k_test(TestArgs g) {
+// neighbours' gathers: four neighbours in flight and 64 registers (one at a
+// time and 108 registers before) take 82 -> 54 us at 10^6 cells.  The grid
+// coordinates are read again for the few slots that the float values leave
+// open; carried along for all of them they cost the registers.
+__global__ void __launch_bounds__(kTestThreads, 8) k_test(const __grid_constant__ TestArgs g) {
   const size_t N = (size_t)g.n;
   const int cur = g.ctl->cur;
   const long long* __restrict__ X = g.X + (size_t)cur * N;

@@ -66,3 +66,21 @@ def test_vertex_model_small_and_with_room_for_many_cells(n):
     assert c[0]["t1_total"] == c[1]["t1_total"] > 0 and c[0]["t2_total"] == c[1]["t2_total"]
     for sim in sims:
         sim.close()
+
+
+def test_cocircular_cells_alone_and_inside_a_large_batch():
+    # a square lattice: every quadruple is cocircular, so float values leave every slot open
+    n, s = 400, 20
+    k = np.arange(n)
+    small = dict(n=n, Lx=float(s), Ly=float(s), p0=3.85, v0=1e-4), k % s + 0.5, k // s + 0.5, np.linspace(0.0, 6.0, n)
+    big = _rep(LARGE, 12)
+    alone = cg.SPV([small[0]], *small[1:], dt=0.002, seed=5)
+    batch = cg.SPV([small[0], big[0]], *(np.concatenate([small[k], big[k]]) for k in (1, 2, 3)), dt=0.002, seed=5)
+    for _ in range(4):
+        alone.step(1)
+        batch.step(1)
+        for a, b in zip(alone.state() + alone.neighbors(), batch.state() + batch.neighbors()):
+            assert np.array_equal(a.cpu().numpy(), b.cpu().numpy()[:n])
+    assert alone.counters()["flagged_total"] > 0
+    alone.close()
+    batch.close()

@@ -79,8 +79,9 @@ __device__ __forceinline__ double2 force_set(double2 k, longlong2 hp, longlong2 
 // 64-bit fixed point in a unit common to the cell, three bits finer than a
 // double holds its largest vertex: FP64 instructions issue at 1/74 of the FP32
 // rate, and 61 per cell remain of 139.  One pass at 262144 cells 94.2 -> 82.9
-// us, at 10^6 315 -> 270; what bounds it now is the latency and issue of the
-// integer sequences at 24 warps per SM.
+// us, at 10^6 315 -> 270; what bounds it now is the issue of the integer
+// sequences (62% of the slots) at 24 warps per SM.  The next neighbour's
+// position is loaded ahead: 270 -> 266.
 //
 // Per ring slot the kernel keeps the circumcentre, then its fixed-point value
 // and the unit vector of the edge ending there, for the force-set pass: the
@@ -128,13 +129,19 @@ __global__ void __launch_bounds__(kGeomThreads, kGeomMinBlocks) k_geom(GeomArgs 
     unsigned __int128 LA = L0;
     long long AX = D0X, AY = D0Y;
     int top = 0;
+    int jq = nb(1);  // the neighbour whose position is loaded ahead
+    long long qX = X[jq], qY = Y[jq];
     for (int a = 0; a < m; ++a) {
       long long BX, BY;
       unsigned __int128 LB;
       if (a + 1 < m) {
-        const int j = nb(a + 1);
-        BX = min_image_i(X[j] - Xi, R.LX);
-        BY = min_image_i(Y[j] - Yi, R.LY);
+        BX = min_image_i(qX - Xi, R.LX);
+        BY = min_image_i(qY - Yi, R.LY);
+        if (a + 2 < m) {
+          jq = nb(a + 2);
+          qX = X[jq];
+          qY = Y[jq];
+        }
         LB = norm2_exact(BX, BY);
       } else {
         BX = D0X; BY = D0Y; LB = L0;

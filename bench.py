@@ -59,7 +59,7 @@ AVM_FLOPS = {"cells_per_cell": 84.0, "vertices_per_vertex": 62.0}
 # DRAM traffic per launch (dram__bytes_read.sum + dram__bytes_write.sum) of
 # the AVM kernels at N = 65536 from one ncu capture of the current kernels
 # (caches flushed before the kernel); None whenever a kernel has changed.
-AVM_DRAM_BYTES_PER_LAUNCH = {"k_avm_cells": 8.14e6, "k_avm_force_move": 7.37e6}
+AVM_DRAM_BYTES_PER_LAUNCH = {"k_avm_cells": 8.15e6, "k_avm_force_move": 7.37e6}
 # AVM storage order: Hilbert re-sort of the vertex and cell slots at creation
 # and every this many steps (Sec. 2.B; results are the same either way).
 AVM_SORT_EVERY = 100
@@ -70,7 +70,7 @@ FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
 # Dominant-kernel DRAM traffic per launch (dram__bytes_read.sum +
 # dram__bytes_write.sum) from one ncu capture of the current k_geom at
 # N = 262144; None whenever the kernel has changed since the capture.
-GEOM_DRAM_BYTES_PER_LAUNCH = 43.99e6
+GEOM_DRAM_BYTES_PER_LAUNCH = 44.49e6
 
 
 def parse():

@@ -136,7 +136,7 @@ typedef struct cg_launch {
 int cg_workspace_bytes(int32_t R, const cg_replica* reps, size_t* bytes);
 
 /* Creates a context and triangulates every replica from scratch: each cell's
- * Voronoi polygon is built by clipping with cell-list candidates, which is the
+ * Delaunay ring is built from the candidates of a cell list, which is the
  * GPU counterpart of the paper's CPU repair (Sec. 2.C.4) applied to all cells.
  *   x, y, theta : any, n_total doubles each, replica-concatenated user order;
  *                 positions must lie in [-L, 2L) and are wrapped into [0, L).

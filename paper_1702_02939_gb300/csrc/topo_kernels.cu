@@ -1,5 +1,5 @@
-// Topology maintenance: cell list, local repair by Voronoi-cell clipping and
-// the ring-consistency check.
+// Topology maintenance: cell list, local repair by gift wrapping (or Voronoi-cell
+// clipping) and the ring-consistency check.
 //
 // The paper repairs flagged cells on the CPU: a candidate "Delaunay 1-ring"
 // from the locality lemma of Chen et al., reduced to the true neighbours with

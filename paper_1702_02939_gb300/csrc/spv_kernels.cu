@@ -849,8 +849,8 @@ void launch_geom(const GeomArgs& a, cudaStream_t st, int blocks) {
   // thread walks by the number of slots: it is faster while the chip is not
   // full (one pass, us, one thread per cell -> slots: 20.5 -> 10.2 at 256
   // cells, 22.5 -> 11.5 at 4096, 22.5 -> 16.4 at 16384, 34.8 -> 32.8 at 65536).
-  // Beyond, the warps of the last slots idle (51 -> 55 at 131072, 83 -> 98 at
-  // 262144, 270 -> 364 at 10^6).  A list (the cells whose rings a step rewrote)
+  // Beyond, the warps of the last slots idle (50 -> 55 at 131072, 82 -> 98 at
+  // 262144, 266 -> 364 at 10^6).  A list (the cells whose rings a step rewrote)
   // is short.
   if (a.list || a.n <= kGeomSlotCells) {
     const int full = (a.n + 31) / 32;
@@ -880,8 +880,8 @@ void launch_force_fix_list(const ForceFixArgs& a, int blocks, cudaStream_t st) {
 void launch_begin_topology(Ctl* ctl, int flip, cudaStream_t st) { k_begin_topology<<<1, 1, 0, st>>>(ctl, flip); }
 void launch_test(const TestArgs& a, cudaStream_t st, int blocks) {
   if (a.n <= 0) return;
-  // As for the force: 13.6 -> 11.4 us at 1024 cells (cell list included),
-  // 16.9 -> 14.0 at 16384, 18.5 -> 19.4 at 65536.
+  // As for the force: 17.0 -> 13.6 us at 16384 cells, 15.7 -> 14.4 at 24576
+  // (cell list included in the slots' times only), 17.2 -> 19.4 at 65536.
   if (a.n <= kTestSlotCells) {
     const int full = (a.n + 31) / 32;
     k_test_slots<<<(blocks > 0 && blocks < full) ? blocks : full, kSlotThreads, 0, st>>>(a);

@@ -538,7 +538,7 @@ __global__ void k_dir_f32(DirArgs g) {
 
 void launch_geom_f32(const GeomArgs& a, cudaStream_t st, int blocks) {
   if (a.n <= 0) return;
-  // up to one resident wave (us: 10.2 -> 8.1 at 256 to 16384 cells; 14.1 -> 14.8
+  // up to one resident wave (us: 10.2 -> 8.1 at 256 to 16384 cells; 13.4 -> 14.8
   // at 65536), and for a list
   if (a.list || a.n <= kGeomF32SlotCells) {
     const int full = (a.n + 31) / 32;

@@ -443,8 +443,9 @@ int cg_avm_sync(cg_avm_ctx* ctx);
 int cg_avm_get_state(cg_avm_ctx* ctx, double* hx, double* hy, double* theta);
 /* Network (layout above); any pointer may be NULL.  Synchronizes. */
 int cg_avm_get_topology(cg_avm_ctx* ctx, int32_t* vc, int32_t* vn, int32_t* cc, int32_t* cv);
-/* Replaces positions (required) and, where not NULL, directors and network
- * arrays, which must describe a valid network of the same N (cell slots).
+/* Replaces positions (required; any finite values, reduced into [0, L)) and,
+ * where not NULL, directors and network arrays, which must describe a valid
+ * network of the same N (cell slots).
  * Synchronizes. */
 int cg_avm_set_state(cg_avm_ctx* ctx, const double* hx, const double* hy, const double* theta, const int32_t* vc,
                      const int32_t* vn, const int32_t* cc, const int32_t* cv);

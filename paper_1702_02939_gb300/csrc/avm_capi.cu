@@ -767,6 +767,7 @@ int cg_avm_set_state(cg_avm_ctx* c, const double* hx, const double* hy, const do
   if ((rc = copy_in(c, c->at<int>(c->off.cc), cc, c->n * sizeof(int)))) return rc;
   if ((rc = copy_in(c, c->at<int>(c->off.cv), cv, c->n * CG_RING * sizeof(int)))) return rc;
   launch_avm_validate(avm_args(c), c->stream);
+  launch_avm_wrap(avm_args(c), c->stream);
   launch_avm_shadow(avm_args(c), c->stream);
   launch_avm_dir(avm_args(c), c->stream);  // director terms of the next step
   return avm_status(c);

@@ -469,6 +469,7 @@ void launch_avm_divide_slots(const DivArgs& d, const int* cslot, const int* vslo
                              int* fv, int* sv, int* svp, cudaStream_t st);
 void launch_avm_divide_begin(const DivArgs& d, cudaStream_t st);
 void launch_avm_divide_round(const DivArgs& d, cudaStream_t st);
+void launch_avm_wrap(const AvmArgs& a, cudaStream_t st);
 void launch_avm_shadow(const AvmArgs& a, cudaStream_t st);
 // Storage order of the AVM (Hilbert re-sort of the vertex and cell slots).
 // Every slot carries a tag, its id in the network as built (and as the API

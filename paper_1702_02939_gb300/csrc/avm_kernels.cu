@@ -264,7 +264,7 @@ __global__ void __launch_bounds__(kSlotThreads, kAvmSlotBlocks) k_avm_cells(AvmA
     return sh > 0 ? make_longlong2(q.x >> sh, q.y >> sh) : make_longlong2(q.x * (1LL << -sh), q.y * (1LL << -sh));
   };
   if (w == kSlotWarps - 1 && m) {
-    PolygonArea area;
+    PolygonArea<> area;
     area.start(vertex(m - 1));
     for (int a = 0; a < m; ++a) area.add(vertex(a));
     const __int128 sum = area.total();

@@ -366,18 +366,25 @@ __device__ __forceinline__ double i64_to_double(long long v, int e2 = 0) {
   return __longlong_as_double((long long)(bits | ((unsigned long long)sgn & 0x8000000000000000ull)));
 }
 
-// ---- polygon of a cell in 64-bit fixed point: vertices as integers below 2^56
-// in a unit common to the cell, 2^(top - 55) with 2^top the leading bit of its
-// largest vertex coordinate ----
+// ---- polygon of a cell in 64-bit fixed point: vertices as integers below 2^61
+// in a unit common to the cell, 2^(top - 60) with 2^top the leading bit of its
+// largest vertex coordinate; area and perimeter in units of 2^(top - 55) ----
+constexpr int kFineBits = 5;
 __device__ __forceinline__ int exponent_of(double x) { return (int)((__double_as_longlong(x) >> 52) & 0x7ff); }
 __device__ __forceinline__ long long to_fixed(double x, int top) {
   const long long b = __double_as_longlong(x);
   const int d = top - (int)((b >> 52) & 0x7ff);
-  const long long m = (((b & 0xFFFFFFFFFFFFFLL) | 0x10000000000000LL) << 3) >> (d < 63 ? (d > 0 ? d : 0) : 63);
+  const long long m =
+      (((b & 0xFFFFFFFFFFFFFLL) | 0x10000000000000LL) << (3 + kFineBits)) >> (d < 63 ? (d > 0 ? d : 0) : 63);
   return b < 0 ? -m : m;
 }
-// The edge from hp to h: its length (truncated to a unit) and its unit vector in
-// Q1.61 (zero for an edge of length zero).
+__device__ __forceinline__ longlong2 to_fixed(double2 h, int top) {
+  return make_longlong2(to_fixed(h.x, top), to_fixed(h.y, top));
+}
+__device__ __forceinline__ int exponent_of(double2 h) { return max(exponent_of(h.x), exponent_of(h.y)); }
+// The edge from hp to h (components below 2^62 apart): its length (truncated to
+// 2^coarser units) and its unit vector in Q1.61 (zero for an edge of length
+// zero).  sh - big + coarser is in [0, 63]: an edge below 2^61, or coarser > 0.
 struct EdgeFixed {
   unsigned long long X, Y, M, r;  // |components| shifted up, squared length, its inverse root
   long long sx, sy;
@@ -398,7 +405,9 @@ struct EdgeFixed {
     r = rsqrt_q63(M);
     return true;
   }
-  __device__ __forceinline__ unsigned long long length() const { return __umul64hi(M, r) >> (sh - big); }
+  __device__ __forceinline__ unsigned long long length(int coarser = 0) const {
+    return __umul64hi(M, r) >> (sh - big + coarser);
+  }
   __device__ __forceinline__ longlong2 unit() const {
     const long long ux = (long long)__umul64hi(X << (1 - big), r), uy = (long long)__umul64hi(Y << (1 - big), r);
     return make_longlong2((ux ^ sx) - sx, (uy ^ sy) - sy);
@@ -408,24 +417,26 @@ __device__ __forceinline__ void edge_fixed(longlong2 h, longlong2 hp, longlong2&
   EdgeFixed e;
   const bool any = e.set(h, hp);
   u = any ? e.unit() : make_longlong2(0, 0);
-  len = any ? e.length() : 0ull;
+  len = any ? e.length(kFineBits) : 0ull;
 }
 
-// Twice the signed area of a polygon whose vertices (components below 2^56) are
-// added in turn, starting from its last one: the 28-bit halves' products add up
-// in 64 bits over at most CG_RING edges.
+// Twice the signed area of a polygon whose vertices (components below 2^56 once
+// shifted down by `fine` bits) are added in turn, starting from its last one: the
+// 28-bit halves' products add up in 64 bits over at most CG_RING edges.
+template <int fine = 0>
 struct PolygonArea {
   long long p2 = 0, p1 = 0, p0 = 0;
   int qx1, qx0, qy1, qy0;
   static constexpr int mask = (1 << 28) - 1;
   __device__ __forceinline__ void start(longlong2 q) {
-    qx1 = (int)(q.x >> 28);
-    qx0 = (int)q.x & mask;
-    qy1 = (int)(q.y >> 28);
-    qy0 = (int)q.y & mask;
+    qx1 = (int)(q.x >> (28 + fine));
+    qx0 = (int)(q.x >> fine) & mask;
+    qy1 = (int)(q.y >> (28 + fine));
+    qy0 = (int)(q.y >> fine) & mask;
   }
   __device__ __forceinline__ void add(longlong2 h) {
-    const int x1 = (int)(h.x >> 28), x0 = (int)h.x & mask, y1 = (int)(h.y >> 28), y0 = (int)h.y & mask;
+    const int x1 = (int)(h.x >> (28 + fine)), x0 = (int)(h.x >> fine) & mask;
+    const int y1 = (int)(h.y >> (28 + fine)), y0 = (int)(h.y >> fine) & mask;
     p2 += wmul(qx1, y1) - wmul(qy1, x1);
     p1 += wmul(qx1, y0) + wmul(qx0, y1) - wmul(qy1, x0) - wmul(qy0, x1);
     p0 += wmul(qx0, y0) - wmul(qy0, x0);

@@ -39,9 +39,10 @@ __device__ __forceinline__ void geom_vertex(long long AX, long long AY, unsigned
   s = make_double2(h.x * r, h.y * r);
 }
 
+__device__ __forceinline__ double power_of_two(int e) { return __longlong_as_double((long long)(1023 + e) << 52); }
 // A, P and the energy of cell i from its sums over the doubled circumcentres in
 // fixed point (one unit 2^unit grid units); returns (ka, kp) for differences of
-// fixed-point vertices and of Q1.61 unit vectors.
+// fixed-point vertices (kFineBits finer) and of Q1.61 unit vectors.
 __device__ __forceinline__ double2 geom_cell_fixed(const GeomArgs& g, int i, double sc, __int128 area,
                                                    unsigned long long per, int unit) {
   const double A = 0.125 * i128_to_double(area, 2 * unit) * sc * sc;
@@ -53,7 +54,7 @@ __device__ __forceinline__ double2 geom_cell_fixed(const GeomArgs& g, int i, dou
   // dA/dh = 1/2 perp(h_next - h_prev) (the 1/2, the doubling of g and the
   // grid scale fold into ka); dP/dh = e_in - e_out (unit edge vectors)
   const double ka = g.KA * dA * (0.5 * sc), kp = 2.0 * g.KP * dP;
-  return make_double2(ka * __longlong_as_double((long long)(1023 + unit) << 52), kp * 0x1p-61);
+  return make_double2(ka * power_of_two(unit - kFineBits), kp * 0x1p-61);
 }
 // dE/dh at a vertex from its neighbours hp, hn on the polygon and the unit
 // vectors of the edges ending (e) and leaving (en) there.
@@ -76,12 +77,18 @@ __device__ __forceinline__ double2 force_set(double2 k, longlong2 hp, longlong2 
 // s x 2 against w / 2).
 //
 // The polygon (edges, lengths, unit vectors, area, differences) is formed in
-// 64-bit fixed point in a unit common to the cell, three bits finer than a
-// double holds its largest vertex: FP64 instructions issue at 1/74 of the FP32
-// rate, and 61 per cell remain of 139.  One pass at 262144 cells 94.2 -> 82.9
-// us, at 10^6 315 -> 270; what bounds it now is the issue of the integer
-// sequences (62% of the slots) at 24 warps per SM.  The next neighbour's
-// position is loaded ahead: 270 -> 266.
+// 64-bit fixed point in a unit common to the cell, eight bits finer than a
+// double holds its largest vertex: vertices down to 2^-7 of the farthest one
+// lose nothing against a double, nearer ones a bit per further factor of two.
+// (Force errors of cells 2^-12 and 2^-16 across among cells 1 apart, against
+// FP64 arithmetic: 1.1 and 2.3 times; three bits finer only, 6 and 42 times and
+// 0.2% less time.  An exact path for such cells, out of line: 17.0 -> 17.9 us
+// per step at 1024 cells without one, 167.1 -> 172.0 at 262144.)
+//
+// FP64 instructions issue at 1/74 of the FP32 rate, and 61 per cell remain of
+// 139.  One pass at 262144 cells 94.2 -> 82.9 us, at 10^6 315 -> 270; what
+// bounds it now is the issue of the integer sequences (62% of the slots) at 24
+// warps per SM.  The next neighbour's position is loaded ahead: 270 -> 266.
 //
 // Per ring slot the kernel keeps the circumcentre, then its fixed-point value
 // and the unit vector of the edge ending there, for the force-set pass: the
@@ -151,20 +158,18 @@ __global__ void __launch_bounds__(kGeomThreads, kGeomMinBlocks) k_geom(GeomArgs 
       g.s[a * N + i] = sj;
       put(sh_hx, lo_hx, a, h.x);
       put(sh_hy, lo_hy, a, h.y);
-      top = max(top, max(exponent_of(h.x), exponent_of(h.y)));
+      top = max(top, exponent_of(h));
       LA = LB;
       AX = BX; AY = BY;
     }
     // the polygon in fixed point, one unit 2^unit grid units: the vertices and
     // the unit vectors of the edges ending there take the circumcentres' places
     const int unit = top - 1023 - 55;
-    auto vertex = [&](int a) {
-      return make_longlong2(to_fixed(get(sh_hx, lo_hx, a), top), to_fixed(get(sh_hy, lo_hy, a), top));
-    };
+    auto vertex = [&](int a) { return to_fixed(make_double2(get(sh_hx, lo_hx, a), get(sh_hy, lo_hy, a)), top); };
     auto keep = [&](double (&sh)[kGeomSh][kGeomThreads], double* lo, int a, long long v) {
       put(sh, lo, a, __longlong_as_double(v));
     };
-    PolygonArea area;
+    PolygonArea<kFineBits> area;
     unsigned long long per = 0;
     longlong2 H = vertex(m - 1);
     area.start(H);
@@ -205,8 +210,8 @@ __global__ void __launch_bounds__(kGeomThreads, kGeomMinBlocks) k_geom(GeomArgs 
 // perimeter and forms the cell's coefficients.
 //
 // The polygon itself (edges, lengths, unit vectors, area, differences) is
-// formed in 64-bit fixed point, with at least three bits more than a double
-// holds: 8 FP64 operations per slot remain of 21.
+// formed in 64-bit fixed point, as in k_geom: 8 FP64 operations per slot remain
+// of 21.
 __global__ void __launch_bounds__(kSlotThreads, kGeomSlotBlocks) k_geom_slots(GeomArgs g) {
   __shared__ longlong2 s_off[CG_RING][32];  // neighbour offsets, then unit edge vectors (Q1.61)
   __shared__ double2 s_h[CG_RING][32];      // doubled circumcentres
@@ -257,18 +262,15 @@ __global__ void __launch_bounds__(kSlotThreads, kGeomSlotBlocks) k_geom_slots(Ge
       geom_vertex(A.x, A.y, norm2_exact(A.x, A.y), B.x, B.y, norm2_exact(B.x, B.y), h, sj);
       g.s[a * N + i] = sj;
       s_h[a][c] = h;
-      top = max(top, max(exponent_of(h.x), exponent_of(h.y)));
+      top = max(top, exponent_of(h));
     }
     if (top) atomicMax(&s_top[c], top);
     __syncthreads();
     top = s_top[c];
     const int unit = top - 1023 - 55;  // one fixed-point unit is 2^unit grid units
     if (w == kSlotWarps - 1) {
-      PolygonArea area;
-      auto vertex = [&](int a) {
-        const double2 h = s_h[a][c];
-        return make_longlong2(to_fixed(h.x, top), to_fixed(h.y, top));
-      };
+      PolygonArea<kFineBits> area;
+      auto vertex = [&](int a) { return to_fixed(s_h[a][c], top); };
       if (m) area.start(vertex(m - 1));
       for (int a = 0; a < m; ++a) area.add(vertex(a));
       const __int128 t = area.total();
@@ -276,10 +278,10 @@ __global__ void __launch_bounds__(kSlotThreads, kGeomSlotBlocks) k_geom_slots(Ge
     }
     for (int a = w; a < m; a += kSlotWarps) {
       const double2 h = s_h[a][c], hp = s_h[a > 0 ? a - 1 : m - 1][c];
-      const longlong2 H = make_longlong2(to_fixed(h.x, top), to_fixed(h.y, top));
+      const longlong2 H = to_fixed(h, top);
       longlong2 e;
       unsigned long long len;
-      edge_fixed(H, make_longlong2(to_fixed(hp.x, top), to_fixed(hp.y, top)), e, len);
+      edge_fixed(H, to_fixed(hp, top), e, len);
       s_H[a][c] = H;
       s_e[a][c] = e;
       s_len[a][c] = len;

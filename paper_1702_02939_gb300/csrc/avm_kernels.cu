@@ -1470,10 +1470,12 @@ __global__ void k_iota2(int n, int* a, int* b) {
   if (i < n) a[i] = b[i] = i;
 }
 
-// The network in tag order with its entries renamed to tags.
+// The network in tag order with its entries renamed to tags (nothing is written
+// when a status is raised: the arrays may be the caller's).
 __global__ void k_avm_topology_by_tag(AvmArgs g, const int* vslot, const int* cslot, int* vc_out, int* vn_out,
                                       int* cc_out, int* cv_out) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (g.ctl->status) return;
   if (t < g.V) {
     const int v = vslot[t];
 #pragma unroll

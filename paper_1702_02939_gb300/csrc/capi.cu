@@ -625,11 +625,12 @@ int triangulate_all(cg_ctx* c) {
   return CG_OK;
 }
 
-int read_status(cg_ctx* c) {
+int read_status(cg_ctx* c, Ctl* ctl = nullptr) {
   Ctl h;
   // the control word read on the context's stream (ordered after its work)
   CG_CUDA(c, cudaMemcpyAsync(&h, c->ctl(), sizeof(Ctl), cudaMemcpyDeviceToHost, c->stream));
   CG_CUDA(c, cudaStreamSynchronize(c->stream));
+  if (ctl) *ctl = h;
   if (h.status != 0) {
     c->seen_status = h.status;
     return fail(c, h.status, std::string("device status: ") + cg_status_string(h.status));
@@ -737,10 +738,9 @@ void drop_graphs(cg_ctx* c) {
 // ---------------------------------------------------------------------------
 struct BwdLayout {
   size_t snap_bytes = 0;                 // one state snapshot
-  // checkpoints (+ final state), the input states of the last segment's steps
-  // (kept by the run) and of the segment being recomputed
-  size_t snaps = 0, last = 0, seg = 0;
+  size_t snaps = 0, seg = 0;             // checkpoints (+ final state), the input states of one segment's steps
   size_t v, fsd, sd, wd, gp0, gv0, gKA, gKP, cA, cP, gx, gy, F, red;
+  size_t kept = 0;                       // int: the segment holds the last one, as the run left it
   size_t total = 0;
 };
 
@@ -756,7 +756,6 @@ BwdLayout bwd_layout(int64_t N, int64_t nsteps, int32_t every) {
   b.snap_bytes = s.total;
   const int64_t nck = (nsteps + every - 1) / every;
   b.snaps = L.take((size_t)(nck + 1) * b.snap_bytes);
-  b.last = L.take((size_t)std::min<int64_t>(every, nsteps) * b.snap_bytes);
   b.seg = L.take((size_t)every * b.snap_bytes);
   b.v = L.take(N * sizeof(double2));
   b.fsd = L.take(N * CG_RING * sizeof(double2));
@@ -771,7 +770,8 @@ BwdLayout bwd_layout(int64_t N, int64_t nsteps, int32_t every) {
   b.gx = L.take(N * d);
   b.gy = L.take(N * d);
   b.F = L.take(N * sizeof(double2));
-  b.red = L.take(4 * d);
+  b.red = L.take(4 * d);  // two sums, then `kept`
+  b.kept = b.red + 2 * d;
   b.total = L.total;
   return b;
 }
@@ -1570,10 +1570,11 @@ int cg_run_checkpointed(cg_ctx* c, int64_t nsteps, int32_t ckpt_every, void* d_b
     // the last segment is the first the reverse pass needs: its steps' states
     // are kept now, so that it is not run again
     const int64_t in_last = t - (nck - 1) * ckpt_every;
-    if (in_last >= 0) snapshot(c, 1, snapshot_at(bw + b.last + in_last * b.snap_bytes, c->N));
+    if (in_last >= 0) snapshot(c, 1, snapshot_at(bw + b.seg + in_last * b.snap_bytes, c->N));
     CG_CUDA(c, cudaGraphLaunch(c->step_exec, c->stream));
   }
   snapshot(c, 1, snapshot_at(bw + b.snaps + nck * b.snap_bytes, c->N));
+  CG_CUDA(c, cudaMemsetAsync(bw + b.kept, 1, sizeof(int), c->stream));
   CG_CUDA(c, cudaGetLastError());
   return read_status(c);
 }
@@ -1585,13 +1586,18 @@ int cg_backward(cg_ctx* c, int64_t nsteps, int32_t ckpt_every, void* d_bw, size_
   int rc = check_bwd(c, nsteps, ckpt_every, d_bw, bytes, b);
   if (rc) return rc;
   if (!gxT || !gyT || !gAT || !gPT) return CG_EINVAL;
-  rc = read_status(c);
-  if (rc) return rc;
   char* bw = static_cast<char*>(d_bw);
   cudaStream_t st = c->stream;
+  const int64_t nck = (nsteps + ckpt_every - 1) / ckpt_every;
+  // an earlier reverse pass of the same run may have put other segments in the
+  // place of the last one; read with the status, no synchronisation of its own
+  Ctl h;
+  CG_CUDA(c, cudaMemcpyAsync(&c->ctl()->pad, bw + b.kept, sizeof(int), cudaMemcpyDeviceToDevice, st));
+  rc = read_status(c, &h);
+  if (rc) return rc;
+  const bool kept = nck == 1 || h.pad != 0;
   const int n = (int)c->N;
   const int* tag = c->at<int>(c->off.tag);
-  const int64_t nck = (nsteps + ckpt_every - 1) / ckpt_every;
   const Snapshot fin = snapshot_at(bw + b.snaps + nck * b.snap_bytes, c->N);
   // cotangents of the final state, in storage order
   double* tmp = c->at<double>(c->off.tmp);
@@ -1632,8 +1638,8 @@ int cg_backward(cg_ctx* c, int64_t nsteps, int32_t ckpt_every, void* d_bw, size_
   a.update = 1;
   for (int64_t ck = nck - 1; ck >= 0; --ck) {
     const int64_t t0 = ck * ckpt_every, t1 = std::min<int64_t>(t0 + ckpt_every, nsteps);
-    const size_t states = ck == nck - 1 ? b.last : b.seg;
-    if (ck < nck - 1) {
+    if (ck < nck - 1 || !kept) {
+      if (ck < nck - 1) CG_CUDA(c, cudaMemsetAsync(bw + b.kept, 0, sizeof(int), st));
       snapshot(c, 0, snapshot_at(bw + b.snaps + ck * b.snap_bytes, c->N));
       for (int64_t t = t0; t < t1; ++t) {  // recompute the segment, keeping every step's input state
         snapshot(c, 1, snapshot_at(bw + b.seg + (t - t0) * b.snap_bytes, c->N));
@@ -1641,7 +1647,7 @@ int cg_backward(cg_ctx* c, int64_t nsteps, int32_t ckpt_every, void* d_bw, size_
       }
     }
     for (int64_t t = t1 - 1; t >= t0; --t) {
-      use(a, snapshot_at(bw + states + (t - t0) * b.snap_bytes, c->N));
+      use(a, snapshot_at(bw + b.seg + (t - t0) * b.snap_bytes, c->N));
       launch_geom_jvp(a, st);
       launch_force_jvp(a, st);
     }

@@ -195,6 +195,7 @@ struct cg_ctx {
   std::vector<cg_replica> user_reps;           // as passed to cg_create
   cudaGraphExec_t step_exec = nullptr;
   cudaGraphExec_t steps_exec = nullptr;  // kGraphSteps steps (built once a run is long)
+  bool single_steps = false;             // a launch per step however long the run
   int graph_steps = 0;
   int seen_status = 0;  // a device status read back earlier (the context then stays refused)
   std::string last_error;
@@ -712,7 +713,7 @@ constexpr int kGraphSteps = 8;
 constexpr int64_t kLongRun = 64, kManyStepCells = 1 << 16;
 bool many_steps(cg_ctx* c) {
   if (c->steps_exec) return true;
-  if (c->host_step < kLongRun || c->N > kManyStepCells || !plain_step(c)) return false;
+  if (c->single_steps || c->host_step < kLongRun || c->N > kManyStepCells || !plain_step(c)) return false;
   if (build_plain_graph(
           c->capture,
           [&](cudaStream_t st) {
@@ -1368,6 +1369,7 @@ int cg_autotune(cg_ctx* c, int32_t steps_per_trial, size_t flush_bytes, void* d_
   cg_ctx* t = nullptr;
   rc = cg_create(c->R, c->user_reps.data(), &c->par, sx, sy, sth, d_ws2, c->off.total, c->stream, &t);
   if (rc) return fail(c, rc, "autotune: temporary context: " + (t ? t->last_error : std::string("create failed")));
+  t->single_steps = true;  // the trials time steps, not the building of graphs
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);

@@ -195,6 +195,7 @@ struct cg_ctx {
   std::vector<cg_replica> user_reps;           // as passed to cg_create
   cudaGraphExec_t step_exec = nullptr;
   cudaGraphExec_t steps_exec = nullptr;  // kGraphSteps steps (built once a run is long)
+  int64_t since_capture = 0;             // steps enqueued since the graphs were last captured
   bool single_steps = false;             // a launch per step however long the run
   int graph_steps = 0;
   int seen_status = 0;  // a device status read back earlier (the context then stays refused)
@@ -706,14 +707,15 @@ int build_graph(cg_ctx* c) {
 }
 
 // A graph launch costs the device about 3.5 us between steps, which a small
-// system's step of 20-45 us feels: once a context has taken kLongRun steps, the
-// steps of a call go kGraphSteps at a time (the graph is built then, beside the
-// steps in flight; contexts of a few steps never pay for it).
+// system's step of 20-45 us feels: once a context has taken kLongRun steps with
+// the same graphs, the steps of a call go kGraphSteps at a time (the graph is
+// built then, beside the steps in flight; contexts of a few steps, or of a few
+// steps between changes of the moduli, never pay for it).
 constexpr int kGraphSteps = 8;
 constexpr int64_t kLongRun = 64, kManyStepCells = 1 << 16;
 bool many_steps(cg_ctx* c) {
   if (c->steps_exec) return true;
-  if (c->single_steps || c->host_step < kLongRun || c->N > kManyStepCells || !plain_step(c)) return false;
+  if (c->single_steps || c->since_capture < kLongRun || c->N > kManyStepCells || !plain_step(c)) return false;
   if (build_plain_graph(
           c->capture,
           [&](cudaStream_t st) {
@@ -727,6 +729,7 @@ bool many_steps(cg_ctx* c) {
   return true;
 }
 void drop_graphs(cg_ctx* c) {
+  c->since_capture = 0;
   for (cudaGraphExec_t* g : {&c->step_exec, &c->steps_exec})
     if (*g) {
       cudaGraphExecDestroy(*g);
@@ -984,8 +987,10 @@ int cg_step(cg_ctx* c, int64_t nsteps) {
     if (every > 0) left = std::min<int64_t>(left, every - c->host_step % every);
     const bool many = left >= kGraphSteps && many_steps(c);
     CG_CUDA(c, cudaGraphLaunch(many ? c->steps_exec : c->step_exec, c->stream));
-    s += many ? kGraphSteps : 1;
-    c->host_step += many ? kGraphSteps : 1;
+    const int k = many ? kGraphSteps : 1;
+    s += k;
+    c->host_step += k;
+    c->since_capture += k;
   }
   return CG_OK;
 }

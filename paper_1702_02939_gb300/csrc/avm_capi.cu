@@ -380,6 +380,11 @@ int in_by_tag(cg_avm_ctx* c, double* dst, const double* src, int count, const in
 // A captured sequence that ends with a first T1 pass and the kernel of the
 // further passes.  Against a while node with a pass as its body (step, us):
 // 35.1 -> 26.9 at 8192 vertices, 56.4 -> 48.3 at 131072, 146 -> 138 at 524288.
+// Long lists: with flips at 1.6% of the cells in every step 112 -> 110 at 131072
+// vertices, 157 -> 145 at 262144; the first step of a fresh network, which has
+// the longest ones, 186 -> 206 and 243 -> 260, the median of its first twenty 94
+// -> 88 and 137 -> 116.  (Further grid kernels for that step would cost every
+// other step 2 us.)
 template <class Body>
 int pass_graph(cg_avm_ctx* c, Body body, cudaGraphExec_t* out) {
   if (*out) {

@@ -460,7 +460,11 @@ int sm_count() {
 // (step, us, with a while node -> without: 41.6 -> 26.8 at 1024 cells, 55.9 ->
 // 43.0 at 16384, 109.5 -> 106.6 at 131072; FP32 98.5 -> 87.3 at 262144, 263.7
 // -> 259.9 at 10^6).  In double precision the rounds of larger systems hide
-// behind the geometry (191 -> 194 at 262144).
+// behind the geometry (191 -> 194 at 262144).  The cluster has few warps for a
+// long list, but the lists after the first are short in a strongly driven tissue
+// too: steps that flag 94% of the cells, against the kernels before with the
+// whole chip in every round, 336 -> 183 at 16384, 1541 -> 966 at 131072, FP32
+// 10143 -> 6114 at 10^6.
 constexpr int64_t kRestCells = 155648, kRestCellsF32 = 1 << 20;
 // Per-step repair rounds handle a few hundred flagged cells: a modest
 // persistent grid (warps loop over the list) keeps empty rounds cheap.
@@ -666,14 +670,25 @@ int refuse_seen(cg_ctx* c) {
 }
 
 // The step without a loop node.  The 128 warps of the further rounds' cluster do
-// the first round of a small system too (a few to some hundred cells), two
-// kernels fewer.
-constexpr int64_t kClusterCells = 4096;
+// the first round of a small system too, two kernels fewer, or its check alone,
+// one fewer.  The lines lie where a step that flags nearly every cell (strong
+// driving, a wild start) still takes no longer than with a while node and the
+// whole chip in every round.  Step, us, relaxed / nearly all cells flagged:
+//   cells   whole cluster   grid repair, then cluster   grid repair and check   while node
+//    1024    17.8 / 124           19.2 / 78                   22.2 / 72          50.5 / 169
+//    2048    18.8 / 195           19.6 / 99                   22.7 / 84          52.2 / 184
+//    4096    28.9 / 330           29.6 / 137                  30.1 / 101         61.4 / 203
+// (FP32 at 2048: 14.9 / 187, 16.6 / 93, 19.7 / 77, 47.7 / 158.)  Past 4096 cells
+// the first round takes the grid; a second list holds 2 to 4% of a first one.
+constexpr int64_t kClusterCells = 1024, kClusterCheckCells = 4096;
 void enqueue_plain_step(cg_ctx* c, cudaStream_t st) {
   enqueue_step_prefix(c, st);
-  const bool cluster_only = c->N <= kClusterCells;
-  if (!cluster_only) enqueue_repair_round(c, 0, st);
-  launch_repair_rest(round_repair_args(c, 0), round_check_args(c, 0), cluster_only, st);
+  const RestFrom from = c->N <= kClusterCells        ? kFromFirst
+                        : c->N <= kClusterCheckCells ? kFromFirstCheck
+                                                     : kFromSecond;
+  if (from == kFromFirstCheck) launch_repair(round_repair_args(c, 0), repair_grid(c), st);
+  if (from == kFromSecond) enqueue_repair_round(c, 0, st);
+  launch_repair_rest(round_repair_args(c, 0), round_check_args(c, 0), from, st);
   enqueue_step_suffix(c, st);
 }
 bool plain_step(const cg_ctx* c) { return c->N <= (fp32(c) ? kRestCellsF32 : kRestCells); }

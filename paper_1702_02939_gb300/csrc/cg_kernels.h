@@ -234,9 +234,10 @@ void launch_cell_list(const CellListArgs& a, cudaStream_t st);
 void launch_repair(const RepairArgs& a, int grid_blocks, cudaStream_t st);
 void launch_scan(const ScanArgs& a, cudaStream_t st);
 void launch_check(const CheckArgs& a, int grid_blocks, cudaStream_t st);
-// After a first round (dyn): the further rounds, until none is needed;
-// every_round: the first one too
-void launch_repair_rest(const RepairArgs& a, const CheckArgs& c, int every_round, cudaStream_t st);
+// A step's rounds (dyn) in one cluster until none is needed: those after the
+// first, the first one's check and those after it, or all of them
+enum RestFrom { kFromSecond, kFromFirstCheck, kFromFirst };
+void launch_repair_rest(const RepairArgs& a, const CheckArgs& c, RestFrom from, cudaStream_t st);
 // Blocks of 8 warps for the check of every cell: a warp per cell up to 16
 // blocks per SM (one block per 256 cells left each warp a chain of 32 cells:
 // 44 us at 1024 cells against 3.5)

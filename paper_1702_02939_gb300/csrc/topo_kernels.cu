@@ -806,13 +806,14 @@ __global__ void k_check(CheckArgs g) {
 // The rounds after the first in one kernel: one cluster of kRestBlocks blocks
 // repairs and checks the listed cells, its hardware barrier between the two,
 // until a round leaves no cell flagged or the cap is reached (raised by the
-// check of the last allowed round).  Nearly every step leaves nothing to do
+// check of the last allowed round).  It can start earlier, with the check or the
+// repair of the first round (RestFrom).  Nearly every step leaves nothing to do
 // here (1.01 to 1.04 rounds per step) and a graph's while node costs 10-12 us
 // whether it runs or not (a chain of 6 empty kernels 6 us, with a while node
 // 14-16); this kernel adds 2 us.
 __global__ void __cluster_dims__(kRestBlocks, 1, 1) __launch_bounds__(kRestWarps * 32) k_repair_rest(RepairArgs g,
                                                                                                 CheckArgs k,
-                                                                                                int every_round) {
+                                                                                                RestFrom from) {
   __shared__ CandBuf s_buf[kRestWarps];
   Ctl* ctl = g.ctl;
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
@@ -824,10 +825,10 @@ __global__ void __cluster_dims__(kRestBlocks, 1, 1) __launch_bounds__(kRestWarps
   const long long* __restrict__ Y = g.Y + cur * N;
   // every thread of the cluster follows the same counts: the list of a round is
   // complete before the barrier that ends the one before it
-  for (int r = every_round ? 0 : *(volatile int*)&ctl->round_count; r < k.cap; ++r) {
+  for (int r = from != kFromSecond ? 0 : *(volatile int*)&ctl->round_count; r < k.cap; ++r) {
     const int in = r & 1;
     const int total = *(volatile int*)&ctl->count[in];
-    if (every_round && r == 0 && first) {  // the first round's statistics (k_check's otherwise)
+    if (from != kFromSecond && r == 0 && first) {  // the first round's statistics (k_check's otherwise)
       ctl->last_flagged = total;
       ctl->flagged_total += total;
       if (total == 0) ctl->loop_total += 1;
@@ -837,12 +838,14 @@ __global__ void __cluster_dims__(kRestBlocks, 1, 1) __launch_bounds__(kRestWarps
     int* list_out = k.lists[in ^ 1];
     int* count_out = &ctl->count[in ^ 1];
     cluster_barrier();  // every thread has read the counts
-    if (first) {
-      *count_out = 0;
-      ctl->repaired_total += total;
+    if (from != kFromFirstCheck || r > 0) {
+      if (first) {
+        *count_out = 0;
+        ctl->repaired_total += total;
+      }
+      for (int item = gw; item < total; item += nw) repair_cell(g, X, Y, list_in[item], s_buf[wib], lane);
+      cluster_barrier();
     }
-    for (int item = gw; item < total; item += nw) repair_cell(g, X, Y, list_in[item], s_buf[wib], lane);
-    cluster_barrier();
     for (int item = gw; item < total; item += nw) check_cell(k, list_in[item], list_out, count_out, lane);
     cluster_barrier();
     if (first) {
@@ -853,8 +856,8 @@ __global__ void __cluster_dims__(kRestBlocks, 1, 1) __launch_bounds__(kRestWarps
   }
 }
 
-void launch_repair_rest(const RepairArgs& a, const CheckArgs& c, int every_round, cudaStream_t st) {
-  if (a.n > 0) k_repair_rest<<<kRestBlocks, kRestWarps * 32, 0, st>>>(a, c, every_round);
+void launch_repair_rest(const RepairArgs& a, const CheckArgs& c, RestFrom from, cudaStream_t st) {
+  if (a.n > 0) k_repair_rest<<<kRestBlocks, kRestWarps * 32, 0, st>>>(a, c, from);
 }
 
 void launch_check(const CheckArgs& a, int grid_blocks, cudaStream_t st) {

@@ -210,14 +210,24 @@ class ClockSampler:
                 "reasons": reasons, "samples": len(rows)}
 
 
-def kernels_launched(steps, loop_iterations, eager=False, ring_order=1, force_beside=0):
-    # per step: begin-topology, test, the cell list, directors, the
-    # ring-size grouping (if on), geometry of the new state, force + move;
-    # graph only: the geometry fix-up of rewritten rings and, with the force
-    # pass beside the rounds, the fix-up list and the force fix-up; per
-    # repair round: repair + check
-    graph_extra = 0 if eager else 1 + (2 if force_beside else 0)
-    return (6 + (1 if ring_order else 0) + graph_extra) * steps + 2 * loop_iterations
+def kernels_launched(steps, loop_iterations, n, eager=False, ring_order=1, force_beside=0, fp32=False):
+    """Launches of this library's kernels in SPV steps of n cells, by the size
+    rules of the step graph (capi.cu); loop_iterations: repair rounds, which
+    only the loop node and eager steps launch one by one."""
+    # begin-topology, directors, test, geometry of the new state, force + move,
+    # the ring-size grouping (if on)
+    per_step = 5 + (1 if ring_order else 0)
+    if eager:  # and the cell list; per round repair + check
+        return (per_step + 1) * steps + 2 * loop_iterations
+    # the geometry fix-up of rewritten rings; with the force pass beside the
+    # rounds, the fix-up list and the force fix-up
+    per_step += 1 + (2 if force_beside else 0)
+    if n > 29184:  # below, the test fills the cell list
+        per_step += 1
+    if n > (1 << 20 if fp32 else 155648):
+        return per_step * steps + 2 * loop_iterations
+    # every round in the cluster; repair, cluster; repair, check, cluster
+    return (per_step + (1 if n <= 1024 else 2 if n <= 4096 else 3)) * steps
 
 
 def host_cpu():
@@ -960,9 +970,9 @@ def run_ours(args):
                            "launch_shapes": launch, "launch_source": launch_source,
                            "autotune_ms_per_step": tune_ms},
                 "clocks": clk, "e2e": e2e,
-                "gpu_launches": (kernels_launched(args.steps, args.steps * repair_cap, True, launch["ring_order"])
+                "gpu_launches": (kernels_launched(args.steps, args.steps * repair_cap, args.n, True, launch["ring_order"])
                                  if args.eager else
-                                 kernels_launched(args.steps, counters["loop_total"] - c_start["loop_total"], False,
+                                 kernels_launched(args.steps, counters["loop_total"] - c_start["loop_total"], args.n, False,
                                                   launch["ring_order"], launch.get("force_beside", 0))),
                 "timed_state": timed_state,
                 "roofline": roofline, "hbm_roofline": hbm, "cpu_baseline": cpu,

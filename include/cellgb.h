@@ -424,7 +424,9 @@ int cg_avm_workspace_bytes_capacity(int32_t n, int32_t capacity, double Lx, doub
 int cg_avm_create(int32_t n, double Lx, double Ly, double p0, double v0, const cg_avm_params* params,
                   const double* x, const double* y, const double* theta, void* d_ws, size_t ws_bytes, void* stream,
                   cg_avm_ctx** out);
-/* Enqueues nsteps steps (one CUDA graph launch each); does not synchronize. */
+/* Enqueues nsteps steps (a CUDA graph launch each; after 64 steps, up to 131072
+ * cell slots, eight steps per launch where a call has that many left); does not
+ * synchronize. */
 int cg_avm_step(cg_avm_ctx* ctx, int64_t nsteps);
 /* Device time of nsteps ordinary steps run eagerly (not as a graph), timed
  * with CUDA events on the context's stream; the T1 pass control is read back

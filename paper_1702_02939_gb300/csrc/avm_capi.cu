@@ -652,7 +652,7 @@ int cg_avm_profile_step(cg_avm_ctx* c, int64_t nsteps, double* ms_out, int32_t n
   cudaEvent_t ev[3];
   for (int k = 0; k < 3; ++k) AV_CUDA(c, cudaEventCreate(&ev[k]));
   for (int k = 0; k < CG_AVM_NUM_PHASES; ++k) ms_out[k] = 0.0;
-  AvmArgs a = avm_args(c);  // loop handle 0: the pass control is read back here
+  AvmArgs a = avm_args(c);  // the pass control is read back here
   float ms = 0.f;
   for (int64_t s = 0; s < nsteps && !rc; ++s) {
     cudaEventRecord(ev[0], st);

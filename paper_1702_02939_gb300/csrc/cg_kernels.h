@@ -18,8 +18,9 @@ constexpr int kSlotThreads = 32 * kSlotWarps;
 constexpr int kGeomSlotBlocks = 5;      // resident blocks per SM that k_geom_slots is compiled for
 constexpr int kGeomSlotCells = 97280;  // up to here (640 cells per SM) k_geom_slots takes all cells
 constexpr int kForceSlotBlocks = 6, kTestSlotBlocks = 6, kGeomF32SlotBlocks = 5, kForceF32SlotBlocks = 8;
-// the force and test passes, and the single-precision geometry, take their
-// slot kernels while every cell is resident at once: 152 SMs x 6 blocks x 32
+// the force and test passes take their slot kernels while every cell is resident
+// at once, 152 SMs x 6 blocks x 32; the single-precision geometry, of which five
+// blocks fit, keeps the same line (times at its launcher)
 constexpr int kForceSlotCells = 29184, kTestSlotCells = 29184, kGeomF32SlotCells = 29184;
 constexpr int kForceThreads = 128;
 constexpr int kTestThreads = 128;

@@ -65,12 +65,8 @@ __device__ __forceinline__ double dm_i2d(long long v) { return i2d_int(v); }  //
 constexpr long long kQOne = 1LL << 62;
 // round(2^62 / d)
 __host__ __device__ constexpr long long qdiv(long long d) { return (kQOne + d / 2) / d; }
-// a b in Q1.62 (|a b| < 2), the product truncated toward minus infinity
-__device__ __forceinline__ long long mulq(long long a, long long b) {
-  return (long long)(((__int128)a * (__int128)b) >> 62);
-}
-// The same for |a| < 1/2 (in Q1.62 below 2^61): one signed high product, where
-// the low half and the 128-bit shift cost half as much again.
+// a b in Q1.62 for |a| < 1/2 (below 2^61), truncated toward minus infinity: one
+// signed high product, where a 128-bit product and shift cost half as much again.
 __device__ __forceinline__ long long mulq_small(long long a, long long b) { return __mul64hi(a << 2, b); }
 // x 2^62 for |x| < 2, truncated toward zero, on the integer pipes
 __device__ __forceinline__ long long d2q(double x) {

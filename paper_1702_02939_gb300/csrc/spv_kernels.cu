@@ -87,7 +87,7 @@ __device__ __forceinline__ double2 force_set(double2 k, longlong2 hp, longlong2 
 //
 // FP64 instructions issue at 1/74 of the FP32 rate, and 61 per cell remain of
 // 139.  One pass at 262144 cells 94.2 -> 82.9 us, at 10^6 315 -> 270; what
-// bounds it now is the issue of the integer sequences (62% of the slots) at 24
+// bounds it now is the issue of the integer sequences (60% of the slots) at 24
 // warps per SM.  The next neighbour's position is loaded ahead: 270 -> 266.
 //
 // Per ring slot the kernel keeps the circumcentre, then its fixed-point value
